@@ -13,6 +13,7 @@ namespace trig {
 // Limits of this implementation.
 constexpr uint32_t kMaxPmt = 4096;          // PMTs per detector
 constexpr uint32_t kSmemDtMaxPmt = 96;      // dt table lives in shared memory up to this P
+constexpr uint32_t kDtRow = 256;            // bytes of a dt row in shared memory (128 PMTs)
 constexpr uint32_t kWideMinPmt = 129;       // from this P on, slices are staged from a bucketed copy
 constexpr uint32_t kBktChunk = 1024;        // buckets per block of the bucket scan
 // A tile plus its halos spans less than 2^20 ns, so a hit's time within the

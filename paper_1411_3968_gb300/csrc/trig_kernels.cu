@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "trig_internal.h"
@@ -700,17 +701,17 @@ struct ItemInfo {
     uint32_t span;      // length of the staged time range (ns)
 };
 
-// Shared memory of the tile kernel, in this order: the staging buffers of
-// CAP 16-byte records (two, or one for the 2048-hit tile: its tile pass
-// hands the buffer back once it has read it, so the next tile's copy
-// overlaps the rest of the pass, and two blocks of it then fit on an SM);
-// the tile's packed keys in merged order (+16 bytes: four end keys that the
-// causal count's 16-byte loads may read past the last key); the keys in
-// bucket order (reused for the seed rounds' lists, then the seed list and
-// seed counts); the charges in bucket order and in merged order; the floor
-// of each merged key; the bucket offsets; the seed mask; the PMT tables
-// (floor, row maximum of dt, and dt itself when the detector's table fits).
-template <int CAP>
+// Shared memory of the tile kernel's sorted builds (EXT), in this order: the
+// staging buffers of CAP 16-byte records (two, or one for the 2048-hit tile:
+// its tile pass hands the buffer back once it has read it, so the next
+// tile's copy overlaps the rest of the pass, and two blocks of it then fit
+// on an SM); the tile's packed keys in merged order (+16 bytes: four end keys
+// that the causal count's 16-byte loads may read past the last key); the
+// keys in bucket order (reused for the seed rounds' lists, then the seed
+// list and seed counts); the charges in bucket order and in merged order;
+// the floor of each merged key; the bucket offsets; the seed mask; the PMT
+// tables (floor, row maximum of dt).
+template <int CAP, bool EXT>
 struct TileLayout {
     // time buckets of the in-tile merge, at most: two per hit slot up to
     // 2048 hits (shorter chains in the floor-coincidence rounds), one at 4096
@@ -732,24 +733,48 @@ struct TileLayout {
     static constexpr size_t oMask = oCnt + kCnt;
     static constexpr size_t oTab = (oMask + kMask + 15) & ~(size_t)15;
     static_assert(oCnt % 16 == 0, "the bucket counts are read as 16-byte vectors");
-    static size_t bytes(uint32_t P, bool smem_dt)
+    static size_t bytes(uint32_t P, bool)
     {
-        size_t b = oTab;
-        b += 2 * (size_t)((P + 7) & ~7u) * 2;              // floor + dmax_row
-        if (smem_dt) b += (size_t)P * P * 2;
-        return (b + 127) & ~(size_t)127;
+        return (oTab + 2 * (size_t)((P + 7) & ~7u) * 2 + 127) & ~(size_t)127;      // floor + dmax_row
     }
 };
 
-// Dynamic shared memory of the tile kernel (layout TileLayout<CAP>).
-extern __shared__ __align__(128) unsigned char g_tile_smem[];
+// Shared memory of the default builds: one staging buffer (handed back after
+// its first read); the keys in bucket order (+16 bytes of end keys); the
+// floor cells, two bits each, whose place the seed list takes; the candidate
+// list (position and charge), whose place the seeds' counts take; the bucket
+// offsets; the mask of fired positions; the dt rows (kDtRow bytes each, 256-byte
+// aligned) when the detector's table fits; the PMT tables.
+template <int CAP>
+struct TileLayout<CAP, false> {
+    static constexpr int NBK = CAP;                        // time buckets
+    static constexpr uint32_t NS = 1;
+    static constexpr uint32_t kCells = 16u * CAP;          // floor cells
+    static constexpr size_t kStage = (size_t)CAP * 16;
+    static constexpr size_t oPk = kStage;
+    static constexpr size_t oCell = oPk + (size_t)CAP * 4 + 16;
+    static constexpr size_t oCand = oCell + (size_t)CAP * 4;
+    static constexpr size_t oCnt = oCand + (size_t)CAP * 4;
+    static constexpr size_t oMask = oCnt + (size_t)(NBK + 1) * 4;
+    static_assert(kCells / 4 == (size_t)CAP * 4, "the cells and the seed list share their place");
+    static constexpr size_t oDt = (oMask + (size_t)(CAP / 32) * 4 + kDtRow - 1) & ~(size_t)(kDtRow - 1);
+    static_assert(oCnt % 16 == 0 && oCell % 16 == 0, "cleared and scanned as 16-byte vectors");
+    __host__ __device__ static size_t tab(uint32_t P, bool smem_dt) { return oDt + (smem_dt ? (size_t)P * kDtRow : 0); }
+    static size_t bytes(uint32_t P, bool smem_dt)
+    {
+        return (tab(P, smem_dt) + 2 * (size_t)((P + 7) & ~7u) * 2 + 127) & ~(size_t)127;
+    }
+};
 
-// The tile kernel's shared-memory regions sit at fixed offsets, so their
+// Dynamic shared memory of the tile kernel (layout TileLayout<CAP, EXT>).
+extern __shared__ __align__(256) unsigned char g_tile_smem[];
+
+// The sorted builds' shared-memory regions sit at fixed offsets, so their
 // addresses are recomputed where used instead of living in registers
 // through every phase; only the PMT-table stride depends on the launch.
 template <int CAP>
-struct TileCtx {
-    using L = TileLayout<CAP>;
+struct SortCtx {
+    using L = TileLayout<CAP, true>;
     uint32_t P;             // PMTs of the loaded slice
     uint32_t pp;            // PMT table stride: the launch's max_pmt rounded up to 8
     const uint16_t *dt_g;   // the loaded slice's dt table in global memory
@@ -767,13 +792,11 @@ struct TileCtx {
     __device__ __forceinline__ uint16_t *chg_b() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oChgB); }
     __device__ __forceinline__ uint16_t *chg_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oChgS); }
     __device__ __forceinline__ uint16_t *flk() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oFlk); }
-    // per-warp lists of the seed rounds (the bucket-order key region, free then)
-    __device__ __forceinline__ uint16_t *live() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oPkB); }
     __device__ __forceinline__ uint32_t *cnt() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCnt); }
     __device__ __forceinline__ uint32_t *mask() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oMask); }
-    // warp w's 4096-bit PMT set of the distinct count above 128 PMTs (extended
-    // builds: the bucket-order charges and the floor keys are no longer read
-    // by then; each region holds CAP / 256 sets)
+    // warp w's 4096-bit PMT set of the distinct count above 128 PMTs (the
+    // bucket-order charges and the floor keys are no longer read by then;
+    // each region holds CAP / 256 sets)
     __device__ __forceinline__ uint32_t *pmt_set(uint32_t w) const
     {
         constexpr uint32_t per = (uint32_t)CAP / 256;
@@ -782,23 +805,47 @@ struct TileCtx {
     }
     __device__ __forceinline__ uint16_t *floor_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oTab); }
     __device__ __forceinline__ uint16_t *dmax_s() const { return floor_s() + pp; }
-    __device__ __forceinline__ uint16_t *dt_s() const { return floor_s() + 2 * (size_t)pp; }
+};
+
+// The same for the default builds.  NARROW: at most 128 PMTs in the batch
+// and every dt table in shared memory.
+template <int CAP, bool NARROW>
+struct TileCtx {
+    using L = TileLayout<CAP, false>;
+    uint32_t P;             // PMTs of the loaded slice
+    uint32_t tab;           // offset of the PMT tables
+    uint32_t pp;            // their stride
+    const uint16_t *dt_g;   // the loaded slice's dt table in global memory
+    __device__ __forceinline__ uint64_t *stage() const { return reinterpret_cast<uint64_t *>(g_tile_smem); }
+    __device__ __forceinline__ uint32_t *pk() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oPk); }
+    __device__ __forceinline__ uint32_t *seeds() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCell); }
+    __device__ __forceinline__ uint32_t *cand() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCand); }
+    __device__ __forceinline__ uint16_t *counts() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oCand); }
+    __device__ __forceinline__ uint32_t *cnt() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCnt); }
+    __device__ __forceinline__ uint32_t *cells() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCell); }
+    __device__ __forceinline__ uint32_t *mask() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oMask); }
+    __device__ __forceinline__ uint16_t *dt_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oDt); }
+    __device__ __forceinline__ uint16_t *floor_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + tab); }
+    __device__ __forceinline__ uint16_t *dmax_s() const { return floor_s() + pp; }
+    // Packed key: time within the staged range (below 2^20 ns) above the PMT.
+    // With at most 128 PMTs the PMT is kept doubled in eight bits, its byte
+    // offset in a dt row; else in twelve bits.
+    static constexpr uint32_t kShift = NARROW ? 8 : 12;
+    static constexpr uint32_t kPmtMask = (1u << kShift) - 1u;
+    static __device__ __forceinline__ uint32_t key(uint32_t t, uint32_t pmt)
+    {
+        return (t << kShift) | (NARROW ? pmt << 1 : pmt);
+    }
+    static __device__ __forceinline__ uint32_t key_t(uint32_t k) { return k >> kShift; }
+    static __device__ __forceinline__ uint32_t key_p(uint32_t k) { return NARROW ? (k & kPmtMask) >> 1 : k & kPmtMask; }
 };
 
 constexpr uint32_t kBarCons = 1;        // named barrier of the consumers
 
-// Floor coincidences in bucket order: candidates of a key checked in the
-// first pass before the rounds take over.
-constexpr uint32_t kFloorPairs = 3;
-
 template <int NC>
 __device__ __forceinline__ void cons_sync() { named_sync(kBarCons, NC); }
 
-__device__ __forceinline__ uint32_t key_t(uint64_t k) { return (uint32_t)(k >> 32); }
-__device__ __forceinline__ uint32_t key_p(uint64_t k) { return (uint32_t)(k >> 16) & 0xffffu; }
-__device__ __forceinline__ uint32_t key_q(uint64_t k) { return (uint32_t)k & 0xffffu; }
-
-// Packed key of the trigger phases: time within the staged range (below
+// Packed key of the sorted builds: time within the staged range (below
 // 2^20 ns) and PMT (below 2^12).  0xffffffff marks "no hit".
 constexpr uint32_t kPkNone = 0xffffffffu;
 __device__ __forceinline__ uint32_t pk_t(uint32_t k) { return k >> 12; }
@@ -907,8 +954,8 @@ __device__ __noinline__ bool coincidence_seed(const uint32_t *pk, uint32_t n, ui
 // A seed's scan range: the keys [j0, j1) of the buckets covering
 // [t_s - d, t_s + d], d its row's maximum (keys beyond fail the causal
 // test), from the sorted tile's bucket offsets.
-template <int CAP, uint32_t NB>
-__device__ __forceinline__ void seed_range(const TileCtx<CAP> &cx, uint32_t ts, uint32_t ps, uint32_t bsh,
+template <uint32_t NB, class CTX>
+__device__ __forceinline__ void seed_range(const CTX &cx, uint32_t ts, uint32_t ps, uint32_t bsh,
                                            uint32_t &j0, uint32_t &j1)
 {
     const uint32_t dm = ps < cx.P ? (uint32_t)cx.dmax_s()[ps] : 0u;
@@ -922,8 +969,8 @@ __device__ __forceinline__ void seed_range(const TileCtx<CAP> &cx, uint32_t ts, 
 // eight lanes per seed each collect a 128-bit PMT set in registers over
 // every eighth key of the seed's scan range, and the sets are OR-ed and
 // counted; above, a warp per seed marks the PMTs in a shared-memory set.
-template <int CAP, int NC, bool SMEM_DT, uint32_t NB>
-__device__ __noinline__ void count_distinct_pmts(const TileCtx<CAP> &cx, const uint32_t *pk, uint32_t n, uint32_t ns,
+template <int CAP, int NC, uint32_t NB>
+__device__ __noinline__ void count_distinct_pmts(const SortCtx<CAP> &cx, const uint32_t *pk, uint32_t n, uint32_t ns,
                                                  const uint16_t *seed_idx, uint32_t bsh, uint16_t *seed_cnt)
 {
     constexpr uint32_t G = 8, NG = NC / G;
@@ -938,14 +985,13 @@ __device__ __noinline__ void count_distinct_pmts(const TileCtx<CAP> &cx, const u
             const uint32_t ks = pk[seed_idx[k]];
             const uint32_t ts = pk_t(ks), ps = pk_p(ks);
             uint32_t j0, j1;
-            seed_range<CAP, NB>(cx, ts, ps, bsh, j0, j1);
+            seed_range<NB>(cx, ts, ps, bsh, j0, j1);
             if (CHECK(12, j1, n + 1) && CHECK(13, ps, P) && CHECK(16, nwords, 129)) {
-                const uint16_t *row_s = cx.dt_s() + (size_t)ps * P;
                 const uint16_t *row_g = cx.dt_g + (size_t)ps * P;
                 for (uint32_t q = j0 + lane; q < j1; q += 32) {
                     const uint32_t kj = pk[q], tj = pk_t(kj), pj = pk_p(kj);
                     if (!CHECK(11, pj, P)) continue;
-                    const uint32_t lim = SMEM_DT ? (uint32_t)row_s[pj] : (uint32_t)__ldg(row_g + pj);
+                    const uint32_t lim = __ldg(row_g + pj);
                     if ((tj > ts ? tj - ts : ts - tj) <= lim) atomicOr(&set[pj >> 5], 1u << (pj & 31u));
                 }
             }
@@ -966,14 +1012,13 @@ __device__ __noinline__ void count_distinct_pmts(const TileCtx<CAP> &cx, const u
             const uint32_t ks = pk[seed_idx[k]];
             const uint32_t ts = pk_t(ks), ps = pk_p(ks);
             uint32_t j0, j1;
-            seed_range<CAP, NB>(cx, ts, ps, bsh, j0, j1);
+            seed_range<NB>(cx, ts, ps, bsh, j0, j1);
             if (CHECK(12, j1, n + 1) && CHECK(13, ps, P)) {
-                const uint16_t *row_s = cx.dt_s() + (size_t)ps * P;
                 const uint16_t *row_g = cx.dt_g + (size_t)ps * P;
                 for (uint32_t q = j0 + gl; q < j1; q += G) {
                     const uint32_t kj = pk[q], tj = pk_t(kj), pj = pk_p(kj);
                     if (!CHECK(11, pj, P)) continue;
-                    const uint32_t lim = SMEM_DT ? (uint32_t)row_s[pj] : (uint32_t)__ldg(row_g + pj);
+                    const uint32_t lim = __ldg(row_g + pj);
                     if ((tj > ts ? tj - ts : ts - tj) > lim) continue;
                     const uint32_t b = 1u << (pj & 31u), h = pj >> 5;
                     m0 |= h == 0 ? b : 0u;
@@ -1087,8 +1132,8 @@ __device__ __noinline__ bool level0_distinct_warp(const uint32_t *pk, uint32_t n
 // lanes per seed,
 // seeds dealt round-robin to the groups, four independent tests per lane in
 // flight.
-template <int CAP, int NC, bool SMEM_DT, uint32_t LG, uint32_t NB>
-__device__ __forceinline__ void count_causal(const TileCtx<CAP> &cx, const uint32_t *pk, uint32_t n, uint32_t ns,
+template <int CAP, int NC, uint32_t LG, uint32_t NB>
+__device__ __forceinline__ void count_causal(const SortCtx<CAP> &cx, const uint32_t *pk, uint32_t n, uint32_t ns,
                                              const uint16_t *seed_idx, uint32_t bsh, uint16_t *seed_cnt)
 {
     constexpr uint32_t G = 1u << LG, NG = NC >> LG;
@@ -1112,18 +1157,17 @@ __device__ __forceinline__ void count_causal(const TileCtx<CAP> &cx, const uint3
             const uint32_t ks = pk[seed_idx[k]];
             const uint32_t ts = pk_t(ks), ps = pk_p(ks);
             uint32_t j0, j1;
-            seed_range<CAP, NB>(cx, ts, ps, bsh, j0, j1);
+            seed_range<NB>(cx, ts, ps, bsh, j0, j1);
 #ifdef TRIG_PHASE_STATS
             keys_seen += gl == 0 ? j1 - j0 : 0u;
 #endif
             if (CHECK(12, j1, n + 1) && CHECK(13, ps, P)) {
-                const uint16_t *row_s = cx.dt_s() + (size_t)ps * P;
                 const uint16_t *row_g = cx.dt_g + (size_t)ps * P;
                 // key kj counts when |t_j - t_s| <= dt[p_s][p_j]
                 auto causal = [&](uint32_t kj) -> uint32_t {
                     const uint32_t tj = pk_t(kj), pj = pk_p(kj);
                     if (!CHECK(11, pj, P)) return 0u;
-                    const uint32_t lim = SMEM_DT ? (uint32_t)row_s[pj] : (uint32_t)__ldg(row_g + pj);
+                    const uint32_t lim = __ldg(row_g + pj);
                     return (tj > ts ? tj - ts : ts - tj) <= lim;
                 };
                 // each lane takes four consecutive keys per 16-byte load, from
@@ -1160,7 +1204,7 @@ constexpr uint32_t kRankUnknown = 0xffffffffu;
 // in [0, span]): the buckets before x's bucket, plus the keys of that bucket
 // below x.  The keys of a bucket are contiguous in bucket order and in
 // sorted order alike.
-template <uint32_t NB>
+template <uint32_t NB, uint32_t SHIFT>
 __device__ __forceinline__ uint32_t keys_before(const uint32_t *pk, const uint32_t *cnt, uint32_t n, uint32_t x,
                                                 uint32_t bsh, uint32_t span)
 {
@@ -1168,7 +1212,7 @@ __device__ __forceinline__ uint32_t keys_before(const uint32_t *pk, const uint32
     const uint32_t b = bucket_of<NB>(x, bsh);
     uint32_t c = cnt[b];
     const uint32_t e = cnt[b + 1];
-    for (uint32_t m = c; m < e; ++m) c += pk_t(pk[m]) < x;
+    for (uint32_t m = c; m < e; ++m) c += (pk[m] >> SHIFT) < x;
     return c;
 }
 
@@ -1182,9 +1226,10 @@ __device__ __forceinline__ uint32_t bucket_shift(uint32_t span)
     return top > nb_bits ? top - nb_bits : 0u;
 }
 
-// One staged tile through the whole trigger: the n records of `stage` (16
-// bytes each, time t_ns, PMT and charge; any order) span [tb, tb + span);
-// the core is t - tb in [lo_t, hi_t).
+// One staged tile through the whole trigger, sorted builds (level 0, seed
+// rule 1, distinct count, row outputs, event extraction): the n records of
+// `stage` (16 bytes each, time t_ns, PMT and charge; any order) span
+// [tb, tb + span); the core is t - tb in [lo_t, hi_t).
 //
 //  A. every record becomes a packed key (t - tb) << 12 | pmt and is counted
 //     in its time bucket (t - tb) >> bsh; the stage buffer is then handed
@@ -1192,35 +1237,28 @@ __device__ __forceinline__ uint32_t bucket_shift(uint32_t span)
 //  B. bucket offsets (exclusive scan of the counts);
 //  C. the k-way merge of the PMT runs ("DAQ system of NEMO Phase II"):
 //     keys, charges and floors scattered to their bucket, about one key per
-//     bucket.  For the default rule that bucket order is the final order;
-//     the builds with the extended rules, row outputs and event extraction
-//     (SORT) also rank each key inside its bucket by (t, pmt, charge);
+//     bucket, then each key ranked inside its bucket by (t, pmt, charge);
 //  D. floor coincidences ("Sorting and triggering in GPU": another PMT of
 //     the same floor within tau), in rounds: round r checks the pair
-//     (i, i + r) of every key i still live.  Sorted, a key stays live while
-//     its next keys lie within tau; in bucket order, while i + r + 1 is
-//     before the end of the bucket holding t_i + tau (every key within tau
-//     after it in that order).  Every pair is checked once, both hits are
-//     marked, and each warp keeps its own list of live keys.  Seed rule 1
-//     and level 0 (SORT builds) test each core key instead;
+//     (i, i + r) of every key i still live, that is whose next keys lie
+//     within tau.  Every pair is checked once, both hits are marked, and
+//     each warp keeps its own list of live keys.  Seed rule 1 and level 0
+//     test each core key instead;
 //  E. the ordered seed list; F. the causal count of every seed over whole
 //     buckets of its scan range, each key tested exactly ("Muon trigger
 //     strategy"); G. the fired seeds, in (t, pmt, charge) order, to out.
 //
 // Returns the counts and c0 = the number of staged keys before the core.
 // cnt and mask are zero on entry and on return.
-template <int CAP, int NC, bool SMEM_DT, bool EXT, bool DENSE>
-__device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span,
+template <int CAP, int NC>
+__device__ CoreOut sorted_pass(SortCtx<CAP> &cx, const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span,
                              uint32_t lo_t, uint32_t hi_t, const TrigParams &tp, trig_trigger *out, uint32_t *wr,
                              bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo, uint64_t *release_bar)
 {
-    constexpr bool SORT = EXT;
     constexpr uint32_t NW = NC / 32;
     constexpr int PER = CAP / NC;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    // buckets of the in-tile merge: the finer grid where it pays (the dense
-    // builds, whose long causal scans dominate, keep one bucket per slot)
-    constexpr uint32_t NB = DENSE ? (uint32_t)CAP : (uint32_t)TileLayout<CAP>::NBK;
+    constexpr uint32_t NB = (uint32_t)TileLayout<CAP, true>::NBK;
     const uint32_t bsh = bucket_shift<NB>(span);
     const uint32_t tau = tp.tau;
     __shared__ uint32_t s_red[NW + 1];
@@ -1284,14 +1322,13 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
     const uint32_t c0 = s_below[0], c1 = s_below[1], d_lo = s_below[2];
     PHASE_MARK(kPhA);
 
-    // C. bucket order (with each key's floor); SORT: then the rank inside
-    //    the bucket
+    // C. bucket order (with each key's floor), then the rank inside the bucket
     uint32_t *pk = cx.pk_s();
     uint16_t *chg = cx.chg_s(), *flk = cx.flk();
-    uint32_t *pk_c = SORT ? cx.pk_b() : pk;
-    uint16_t *chg_c = SORT ? cx.chg_b() : chg;
+    uint32_t *pk_c = cx.pk_b();
+    uint16_t *chg_c = cx.chg_b();
     const uint16_t *fl = cx.floor_s();
-    const bool charge_rule = !(EXT && tp.seed_rule == 1);
+    const bool charge_rule = tp.seed_rule != 1;
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
         if (key[r] != kPkNone) {
@@ -1300,49 +1337,42 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
             if (CHECK(22, pos, CAP)) {
                 pk_c[pos] = key[r];
                 chg_c[pos] = (uint16_t)(cs[r] >> 16);
-                if (!SORT) {
-                    flk[pos] = fl[key[r] & 0xfffu];
-                    if (charge_rule && (cs[r] >> 16) >= tp.q_seed && tr >= lo_t && tr < hi_t)
-                        atomicOr(&mask[pos >> 5], 1u << (pos & 31u));
-                }
             }
         }
     }
     if (tid < 4) pk[n + tid] = 0xfffff000u;           // end keys (time 2^20 - 1, PMT 0)
     cons_sync<NC>();
     PHASE_MARK(kPhB);
-    if (SORT) {
 #pragma unroll
-        for (int r = 0; r < PER; ++r) {
-            const uint32_t k = key[r];
-            if (k == kPkNone) continue;
-            const uint32_t b = bucket_of<NB>(k >> 12, bsh);
-            const uint32_t s0 = cnt[b], s1 = cnt[b + 1], q = cs[r] >> 16, pos = s0 + (cs[r] & 0xffffu);
-            uint32_t rk = s0;
-            for (uint32_t m = s0; m < s1; ++m) {
-                const uint32_t o = pk_c[m];
-                rk += o < k;
-                if (o == k) {                      // equal time and PMT: charge, then position
-                    const uint32_t oq = chg_c[m];
-                    rk += oq < q || (oq == q && m < pos);
-                }
-            }
-            if (CHECK(23, rk, CAP)) {
-                pk[rk] = k;
-                chg[rk] = (uint16_t)q;
-                flk[rk] = fl[k & 0xfffu];
-                const uint32_t tr = k >> 12;
-                if (charge_rule && q >= tp.q_seed && tr >= lo_t && tr < hi_t)
-                    atomicOr(&mask[rk >> 5], 1u << (rk & 31u));
+    for (int r = 0; r < PER; ++r) {
+        const uint32_t k = key[r];
+        if (k == kPkNone) continue;
+        const uint32_t b = bucket_of<NB>(k >> 12, bsh);
+        const uint32_t s0 = cnt[b], s1 = cnt[b + 1], q = cs[r] >> 16, pos = s0 + (cs[r] & 0xffffu);
+        uint32_t rk = s0;
+        for (uint32_t m = s0; m < s1; ++m) {
+            const uint32_t o = pk_c[m];
+            rk += o < k;
+            if (o == k) {                      // equal time and PMT: charge, then position
+                const uint32_t oq = chg_c[m];
+                rk += oq < q || (oq == q && m < pos);
             }
         }
-        cons_sync<NC>();
+        if (CHECK(23, rk, CAP)) {
+            pk[rk] = k;
+            chg[rk] = (uint16_t)q;
+            flk[rk] = fl[k & 0xfffu];
+            const uint32_t tr = k >> 12;
+            if (charge_rule && q >= tp.q_seed && tr >= lo_t && tr < hi_t)
+                atomicOr(&mask[rk >> 5], 1u << (rk & 31u));
+        }
     }
+    cons_sync<NC>();
     PHASE_MARK(kPhC);
 
     // D. seed flags of the core keys
     const uint32_t P = cx.P;
-    if (EXT && tp.seed_rule == 1) {
+    if (tp.seed_rule == 1) {
         for (uint32_t base = c0 & ~31u; base < c1; base += NC) {
             const uint32_t i = base + tid;
             const bool seed = i >= c0 && i < c1 && coincidence_seed(pk, n, i, tp.rel, P, tp.sc_w, tp.fc_w, tp.afc_w);
@@ -1350,85 +1380,61 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
             if (lane == 0 && m) atomicOr(&mask[(base >> 5) + warp], m);
         }
     } else {
-        // the keys that can pair with a core key -- sorted: [d_lo, c1); in
-        // bucket order: the buckets from t = lo_t - tau to hi_t + tau - 1 --
-        // in contiguous shares per warp; a live entry is (end << 16) | i
-        // with end the first position past i's candidates
+        // the keys [d_lo, c1) can pair with a core key, in contiguous shares
+        // per warp
         const uint32_t lt = (1u << lane) - 1u;
-        const uint32_t r_lo = SORT ? d_lo : cnt[bucket_of<NB>(lo_t > tau ? lo_t - tau : 0u, bsh)];
-        const uint32_t r_hi = SORT ? c1 : cnt[bucket_of<NB>(hi_t + tau - 1u, bsh) + 1];
-        const uint32_t d_n = r_hi > r_lo ? r_hi - r_lo : 0u;
+        const uint32_t d_n = c1 > d_lo ? c1 - d_lo : 0u;
         const uint32_t share = ((d_n + NW - 1) / NW + 31u) & ~31u;
-        const uint32_t w_begin = min(r_lo + warp * share, r_hi), w_end = min(w_begin + share, r_hi);
+        const uint32_t w_begin = min(d_lo + warp * share, c1), w_end = min(w_begin + share, c1);
         uint32_t *live = cx.pk_b() + warp * (CAP / NW);
-        auto core = [&](uint32_t i, uint32_t ti) { return SORT ? (i >= c0 && i < c1) : (ti >= lo_t && ti < hi_t); };
         auto pair = [&](uint32_t i, uint32_t j, uint32_t ki, uint32_t kj) {
-            const uint32_t ti = ki >> 12, tj = kj >> 12;
-            if ((SORT || (tj > ti ? tj - ti : ti - tj) <= tau) && (ki & 0xfffu) != (kj & 0xfffu) && flk[i] == flk[j]) {
-                if (core(i, ti)) atomicOr(&mask[i >> 5], 1u << (i & 31u));
-                if (core(j, tj)) atomicOr(&mask[j >> 5], 1u << (j & 31u));
+            if ((ki & 0xfffu) != (kj & 0xfffu) && flk[i] == flk[j]) {
+                if (i >= c0 && i < c1) atomicOr(&mask[i >> 5], 1u << (i & 31u));
+                if (j >= c0 && j < c1) atomicOr(&mask[j >> 5], 1u << (j & 31u));
             }
         };
         uint32_t nlive = 0;
         for (uint32_t x = w_begin; x < w_end; x += 32) {
             const uint32_t i = x + lane;
             bool alive = false;
-            uint32_t end = 0;
             if (i < w_end) {
-                const uint32_t ki = pk[i], ti = ki >> 12;
-                if (SORT) {
-                    // i + 1 <= c1 <= n: an end key at worst
-                    const uint32_t kj = pk[i + 1];
-                    if ((kj >> 12) - ti <= tau && i + 1 < n) {
-                        alive = true;
-                        pair(i, i + 1, ki, kj);
-                    }
-                } else if (ti + tau >= lo_t && ti < hi_t + tau) {
-                    // the first kFloorPairs candidates inline (most keys
-                    // have no more), the rest in the rounds below
-                    end = cnt[bucket_of<NB>(ti + tau, bsh) + 1];
-#pragma unroll
-                    for (uint32_t r = 1; r <= kFloorPairs; ++r)
-                        if (i + r < end) pair(i, i + r, ki, pk[i + r]);
-                    alive = i + kFloorPairs + 1 < end;
+                const uint32_t ki = pk[i], kj = pk[i + 1];     // i + 1 <= c1 <= n: an end key at worst
+                if ((kj >> 12) - (ki >> 12) <= tau && i + 1 < n) {
+                    alive = true;
+                    pair(i, i + 1, ki, kj);
                 }
             }
             const uint32_t m = __ballot_sync(0xffffffffu, alive);
-            if (alive) live[nlive + __popc(m & lt)] = (end << 16) | i;
+            if (alive) live[nlive + __popc(m & lt)] = i;
             nlive += __popc(m);
         }
-        for (uint32_t d = SORT ? 2u : kFloorPairs + 1; nlive; ++d) {
+        for (uint32_t d = 2u; nlive; ++d) {
             uint32_t next = 0;
             for (uint32_t x = 0; x < nlive; x += 32) {
                 bool alive = false;
-                uint32_t e = 0;
+                uint32_t i = 0;
                 if (x + lane < nlive) {
-                    e = live[x + lane];
-                    const uint32_t i = e & 0xffffu, j = i + d;
-                    if (SORT) {
-                        if (j < n) {
-                            const uint32_t ki = pk[i], kj = pk[j];
-                            if ((kj >> 12) - (ki >> 12) <= tau) {
-                                alive = true;
-                                pair(i, j, ki, kj);
-                            }
+                    i = live[x + lane];
+                    const uint32_t j = i + d;
+                    if (j < n) {
+                        const uint32_t ki = pk[i], kj = pk[j];
+                        if ((kj >> 12) - (ki >> 12) <= tau) {
+                            alive = true;
+                            pair(i, j, ki, kj);
                         }
-                    } else {
-                        pair(i, j, pk[i], pk[j]);           // j < end by the list
-                        alive = j + 1 < (e >> 16);
                     }
                 }
                 // the ballot orders this batch's reads of the list before
                 // the writes below (which land at or before x + 31)
                 const uint32_t m = __ballot_sync(0xffffffffu, alive);
-                if (alive) live[next + __popc(m & lt)] = e;
+                if (alive) live[next + __popc(m & lt)] = i;
                 next += __popc(m);
             }
             nlive = next;
         }
     }
     cons_sync<NC>();
-    if (EXT && tp.l0_hits) {
+    if (tp.l0_hits) {
         // level 0 (N hits within TW) before the seed triggers count
         if (tp.l0_distinct && P > 128) {
             // a warp per seed, its PMT set in the bucket-order key region
@@ -1463,12 +1469,9 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
 
     // E. ordered seed list: thread x takes mask word w_lo + x (at most
     //    CAP / 32 <= NC words); each word's offset adds the totals of the
-    //    warps before it.  Marks lie in the core: sorted, positions
-    //    [c0, c1); in bucket order, the buckets of [lo_t, hi_t)
-    uint16_t *seed_idx = SORT ? cx.seed_idx() : cx.flk();
-    const uint32_t p_lo = SORT ? c0 : cnt[bucket_of<NB>(lo_t, bsh)];
-    const uint32_t p_hi = SORT ? c1 : cnt[bucket_of<NB>(hi_t > 0 ? hi_t - 1 : 0, bsh) + 1];
-    const uint32_t w_lo = p_lo >> 5, w_hi = (p_hi + 31) >> 5;
+    //    warps before it.  Marks lie in the core: positions [c0, c1)
+    uint16_t *seed_idx = cx.seed_idx();
+    const uint32_t w_lo = c0 >> 5, w_hi = (c1 + 31) >> 5;
     const uint32_t nwords = w_hi - w_lo;
     const uint32_t nw_used = (nwords + 31) >> 5;
     uint32_t *wtot = s_tot;                               // [NW]
@@ -1498,15 +1501,13 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
     PHASE_MARK(kPhE);
     if (tid == 0) PHASE_ADD(kPhSeeds, ns);
 
-    // F. causal count c(s) over each seed's scan range (sparse batches give
-    //    each seed 4 lanes, dense ones a warp), or its distinct-PMT form
-    // (in bucket order the seed list sits in the floor array, so the
-    // counts take the second half of the bucket-order key region)
+    // F. causal count c(s) over each seed's scan range, 4 lanes per seed, or
+    //    its distinct-PMT form
     uint16_t *seed_cnt = cx.seed_cnt();
-    if (EXT && tp.count_distinct) {
-        count_distinct_pmts<CAP, NC, SMEM_DT, NB>(cx, pk, n, ns, seed_idx, bsh, seed_cnt);
+    if (tp.count_distinct) {
+        count_distinct_pmts<CAP, NC, NB>(cx, pk, n, ns, seed_idx, bsh, seed_cnt);
     } else {
-        count_causal<CAP, NC, SMEM_DT, DENSE ? 5u : 2u, NB>(cx, pk, n, ns, seed_idx, bsh, seed_cnt);
+        count_causal<CAP, NC, 2u, NB>(cx, pk, n, ns, seed_idx, bsh, seed_cnt);
     }
     cons_sync<NC>();
     PHASE_MARK(kPhF);
@@ -1514,8 +1515,6 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
 
     // G. emit the fired seeds in order: warp w takes a contiguous range of
     //    the seed list and adds up the fired totals of the warps before it.
-    //    In bucket order a fired seed's rank also counts the fired seeds of
-    //    its bucket (adjacent in the list) with a smaller (t, pmt, charge).
     const uint32_t threshold = tp.threshold;
     const uint32_t per_w = (ns + NW - 1) / NW;
     const uint32_t k_begin = min(ns, warp * per_w), k_end = min(ns, k_begin + per_w);
@@ -1546,23 +1545,7 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
             const uint32_t i = seed_idx[k];
             const uint32_t ks = pk[i];
             const uint32_t q = chg[i];
-            uint32_t o_ = F + __popc(m & ((1u << lane) - 1u));
-            if (!SORT) {
-                // fired seeds of the same bucket before k that order after
-                // it, and after k that order before it
-                const uint32_t bk = bucket_of<NB>(ks >> 12, bsh);
-                const uint64_t key_k = ((uint64_t)ks << 16) | q;
-                for (uint32_t k2 = k; k2-- > 0;) {
-                    const uint32_t i2 = seed_idx[k2];
-                    if (bucket_of<NB>(pk[i2] >> 12, bsh) != bk) break;
-                    if (count_of(k2) >= threshold && (((uint64_t)pk[i2] << 16) | chg[i2]) > key_k) --o_;
-                }
-                for (uint32_t k2 = k + 1; k2 < ns; ++k2) {
-                    const uint32_t i2 = seed_idx[k2];
-                    if (bucket_of<NB>(pk[i2] >> 12, bsh) != bk) break;
-                    if (count_of(k2) >= threshold && (((uint64_t)pk[i2] << 16) | chg[i2]) < key_k) ++o_;
-                }
-            }
+            const uint32_t o_ = F + __popc(m & ((1u << lane) - 1u));
             trig_trigger tr;
             tr.t_ns = tb + (int64_t)(ks >> 12);
             tr.pmt = (uint16_t)(ks & 0xfffu);
@@ -1575,21 +1558,21 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
                 // that bound lies in the staged range (else kRankUnknown:
                 // the window pass searches for it)
                 const uint32_t ts = ks >> 12, wh = tp.win_half;
-                const uint32_t r_lo = ts >= wh ? rank_base + keys_before<NB>(pk, cnt, n, ts - wh, bsh, span)
+                const uint32_t r_lo = ts >= wh ? rank_base + keys_before<NB, 12>(pk, cnt, n, ts - wh, bsh, span)
                                                : kRankUnknown;
                 const uint32_t r_hi = ts + wh + 1u <= span
-                                          ? rank_base + keys_before<NB>(pk, cnt, n, ts + wh + 1u, bsh, span)
+                                          ? rank_base + keys_before<NB, 12>(pk, cnt, n, ts + wh + 1u, bsh, span)
                                           : kRankUnknown;
                 *reinterpret_cast<uint2 *>(wr + 2 * ((out_at_c0 ? c0 : 0u) + o_)) = make_uint2(r_lo, r_hi);
             }
         }
         F += __popc(m);
     }
-    // optional row outputs (SORT builds): the merged core rows
+    // optional row outputs: the merged core rows
     // (verification, and the merged stream of event extraction) and each
     // row's causal count (verification only); rows are indexed by merged
     // rank minus the rank of the slice's first owned hit
-    if (SORT && tp.dbg_merged) {
+    if (tp.dbg_merged) {
         const uint64_t dbg_base = (uint64_t)(dbg_rank_lo + (int64_t)c0);
         for (uint32_t i = tid; i < c1 - c0; i += NC) {
             const uint32_t k = pk[c0 + i];
@@ -1621,14 +1604,381 @@ __device__ CoreOut tile_pass(TileCtx<CAP> &cx, const uint64_t *stage, uint32_t n
     return co;
 }
 
-// Overflow path: the tile holds more than CAP hits with its halo.  Split
+// Causal count c(s) = #{ j : |t_j - t_s| <= min(dt_max[p_s][p_j], W) } over
+// each seed's scan range keys [j0, j1) (seed_range), a group of 2^lg lanes
+// per seed; a fired seed sets its position in mask.
+//
+// Bound by the issue slots and the shared-memory reads of its inner loop (the
+// row lookups of 32 lanes meet in 3.4 banks' turns), so a key costs six
+// instructions: a quarter of a 16-byte key load, the row
+// lookup whose address is one logical operation (kDtRow-aligned rows, the
+// key's low byte is the offset in the row), shift, absolute difference,
+// compare, count.  No key outside [j0, j1) can pass: those before j0 lie in
+// earlier buckets, more than dmax_row(p_s) >= dt before t_s, those from j1
+// on in later buckets, and the four end keys past the last key are beyond
+// any dt as well, so whole groups of four from j0 rounded down are taken.
+template <int CAP, int NC, bool NARROW, uint32_t NB>
+__device__ __forceinline__ void count_seeds(const TileCtx<CAP, NARROW> &cx, uint32_t n, uint32_t ns, uint32_t bsh,
+                                            uint32_t lg, uint32_t threshold)
+{
+    using C = TileCtx<CAP, NARROW>;
+    const uint32_t tid = threadIdx.x, G = 1u << lg, gl = tid & (G - 1u), gid = tid >> lg, NG = NC >> lg;
+    const uint32_t *pk = cx.pk();
+    const uint32_t *seeds = cx.seeds();
+    const uint32_t rounds = (ns + NG - 1) / NG;
+    for (uint32_t r = 0; r < rounds; ++r) {
+        const uint32_t k = r * NG + gid;
+        uint32_t c = 0, pos = 0;
+        if (k < ns) {
+            pos = seeds[k] & 0xffffu;
+            const uint32_t ks = pk[pos];
+            const uint32_t ts = C::key_t(ks), ps = C::key_p(ks);
+            uint32_t j0, j1;
+            seed_range<NB>(cx, ts, ps, bsh, j0, j1);
+            if (CHECK(12, j1, n + 1) && CHECK(13, ps, cx.P)) {
+                const uint32_t row_s = (uint32_t)TileCtx<CAP, NARROW>::L::oDt + ps * kDtRow;
+                const uint16_t *row_g = cx.dt_g + (size_t)ps * cx.P;
+                auto causal = [&](uint32_t kj) -> uint32_t {
+                    uint32_t lim;
+                    if (NARROW) {
+                        lim = *reinterpret_cast<const uint16_t *>(g_tile_smem + (row_s | (kj & C::kPmtMask)));
+                    } else {
+                        const uint32_t pj = C::key_p(kj);
+                        if (!CHECK(11, pj, cx.P)) return 0u;
+                        lim = __ldg(row_g + pj);
+                    }
+                    return __usad(C::key_t(kj), ts, 0u) <= lim;
+                };
+                uint32_t ca = 0, cb = 0, cc = 0, cd = 0;
+                for (uint32_t q = (j0 & ~3u) + 4 * gl; q < j1; q += 4 * G) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(pk + q);
+                    ca += causal(v.x);
+                    cb += causal(v.y);
+                    cc += causal(v.z);
+                    cd += causal(v.w);
+                }
+                c = ca + cb + cc + cd;
+            }
+        }
+        for (uint32_t off = G >> 1; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+        if (k < ns && gl == 0) {
+            cx.counts()[k] = (uint16_t)c;
+            if (c >= threshold) atomicOr(&cx.mask()[pos >> 5], 1u << (pos & 31u));
+        }
+    }
+}
+
+// One staged tile through the whole trigger, default rule: the n records of
+// `stage` (16 bytes each, any order) span [tb, tb + span); the core is
+// t - tb in [lo_t, hi_t).
+//
+//  A. every record becomes a packed key (TileCtx::key), is counted in its
+//     time bucket (t - tb) >> bsh and marked in its floor cell (floor, and
+//     time in steps of 2^csh > tau: two bits, one hit and more than one);
+//  B. bucket offsets (exclusive scan of the counts), and a mark on each floor
+//     cell with another hit in it or in a neighbouring cell;
+//  C. the k-way merge of the PMT runs ("DAQ system of NEMO Phase II"): keys
+//     scattered to bucket order, about one key per bucket.  A core hit
+//     over the charge threshold or in a marked cell becomes a candidate;
+//  D. floor coincidences ("Sorting and triggering in GPU": another PMT of
+//     the same floor within tau): each candidate looks through the buckets
+//     of [t - tau, t + tau];
+//  E. the causal counts (count_seeds);
+//  F. the fired seeds to out, in (t, pmt, charge) order: a seed's rank is
+//     the number of fired positions before it, corrected inside its bucket.
+//
+// Bound by the shared-memory pipe (60 % busy) and the latency of the phases'
+// chains of lookups, then by instruction issue (54 %), not by HBM (11 %).  So
+// each phase reads shared memory as seldom as it can: the floor cells leave
+// about one hit in six for phase D's search (a search from every hit took a
+// third of the pass), charges travel with the candidates instead of being
+// scattered with every key, and two lanes share a seed's emission.  The 64
+// slices of both towers (205 M hits, tiles of 2048 at 90 %) take 3.50 ms,
+// 4.43 ms with the search from every hit and an ordered seed list; the
+// 2688-PMT slice 1.22 ms, 2.05 before.
+// The bucket counts, cells and mask are zero on entry and on return.
+template <int CAP, int NC, bool NARROW, bool DENSE>
+__device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span,
+                             uint32_t lo_t, uint32_t hi_t, const TrigParams &tp, trig_trigger *out, uint32_t *wr,
+                             bool out_at_c0, uint32_t rank_base, uint64_t *release_bar)
+{
+    using C = TileCtx<CAP, NARROW>;
+    using L = typename C::L;
+    constexpr uint32_t NW = NC / 32;
+    constexpr int PER = CAP / NC;
+    constexpr uint32_t NB = L::NBK;
+    constexpr uint32_t M = L::kCells;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, lt = (1u << lane) - 1u;
+    const uint32_t bsh = bucket_shift<NB>(span);
+    const uint32_t tau = tp.tau;
+    __shared__ uint32_t s_red[NW];
+    __shared__ uint32_t s_n[3];             // candidates, seeds, keys before the core
+    uint32_t *cnt = cx.cnt(), *mask = cx.mask(), *cells = cx.cells();
+    uint32_t *pk = cx.pk(), *seeds = cx.seeds(), *cand = cx.cand();
+    const uint16_t *fl = cx.floor_s();
+    // floor cells of 2^csh ns; the floors' ranges of cells follow each other,
+    // taken modulo M (two hits that share a cell by chance only cost a search)
+    const uint32_t csh = 32u - __clz(tau), fstep = (span >> csh) + 2u;
+#ifdef TRIG_PHASE_STATS
+    long long t_ph = clock64();
+#define PHASE_MARK(i)                                   \
+    do {                                                \
+        if (tid == 0) {                                 \
+            const long long now_ = clock64();           \
+            PHASE_ADD((i), now_ - t_ph);                \
+            t_ph = now_;                                \
+        }                                               \
+    } while (0)
+#else
+#define PHASE_MARK(i) ((void)0)
+#endif
+
+    // A. keys, bucket counts, floor cells
+    uint32_t key[PER], cs[PER], hc[PER];  // packed key; charge << 16 | slot in the bucket; floor cell
+    if (tid == 0) s_n[0] = s_n[1] = 0;
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+        const uint32_t i = tid + r * NC;
+        key[r] = kPkNone;
+        cs[r] = hc[r] = 0;
+        if (i < n) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(stage + 2 * i);
+            // t - tb in 32 bits (the staged range spans less than 2^20 ns)
+            const uint32_t tr = min(v.x - (uint32_t)tb, span - 1u), p = v.z & 0xfffu;
+            key[r] = C::key(tr, p);
+            cs[r] = (v.z & 0xffff0000u) | atomicAdd(&cnt[tr >> bsh], 1u);
+            const uint32_t h = (fl[p] * fstep + (tr >> csh)) & (M - 1u), bit = 1u << (2u * (h & 15u));
+            hc[r] = h;
+            if (atomicOr(&cells[h >> 4], bit) & bit) atomicOr(&cells[h >> 4], bit << 1);
+        }
+    }
+    // the stage buffer has been read: order those reads before the
+    // producer's next bulk copy into it, then hand it back
+    if (release_bar) fence_proxy_async_smem();
+    cons_sync<NC>();
+    if (release_bar && tid == 0) mbar_arrive(release_bar);
+    PHASE_MARK(kPhA);
+
+    // B. bucket offsets; and each floor cell's two bits become one: another
+    //    hit in the cell, or one in a neighbouring cell
+    {
+        constexpr uint32_t MV = M / 64 / NC;              // 16-byte vectors of cells per thread
+        static_assert(M % (64 * NC) == 0, "each thread folds whole 16-byte vectors of cells");
+        uint4 *m4 = reinterpret_cast<uint4 *>(cells) + tid * MV;
+        uint32_t fold[4 * MV];
+        {
+            uint32_t prev = cells[(tid * 4 * MV - 1u) & (M / 16 - 1u)];
+            const uint32_t last = cells[(tid * 4 * MV + 4 * MV) & (M / 16 - 1u)];
+            uint32_t w[4 * MV + 1];
+#pragma unroll
+            for (uint32_t i = 0; i < MV; ++i) {
+                const uint4 c = m4[i];
+                w[4 * i] = c.x, w[4 * i + 1] = c.y, w[4 * i + 2] = c.z, w[4 * i + 3] = c.w;
+            }
+            w[4 * MV] = last;
+#pragma unroll
+            for (uint32_t i = 0; i < 4 * MV; ++i) {
+                fold[i] = (w[i] >> 1) | __funnelshift_l(prev, w[i], 2) | __funnelshift_r(w[i], w[i + 1], 2);
+                prev = w[i];
+            }
+        }
+        constexpr uint32_t V = NB / NC / 4;
+        static_assert(NB % (4 * NC) == 0, "each thread scans whole 16-byte vectors");
+        uint4 *c4 = reinterpret_cast<uint4 *>(cnt) + tid * V;
+        uint4 v[V];
+        uint32_t local = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < V; ++i) {
+            v[i] = c4[i];
+            local += v[i].x + v[i].y + v[i].z + v[i].w;
+        }
+        const uint32_t incl = warp_incl_scan(local);
+        if (lane == 31) s_red[warp] = incl;
+        cons_sync<NC>();
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? s_red[lane % NW] : 0u);
+        uint32_t run = before + incl - local;
+#pragma unroll
+        for (uint32_t i = 0; i < V; ++i) {
+            uint4 o;
+            o.x = run;
+            o.y = o.x + v[i].x;
+            o.z = o.y + v[i].y;
+            o.w = o.z + v[i].z;
+            run = o.w + v[i].w;
+            c4[i] = o;
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < MV; ++i)
+            m4[i] = make_uint4(fold[4 * i], fold[4 * i + 1], fold[4 * i + 2], fold[4 * i + 3]);
+        if (tid == NC - 1) cnt[NB] = run;
+        if (tid < 4) pk[n + tid] = ~C::kPmtMask;          // end keys (the last time, PMT 0)
+    }
+    cons_sync<NC>();
+    PHASE_MARK(kPhB);
+
+    // C. bucket order and candidates (charge << 16 | position, with bit 15
+    //    set for a charge over the threshold)
+    {
+        uint32_t m[PER], total = 0;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            bool c = false;
+            if (key[r] != kPkNone) {
+                const uint32_t tr = C::key_t(key[r]);
+                const uint32_t pos = cnt[tr >> bsh] + (cs[r] & 0xffffu);
+                if (CHECK(22, pos, CAP)) pk[pos] = key[r];
+                if (tr - lo_t < hi_t - lo_t) {
+                    const bool over = (cs[r] >> 16) >= tp.q_seed;
+                    c = over || ((cells[hc[r] >> 4] >> (2u * (hc[r] & 15u))) & 1u);
+                    cs[r] = (cs[r] & 0xffff0000u) | pos | (over ? 0x8000u : 0u);
+                }
+            }
+            m[r] = __ballot_sync(0xffffffffu, c);
+            total += __popc(m[r]);
+        }
+        uint32_t at = 0;
+        if (lane == 0 && total) at = atomicAdd(&s_n[0], total);
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            if ((m[r] >> lane) & 1u) cand[at + __popc(m[r] & lt)] = cs[r];
+            at += __popc(m[r]);
+        }
+    }
+    cons_sync<NC>();
+    PHASE_MARK(kPhC);
+
+    // D. floor coincidences of the candidates, four keys of the range at a
+    //    time; the seeds take the cells' place
+    {
+        const uint32_t nc = s_n[0];
+        for (uint32_t x = warp * 32; x < nc; x += NC) {
+            bool seed = false;
+            uint32_t e = 0;
+            if (x + lane < nc) {
+                e = cand[x + lane];
+                seed = (e >> 15) & 1u;
+                e &= 0xffff7fffu;
+                if (!seed) {
+                    const uint32_t ki = pk[e & 0xffffu], ti = C::key_t(ki), pi = C::key_p(ki), fi = fl[pi];
+                    uint32_t j = cnt[(ti > tau ? ti - tau : 0u) >> bsh];
+                    const uint32_t je = cnt[bucket_of<NB>(ti + tau, bsh) + 1];
+                    for (; j < je; j += 4) {
+                        uint32_t kj[4], fj[4];
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u) kj[u] = pk[min(j + u, je - 1u)];
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u) fj[u] = fl[C::key_p(kj[u])];
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u)
+                            seed = seed || (__usad(C::key_t(kj[u]), ti, 0u) <= tau && C::key_p(kj[u]) != pi && fj[u] == fi);
+                    }
+                }
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, seed);
+            uint32_t at = 0;
+            if (lane == 0 && m) at = atomicAdd(&s_n[1], __popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (seed && CHECK(2, at + __popc(m & lt), CAP)) seeds[at + __popc(m & lt)] = e;
+        }
+        // keys before the core: the fired seeds' place in the slice's staging
+        if (tid == NC - 1) s_n[2] = keys_before<NB, C::kShift>(pk, cnt, n, lo_t, bsh, span);
+    }
+    cons_sync<NC>();
+    PHASE_MARK(kPhD);
+    const uint32_t ns = s_n[1], c0 = s_n[2];
+    if (tid == 0) PHASE_ADD(kPhSeeds, ns);
+
+    // E. causal counts: the dense builds (hundreds of keys per seed) take a
+    //    warp per seed; the others four lanes, or more while all seeds of
+    //    the tile still fit in one round
+    uint32_t lg = 5;
+    if (!DENSE) {
+        lg = 2;
+        while (lg < 5 && (ns << (lg + 1)) <= NC) ++lg;
+    }
+    count_seeds<CAP, NC, NARROW, NB>(cx, n, ns, bsh, lg, tp.threshold);
+    cons_sync<NC>();
+    PHASE_MARK(kPhE);
+
+    // F. each warp counts the fired positions before each mask word (a lane
+    //    takes PW consecutive words), then takes 16 seeds at a time, two
+    //    lanes per seed: one finds the merged rank of the first hit of the
+    //    seed's event window [t - h, t + h], the other of the first hit past
+    //    it, where that bound lies in the staged range (else kRankUnknown:
+    //    the window pass searches for it)
+    constexpr uint32_t PW = CAP / 32 / 32;
+    uint32_t wn[PW], own = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < PW; ++w) {
+        wn[w] = __popc(mask[lane * PW + w]);
+        own += wn[w];
+    }
+    const uint32_t incl = warp_incl_scan(own), wpre = incl - own;
+    const uint32_t n_fired = __shfl_sync(0xffffffffu, incl, 31);
+    const size_t out_at = out_at_c0 ? c0 : 0u;
+    for (uint32_t k0 = warp * 16; k0 < ns; k0 += NW * 16) {
+        const uint32_t k = k0 + (lane >> 1), side = lane & 1u;
+        const uint32_t e = k < ns ? seeds[k] : 0u, c = k < ns ? cx.counts()[k] : 0u;
+        const uint32_t pos = e & 0xffffu, w = pos >> 5;
+        // fired positions before pos: the words before its word ...
+        uint32_t o = __shfl_sync(0xffffffffu, wpre, w / PW);
+#pragma unroll
+        for (uint32_t x = 0; x + 1 < PW; ++x) {
+            const uint32_t v = __shfl_sync(0xffffffffu, wn[x], w / PW);
+            o += x < w % PW ? v : 0u;
+        }
+        if (k >= ns || c < tp.threshold) continue;
+        // ... and those before it in the word
+        o += __popc(mask[w] & ((1u << (pos & 31u)) - 1u));
+        const uint32_t ks = pk[pos], ts = C::key_t(ks), b = ts >> bsh;
+        // fired seeds of its bucket that order the other way round
+        for (uint32_t j = cnt[b], je = cnt[b + 1]; j < je; ++j) {
+            if (j == pos || !((mask[j >> 5] >> (j & 31u)) & 1u)) continue;
+            const uint32_t kj = pk[j];
+            bool less = kj < ks, more = kj > ks;
+            if (kj == ks)                        // the same time and PMT: by charge (kept in the list)
+                for (uint32_t y = 0; y < ns; ++y)
+                    if ((seeds[y] & 0xffffu) == j) {
+                        less = (seeds[y] >> 16) < (e >> 16);
+                        more = (seeds[y] >> 16) > (e >> 16);
+                    }
+            o += j > pos && less ? 1u : 0u;
+            o -= j < pos && more ? 1u : 0u;
+        }
+        if (!CHECK(3, o, n_fired)) continue;
+        const uint32_t wh = tp.win_half, x = side ? ts + wh + 1u : ts - wh;
+        const bool known = side ? x <= span : ts >= wh;
+        wr[2 * (out_at + o) + side] = known ? rank_base + keys_before<NB, C::kShift>(pk, cnt, n, x, bsh, span) : kRankUnknown;
+        // the trigger's two halves: time; PMT, charge and count
+        const uint64_t half = side ? (uint64_t)c << 32 | (e & 0xffff0000u) | C::key_p(ks) : (uint64_t)(tb + (int64_t)ts);
+        reinterpret_cast<uint64_t *>(out + out_at + o)[side] = half;
+    }
+    // leave the bucket counts, cells and mask zero for the next tile
+    cons_sync<NC>();
+    PHASE_MARK(kPhF);
+    {
+        uint4 *z = reinterpret_cast<uint4 *>(cnt);
+        uint4 *y = reinterpret_cast<uint4 *>(cells);
+        for (uint32_t i = tid; i < NB / 4; i += NC) z[i] = y[i] = make_uint4(0, 0, 0, 0);
+        for (uint32_t i = tid; i < (uint32_t)CAP / 32; i += NC) mask[i] = 0;
+    }
+    cons_sync<NC>();
+    PHASE_MARK(kPhG);
+#undef PHASE_MARK
+    CoreOut co;
+    co.n_fired = n_fired;
+    co.n_seeds = ns;
+    co.c0 = c0;
+    return co;
+}
+
 // Overflow path: the tile holds more than CAP hits with its halo.  Split
 // its core in halves until each piece fits; pieces are staged with plain
 // loads after per-PMT binary searches.  A 1 ns core that still does not
 // fit is reported (TRIG_FLAG_TILE_FULL) and skipped.
-template <int CAP, int NC, bool SMEM_DT, bool EXT, bool DENSE>
-__device__ void tile_overflow(TileCtx<CAP> &cx, uint64_t *buf, const SliceDesc &d, const TrigParams &tp, uint32_t g,
-                              uint32_t *red, int64_t *stk)
+template <int CAP, int NC, class PASS>
+__device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint32_t g, uint32_t *red, int64_t *stk)
 {
     constexpr uint32_t NW = NC / 32;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
@@ -1737,11 +2087,9 @@ __device__ void tile_overflow(TileCtx<CAP> &cx, uint64_t *buf, const SliceDesc &
         const int64_t tb = lo - (int64_t)H;
         const uint32_t span = (uint32_t)(hi - lo) + 2 * H;
         const uint32_t fired0 = red[5];
-        CoreOut co = tile_pass<CAP, NC, SMEM_DT, EXT, DENSE>(cx, buf, total, tb, span, H, H + (uint32_t)(hi - lo), tp,
-                                                             d.stage + tile_rank + fired0,
-                                                             d.wrank + 2 * (size_t)(tile_rank + fired0), false,
-                                                             rank_lo, (int64_t)rank_lo - (int64_t)d.dbg_rank0,
-                                                             nullptr);
+        CoreOut co = pass(buf, total, tb, span, H, H + (uint32_t)(hi - lo), d.stage + tile_rank + fired0,
+                          d.wrank + 2 * (size_t)(tile_rank + fired0), false, rank_lo,
+                          (int64_t)rank_lo - (int64_t)d.dbg_rank0, nullptr);
         if (tid == 0) {
             red[5] = fired0 + co.n_fired;
             red[6] += co.n_seeds;
@@ -1762,16 +2110,19 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                                                                           uint32_t max_pmt)
 {
     constexpr uint32_t NW = NC / 32;
-    constexpr uint32_t NSTG = TileLayout<CAP>::NS;
+    using L = TileLayout<CAP, EXT>;
+    constexpr uint32_t NSTG = L::NS;
     __shared__ uint64_t full_bar[2], empty_bar[2];
     __shared__ ItemInfo info[2];
     __shared__ __align__(16) uint32_t red[64 + 64];
     __shared__ int64_t stk[128];
 
-    TileCtx<CAP> cx;
+    std::conditional_t<EXT, SortCtx<CAP>, TileCtx<CAP, SMEM_DT>> cx;
     cx.pp = (max_pmt + 7) & ~7u;
     cx.dt_g = nullptr;
     cx.P = 0;
+    if constexpr (!EXT) cx.tab = (uint32_t)L::tab(max_pmt, SMEM_DT);
+    auto stage_of = [&](uint32_t b) { return reinterpret_cast<uint64_t *>(g_tile_smem + (size_t)b * L::kStage); };
 
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     if (tid == 0) {
@@ -1914,7 +2265,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             __syncwarp();
             if (mode == 0 && wide) {
                 if (lane == 0 && CHECK(7, rlo + tot, d->n_hits + 1))
-                    bulk_g2s(cx.stage(b), d->tbuf + rlo, (uint32_t)tot * 16u, &full_bar[b]);
+                    bulk_g2s(stage_of(b), d->tbuf + rlo, (uint32_t)tot * 16u, &full_bar[b]);
             } else if (mode == 0) {
                 uint32_t dst = 0;
 #pragma unroll
@@ -1923,7 +2274,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                     const uint64_t a = ra[r];
                     const uint32_t incl = warp_incl_scan(len);
                     if (len && CHECK(6, dst + incl, CAP + 1) && CHECK(7, a + len, d->n_hits + 1))
-                        bulk_g2s(cx.stage(b) + 2 * (size_t)(dst + incl - len), d->hits + a, len * 16u, &full_bar[b]);
+                        bulk_g2s(stage_of(b) + 2 * (size_t)(dst + incl - len), d->hits + a, len * 16u, &full_bar[b]);
                     dst += __shfl_sync(0xffffffffu, incl, 31);
                 }
             }
@@ -1936,9 +2287,11 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     }
 
     // ---------------------------------------------------- consumer warps
-    // the tile pass expects zero bucket counts and seed mask (and leaves them so)
-    for (uint32_t i = tid; i < (uint32_t)TileLayout<CAP>::NBK; i += NC) cx.cnt()[i] = 0;
+    // the tile pass expects zero bucket counts, masks and bitmaps (and leaves them so)
+    for (uint32_t i = tid; i < (uint32_t)L::NBK; i += NC) cx.cnt()[i] = 0;
     for (uint32_t i = tid; i < (uint32_t)CAP / 32; i += NC) cx.mask()[i] = 0;
+    if constexpr (!EXT)
+        for (uint32_t i = tid; i < L::kCells / 16; i += NC) cx.cells()[i] = 0;
     cons_sync<NC>();
     const SliceDesc *loaded = nullptr;
     // the slice's trigger parameters live in shared memory (written by one
@@ -1947,6 +2300,16 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     // the loaded slice's tile width, t0, length and merged rank of its first
     // owned hit, also kept in shared memory
     __shared__ int64_t sl[4];
+    auto pass = [&](const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span, uint32_t lo_t, uint32_t hi_t,
+                    trig_trigger *out, uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo,
+                    uint64_t *release_bar) {
+        if constexpr (EXT)
+            return sorted_pass<CAP, NC>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0, rank_base,
+                                        dbg_rank_lo, release_bar);
+        else
+            return tile_pass<CAP, NC, SMEM_DT, DENSE>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0,
+                                                      rank_base, release_bar);
+    };
     for (uint32_t it = 0;; ++it) {
         const uint32_t b = it % NSTG, use = it / NSTG;
         // every thread waits (bounded) for the staged tile; the barrier
@@ -1978,8 +2341,8 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 cx.floor_s()[p] = d.floor[p];
                 cx.dmax_s()[p] = d.dmax_row[p];
             }
-            if (SMEM_DT && P <= kSmemDtMaxPmt)
-                for (uint32_t i = tid; i < P * P; i += NC) cx.dt_s()[i] = d.dt[i];
+            if constexpr (!EXT && SMEM_DT)
+                for (uint32_t i = tid; i < P * P; i += NC) cx.dt_s()[(i / P) * (kDtRow / 2) + i % P] = d.dt[i];
             cx.dt_g = d.dt;
             cx.P = P;
             loaded = &d;
@@ -2015,7 +2378,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 d.tile_rank[inf.g] = 0;
             }
         } else if (inf.mode == 1) {
-            tile_overflow<CAP, NC, SMEM_DT, EXT, DENSE>(cx, cx.stage(b), d, tp, inf.g, red, stk);
+            tile_overflow<CAP, NC>(pass, stage_of(b), d, inf.g, red, stk);
         } else {
             const int64_t W = sl[0];
             const uint32_t g = inf.g, n_st = inf.n, rank_lo = inf.rank_lo, span = inf.span;
@@ -2028,10 +2391,8 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             // the pass hands the buffer back as soon as it has read it (inf
             // is not read after that); the core's first hit has merged rank
             // rank_lo + c0
-            CoreOut co = tile_pass<CAP, NC, SMEM_DT, EXT, DENSE>(cx, cx.stage(b), n_st, tb, span, lo_t, hi_t, tp,
-                                                                 d.stage + rank_lo, d.wrank + 2 * (size_t)rank_lo,
-                                                                 true, rank_lo, (int64_t)rank_lo - sl[3],
-                                                                 &empty_bar[b]);
+            CoreOut co = pass(stage_of(b), n_st, tb, span, lo_t, hi_t, d.stage + rank_lo, d.wrank + 2 * (size_t)rank_lo,
+                              true, rank_lo, (int64_t)rank_lo - sl[3], &empty_bar[b]);
             const uint32_t tile_rank = rank_lo + co.c0;
             if (tid == 0 && CHECK(14, (uint64_t)tile_rank + co.n_fired, d.n_hits + 1) && CHECK(15, g, d.n_tiles)) {
                 d.tile_nfired[g] = co.n_fired;
@@ -2710,7 +3071,7 @@ template <int CAP, int NC, bool SMEM_DT, bool EXT = false, bool DENSE = false>
 static cudaError_t launch_tile(BatchHeader *hdr, SliceDesc *desc, uint32_t max_pmt, cudaStream_t st)
 {
     static bool limit_set[64] = {};
-    size_t smem = TileLayout<CAP>::bytes(max_pmt, SMEM_DT);
+    size_t smem = TileLayout<CAP, EXT>::bytes(max_pmt, SMEM_DT);
     auto kern = k_tile<CAP, NC, SMEM_DT, EXT, DENSE>;
     cudaError_t e = raise_smem_limit(kern, limit_set);
     if (e != cudaSuccess) return e;

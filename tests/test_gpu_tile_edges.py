@@ -1,0 +1,85 @@
+"""The tile pass of the default rule where its phases can go wrong: floor
+cells (tau at and around powers of two, 0 and the largest), seed lists that
+hold every hit, detectors at the edges of the shared-memory dt table and of
+the bucketed path, equal times, and tile fills around a full tile.  Whole
+numbers, equal to the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+    import paper_1411_3968_gb300 as p
+    from paper_1411_3968_gb300 import build
+    build.build()
+    p.load()
+    torch.cuda.init()
+    return p
+
+
+def _detector(n_pmt, per_floor=6):
+    k = np.arange(n_pmt)
+    xyz = np.stack([1000 * (k % per_floor), np.zeros_like(k), 40_000 * (k // per_floor)], 1).astype(np.int32)
+    return xyz, (k // per_floor).astype(np.uint32)
+
+
+def _hits(rng, n, n_pmt, lo, hi, step=1):
+    hits = np.zeros(n, workload.HIT_DTYPE)
+    hits["t"] = lo + rng.integers(0, max(1, (hi - lo) // step), n) * step
+    hits["pmt"] = rng.integers(0, n_pmt, n)
+    hits["charge"] = rng.integers(1, 400, n)
+    hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    return hits, off
+
+
+@pytest.mark.parametrize("shape", [(2048, 16, 90), (1024, 4, 75), (4096, 8, 60)])
+@pytest.mark.parametrize("n_pmt,n,slice_ns,step,extra", [
+    (32, 6000, 300_000, 1, dict(floor_tau_ns=0)),
+    (32, 6000, 300_000, 1, dict(floor_tau_ns=1)),
+    (84, 9000, 300_000, 1, dict(floor_tau_ns=31)),
+    (84, 9000, 300_000, 1, dict(floor_tau_ns=32)),
+    (84, 500, 2_000_000, 1, dict(floor_tau_ns=60_000)),
+    (84, 9000, 300_000, 1, dict(q_seed_adc=0)),
+    (84, 4000, 200_000, 40, dict(q_seed_adc=150)),         # many equal times
+    (1, 900, 900_000, 1, dict(q_seed_adc=300, threshold=1)),
+    (96, 9000, 400_000, 1, {}),
+    (97, 9000, 400_000, 1, {}),
+    (128, 9000, 400_000, 1, {}),
+    (129, 9000, 400_000, 1, {}),
+    (129, 9000, 400_000, 1, dict(q_seed_adc=0)),
+    (84, 30_000, 150_000, 1, {}),                            # hundreds of keys in each scan range
+    (32, 2000, 40_000_000, 1, dict(threshold=1)),            # a few hits in the widest tiles
+])
+def test_tile_pass_edges(pkg, params, shape, n_pmt, n, slice_ns, step, extra):
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(n_pmt * 1000 + n))
+    par = dict(params, slice_ns=slice_ns, **extra)
+    halo = max(par["corr_window_ns"], par["win_half_ns"], par["floor_tau_ns"])
+    t0 = 1_000_000
+    xyz, floor = _detector(n_pmt)
+    hits, off = _hits(rng, n, n_pmt, t0 - halo, t0 + slice_ns + halo, step)
+    old = pkg.trig_get_tile_config()
+    try:
+        pkg.trig_set_tile_config(*shape)
+        det = pkg.Detector(xyz, floor, par)
+        b = DeviceBatch([SliceIn(det, t0, hits, off)])
+        b.run()
+        (stats, trig, win), = b.results()
+    finally:
+        pkg.trig_set_tile_config(*old)
+    ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+    assert int(stats["status"]) == 0
+    assert int(stats["n_seeds"]) == len(ref.seeds) and len(trig) == len(ref.triggers) and len(win) == len(ref.windows)
+    for f in ("t", "pmt", "charge", "count"):
+        assert np.array_equal(trig[f], ref.triggers[f]), f
+    for f in ("lo", "hi", "n_hits", "n_triggers"):
+        assert np.array_equal(win[f], ref.windows[f]), f
+    det.close()
