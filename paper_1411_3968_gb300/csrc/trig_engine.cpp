@@ -404,7 +404,7 @@ static int64_t choose_tile_w(const trig_detector *det, uint64_t n_hits, const Ti
     // a tile plus its halos spans less than kMaxTileSpan ns
     const double w_max = std::max(1.0, (double)(kMaxTileSpan - 1) - 2.0 * det->tile_halo);
     if (w > w_max) w = w_max;
-    return (int64_t)w;
+    return std::max<int64_t>((int64_t)w, 2);        // ceil(2^32 / W) is kept in 32 bits
 }
 
 // Bucket grid of a wide slice: buckets of Wb ns from O = t0 - lead * Wb,
@@ -558,11 +558,12 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             d.tbuf = reinterpret_cast<trig_hit *>(base + off);
             off += align256((size_t)x.n_hits * sizeof(trig_hit));
         } else {
-            const size_t eb = (size_t)d.n_tiles * P * 4;
-            d.e_lo = reinterpret_cast<uint32_t *>(base + off);
-            off += align256(eb);
-            d.e_hi = reinterpret_cast<uint32_t *>(base + off);
-            off += align256(eb);
+            const uint32_t D = 2u * d.halo + (uint32_t)W;
+            d.edge_a = D / (uint32_t)W;
+            d.edge_b = D % (uint32_t)W;
+            d.n_edges = 2u * (d.n_tiles + d.edge_a) + 2u;
+            d.edge = reinterpret_cast<uint32_t *>(base + off);
+            off += align256((size_t)d.n_edges * P * 4);
         }
         d.tile_nfired = reinterpret_cast<uint32_t *>(base + off);
         off += align256((size_t)d.n_tiles * 4);

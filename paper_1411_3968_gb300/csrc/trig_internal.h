@@ -69,8 +69,9 @@ struct SliceDesc {
     uint32_t n_tiles;       // NG (<= 2^20)
     uint32_t item0;         // first work item (tile) of this slice
     uint32_t chunk0;        // first structure-pass chunk of this slice
-    uint32_t *e_lo;         // [NG][P] first hit index with t >= B_g - H (narrow slices)
-    uint32_t *e_hi;         // [NG][P] first hit index with t >= B_{g+1} + H (narrow slices)
+    uint32_t *edge;         // [n_edges][P] first hit index at or past each tile edge (narrow slices):
+                            //   edge 2g is B_g - H, edge 2 (g + edge_a) + 1 is B_{g+1} + H
+    uint32_t n_edges, edge_a, edge_b;       // 2H + W = edge_a W + edge_b
     // Wide slices (P >= kWideMinPmt): the hits are also copied, grouped by
     // time bucket [O + b Wb, O + (b+1) Wb), into tbuf; tile g's core is the
     // buckets [lead + g m, lead + (g+1) m) and it stages those plus `hh`
@@ -136,7 +137,7 @@ constexpr uint64_t kDefaultWaitNs = 1000000000ull;     // one second
 // from which the causal count gives each seed a warp instead of 4 lanes.
 constexpr double kDenseKeys = 600.0;
 
-constexpr uint32_t kChunkHits = 4096;       // structure-pass chunk
+constexpr uint32_t kChunkHits = 992;        // structure-pass chunk: 8 warps of 4 x 31 hits
 
 // Kernel launch helpers implemented in trig_kernels.cu.
 cudaError_t launch_dtmax(const int32_t *xyz, uint32_t n_pmt, uint32_t tol, uint32_t n_num, uint32_t n_den,

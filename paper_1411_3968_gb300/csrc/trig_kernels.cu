@@ -5,7 +5,7 @@
 //   k_bounds   structure pass of the k-way merge ("DAQ system": the Hit
 //              Manager merges the PMT streams into time slices).  One read
 //              of every hit: validates the CSR layout and ordering, and for
-//              every time tile g and PMT p records where p's stream crosses
+//              every tile g and PMT p records where p's stream crosses
 //              the tile's halo edges B_g - H and B_{g+1} + H.
 //   k_tile     persistent, warp-specialised: a producer warp dequeues tiles
 //              and stages each tile's hits (one contiguous run per PMT) into
@@ -364,28 +364,6 @@ __global__ void k_prep(BatchHeader *hdr, const SliceDesc *desc)
 
 // ---------------------------------------------------------------- k_bounds
 
-// Number of tile edges v_g = base + g * W (g in [0, NG)) with v_g <= t,
-// i.e. floor((t - base) / W) + 1 clamped to [0, NG].  (Slices longer than
-// about 2 s; kept out of line.)
-__device__ __noinline__ uint32_t edges_le64(int64_t t, int64_t base, int64_t W, uint32_t ng)
-{
-    const int64_t rel = t - base;
-    if (rel < 0) return 0u;
-    const int64_t q = rel / W;
-    return q + 1 >= (int64_t)ng ? ng : (uint32_t)(q + 1);
-}
-
-// Same for 0 <= rel < 2^31 and W < 2^31: the high half of rel * ceil(2^32 / W)
-// is the quotient or one more; one multiply corrects it.
-__device__ __forceinline__ uint32_t edges_le32(int64_t rel64, uint32_t W, uint32_t magic, uint32_t ng)
-{
-    if (rel64 < 0) return 0u;
-    const uint32_t rel = (uint32_t)rel64;
-    uint32_t q = __umulhi(rel, magic);
-    if (q * W > rel) --q;
-    return q + 1 >= ng ? ng : q + 1;
-}
-
 __device__ __forceinline__ void fill_edges(uint32_t *e, uint32_t P, uint32_t p, uint32_t g0, uint32_t g1,
                                            uint32_t v)
 {
@@ -394,194 +372,177 @@ __device__ __forceinline__ void fill_edges(uint32_t *e, uint32_t P, uint32_t p, 
 }
 
 // Edges after a PMT's last hit, and all edges of the empty PMTs that follow.
-__device__ __noinline__ void fill_run_end(uint32_t *e_lo, uint32_t *e_hi, const uint64_t *poff, uint32_t P,
-                                          uint32_t NG, uint32_t p, uint32_t lo_to, uint32_t hi_to, uint32_t ep)
+__device__ __noinline__ void fill_run_end(uint32_t *edge, const uint64_t *poff, uint32_t P, uint32_t NE, uint32_t p,
+                                          uint32_t from, uint32_t ep)
 {
-    fill_edges(e_lo, P, p, lo_to, NG, ep);
-    fill_edges(e_hi, P, p, hi_to, NG, ep);
-    for (uint32_t q = p + 1; q < P && poff[q] == poff[q + 1]; ++q) {
-        fill_edges(e_lo, P, q, 0, NG, ep);
-        fill_edges(e_hi, P, q, 0, NG, ep);
-    }
-}
-
-// All edges of the empty PMTs before the slice's first hit.
-__device__ __noinline__ void fill_leading_empty(uint32_t *e_lo, uint32_t *e_hi, uint32_t P, uint32_t NG, uint32_t p)
-{
-    for (uint32_t q = 0; q < p; ++q) {
-        fill_edges(e_lo, P, q, 0, NG, 0u);
-        fill_edges(e_hi, P, q, 0, NG, 0u);
-    }
+    fill_edges(edge, P, p, from, NE, ep);
+    for (uint32_t q = p + 1; q < P && poff[q] == poff[q + 1]; ++q) fill_edges(edge, P, q, 0, NE, ep);
 }
 
 constexpr int kBoundsThreads = 256;
 constexpr int kBoundsUnroll = 4;
 constexpr uint32_t kBoundsPerWarp = kChunkHits / (kBoundsThreads / 32);    // consecutive hits per warp
+static_assert(kBoundsPerWarp == 31 * kBoundsUnroll, "a warp steps through 31 hits at a time");
 
-// Structure pass over one chunk of a wide slice: the same checks of the CSR
-// layout and time order, then each valid hit counted in its time bucket.
-__device__ __noinline__ void bounds_wide_chunk(const SliceDesc &d, uint64_t first)
+// A slice's tile edges in time order.  Tile g's staged range starts at x = g W
+// (its lo edge; x = t - (t0 - H)) and ends at g W + D, D = 2H + W = a W + b
+// (its hi edge), so with x = q W + r the edges at or before x are
+// 2 q + 1 + (r >= b): edge 2g is tile g's lo edge, edge 2 (g + a) + 1 its hi
+// edge (the odd ones below 2a + 1 are no tile's).  One number per hit then
+// tells both, and passing either kind of edge is the same store.
+struct EdgeCount {
+    uint32_t W, magic, b, NE;
+    __device__ __forceinline__ explicit EdgeCount(const SliceDesc &d)
+        : W((uint32_t)d.tile_w), magic(d.w_magic), b(d.edge_b), NE(d.n_edges)
+    {
+    }
+    // x below 2^31: the high half of x * ceil(2^32 / W) is the quotient or
+    // one more
+    __device__ __forceinline__ uint32_t of32(int32_t x) const
+    {
+        if (x < 0) return 0u;
+        uint32_t q = __umulhi((uint32_t)x, magic);
+        uint32_t r = (uint32_t)x - q * W;
+        if ((int32_t)r < 0) --q, r += W;
+        return min(2u * q + (r >= b ? 2u : 1u), NE);
+    }
+    __device__ __forceinline__ uint32_t of64(int64_t x) const
+    {
+        if (x < 0) return 0u;
+        const int64_t q = x / (int64_t)W;
+        if (q >= (int64_t)(NE / 2u)) return NE;
+        return min(2u * (uint32_t)q + (x - q * (int64_t)W >= (int64_t)b ? 2u : 1u), NE);
+    }
+};
+
+// Hit li of a slice where something other than a tile edge happens: the
+// first or last hit of a PMT's run or of the slice, an out-of-range time, a
+// step back.  It looks at the hit and its predecessor again (a run has
+// thousands of hits, so few come here).
+__device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
 {
-    const uint32_t lane = lane_id(), P = d.n_pmt;
+    const SliceDesc &d = *dp;
+    const uint32_t P = d.n_pmt, NE = d.n_edges;
+    const uint64_t *poff = d.pmt_off;
     const uint64_t n_hits = d.n_hits;
+    const trig_hit h = load_hit(d.hits + li);
+    trig_hit l = h;
+    if (li > 0) l = load_hit(d.hits + li - 1);
+    const uint32_t p = h.pmt, pl = l.pmt;
+    const bool is_first = li == 0 || pl != p, narrow = !d.wide;
+    uint32_t e = 0, el = 0;
+    if (narrow) {
+        const EdgeCount ec(d);
+        const int64_t x0 = d.t0 - (int64_t)d.halo;
+        e = ec.of64(h.t_ns - x0);
+        el = ec.of64(l.t_ns - x0);
+    }
+    uint32_t bad = 0;
+    if (is_first && li > 0 && pl < P) {
+        // hit li - 1 was the last of PMT pl's run
+        if (poff[pl + 1] != li) bad |= TRIG_FLAG_BAD_PMT;
+        if (narrow) fill_run_end(d.edge, poff, P, NE, pl, el, (uint32_t)li);
+    }
+    if (p >= P) bad |= TRIG_FLAG_BAD_PMT;
+    else {
+        if (is_first && poff[p] != li) bad |= TRIG_FLAG_BAD_PMT;
+        if (li + 1 == n_hits && (poff[p + 1] != n_hits || poff[P] != n_hits)) bad |= TRIG_FLAG_BAD_PMT;
+    }
+    if (h.t_ns < d.in_lo || h.t_ns >= d.in_hi) bad |= TRIG_FLAG_OUT_OF_RANGE;
+    if (!is_first && l.t_ns > h.t_ns) bad |= TRIG_FLAG_UNSORTED;
+    if (bad) {
+        report(d, bad);
+        return;
+    }
+    if (!narrow) {
+        atomicAdd(&d.bkt_cnt[bkt_index(d, h.t_ns)], 1u);
+        return;
+    }
+    fill_edges(d.edge, P, p, is_first ? 0u : el, e, (uint32_t)li);
+    if (li + 1 == n_hits) fill_run_end(d.edge, poff, P, NE, p, e, (uint32_t)n_hits);
+    if (li == 0)
+        for (uint32_t q = 0; q < p; ++q) fill_edges(d.edge, P, q, 0, NE, 0u);       // empty PMTs before the first hit
+}
+
+// Chunks [c, c_end) of one slice, block-wide.  A warp takes 31 new hits per
+// step: lane 0 holds the hit before them, so every other lane's predecessor
+// is its neighbour's and nothing is carried from step to step.  A lane whose
+// hit has its predecessor's PMT and edge count, in order and in range, is
+// done after that comparison; one that passes a tile edge writes its index.
+// Bound by instruction issue (nearly every step of 31 hits has a lane on the
+// edge path), then by HBM: the 64 slices of both towers (205 M hits) take
+// 0.95 ms, 1.42 with two edge counts per hit carried along walks of 512
+// hits; one 320 k-hit slice 8 us, 13 before.
+template <bool WIDE, bool S32>
+__device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, uint32_t c_end)
+{
+    using T = std::conditional_t<S32, uint32_t, int64_t>;
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, P = d.n_pmt;
+    const uint32_t n_hits = (uint32_t)d.n_hits;                 // below 2^32 - 16
     const trig_hit *__restrict__ hits = d.hits;
-    const uint64_t *__restrict__ poff = d.pmt_off;
-    for (uint32_t k0 = 0; k0 < kChunkHits; k0 += kBoundsThreads) {
-        const uint64_t li = first + k0 + threadIdx.x;
-        const bool valid = li < n_hits;
-        trig_hit h;
-        if (valid) h = load_hit(hits + li);
-        else h.t_ns = 0, h.pmt = 0xffff;
-        const uint32_t p = h.pmt;
-        const int64_t t = h.t_ns;
-        uint32_t pp = __shfl_up_sync(0xffffffffu, p, 1);
-        int64_t tp = __shfl_up_sync(0xffffffffu, t, 1);
-        uint32_t pn = __shfl_down_sync(0xffffffffu, p, 1);
-        if (!valid) continue;
-        if (lane == 0 && li > 0) {
-            const trig_hit q = load_hit(hits + li - 1);
-            pp = q.pmt;
-            tp = q.t_ns;
+    const int64_t in_lo = d.in_lo;
+    const T in_span = (T)(d.in_hi - in_lo);
+    const T x0 = (T)(d.t0 - (int64_t)d.halo - in_lo);           // the first edge, from in_lo
+    const EdgeCount ec(d);
+    for (; c < c_end; ++c) {
+        const uint32_t wbase = (c - d.chunk0) * kChunkHits + warp * kBoundsPerWarp;
+        if (wbase >= n_hits) continue;
+        uint4 v[kBoundsUnroll];
+        uint32_t special = 0;
+#pragma unroll
+        for (int u = 0; u < kBoundsUnroll; ++u) {
+            const uint32_t li = wbase + u * 31 + lane - 1u;      // wraps to 2^32 - 1 before the first hit
+            v[u] = li < n_hits ? __ldg(reinterpret_cast<const uint4 *>(hits + li)) : make_uint4(0, 0, 0xffffu, 0);
         }
-        if (lane == 31 && li + 1 < n_hits) pn = hits[li + 1].pmt;
-        const bool is_first = li == 0 || pp != p;
-        const bool is_last = li + 1 == n_hits || pn != p;
-        uint32_t bad = 0;
-        if (p >= P) bad |= TRIG_FLAG_BAD_PMT;
-        else {
-            if (is_first && poff[p] != li) bad |= TRIG_FLAG_BAD_PMT;
-            if (is_last && poff[p + 1] != li + 1) bad |= TRIG_FLAG_BAD_PMT;
-            if (li + 1 == n_hits && poff[P] != n_hits) bad |= TRIG_FLAG_BAD_PMT;
+#pragma unroll
+        for (int u = 0; u < kBoundsUnroll; ++u) {
+            const uint32_t li = wbase + u * 31 + lane - 1u;
+            const int64_t t = (int64_t)(((uint64_t)v[u].y << 32) | v[u].x);
+            const uint64_t rel = (uint64_t)t - (uint64_t)in_lo;
+            const T r = (T)rel;
+            const bool valid = li < n_hits, in = S32 ? (rel >> 32) == 0 && r < in_span : rel < (uint64_t)in_span;
+            // PMT label; bits 16, 17: out of range, no such hit
+            const uint32_t p = v[u].z & 0xffffu, pc = valid ? (in ? p : p | 0x10000u) : 0x2ffffu;
+            uint32_t e = 0;
+            if (!WIDE && in) e = S32 ? ec.of32((int32_t)(r - x0)) : ec.of64((int64_t)(r - x0));
+            const uint32_t pcl = __shfl_up_sync(0xffffffffu, pc, 1);
+            const T rl = __shfl_up_sync(0xffffffffu, r, 1);
+            const uint32_t el = WIDE ? 0u : __shfl_up_sync(0xffffffffu, e, 1);
+            if (lane == 0 || !valid) continue;
+            if (pc != pcl || rl > r || !in || li + 1 == n_hits) special |= 1u << u;
+            else if (WIDE) atomicAdd(&d.bkt_cnt[bkt_index(d, t)], 1u);
+            else if (e != el && p < P) fill_edges(d.edge, P, p, el, e, li);
         }
-        if (t < d.in_lo || t >= d.in_hi) bad |= TRIG_FLAG_OUT_OF_RANGE;
-        if (!is_first && tp > t) bad |= TRIG_FLAG_UNSORTED;
-        if (bad) {
-            report(d, bad);
-            continue;
-        }
-        atomicAdd(&d.bkt_cnt[bkt_index(d, t)], 1u);
+        for (; special; special &= special - 1u)
+            bounds_special(&d, wbase + (__ffs(special) - 1) * 31 + lane - 1u);
     }
 }
 
-// One read of every hit.  Per hit: CSR layout and time order are checked
-// (run starts and ends against pmt_off, neighbours from adjacent lanes), and
-// the tile edges passed between the previous hit of the PMT and this one
-// get this hit's index.
-__global__ void __launch_bounds__(kBoundsThreads, 4) k_bounds(const BatchHeader *__restrict__ hdr,
+// Slices longer than about two seconds, in 64-bit times.
+__device__ __noinline__ void bounds_chunks_long(const SliceDesc &d, uint32_t c, uint32_t c_end)
+{
+    bounds_chunks<false, false>(d, c, c_end);
+}
+
+// Structure pass: one read of every hit.  The CSR layout and the time order
+// are checked (run starts and ends against pmt_off, each hit against its
+// predecessor); narrow slices record where each PMT's stream crosses the
+// tile edges, wide ones count their time buckets.  Each block takes a
+// contiguous share of the chunks, so it looks its slice up once.
+__global__ void __launch_bounds__(kBoundsThreads, 3) k_bounds(const BatchHeader *__restrict__ hdr,
                                                            const SliceDesc *__restrict__ desc)
 {
     const uint32_t n_slices = hdr->n_slices, n_chunks = hdr->n_chunks;
-    const uint32_t lane = lane_id();
-    for (uint32_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-        const uint32_t s = find_slice_by_chunk(desc, n_slices, c);
+    uint32_t c = (uint32_t)((uint64_t)n_chunks * blockIdx.x / gridDim.x);
+    const uint32_t c1 = (uint32_t)((uint64_t)n_chunks * (blockIdx.x + 1) / gridDim.x);
+    if (c >= c1) return;
+    for (uint32_t s = find_slice_by_chunk(desc, n_slices, c); c < c1; ++s) {
         const SliceDesc &d = desc[s];
-        const uint32_t P = d.n_pmt, NG = d.n_tiles;
-        const int64_t W = d.tile_w;
-        const uint32_t W32 = (uint32_t)W, magic = d.w_magic;
-        const bool span32 = d.span32 != 0;
-        const int64_t base_lo = d.t0 - (int64_t)d.halo;             // lo edge g: t0 - H + g W
-        const int64_t base_hi = d.t0 + (int64_t)d.halo + W;         // hi edge g: t0 + H + (g + 1) W
-        const uint64_t first = (uint64_t)(c - d.chunk0) * kChunkHits;
-        const uint64_t n_hits = d.n_hits;
-        const trig_hit *__restrict__ hits = d.hits;
-        const uint64_t *__restrict__ poff = d.pmt_off;
-        uint32_t *__restrict__ e_lo = d.e_lo;
-        uint32_t *__restrict__ e_hi = d.e_hi;
-        const int64_t in_lo = d.in_lo, in_hi = d.in_hi;
-        if (d.wide) {
-            bounds_wide_chunk(d, first);
-            continue;
-        }
-        // tile edges at or below t: lo edge g at base_lo + g W, hi edge g at
-        // base_lo + D + g W with D = 2H + W = a W + b; with t - base_lo =
-        // q W + r the hi count is q - a + 1 - (r < b), so one division
-        // serves both
-        const uint32_t D32 = 2u * d.halo + W32, a32 = span32 ? D32 / W32 : 0u, b32 = D32 - a32 * W32;
-        auto edges = [&](int64_t t, uint32_t &lo, uint32_t &hi) {
-            if (span32) {
-                const int64_t x64 = t - base_lo;
-                if (x64 < 0) {
-                    lo = hi = 0u;
-                    return;
-                }
-                const uint32_t x = (uint32_t)x64;
-                uint32_t q = __umulhi(x, magic);
-                if (q * W32 > x) --q;
-                const uint32_t r = x - q * W32;
-                lo = q + 1 >= NG ? NG : q + 1;
-                const int32_t qh = (int32_t)q - (int32_t)a32 + 1 - (r < b32 ? 1 : 0);
-                hi = qh <= 0 ? 0u : ((uint32_t)qh >= NG ? NG : (uint32_t)qh);
-            } else {
-                lo = edges_le64(t, base_lo, W, NG);
-                hi = edges_le64(t, base_hi, W, NG);
-            }
-        };
-        // each warp walks kBoundsPerWarp consecutive hits, 32 at a time: a
-        // hit's predecessor is the previous lane's (lane 0: the previous
-        // step's lane 31; the first step loads it).  The first hit of a run
-        // closes the previous PMT's run.
-        const uint32_t warp = threadIdx.x >> 5;
-        const uint64_t wbase = first + (uint64_t)warp * kBoundsPerWarp;
-        uint32_t c_p = 0xffffu, c_lo = 0u, c_hi = 0u;
-        int64_t c_t = 0;
-        if (wbase > 0 && wbase <= n_hits) {
-            const trig_hit q = load_hit(hits + wbase - 1);
-            c_p = q.pmt;
-            c_t = q.t_ns;
-            edges(c_t, c_lo, c_hi);
-        }
-        for (uint32_t k0 = 0; k0 < kBoundsPerWarp; k0 += 32 * kBoundsUnroll) {
-            trig_hit h[kBoundsUnroll];
-#pragma unroll
-            for (int u = 0; u < kBoundsUnroll; ++u) {
-                const uint64_t li = wbase + k0 + u * 32 + lane;
-                if (li < n_hits) h[u] = load_hit(hits + li);
-                else h[u].t_ns = 0, h[u].pmt = 0xffff;
-            }
-#pragma unroll
-            for (int u = 0; u < kBoundsUnroll; ++u) {
-                const uint64_t li = wbase + k0 + u * 32 + lane;
-                const bool valid = li < n_hits;
-                const uint32_t p = h[u].pmt;
-                const int64_t t = h[u].t_ns;
-                uint32_t lo_to = 0u, hi_to = 0u;
-                if (valid) edges(t, lo_to, hi_to);
-                uint32_t pp = __shfl_up_sync(0xffffffffu, p, 1);
-                int64_t tp = __shfl_up_sync(0xffffffffu, t, 1);
-                uint32_t lo_p = __shfl_up_sync(0xffffffffu, lo_to, 1);
-                uint32_t hi_p = __shfl_up_sync(0xffffffffu, hi_to, 1);
-                if (lane == 0) {
-                    pp = c_p;
-                    tp = c_t;
-                    lo_p = c_lo;
-                    hi_p = c_hi;
-                }
-                c_p = __shfl_sync(0xffffffffu, p, 31);
-                c_t = __shfl_sync(0xffffffffu, t, 31);
-                c_lo = __shfl_sync(0xffffffffu, lo_to, 31);
-                c_hi = __shfl_sync(0xffffffffu, hi_to, 31);
-                if (!valid) continue;
-                const bool is_first = li == 0 || pp != p;
-                uint32_t bad = 0;
-                if (is_first && li > 0 && pp < P) {
-                    // hit li - 1 was the last of PMT pp's run
-                    if (poff[pp + 1] != li) bad |= TRIG_FLAG_BAD_PMT;
-                    fill_run_end(e_lo, e_hi, poff, P, NG, pp, lo_p, hi_p, (uint32_t)li);
-                }
-                if (p >= P) bad |= TRIG_FLAG_BAD_PMT;
-                else {
-                    if (is_first && poff[p] != li) bad |= TRIG_FLAG_BAD_PMT;
-                    if (li + 1 == n_hits && (poff[p + 1] != n_hits || poff[P] != n_hits)) bad |= TRIG_FLAG_BAD_PMT;
-                }
-                if (t < in_lo || t >= in_hi) bad |= TRIG_FLAG_OUT_OF_RANGE;
-                if (!is_first && tp > t) bad |= TRIG_FLAG_UNSORTED;
-                if (bad) { report(d, bad); continue; }
-                fill_edges(e_lo, P, p, is_first ? 0u : lo_p, lo_to, (uint32_t)li);
-                fill_edges(e_hi, P, p, is_first ? 0u : hi_p, hi_to, (uint32_t)li);
-                if (li + 1 == n_hits) fill_run_end(e_lo, e_hi, poff, P, NG, p, lo_to, hi_to, (uint32_t)(li + 1));
-                if (li == 0 && p > 0) fill_leading_empty(e_lo, e_hi, P, NG, p);
-            }
-        }
+        const uint32_t end = min(c1, s + 1 < n_slices ? desc[s + 1].chunk0 : n_chunks);
+        if (d.wide) bounds_chunks<true, false>(d, c, end);
+        else if (d.span32) bounds_chunks<false, true>(d, c, end);
+        else bounds_chunks_long(d, c, end);
+        c = end;
     }
 }
 
@@ -2157,9 +2118,8 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             const long long tp0 = clock64();
 #endif
             uint32_t g = 0, P = 0, mode = 2, lo_t = 0, span = 0;
-            uint64_t ra[R];
-            uint32_t rl[R];
-            uint64_t tot = 0, rlo = 0;
+            uint32_t ra[R], rl[R];                  // hit indices are below 2^32 - 16
+            uint32_t tot = 0, rlo = 0;
             bool wide = false;
             if (item < n_items) {
                 // items arrive in increasing order: walk the slice index forward
@@ -2187,8 +2147,8 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                     }
                 } else {
                     // the PMTs' runs [lb(B_g - H), lb(B_{g+1} + H)), P <= 32 R
-                    const uint32_t *elo = d->e_lo + (size_t)g * P;
-                    const uint32_t *ehi = d->e_hi + (size_t)g * P;
+                    const uint32_t *elo = d->edge + (size_t)(2u * g) * P;
+                    const uint32_t *ehi = d->edge + (size_t)(2u * (g + d->edge_a) + 1u) * P;
                     const uint64_t *poff = d->pmt_off;
                     lo_t = d->halo;
                     span = (uint32_t)d->tile_w + 2u * d->halo;
@@ -2196,25 +2156,25 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
 #pragma unroll
                         for (int r = 0; r < R; ++r) {
                             const uint32_t p = r * 32 + lane;
-                            uint64_t a = 0, e = 0, sp_ = 0, ep_ = 0;
+                            uint32_t a = 0, e = 0, sp_ = 0, ep_ = 0;
                             if (p < P) {
                                 a = __ldg(elo + p);
                                 e = __ldg(ehi + p);
-                                sp_ = __ldg(poff + p);
-                                ep_ = __ldg(poff + p + 1);
+                                sp_ = (uint32_t)__ldg(poff + p);
+                                ep_ = (uint32_t)__ldg(poff + p + 1);
                                 a = min(max(a, sp_), ep_);
                                 e = min(max(e, a), ep_);
                             }
                             ra[r] = a;
-                            rl[r] = (uint32_t)(e - a);
+                            rl[r] = e - a;
                             tot += e - a;
                             rlo += a - sp_;
                         }
                     }
-                    tot = warp_sum_u64(tot);
-                    rlo = warp_sum_u64(rlo);
+                    tot = __reduce_add_sync(0xffffffffu, tot);
+                    rlo = __reduce_add_sync(0xffffffffu, rlo);
                 }
-                mode = bad ? 2u : (tot > (uint64_t)CAP ? 1u : (tot == 0 ? 2u : 0u));
+                mode = bad ? 2u : (tot > (uint32_t)CAP ? 1u : (tot == 0 ? 2u : 0u));
             }
             uint32_t next = 0;
             if (item < n_items) {
@@ -2254,26 +2214,25 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 info[b].item = (int32_t)item;
                 info[b].slice = s;
                 info[b].g = g;
-                info[b].n = (uint32_t)min(tot, (uint64_t)CAP);
-                info[b].rank_lo = (uint32_t)rlo;
+                info[b].n = min(tot, (uint32_t)CAP);
+                info[b].rank_lo = rlo;
                 info[b].mode = mode;
                 info[b].lo_t = lo_t;
                 info[b].span = span;
-                if (mode == 0) mbar_arrive_expect_tx(&full_bar[b], (uint32_t)tot * 16u);
+                if (mode == 0) mbar_arrive_expect_tx(&full_bar[b], tot * 16u);
                 else mbar_arrive(&full_bar[b]);
             }
             __syncwarp();
             if (mode == 0 && wide) {
-                if (lane == 0 && CHECK(7, rlo + tot, d->n_hits + 1))
-                    bulk_g2s(stage_of(b), d->tbuf + rlo, (uint32_t)tot * 16u, &full_bar[b]);
+                if (lane == 0 && CHECK(7, (uint64_t)rlo + tot, d->n_hits + 1))
+                    bulk_g2s(stage_of(b), d->tbuf + rlo, tot * 16u, &full_bar[b]);
             } else if (mode == 0) {
                 uint32_t dst = 0;
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const uint32_t len = rl[r];
-                    const uint64_t a = ra[r];
+                    const uint32_t len = rl[r], a = ra[r];
                     const uint32_t incl = warp_incl_scan(len);
-                    if (len && CHECK(6, dst + incl, CAP + 1) && CHECK(7, a + len, d->n_hits + 1))
+                    if (len && CHECK(6, dst + incl, CAP + 1) && CHECK(7, (uint64_t)a + len, d->n_hits + 1))
                         bulk_g2s(stage_of(b) + 2 * (size_t)(dst + incl - len), d->hits + a, len * 16u, &full_bar[b]);
                     dst += __shfl_sync(0xffffffffu, incl, 31);
                 }
@@ -2594,21 +2553,21 @@ __global__ void __launch_bounds__(256) k_wwrite(const BatchHeader *__restrict__ 
 // ---------------------------------------------------------------- k_wcount
 
 // Hit rank of time x in PMT p's stream, narrowed by the tile edges the
-// structure pass recorded: x in tile g's core lies between the PMT's
-// offsets at B_g - H and B_{g+1} + H, so the binary search covers a handful
-// of hits.  Outside the slice the first or last tile's outer edge bounds it.
+// structure pass recorded: x between the edges B_g - H and B_{g+1} - H lies
+// between the PMT's offsets there, so the binary search covers a handful of
+// hits.  Outside the edges the first or last one bounds it.
 __device__ __forceinline__ uint64_t rank_in_pmt(const SliceDesc &d, uint32_t p, int64_t x, uint64_t sp, uint64_t ep)
 {
-    const int64_t W = d.tile_w;
-    const int64_t rel = x - d.t0;
-    int64_t g = rel < 0 ? 0 : rel / W;
-    if (g >= (int64_t)d.n_tiles) g = (int64_t)d.n_tiles - 1;
-    const int64_t Bg = d.t0 + g * W;
-    const size_t at = (size_t)g * d.n_pmt + p;
+    const int64_t rel = x - (d.t0 - (int64_t)d.halo);
     uint64_t lo = sp, hi = ep;
-    const uint64_t a = d.e_lo[at], b = d.e_hi[at];
-    if (x >= Bg - (int64_t)d.halo) lo = max(lo, min(a, ep));
-    if (x <= Bg + W + (int64_t)d.halo) hi = min(hi, max(b, lo));
+    if (rel >= 0) {
+        const int64_t g = min(rel / d.tile_w, (int64_t)d.n_tiles);
+        const uint32_t *at = d.edge + (size_t)(2 * g) * d.n_pmt + p;
+        lo = max(lo, min((uint64_t)at[0], ep));
+        if (g < (int64_t)d.n_tiles) hi = min(hi, max((uint64_t)at[2 * (size_t)d.n_pmt], lo));
+    } else if (d.n_tiles) {
+        hi = min(hi, max((uint64_t)d.edge[p], lo));
+    }
     return lb_time(d.hits, lo, hi, x);
 }
 
@@ -3099,7 +3058,7 @@ cudaError_t launch_batch(BatchHeader *d_hdr, SliceDesc *d_desc, uint32_t n_slice
     mark(0);
     k_prep<<<any_wide ? sms : 1, 256, 0, st>>>(d_hdr, d_desc);
     mark(1);
-    k_bounds<<<sms * 8, kBoundsThreads, 0, st>>>(d_hdr, d_desc);
+    k_bounds<<<sms * 6, kBoundsThreads, 0, st>>>(d_hdr, d_desc);
     nl += 2;
     if (rows) {
         k_rank0<<<n_slices, 256, 0, st>>>(d_hdr, d_desc);
