@@ -470,7 +470,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
     if (shape_out) *shape_out = cfg;
     size_t off = align256(sizeof(BatchHeader));
     off += align256(sizeof(SliceDesc) * n);
-    uint32_t items = 0, chunks = 0;
+    uint32_t items = 0, chunks = 0, fins = 0;
     max_pmt = 0;
     smem_dt = true;
     any_wide = false;
@@ -569,18 +569,12 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
         off += align256((size_t)d.n_tiles * 4);
         d.tile_rank = reinterpret_cast<uint32_t *>(base + off);
         off += align256((size_t)d.n_tiles * 4);
-        d.tile_out = reinterpret_cast<uint32_t *>(base + off);
-        off += align256((size_t)d.n_tiles * 4);
-        d.tile_nwin = reinterpret_cast<uint32_t *>(base + off);
-        off += align256((size_t)d.n_tiles * 4);
-        d.tile_wout = reinterpret_cast<uint32_t *>(base + off);
-        off += align256((size_t)d.n_tiles * 4);
+        d.fin0 = fins;
+        fins += std::max(1u, (d.n_tiles + kFinTiles - 1) / kFinTiles);
         d.stage = reinterpret_cast<trig_trigger *>(base + off);
         off += align256((size_t)x.n_hits * sizeof(trig_trigger));
         d.wrank = reinterpret_cast<uint32_t *>(base + off);
         off += align256((size_t)x.n_hits * 8);
-        d.win_r = reinterpret_cast<uint32_t *>(base + off);
-        off += align256((size_t)x.win_cap * 8);
         d.triggers = x.triggers;
         d.trig_cap = x.trig_cap;
         d.windows = x.windows;
@@ -616,6 +610,10 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
     hdr.dense = dense ? 1u : 0u;
     hdr.n_items = items;
     hdr.n_chunks = chunks;
+    hdr.n_fin = fins;
+    hdr.fin = reinterpret_cast<unsigned char *>(base + off);
+    off += align256((size_t)fins * kFinStateBytes);
+    for (uint32_t s = 0; s < n; ++s) desc[s].fin = hdr.fin + (size_t)desc[s].fin0 * kFinStateBytes;
     hdr.wait_ns = g_wait_ns.load();
     hdr.stall = g_stall.load();
     bytes = off;
@@ -675,7 +673,6 @@ struct GraphKey {
 
 struct GraphEntry {
     cudaGraphExec_t exec = nullptr;
-    unsigned char *pinned = nullptr;     // header + descriptors, copied by the graph's first node
     std::vector<unsigned char> plan;     // the plan bytes (hash collisions are checked against it)
     cudaEvent_t done = nullptr;          // last replay finished
     bool launched = false;
@@ -700,7 +697,6 @@ static void drop_graph(GraphEntry &ge)
     if (ge.launched) cudaEventSynchronize(ge.done);
     if (ge.exec) cudaGraphExecDestroy(ge.exec);
     if (ge.done) cudaEventDestroy(ge.done);
-    if (ge.pinned) cudaFreeHost(ge.pinned);
     ge = GraphEntry{};
 }
 
@@ -733,9 +729,7 @@ static int run_graph(const Plan &pl, void *scratch, cudaStream_t st)
             g_graphs.erase(key);
             return rc;
         };
-        if ((e = cudaMallocHost(&ge.pinned, host.size()))) return forget(cuda_fail(e, "graph: pinned descriptors"));
         if ((e = cudaEventCreateWithFlags(&ge.done, cudaEventDisableTiming))) return forget(cuda_fail(e, "graph: event"));
-        std::memcpy(ge.pinned, host.data(), host.size());
         ge.plan = host;
         // capture on a private stream (the caller's may be the legacy default
         // stream, which cannot capture); replays go to the caller's stream
@@ -747,13 +741,9 @@ static int run_graph(const Plan &pl, void *scratch, cudaStream_t st)
             return forget(cuda_fail(e, "graph: capture"));
         }
         uint64_t nl = 0;
-        cudaError_t ce = cudaMemcpyAsync(scratch, ge.pinned, host.size(), cudaMemcpyHostToDevice, cap);
-        if (!ce)
-            ce = launch_batch(reinterpret_cast<BatchHeader *>(scratch),
-                              reinterpret_cast<SliceDesc *>((char *)scratch + align256(sizeof(BatchHeader))),
-                              pl.hdr.n_slices, pl.max_pmt, pl.smem_dt, pl.any_wide, pl.any_events,
-                              pl.hdr.any_ext != 0, pl.hdr.dense != 0, cfg, cap, &nl,
-                              false);
+        cudaError_t ce = launch_batch(pl.hdr, pl.desc.data(), reinterpret_cast<BatchHeader *>(scratch),
+                                      reinterpret_cast<SliceDesc *>((char *)scratch + align256(sizeof(BatchHeader))),
+                                      pl.max_pmt, pl.smem_dt, cfg, cap, &nl, false);
         ge.launches = nl;
         e = cudaStreamEndCapture(cap, &graph);
         cudaStreamDestroy(cap);
@@ -836,10 +826,6 @@ static int run_plan(const Plan &pl, void *scratch, size_t scratch_bytes, cudaStr
     if (scratch_bytes < pl.bytes) return fail(TRIG_EINVAL, "scratch too small (see trig_batch_scratch_bytes)");
     if ((flags & TRIG_RUN_GRAPH) && (flags & TRIG_RUN_TIMED)) return fail(TRIG_EINVAL, "TIMED runs cannot use GRAPH");
     if ((flags & TRIG_RUN_GRAPH) && !rows) return run_graph(pl, scratch, st);
-    std::vector<unsigned char> host;
-    pack_plan(pl, host);
-    cudaError_t e = cudaMemcpyAsync(scratch, host.data(), host.size(), cudaMemcpyHostToDevice, st);
-    if (e) return cuda_fail(e, "copy descriptors");
     TimedRun tr{};
     const bool timed = (flags & TRIG_RUN_TIMED) && !rows;
     if (timed) {
@@ -847,11 +833,9 @@ static int run_plan(const Plan &pl, void *scratch, size_t scratch_bytes, cudaStr
         if (rc) return rc;
     }
     uint64_t nl = 0;
-    e = launch_batch(reinterpret_cast<BatchHeader *>(scratch),
-                     reinterpret_cast<SliceDesc *>((char *)scratch + align256(sizeof(BatchHeader))), pl.hdr.n_slices,
-                     pl.max_pmt, pl.smem_dt, pl.any_wide, pl.any_events, pl.hdr.any_ext != 0, pl.hdr.dense != 0, cfg,
-                     st, &nl, rows,
-                     timed ? tr.ev : nullptr);
+    cudaError_t e = launch_batch(pl.hdr, pl.desc.data(), reinterpret_cast<BatchHeader *>(scratch),
+                                 reinterpret_cast<SliceDesc *>((char *)scratch + align256(sizeof(BatchHeader))),
+                                 pl.max_pmt, pl.smem_dt, cfg, st, &nl, rows, timed ? tr.ev : nullptr);
     g_launches += nl;
     if (timed) {
         std::lock_guard<std::mutex> lk(g_time_mu);
@@ -1072,23 +1056,20 @@ extern "C" int trig_batch_run_noalloc(const trig_slice_dev *slices, uint32_t n_s
     e = static_scratch(&scratch, &cap);
     if (e) return cuda_fail(e, "trig_batch_run_noalloc: static scratch address");
     const TileConfig cfg = current_cfg();
-    NoallocPlan plan;
+    BatchHeader hdr;
+    SliceDesc desc[TRIG_NOALLOC_MAX_SLICES];
     size_t bytes = 0;
     uint32_t max_pmt = 0;
     bool smem_dt = true, any_wide = false;
     TileConfig shape{};
-    int rc = plan_into(slices, n_slices, (uintptr_t)scratch, cfg, plan.hdr, plan.desc, bytes, max_pmt, smem_dt,
+    int rc = plan_into(slices, n_slices, (uintptr_t)scratch, cfg, hdr, desc, bytes, max_pmt, smem_dt,
                        any_wide, &shape);
     if (rc) return rc;
     if (bytes > cap) return fail(TRIG_ECAPACITY, "trig_batch_run_noalloc: batch needs more than TRIG_NOALLOC_SCRATCH_BYTES of scratch");
-    plan.n = n_slices;
     BatchHeader *d_hdr = reinterpret_cast<BatchHeader *>(scratch);
     SliceDesc *d_desc = reinterpret_cast<SliceDesc *>((char *)scratch + align256(sizeof(BatchHeader)));
-    e = launch_put_plan(plan, d_hdr, d_desc, st);
-    if (e) return cuda_fail(e, "trig_batch_run_noalloc: descriptors");
-    uint64_t nl = 1;
-    e = launch_batch(d_hdr, d_desc, n_slices, max_pmt, smem_dt, any_wide, false, plan.hdr.any_ext != 0,
-                     plan.hdr.dense != 0, shape, st, &nl, false);
+    uint64_t nl = 0;
+    e = launch_batch(hdr, desc, d_hdr, d_desc, max_pmt, smem_dt, shape, st, &nl, false);
     g_launches += nl;
     if (e) return cuda_fail(e, "trig_batch_run_noalloc: launch");
     return TRIG_OK;

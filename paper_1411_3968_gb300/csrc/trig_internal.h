@@ -92,13 +92,10 @@ struct SliceDesc {
     trig_trigger *stage;    // [n_hits] fired seeds at their merged rank
     uint32_t *wrank;        // [n_hits][2] beside each staged fired seed: the merged ranks of the
                             //   first hit at or after t - win_half and of the first after t + win_half
-    uint32_t *win_r;        // [win_cap][2] a window's first-hit rank (from its first trigger)
-                            //   and its one-past-last rank (from its last trigger)
     uint32_t *tile_nfired;  // [NG]
     uint32_t *tile_rank;    // [NG] merged rank of the tile's first core hit
-    uint32_t *tile_out;     // [NG] exclusive prefix of tile_nfired
-    uint32_t *tile_nwin;    // [NG] window heads among the tile's triggers
-    uint32_t *tile_wout;    // [NG] exclusive prefix of tile_nwin
+    unsigned char *fin;     // this slice's chunks of tiles (FinState each), of the batch's
+    uint32_t fin0;          // first of them in the batch
     trig_trigger *triggers;
     uint64_t trig_cap;
     trig_window *windows;
@@ -128,6 +125,9 @@ struct BatchHeader {
     uint32_t any_ext;       // a slice uses level 0, seed rule 1 or the distinct count
     uint32_t dense;         // a slice expects kDenseKeys or more keys per causal scan range
     uint32_t stall;         // test control: the tile pass's stagers fill nothing, so its waits run out
+    uint32_t n_fin;         // chunks of kFinTiles tiles, at least one for each slice
+    uint32_t fin_queue;     // next of them
+    unsigned char *fin;     // their states
     uint64_t wait_ns;       // limit of every device wait (ns); a wait that runs out sets TRIG_FLAG_TIMEOUT
 };
 
@@ -136,6 +136,10 @@ constexpr uint64_t kDefaultWaitNs = 1000000000ull;     // one second
 // Expected keys in a seed's scan range (2H + 1 ns at the slice's mean rate)
 // from which the causal count gives each seed a warp instead of 4 lanes.
 constexpr double kDenseKeys = 600.0;
+
+constexpr uint32_t kFinTiles = 32;          // tiles whose seeds a block of k_final takes at a time
+constexpr uint32_t kFinStateBytes = 104;    // what such a chunk publishes
+constexpr uint32_t kPutSlices = 64;         // descriptors a launch of k_put carries at most
 
 constexpr uint32_t kChunkHits = 992;        // structure-pass chunk: 8 warps of 4 x 31 hits
 
@@ -159,24 +163,22 @@ inline bool valid_tile_shape(uint32_t cap, uint32_t warps)
 }
 constexpr uint32_t kMaxTilesPerSlice = 1u << 20;
 
-// Enqueues the batch pipeline; header/desc already copied to device scratch.
-constexpr int kPipelineKernels = 15;
+constexpr int kPipelineKernels = 11;
 extern const char *const kKernelNames[kPipelineKernels];
 
-// any_wide: the batch holds a wide slice (the bucket sums, scan and
-// scatter kernels run only then); any_events: a slice extracts events (the
-// halo, event-offset and event-copy kernels run only then); any_ext: a slice
-// uses level 0, seed rule 1 or the distinct count (the tile kernel built
-// with those rules runs, else the one without them); dense: the tile kernel
-// built with a warp per seed in the causal count runs.  ev (optional, kPipelineKernels + 1 events): ev[i]
-// is recorded before pipeline kernel i and ev[kPipelineKernels] after the
-// last one (a kernel that does not run gets an empty interval).
-// *launches is increased by the number of kernels launched.
-cudaError_t launch_batch(BatchHeader *d_hdr, SliceDesc *d_desc, uint32_t n_slices, uint32_t max_pmt,
-                         bool any_smem_dt, bool any_wide, bool any_events, bool any_ext, bool dense,
-                         const TileConfig &cfg,
-                         cudaStream_t st,
-                         uint64_t *launches, bool rows, cudaEvent_t *ev = nullptr);
+// Enqueues the batch pipeline, the copy of its header and descriptors to
+// d_hdr and d_desc included.  hdr.any_wide: the bucket sums, scan and scatter
+// kernels run only then; any_events: the halo, event-offset, event-copy and
+// status kernels run only then; any_ext: the tile kernel built with level 0,
+// seed rule 1 and the distinct count runs, else the one without them; dense:
+// the tile kernel built with a warp per seed in the causal count runs.  ev
+// (optional, kPipelineKernels + 1 events): ev[i] is recorded before pipeline
+// kernel i and ev[kPipelineKernels] after the last one (a kernel that does
+// not run gets an empty interval).  *launches is increased by the number of
+// kernels launched.
+cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHeader *d_hdr, SliceDesc *d_desc,
+                         uint32_t max_pmt, bool any_smem_dt, const TileConfig &cfg, cudaStream_t st, uint64_t *launches,
+                         bool rows, cudaEvent_t *ev = nullptr);
 
 int device_sm_count();
 
@@ -203,16 +205,5 @@ void count_launches(uint64_t n);
 
 // Address and size of the library's static scratch array on the current device.
 cudaError_t static_scratch(void **ptr, size_t *bytes);
-
-// A no-allocation batch's header and descriptors, passed by value to the
-// kernel that writes them into the static scratch array.
-struct NoallocPlan {
-    BatchHeader hdr;
-    SliceDesc desc[TRIG_NOALLOC_MAX_SLICES];
-    uint32_t n;
-};
-static_assert(sizeof(BatchHeader) % 4 == 0 && sizeof(SliceDesc) % 4 == 0, "copied as 32-bit words");
-static_assert(sizeof(NoallocPlan) <= 32000, "kernel parameter space");
-cudaError_t launch_put_plan(const NoallocPlan &plan, BatchHeader *hdr, SliceDesc *desc, cudaStream_t st);
 
 }  // namespace trig
