@@ -507,6 +507,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
         d.afc_w = det->par.afc_window_ns;
         d.count_distinct = det->par.count_distinct_pmts;
         d.rel = det->dev.rel;
+        d.rel_in_dt = det->par.seed_rule == 1 && det->par.corr_window_ns < (1u << kRelShift) ? 1u : 0u;
         d.win_half = det->par.win_half_ns;
         d.t0 = x.t0_ns;
         d.slice_ns = det->par.slice_ns;

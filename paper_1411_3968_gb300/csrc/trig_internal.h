@@ -38,6 +38,9 @@ struct DetDev {
 constexpr uint8_t kRelFloor = 1;        // another PMT of the same floor (FC)
 constexpr uint8_t kRelAdjacent = 2;     // adjacent PMT: same floor, within sc_dist (SC)
 constexpr uint8_t kRelNextFloor = 4;    // PMT on a consecutive floor of the same tower (AFC)
+// In shared memory the relation sits above the dt entry, which then has
+// kRelShift bits (corr_window_ns below 2^13; the workloads' is 3000).
+constexpr uint32_t kRelShift = 13;
 
 // Per-slice descriptor in device scratch, written by the host each run.
 struct SliceDesc {
@@ -59,6 +62,7 @@ struct SliceDesc {
     uint32_t sc_w, fc_w, afc_w;     // coincidence windows of seed rule 1 (ns)
     uint32_t count_distinct;        // c(s) counts different PMTs (P <= 128)
     const uint8_t *rel;     // [P*P] kRel* bits (seed rule 1)
+    uint32_t rel_in_dt;     // seed rule 1 and every dt below 2^kRelShift
     int64_t t0;
     int64_t slice_ns;
     int64_t in_lo, in_hi;   // accepted hit times [in_lo, in_hi)

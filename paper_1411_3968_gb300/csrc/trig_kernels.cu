@@ -636,55 +636,20 @@ struct ItemInfo {
     uint32_t span;      // length of the staged time range (ns)
 };
 
-// Shared memory of the tile kernel's sorted builds (EXT), in this order: the
-// staging buffers of CAP 16-byte records (two, or one for the 2048-hit tile:
-// its tile pass hands the buffer back once it has read it, so the next
-// tile's copy overlaps the rest of the pass, and two blocks of it then fit
-// on an SM); the tile's packed keys in merged order (+16 bytes: four end keys
-// that the causal count's 16-byte loads may read past the last key); the
-// keys in bucket order (reused for the seed rounds' lists, then the seed
-// list and seed counts); the charges in bucket order and in merged order;
-// the floor of each merged key; the bucket offsets; the seed mask; the PMT
-// tables (floor, row maximum of dt).
-template <int CAP, bool EXT>
+// Shared memory of the tile kernel, in this order: the staging buffer (handed
+// back after its first read, so the next tile's copy overlaps the rest of the
+// pass); the keys in bucket order (+16 bytes of end keys that the causal
+// count's 16-byte loads may read past the last key); the floor cells, two
+// bits each, whose place the seed list takes; the candidate list (position
+// and charge), whose place the seeds' counts take; the bucket offsets; the
+// mask of fired positions; the extended builds' (EXT) charges in key order
+// and, for detectors above 128 PMTs, a 4096-bit PMT set per warp; the dt rows
+// (kDtRow bytes each, 256-byte aligned) when the detector's table fits
+// (NARROW); the PMT tables (floor, row maximum of dt).
+template <int CAP, int NC, bool NARROW, bool EXT>
 struct TileLayout {
-    // time buckets of the in-tile merge, at most: two per hit slot up to
-    // 2048 hits (shorter chains in the floor-coincidence rounds), one at 4096
-    static constexpr int NBK = CAP <= 2048 ? 2 * CAP : CAP;
-    static constexpr uint32_t NS = CAP == 2048 ? 1u : 2u;  // staging buffers
-    static constexpr size_t kStage = (size_t)CAP * 16;     // one staging buffer
-    static constexpr size_t kPkS = (size_t)CAP * 4 + 16;
-    static constexpr size_t kPkB = (size_t)CAP * 4;
-    static constexpr size_t kChg = (size_t)CAP * 2;
-    static constexpr size_t kFlk = (size_t)CAP * 2;
-    static constexpr size_t kCnt = (size_t)(NBK + 1) * 4;
-    static constexpr size_t kMask = (size_t)(CAP / 32) * 4;
-    static constexpr size_t oPkS = NS * kStage;
-    static constexpr size_t oPkB = oPkS + kPkS;
-    static constexpr size_t oChgB = oPkB + kPkB;
-    static constexpr size_t oChgS = oChgB + kChg;
-    static constexpr size_t oFlk = oChgS + kChg;
-    static constexpr size_t oCnt = oFlk + kFlk;
-    static constexpr size_t oMask = oCnt + kCnt;
-    static constexpr size_t oTab = (oMask + kMask + 15) & ~(size_t)15;
-    static_assert(oCnt % 16 == 0, "the bucket counts are read as 16-byte vectors");
-    static size_t bytes(uint32_t P, bool)
-    {
-        return (oTab + 2 * (size_t)((P + 7) & ~7u) * 2 + 127) & ~(size_t)127;      // floor + dmax_row
-    }
-};
-
-// Shared memory of the default builds: one staging buffer (handed back after
-// its first read); the keys in bucket order (+16 bytes of end keys); the
-// floor cells, two bits each, whose place the seed list takes; the candidate
-// list (position and charge), whose place the seeds' counts take; the bucket
-// offsets; the mask of fired positions; the dt rows (kDtRow bytes each, 256-byte
-// aligned) when the detector's table fits; the PMT tables.
-template <int CAP>
-struct TileLayout<CAP, false> {
-    static constexpr int NBK = CAP;                        // time buckets
-    static constexpr uint32_t NS = 1;
     static constexpr uint32_t kCells = 16u * CAP;          // floor cells
+    static constexpr int NBK = CAP;                        // time buckets
     static constexpr size_t kStage = (size_t)CAP * 16;
     static constexpr size_t oPk = kStage;
     static constexpr size_t oCell = oPk + (size_t)CAP * 4 + 16;
@@ -692,61 +657,24 @@ struct TileLayout<CAP, false> {
     static constexpr size_t oCnt = oCand + (size_t)CAP * 4;
     static constexpr size_t oMask = oCnt + (size_t)(NBK + 1) * 4;
     static_assert(kCells / 4 == (size_t)CAP * 4, "the cells and the seed list share their place");
-    static constexpr size_t oDt = (oMask + (size_t)(CAP / 32) * 4 + kDtRow - 1) & ~(size_t)(kDtRow - 1);
+    static constexpr size_t oChg = oMask + (size_t)(CAP / 32) * 4;
+    static constexpr size_t oSet = oChg + (EXT ? (size_t)CAP * 2 : 0);
+    static constexpr size_t oDt = (oSet + (EXT && !NARROW ? (size_t)NC / 32 * 512 : 0) + kDtRow - 1) & ~(size_t)(kDtRow - 1);
     static_assert(oCnt % 16 == 0 && oCell % 16 == 0, "cleared and scanned as 16-byte vectors");
-    __host__ __device__ static size_t tab(uint32_t P, bool smem_dt) { return oDt + (smem_dt ? (size_t)P * kDtRow : 0); }
-    static size_t bytes(uint32_t P, bool smem_dt)
-    {
-        return (tab(P, smem_dt) + 2 * (size_t)((P + 7) & ~7u) * 2 + 127) & ~(size_t)127;
-    }
+    __host__ __device__ static size_t tab(uint32_t P) { return oDt + (NARROW ? (size_t)P * kDtRow : 0); }
+    static size_t bytes(uint32_t P) { return (tab(P) + 2 * (size_t)((P + 7) & ~7u) * 2 + 127) & ~(size_t)127; }
 };
 
-// Dynamic shared memory of the tile kernel (layout TileLayout<CAP, EXT>).
+// Dynamic shared memory of the tile kernel (layout TileLayout).
 extern __shared__ __align__(256) unsigned char g_tile_smem[];
 
-// The sorted builds' shared-memory regions sit at fixed offsets, so their
-// addresses are recomputed where used instead of living in registers
-// through every phase; only the PMT-table stride depends on the launch.
-template <int CAP>
-struct SortCtx {
-    using L = TileLayout<CAP, true>;
-    uint32_t P;             // PMTs of the loaded slice
-    uint32_t pp;            // PMT table stride: the launch's max_pmt rounded up to 8
-    const uint16_t *dt_g;   // the loaded slice's dt table in global memory
-    __device__ __forceinline__ uint64_t *stage(uint32_t b) const
-    {
-        return reinterpret_cast<uint64_t *>(g_tile_smem + (size_t)b * L::kStage);
-    }
-    __device__ __forceinline__ uint32_t *pk_s() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oPkS); }
-    __device__ __forceinline__ uint32_t *pk_b() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oPkB); }
-    __device__ __forceinline__ uint16_t *seed_idx() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oPkB); }
-    __device__ __forceinline__ uint16_t *seed_cnt() const
-    {
-        return reinterpret_cast<uint16_t *>(g_tile_smem + L::oPkB) + CAP;
-    }
-    __device__ __forceinline__ uint16_t *chg_b() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oChgB); }
-    __device__ __forceinline__ uint16_t *chg_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oChgS); }
-    __device__ __forceinline__ uint16_t *flk() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oFlk); }
-    __device__ __forceinline__ uint32_t *cnt() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCnt); }
-    __device__ __forceinline__ uint32_t *mask() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oMask); }
-    // warp w's 4096-bit PMT set of the distinct count above 128 PMTs (the
-    // bucket-order charges and the floor keys are no longer read by then;
-    // each region holds CAP / 256 sets)
-    __device__ __forceinline__ uint32_t *pmt_set(uint32_t w) const
-    {
-        constexpr uint32_t per = (uint32_t)CAP / 256;
-        return w < per ? reinterpret_cast<uint32_t *>(g_tile_smem + L::oChgB) + 128 * w
-                       : reinterpret_cast<uint32_t *>(g_tile_smem + L::oFlk) + 128 * (w - per);
-    }
-    __device__ __forceinline__ uint16_t *floor_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oTab); }
-    __device__ __forceinline__ uint16_t *dmax_s() const { return floor_s() + pp; }
-};
-
-// The same for the default builds.  NARROW: at most 128 PMTs in the batch
-// and every dt table in shared memory.
-template <int CAP, bool NARROW>
+// The tile kernel's shared-memory regions sit at fixed offsets, so their
+// addresses are recomputed where used instead of living in registers through
+// every phase; only the PMT tables' place depends on the launch.  NARROW: at
+// most kSmemDtMaxPmt PMTs in the batch and every dt table in shared memory.
+template <int CAP, int NC, bool NARROW, bool EXT>
 struct TileCtx {
-    using L = TileLayout<CAP, false>;
+    using L = TileLayout<CAP, NC, NARROW, EXT>;
     uint32_t P;             // PMTs of the loaded slice
     uint32_t tab;           // offset of the PMT tables
     uint32_t pp;            // their stride
@@ -759,6 +687,12 @@ struct TileCtx {
     __device__ __forceinline__ uint32_t *cnt() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCnt); }
     __device__ __forceinline__ uint32_t *cells() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCell); }
     __device__ __forceinline__ uint32_t *mask() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oMask); }
+    // the extended builds' charges, and warp w's PMT set
+    __device__ __forceinline__ uint16_t *chg() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oChg); }
+    __device__ __forceinline__ uint32_t *pmt_set(uint32_t w) const
+    {
+        return reinterpret_cast<uint32_t *>(g_tile_smem + L::oSet) + 128 * w;
+    }
     __device__ __forceinline__ uint16_t *dt_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oDt); }
     __device__ __forceinline__ uint16_t *floor_s() const { return reinterpret_cast<uint16_t *>(g_tile_smem + tab); }
     __device__ __forceinline__ uint16_t *dmax_s() const { return floor_s() + pp; }
@@ -771,6 +705,20 @@ struct TileCtx {
     {
         return (t << kShift) | (NARROW ? pmt << 1 : pmt);
     }
+    // dt entry of a row (seed rule 1 keeps the PMT relation in its upper bits)
+    struct Row {
+        uint32_t s;
+        const uint16_t *g;
+        __device__ __forceinline__ uint32_t at(uint32_t k) const
+        {
+            if (NARROW) return *reinterpret_cast<const uint16_t *>(g_tile_smem + (s | (k & kPmtMask)));
+            return __ldg(g + key_p(k));
+        }
+    };
+    __device__ __forceinline__ Row row(uint32_t p) const
+    {
+        return Row{(uint32_t)L::oDt + p * kDtRow, dt_g + (size_t)p * P};
+    }
     static __device__ __forceinline__ uint32_t key_t(uint32_t k) { return k >> kShift; }
     static __device__ __forceinline__ uint32_t key_p(uint32_t k) { return NARROW ? (k & kPmtMask) >> 1 : k & kPmtMask; }
 };
@@ -780,52 +728,7 @@ constexpr uint32_t kBarCons = 1;        // named barrier of the consumers
 template <int NC>
 __device__ __forceinline__ void cons_sync() { named_sync(kBarCons, NC); }
 
-// Packed key of the sorted builds: time within the staged range (below
-// 2^20 ns) and PMT (below 2^12).  0xffffffff marks "no hit".
-constexpr uint32_t kPkNone = 0xffffffffu;
-__device__ __forceinline__ uint32_t pk_t(uint32_t k) { return k >> 12; }
-__device__ __forceinline__ uint32_t pk_p(uint32_t k) { return k & 0xfffu; }
-
-// Consumer-wide exclusive scan of cnt[0..nb), nb a multiple of NC; writes
-// the total to cnt[nb].  Scratch words red[0..NC/32].
-template <int NC, uint32_t NB>
-__device__ void cons_exclusive_scan(uint32_t *cnt, uint32_t *red)
-{
-    constexpr uint32_t NW = NC / 32, PER = NB / NC, V = PER / 4;
-    static_assert(NB % NC == 0 && PER % 4 == 0, "each thread scans whole 16-byte vectors");
-    const uint32_t tid = threadIdx.x;
-    uint4 *c4 = reinterpret_cast<uint4 *>(cnt) + tid * V;
-    uint4 v[V];
-    uint32_t local = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < V; ++i) {
-        v[i] = c4[i];
-        local += v[i].x + v[i].y + v[i].z + v[i].w;
-    }
-    uint32_t incl = warp_incl_scan(local);
-    if (lane_id() == 31) red[tid >> 5] = incl;
-    cons_sync<NC>();
-    if (tid < 32) {
-        uint32_t w = tid < NW ? red[tid] : 0u;
-        uint32_t wi = warp_incl_scan(w);
-        if (tid < NW) red[tid] = wi - w;
-        if (tid == NW - 1) red[NW] = wi;
-    }
-    cons_sync<NC>();
-    uint32_t run = red[tid >> 5] + incl - local;
-#pragma unroll
-    for (uint32_t i = 0; i < V; ++i) {
-        uint4 o;
-        o.x = run;
-        o.y = o.x + v[i].x;
-        o.z = o.y + v[i].y;
-        o.w = o.z + v[i].z;
-        run = o.w + v[i].w;
-        c4[i] = o;
-    }
-    if (tid == 0) cnt[NB] = red[NW];
-    cons_sync<NC>();
-}
+constexpr uint32_t kPkNone = 0xffffffffu;       // "no hit", above every key
 
 // Bucket of a time relative to the tile base: t_rel >> bsh, the last of
 // the NB buckets taking everything beyond.
@@ -842,48 +745,49 @@ struct CoreOut {
     uint32_t c0;
 };
 
-// Seeds, causal counts and emission over the sorted tile keys[0..n).  The
-// core is t_rel in [H, H + core_w).  Fired seeds go to out[0..n_fired).
+// The loaded slice's trigger parameters.
 struct TrigParams {
     uint32_t H, tau, q_seed, threshold, win_half;
     uint32_t l0_hits, l0_window, l0_distinct;
     uint32_t seed_rule, sc_w, fc_w, afc_w, count_distinct;
+    uint32_t dt_mask;       // the dt bits of a shared-memory row's entry
     const uint8_t *rel;
     trig_hit *dbg_merged;
     uint32_t *dbg_seedcnt;
 };
 
-// Seed rule 1 at sorted index i: [SC and AFC] or [FC and AFC].  Walks the
-// keys within the widest of the three windows on both sides (all staged:
-// the tile halo covers it) and looks each pair up in the PMT relation row
-// of p_i.
-__device__ __noinline__ bool coincidence_seed(const uint32_t *pk, uint32_t n, uint32_t i, const uint8_t *rel,
-                                              uint32_t P, uint32_t sc, uint32_t fc, uint32_t afc)
+// Seed rule 1 for the key at position i: [SC and AFC] or [FC and AFC].  Looks
+// through the buckets of the widest of the three windows, four keys at a
+// time (all staged: the tile halo covers it), and each pair up in the PMT
+// relation row of p_i: the upper bits of the dt row where they hold it, else
+// the table in global memory.
+template <uint32_t NB, class CTX>
+__device__ __forceinline__ bool coincidence_seed(const CTX &cx, const TrigParams &tp, uint32_t i, uint32_t bsh)
 {
-    const uint32_t ki = pk[i], ti = pk_t(ki), pi = pk_p(ki);
-    if (!CHECK(14, pi, P)) return false;
-    const uint8_t *row = rel + (size_t)pi * P;
-    const uint32_t wmax = max(sc, max(fc, afc));
+    const uint32_t *pk = cx.pk(), *cnt = cx.cnt();
+    const uint32_t ki = pk[i], ti = CTX::key_t(ki), pi = CTX::key_p(ki);
+    if (!CHECK(14, pi, cx.P)) return false;
+    const uint8_t *rel = tp.rel + (size_t)pi * cx.P;
+    const auto row = cx.row(pi);
+    const bool packed = tp.dt_mask != 0xffffu;
+    const uint32_t sc = tp.sc_w, fc = tp.fc_w, afc = tp.afc_w, w = max(sc, max(fc, afc));
+    uint32_t j = cnt[(ti > w ? ti - w : 0u) >> bsh];
+    const uint32_t je = cnt[bucket_of<NB>(ti + w, bsh) + 1];
     bool c = false, a = false;
-    for (uint32_t j = i + 1; j < n; ++j) {
-        const uint32_t kj = pk[j], d = pk_t(kj) - ti;
-        if (d > wmax) break;
-        if (!CHECK(15, pk_p(kj), P)) continue;
-        const uint32_t r = __ldg(row + pk_p(kj));
-        c = c || ((r & kRelAdjacent) && d <= sc) || ((r & kRelFloor) && d <= fc);
-        a = a || ((r & kRelNextFloor) && d <= afc);
-        if (a && c) return true;
+    for (; j < je && !(a && c); j += 4) {
+        uint32_t kj[4], r[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) kj[u] = pk[min(j + u, je - 1u)];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) r[u] = packed ? row.at(kj[u]) >> kRelShift : __ldg(rel + CTX::key_p(kj[u]));
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            const uint32_t d = __usad(CTX::key_t(kj[u]), ti, 0u);
+            c = c || ((r[u] & kRelAdjacent) && d <= sc) || ((r[u] & kRelFloor) && d <= fc);
+            a = a || ((r[u] & kRelNextFloor) && d <= afc);
+        }
     }
-    for (uint32_t j = i; j-- > 0;) {
-        const uint32_t kj = pk[j], d = ti - pk_t(kj);
-        if (d > wmax) break;
-        if (!CHECK(15, pk_p(kj), P)) continue;
-        const uint32_t r = __ldg(row + pk_p(kj));
-        c = c || ((r & kRelAdjacent) && d <= sc) || ((r & kRelFloor) && d <= fc);
-        a = a || ((r & kRelNextFloor) && d <= afc);
-        if (a && c) return true;
-    }
-    return false;
+    return a && c;
 }
 
 // A seed's scan range: the keys [j0, j1) of the buckets covering
@@ -901,40 +805,44 @@ __device__ __forceinline__ void seed_range(const CTX &cx, uint32_t ts, uint32_t 
 
 // Distinct-PMT causal count: c(s) = the number of different PMTs among the
 // keys j with |t_j - t_s| <= min(dt_max[p_s][p_j], W).  Up to 128 PMTs,
-// eight lanes per seed each collect a 128-bit PMT set in registers over
-// every eighth key of the seed's scan range, and the sets are OR-ed and
-// counted; above, a warp per seed marks the PMTs in a shared-memory set.
-template <int CAP, int NC, uint32_t NB>
-__device__ __noinline__ void count_distinct_pmts(const SortCtx<CAP> &cx, const uint32_t *pk, uint32_t n, uint32_t ns,
-                                                 const uint16_t *seed_idx, uint32_t bsh, uint16_t *seed_cnt)
+// eight lanes per seed each collect a 128-bit PMT set in registers over four
+// consecutive keys at a time of the seed's scan range (keys outside it fail
+// the test, see count_seeds), and the sets are OR-ed and counted; above, a
+// warp per seed marks the PMTs in a shared-memory set.
+template <uint32_t NB, int NC, class CTX>
+__device__ __forceinline__ void count_distinct_pmts(const CTX &cx, uint32_t n, uint32_t ns, uint32_t bsh, uint32_t threshold,
+                                                    uint32_t dt_mask)
 {
     constexpr uint32_t G = 8, NG = NC / G;
-    static_assert(NC / 32 <= CAP / 128, "a PMT set per consumer warp");
     const uint32_t tid = threadIdx.x, gl = tid & (G - 1u), gid = tid / G, P = cx.P;
+    const uint32_t *pk = cx.pk(), *seeds = cx.seeds();
+    auto done = [&](uint32_t k, uint32_t pos, uint32_t c) {
+        cx.counts()[k] = (uint16_t)c;
+        if (c >= threshold) atomicOr(&cx.mask()[pos >> 5], 1u << (pos & 31u));
+    };
     if (P > 128) {
         const uint32_t warp = tid >> 5, lane = tid & 31u, nwords = (P + 31u) >> 5;
         uint32_t *set = cx.pmt_set(warp);
         for (uint32_t k = warp; k < ns; k += NC / 32) {
             for (uint32_t w = lane; w < nwords; w += 32) set[w] = 0u;
             __syncwarp();
-            const uint32_t ks = pk[seed_idx[k]];
-            const uint32_t ts = pk_t(ks), ps = pk_p(ks);
+            const uint32_t pos = seeds[k] & 0xffffu, ks = pk[pos];
+            const uint32_t ts = CTX::key_t(ks), ps = CTX::key_p(ks);
             uint32_t j0, j1;
             seed_range<NB>(cx, ts, ps, bsh, j0, j1);
             if (CHECK(12, j1, n + 1) && CHECK(13, ps, P) && CHECK(16, nwords, 129)) {
-                const uint16_t *row_g = cx.dt_g + (size_t)ps * P;
+                const auto row = cx.row(ps);
                 for (uint32_t q = j0 + lane; q < j1; q += 32) {
-                    const uint32_t kj = pk[q], tj = pk_t(kj), pj = pk_p(kj);
+                    const uint32_t kj = pk[q], tj = CTX::key_t(kj), pj = CTX::key_p(kj);
                     if (!CHECK(11, pj, P)) continue;
-                    const uint32_t lim = __ldg(row_g + pj);
-                    if ((tj > ts ? tj - ts : ts - tj) <= lim) atomicOr(&set[pj >> 5], 1u << (pj & 31u));
+                    if (__usad(tj, ts, 0u) <= row.at(kj)) atomicOr(&set[pj >> 5], 1u << (pj & 31u));
                 }
             }
             __syncwarp();
             uint32_t c = 0;
             for (uint32_t w = lane; w < nwords; w += 32) c += __popc(set[w]);
             c = __reduce_add_sync(0xffffffffu, c);
-            if (lane == 0) seed_cnt[k] = (uint16_t)c;
+            if (lane == 0) done(k, pos, c);
             __syncwarp();                       // the set is read before the next seed clears it
         }
         return;
@@ -942,24 +850,30 @@ __device__ __noinline__ void count_distinct_pmts(const SortCtx<CAP> &cx, const u
     const uint32_t rounds = (ns + NG - 1) / NG;
     for (uint32_t r = 0; r < rounds; ++r) {
         const uint32_t k = r * NG + gid;
-        uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+        uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0, pos = 0;
         if (k < ns) {
-            const uint32_t ks = pk[seed_idx[k]];
-            const uint32_t ts = pk_t(ks), ps = pk_p(ks);
+            pos = seeds[k] & 0xffffu;
+            const uint32_t ks = pk[pos], ts = CTX::key_t(ks), ps = CTX::key_p(ks);
             uint32_t j0, j1;
             seed_range<NB>(cx, ts, ps, bsh, j0, j1);
             if (CHECK(12, j1, n + 1) && CHECK(13, ps, P)) {
-                const uint16_t *row_g = cx.dt_g + (size_t)ps * P;
-                for (uint32_t q = j0 + gl; q < j1; q += G) {
-                    const uint32_t kj = pk[q], tj = pk_t(kj), pj = pk_p(kj);
-                    if (!CHECK(11, pj, P)) continue;
-                    const uint32_t lim = __ldg(row_g + pj);
-                    if ((tj > ts ? tj - ts : ts - tj) > lim) continue;
-                    const uint32_t b = 1u << (pj & 31u), h = pj >> 5;
+                const auto row = cx.row(ps);
+                auto mark = [&](uint32_t kj) {
+                    const uint32_t pj = CTX::key_p(kj);
+                    if (!CHECK(11, pj, P)) return;
+                    const bool in = __usad(CTX::key_t(kj), ts, 0u) <= (row.at(kj) & dt_mask);
+                    const uint32_t b = in ? 1u << (pj & 31u) : 0u, h = pj >> 5;
                     m0 |= h == 0 ? b : 0u;
                     m1 |= h == 1 ? b : 0u;
                     m2 |= h == 2 ? b : 0u;
                     m3 |= h == 3 ? b : 0u;
+                };
+                for (uint32_t q = (j0 & ~3u) + 4 * gl; q < j1; q += 4 * G) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(pk + q);
+                    mark(v.x);
+                    mark(v.y);
+                    mark(v.z);
+                    mark(v.w);
                 }
             }
         }
@@ -969,7 +883,7 @@ __device__ __noinline__ void count_distinct_pmts(const SortCtx<CAP> &cx, const u
             m2 |= __shfl_xor_sync(0xffffffffu, m2, off);
             m3 |= __shfl_xor_sync(0xffffffffu, m3, off);
         }
-        if (k < ns && gl == 0) seed_cnt[k] = (uint16_t)(__popc(m0) + __popc(m1) + __popc(m2) + __popc(m3));
+        if (k < ns && gl == 0) done(k, pos, __popc(m0) + __popc(m1) + __popc(m2) + __popc(m3));
     }
 }
 
@@ -979,20 +893,21 @@ __device__ __noinline__ void count_distinct_pmts(const SortCtx<CAP> &cx, const u
 // hit within TW of a core hit is staged (the tile halo covers TW).  The
 // distinct count slides the window back start by start, keeping per-PMT
 // counts, so it reads each hit within 2 TW once.
+template <class CTX>
 __device__ __noinline__ bool level0_pass(const uint32_t *pk, uint32_t n, uint32_t i, uint32_t N, uint32_t TW,
                                          bool distinct)
 {
-    const uint32_t ts = pk_t(pk[i]);
+    const uint32_t ts = CTX::key_t(pk[i]);
     uint32_t j = i;
-    while (j > 0 && pk_t(pk[j - 1]) == ts) --j;             // first index of t_i
+    while (j > 0 && CTX::key_t(pk[j - 1]) == ts) --j;             // first index of t_i
     if (!distinct) {
         for (;;) {
-            const uint32_t tj = pk_t(pk[j]);
-            if (j + N - 1 < n && pk_t(pk[j + N - 1]) - tj < TW) return true;
+            const uint32_t tj = CTX::key_t(pk[j]);
+            if (j + N - 1 < n && CTX::key_t(pk[j + N - 1]) - tj < TW) return true;
             if (j == 0) return false;
-            const uint32_t tp = pk_t(pk[j - 1]);
+            const uint32_t tp = CTX::key_t(pk[j - 1]);
             if (ts - tp >= TW) return false;
-            for (--j; j > 0 && pk_t(pk[j - 1]) == tp; --j) {
+            for (--j; j > 0 && CTX::key_t(pk[j - 1]) == tp; --j) {
             }
         }
     }
@@ -1000,23 +915,23 @@ __device__ __noinline__ bool level0_pass(const uint32_t *pk, uint32_t n, uint32_
     for (uint32_t p = 0; p < 128; ++p) cnt[p] = 0;
     uint32_t distinct_n = 0, e = j;
     for (;;) {
-        const uint32_t tj = pk_t(pk[j]);
-        while (e < n && pk_t(pk[e]) - tj < TW) {                // extend the end
-            if (cnt[pk_p(pk[e]) & 127u]++ == 0) ++distinct_n;
+        const uint32_t tj = CTX::key_t(pk[j]);
+        while (e < n && CTX::key_t(pk[e]) - tj < TW) {                // extend the end
+            if (cnt[CTX::key_p(pk[e]) & 127u]++ == 0) ++distinct_n;
             ++e;
         }
         if (distinct_n >= N) return true;
         if (j == 0) return false;
-        const uint32_t tp = pk_t(pk[j - 1]);
+        const uint32_t tp = CTX::key_t(pk[j - 1]);
         if (ts - tp >= TW) return false;
         // the previous start: add its hits, drop hits at or past tp + TW
         uint32_t nj = j - 1;
-        while (nj > 0 && pk_t(pk[nj - 1]) == tp) --nj;
+        while (nj > 0 && CTX::key_t(pk[nj - 1]) == tp) --nj;
         for (uint32_t q = nj; q < j; ++q)
-            if (cnt[pk_p(pk[q]) & 127u]++ == 0) ++distinct_n;
-        while (e > j && pk_t(pk[e - 1]) - tp >= TW) {
+            if (cnt[CTX::key_p(pk[q]) & 127u]++ == 0) ++distinct_n;
+        while (e > j && CTX::key_t(pk[e - 1]) - tp >= TW) {
             --e;
-            if (--cnt[pk_p(pk[e]) & 127u] == 0) --distinct_n;
+            if (--cnt[CTX::key_p(pk[e]) & 127u] == 0) --distinct_n;
         }
         j = nj;
     }
@@ -1026,15 +941,16 @@ __device__ __noinline__ bool level0_pass(const uint32_t *pk, uint32_t n, uint32_
 // starts as level0_pass (each first index of a time within TW before t_i),
 // each window's PMTs marked in the warp's 4096-bit set in shared memory and
 // counted; the first window with N different PMTs ends the search.
+template <class CTX>
 __device__ __noinline__ bool level0_distinct_warp(const uint32_t *pk, uint32_t n, uint32_t i, uint32_t N, uint32_t TW,
                                                   uint32_t P, uint32_t *set)
 {
     const uint32_t lane = lane_id(), nwords = (P + 31u) >> 5;
-    const uint32_t ts = pk_t(pk[i]);
+    const uint32_t ts = CTX::key_t(pk[i]);
     uint32_t j = i;
-    while (j > 0 && pk_t(pk[j - 1]) == ts) --j;             // first index of t_i
+    while (j > 0 && CTX::key_t(pk[j - 1]) == ts) --j;             // first index of t_i
     for (;;) {
-        const uint32_t tj = pk_t(pk[j]);
+        const uint32_t tj = CTX::key_t(pk[j]);
         for (uint32_t w = lane; w < nwords; w += 32) set[w] = 0u;
         __syncwarp();
         // the window [t_j, t_j + TW): keys from j on, in time order
@@ -1042,8 +958,8 @@ __device__ __noinline__ bool level0_distinct_warp(const uint32_t *pk, uint32_t n
             const uint32_t k = k0 + lane;
             bool in = false;
             if (k < n) {
-                const uint32_t kk = pk[k], pj = pk_p(kk);
-                in = pk_t(kk) - tj < TW;
+                const uint32_t kk = pk[k], pj = CTX::key_p(kk);
+                in = CTX::key_t(kk) - tj < TW;
                 if (in && CHECK(27, pj, P)) atomicOr(&set[pj >> 5], 1u << (pj & 31u));
             }
             if (!__any_sync(0xffffffffu, in)) break;
@@ -1055,80 +971,10 @@ __device__ __noinline__ bool level0_distinct_warp(const uint32_t *pk, uint32_t n
         __syncwarp();                                       // the set is read before it is cleared again
         if (c >= N) return true;
         if (j == 0) return false;
-        const uint32_t tp = pk_t(pk[j - 1]);
+        const uint32_t tp = CTX::key_t(pk[j - 1]);
         if (ts - tp >= TW) return false;
-        for (--j; j > 0 && pk_t(pk[j - 1]) == tp; --j) {
+        for (--j; j > 0 && CTX::key_t(pk[j - 1]) == tp; --j) {
         }
-    }
-}
-
-// Causal count c(s) = #{ j : |t_j - t_s| <= min(dt_max[p_s][p_j], W) }
-// over each seed's scan range keys [j0, j1) (seed_range): a group of 2^LG
-// lanes per seed,
-// seeds dealt round-robin to the groups, four independent tests per lane in
-// flight.
-template <int CAP, int NC, uint32_t LG, uint32_t NB>
-__device__ __forceinline__ void count_causal(const SortCtx<CAP> &cx, const uint32_t *pk, uint32_t n, uint32_t ns,
-                                             const uint16_t *seed_idx, uint32_t bsh, uint16_t *seed_cnt)
-{
-    constexpr uint32_t G = 1u << LG, NG = NC >> LG;
-    const uint32_t tid = threadIdx.x, gl = tid & (G - 1u), gid = tid >> LG, P = cx.P;
-    const uint32_t rounds = (ns + NG - 1) / NG;
-#ifdef TRIG_PHASE_STATS
-    uint32_t keys_seen = 0;
-    struct Flush {
-        uint32_t &k;
-        __device__ ~Flush()
-        {
-            const uint32_t w = __reduce_add_sync(0xffffffffu, k);
-            if ((threadIdx.x & 31u) == 0 && w) PHASE_ADD(kPhKeys, w);
-        }
-    } flush{keys_seen};
-#endif
-    for (uint32_t r = 0; r < rounds; ++r) {
-        const uint32_t k = r * NG + gid;
-        uint32_t c = 0;
-        if (k < ns) {
-            const uint32_t ks = pk[seed_idx[k]];
-            const uint32_t ts = pk_t(ks), ps = pk_p(ks);
-            uint32_t j0, j1;
-            seed_range<NB>(cx, ts, ps, bsh, j0, j1);
-#ifdef TRIG_PHASE_STATS
-            keys_seen += gl == 0 ? j1 - j0 : 0u;
-#endif
-            if (CHECK(12, j1, n + 1) && CHECK(13, ps, P)) {
-                const uint16_t *row_g = cx.dt_g + (size_t)ps * P;
-                // key kj counts when |t_j - t_s| <= dt[p_s][p_j]
-                auto causal = [&](uint32_t kj) -> uint32_t {
-                    const uint32_t tj = pk_t(kj), pj = pk_p(kj);
-                    if (!CHECK(11, pj, P)) return 0u;
-                    const uint32_t lim = __ldg(row_g + pj);
-                    return (tj > ts ? tj - ts : ts - tj) <= lim;
-                };
-                // each lane takes four consecutive keys per 16-byte load, from
-                // j0 rounded down to a multiple of 4.  No key outside
-                // [j0, j1) can pass: those before j0 lie in earlier buckets,
-                // more than dmax_row(p_s) >= dt before t_s, those from j1 on
-                // in later buckets, and the four end keys past the last key
-                // (time 2^20 - 1, PMT 0) are beyond any dt as well
-                uint32_t ca = 0, cb = 0, cc = 0, cd = 0;
-                for (uint32_t q = (j0 & ~3u) + 4 * gl; q < j1; q += 4 * G) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(pk + q);
-                    ca += causal(v.x);
-                    cb += causal(v.y);
-                    cc += causal(v.z);
-                    cd += causal(v.w);
-                }
-                c = ca + cb + cc + cd;
-            }
-        }
-        if (LG == 5) {
-            c = __reduce_add_sync(0xffffffffu, c);
-        } else {
-#pragma unroll
-            for (uint32_t off = G >> 1; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-        }
-        if (k < ns && gl == 0) seed_cnt[k] = (uint16_t)c;
     }
 }
 
@@ -1161,384 +1007,6 @@ __device__ __forceinline__ uint32_t bucket_shift(uint32_t span)
     return top > nb_bits ? top - nb_bits : 0u;
 }
 
-// One staged tile through the whole trigger, sorted builds (level 0, seed
-// rule 1, distinct count, row outputs, event extraction): the n records of
-// `stage` (16 bytes each, time t_ns, PMT and charge; any order) span
-// [tb, tb + span); the core is t - tb in [lo_t, hi_t).
-//
-//  A. every record becomes a packed key (t - tb) << 12 | pmt and is counted
-//     in its time bucket (t - tb) >> bsh; the stage buffer is then handed
-//     back to the producer (release_bar), the rest works on the keys;
-//  B. bucket offsets (exclusive scan of the counts);
-//  C. the k-way merge of the PMT runs ("DAQ system of NEMO Phase II"):
-//     keys, charges and floors scattered to their bucket, about one key per
-//     bucket, then each key ranked inside its bucket by (t, pmt, charge);
-//  D. floor coincidences ("Sorting and triggering in GPU": another PMT of
-//     the same floor within tau), in rounds: round r checks the pair
-//     (i, i + r) of every key i still live, that is whose next keys lie
-//     within tau.  Every pair is checked once, both hits are marked, and
-//     each warp keeps its own list of live keys.  Seed rule 1 and level 0
-//     test each core key instead;
-//  E. the ordered seed list; F. the causal count of every seed over whole
-//     buckets of its scan range, each key tested exactly ("Muon trigger
-//     strategy"); G. the fired seeds, in (t, pmt, charge) order, to out.
-//
-// Returns the counts and c0 = the number of staged keys before the core.
-// cnt and mask are zero on entry and on return.
-template <int CAP, int NC>
-__device__ CoreOut sorted_pass(SortCtx<CAP> &cx, const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span,
-                             uint32_t lo_t, uint32_t hi_t, const TrigParams &tp, trig_trigger *out, uint32_t *wr,
-                             bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo, uint64_t *release_bar)
-{
-    constexpr uint32_t NW = NC / 32;
-    constexpr int PER = CAP / NC;
-    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    constexpr uint32_t NB = (uint32_t)TileLayout<CAP, true>::NBK;
-    const uint32_t bsh = bucket_shift<NB>(span);
-    const uint32_t tau = tp.tau;
-    __shared__ uint32_t s_red[NW + 1];
-    __shared__ uint32_t s_below[3];
-    __shared__ uint32_t s_tot[2 * NW];
-    uint32_t *cnt = cx.cnt();
-    uint32_t *mask = cx.mask();
-#ifdef TRIG_PHASE_STATS
-    long long t_ph = clock64();
-#define PHASE_MARK(i)                                   \
-    do {                                                \
-        if (tid == 0) {                                 \
-            const long long now_ = clock64();           \
-            PHASE_ADD((i), now_ - t_ph);                \
-            t_ph = now_;                                \
-        }                                               \
-    } while (0)
-#else
-#define PHASE_MARK(i) ((void)0)
-#endif
-
-    // A. keys and bucket counts; keys before the core, before its end, and
-    //    too early to pair with a core key (t + tau < lo_t)
-    uint32_t key[PER], cs[PER];           // packed key; charge << 16 | slot in the bucket
-    uint32_t below_lo = 0, below_hi = 0, below_w = 0;
-#pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        const uint32_t i = tid + r * NC;
-        key[r] = kPkNone;
-        cs[r] = 0;
-        if (i < n) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(stage + 2 * i);
-            // t - tb in 32 bits (the staged range spans less than 2^20 ns)
-            const uint32_t tr = min(v.x - (uint32_t)tb, span - 1u);
-            key[r] = (tr << 12) | (v.z & 0xfffu);
-            const uint32_t slot = atomicAdd(&cnt[bucket_of<NB>(tr, bsh)], 1u);
-            cs[r] = (v.z & 0xffff0000u) | slot;
-            below_lo += tr < lo_t;
-            below_hi += tr < hi_t;
-            below_w += tr + tau < lo_t;
-        }
-    }
-    below_lo = __reduce_add_sync(0xffffffffu, below_lo);
-    below_hi = __reduce_add_sync(0xffffffffu, below_hi);
-    below_w = __reduce_add_sync(0xffffffffu, below_w);
-    if (tid == 0) s_below[0] = s_below[1] = s_below[2] = 0;
-    cons_sync<NC>();
-    if (lane == 0) {
-        if (below_lo) atomicAdd(&s_below[0], below_lo);
-        if (below_hi) atomicAdd(&s_below[1], below_hi);
-        if (below_w) atomicAdd(&s_below[2], below_w);
-    }
-    // the stage buffer has been read: order those reads before the
-    // producer's next bulk copy into it, then hand it back
-    if (release_bar) fence_proxy_async_smem();
-
-    // B. bucket offsets (the scan's barriers also publish s_below and end
-    //    every read of the stage buffer)
-    cons_exclusive_scan<NC, NB>(cnt, s_red);
-    if (release_bar && tid == 0) mbar_arrive(release_bar);
-    const uint32_t c0 = s_below[0], c1 = s_below[1], d_lo = s_below[2];
-    PHASE_MARK(kPhA);
-
-    // C. bucket order (with each key's floor), then the rank inside the bucket
-    uint32_t *pk = cx.pk_s();
-    uint16_t *chg = cx.chg_s(), *flk = cx.flk();
-    uint32_t *pk_c = cx.pk_b();
-    uint16_t *chg_c = cx.chg_b();
-    const uint16_t *fl = cx.floor_s();
-    const bool charge_rule = tp.seed_rule != 1;
-#pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        if (key[r] != kPkNone) {
-            const uint32_t tr = key[r] >> 12;
-            const uint32_t pos = cnt[bucket_of<NB>(tr, bsh)] + (cs[r] & 0xffffu);
-            if (CHECK(22, pos, CAP)) {
-                pk_c[pos] = key[r];
-                chg_c[pos] = (uint16_t)(cs[r] >> 16);
-            }
-        }
-    }
-    if (tid < 4) pk[n + tid] = 0xfffff000u;           // end keys (time 2^20 - 1, PMT 0)
-    cons_sync<NC>();
-    PHASE_MARK(kPhB);
-#pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        const uint32_t k = key[r];
-        if (k == kPkNone) continue;
-        const uint32_t b = bucket_of<NB>(k >> 12, bsh);
-        const uint32_t s0 = cnt[b], s1 = cnt[b + 1], q = cs[r] >> 16, pos = s0 + (cs[r] & 0xffffu);
-        uint32_t rk = s0;
-        for (uint32_t m = s0; m < s1; ++m) {
-            const uint32_t o = pk_c[m];
-            rk += o < k;
-            if (o == k) {                      // equal time and PMT: charge, then position
-                const uint32_t oq = chg_c[m];
-                rk += oq < q || (oq == q && m < pos);
-            }
-        }
-        if (CHECK(23, rk, CAP)) {
-            pk[rk] = k;
-            chg[rk] = (uint16_t)q;
-            flk[rk] = fl[k & 0xfffu];
-            const uint32_t tr = k >> 12;
-            if (charge_rule && q >= tp.q_seed && tr >= lo_t && tr < hi_t)
-                atomicOr(&mask[rk >> 5], 1u << (rk & 31u));
-        }
-    }
-    cons_sync<NC>();
-    PHASE_MARK(kPhC);
-
-    // D. seed flags of the core keys
-    const uint32_t P = cx.P;
-    if (tp.seed_rule == 1) {
-        for (uint32_t base = c0 & ~31u; base < c1; base += NC) {
-            const uint32_t i = base + tid;
-            const bool seed = i >= c0 && i < c1 && coincidence_seed(pk, n, i, tp.rel, P, tp.sc_w, tp.fc_w, tp.afc_w);
-            const uint32_t m = __ballot_sync(0xffffffffu, seed);
-            if (lane == 0 && m) atomicOr(&mask[(base >> 5) + warp], m);
-        }
-    } else {
-        // the keys [d_lo, c1) can pair with a core key, in contiguous shares
-        // per warp
-        const uint32_t lt = (1u << lane) - 1u;
-        const uint32_t d_n = c1 > d_lo ? c1 - d_lo : 0u;
-        const uint32_t share = ((d_n + NW - 1) / NW + 31u) & ~31u;
-        const uint32_t w_begin = min(d_lo + warp * share, c1), w_end = min(w_begin + share, c1);
-        uint32_t *live = cx.pk_b() + warp * (CAP / NW);
-        auto pair = [&](uint32_t i, uint32_t j, uint32_t ki, uint32_t kj) {
-            if ((ki & 0xfffu) != (kj & 0xfffu) && flk[i] == flk[j]) {
-                if (i >= c0 && i < c1) atomicOr(&mask[i >> 5], 1u << (i & 31u));
-                if (j >= c0 && j < c1) atomicOr(&mask[j >> 5], 1u << (j & 31u));
-            }
-        };
-        uint32_t nlive = 0;
-        for (uint32_t x = w_begin; x < w_end; x += 32) {
-            const uint32_t i = x + lane;
-            bool alive = false;
-            if (i < w_end) {
-                const uint32_t ki = pk[i], kj = pk[i + 1];     // i + 1 <= c1 <= n: an end key at worst
-                if ((kj >> 12) - (ki >> 12) <= tau && i + 1 < n) {
-                    alive = true;
-                    pair(i, i + 1, ki, kj);
-                }
-            }
-            const uint32_t m = __ballot_sync(0xffffffffu, alive);
-            if (alive) live[nlive + __popc(m & lt)] = i;
-            nlive += __popc(m);
-        }
-        for (uint32_t d = 2u; nlive; ++d) {
-            uint32_t next = 0;
-            for (uint32_t x = 0; x < nlive; x += 32) {
-                bool alive = false;
-                uint32_t i = 0;
-                if (x + lane < nlive) {
-                    i = live[x + lane];
-                    const uint32_t j = i + d;
-                    if (j < n) {
-                        const uint32_t ki = pk[i], kj = pk[j];
-                        if ((kj >> 12) - (ki >> 12) <= tau) {
-                            alive = true;
-                            pair(i, j, ki, kj);
-                        }
-                    }
-                }
-                // the ballot orders this batch's reads of the list before
-                // the writes below (which land at or before x + 31)
-                const uint32_t m = __ballot_sync(0xffffffffu, alive);
-                if (alive) live[next + __popc(m & lt)] = i;
-                next += __popc(m);
-            }
-            nlive = next;
-        }
-    }
-    cons_sync<NC>();
-    if (tp.l0_hits) {
-        // level 0 (N hits within TW) before the seed triggers count
-        if (tp.l0_distinct && P > 128) {
-            // a warp per seed, its PMT set in the bucket-order key region
-            // (free between the floor coincidences and the seed list)
-            static_assert(NC / 32 * 128 <= CAP, "a 4096-bit PMT set per consumer warp");
-            uint32_t *set = cx.pk_b() + warp * 128;
-            for (uint32_t base = (c0 & ~31u) + warp * 32; base < c1; base += NC) {
-                const uint32_t i = base + lane;
-                const uint32_t w = (i >= c0 && i < c1) ? mask[i >> 5] : 0u;
-                uint32_t cand = __ballot_sync(0xffffffffu, (w >> (i & 31u)) & 1u);
-                uint32_t drop = 0;
-                while (cand) {
-                    const uint32_t b = __ffs(cand) - 1;
-                    cand &= cand - 1;
-                    if (!level0_distinct_warp(pk, n, base + b, tp.l0_hits, tp.l0_window, P, set)) drop |= 1u << b;
-                }
-                if (lane == 0 && drop) atomicAnd(&mask[base >> 5], ~drop);
-            }
-        } else {
-            for (uint32_t base = c0 & ~31u; base < c1; base += NC) {
-                const uint32_t i = base + tid;
-                const uint32_t w = (i >= c0 && i < c1) ? mask[i >> 5] : 0u;
-                const bool drop = ((w >> (i & 31u)) & 1u) &&
-                                  !level0_pass(pk, n, i, tp.l0_hits, tp.l0_window, tp.l0_distinct != 0);
-                const uint32_t m = __ballot_sync(0xffffffffu, drop);
-                if (lane == 0 && m) atomicAnd(&mask[(base >> 5) + warp], ~m);
-            }
-        }
-        cons_sync<NC>();
-    }
-    PHASE_MARK(kPhD);
-
-    // E. ordered seed list: thread x takes mask word w_lo + x (at most
-    //    CAP / 32 <= NC words); each word's offset adds the totals of the
-    //    warps before it.  Marks lie in the core: positions [c0, c1)
-    uint16_t *seed_idx = cx.seed_idx();
-    const uint32_t w_lo = c0 >> 5, w_hi = (c1 + 31) >> 5;
-    const uint32_t nwords = w_hi - w_lo;
-    const uint32_t nw_used = (nwords + 31) >> 5;
-    uint32_t *wtot = s_tot;                               // [NW]
-    uint32_t ns = 0;
-    {
-        const uint32_t m = tid < nwords ? mask[w_lo + tid] : 0u;
-        const uint32_t c = __popc(m);
-        const uint32_t incl = warp < nw_used ? warp_incl_scan(c) : 0u;
-        if (warp < nw_used && lane == 31) wtot[warp] = incl;
-        cons_sync<NC>();
-        uint32_t before = 0;
-        for (uint32_t w2 = 0; w2 < nw_used; ++w2) {
-            const uint32_t v = wtot[w2];
-            before += w2 < warp ? v : 0u;
-            ns += v;
-        }
-        uint32_t at = before + incl - c;
-        uint32_t mm = m;
-        while (mm) {
-            const uint32_t bit = __ffs(mm) - 1;
-            mm &= mm - 1;
-            if (CHECK(2, at, CAP)) seed_idx[at] = (uint16_t)((w_lo + tid) * 32 + bit);
-            ++at;
-        }
-    }
-    cons_sync<NC>();
-    PHASE_MARK(kPhE);
-    if (tid == 0) PHASE_ADD(kPhSeeds, ns);
-
-    // F. causal count c(s) over each seed's scan range, 4 lanes per seed, or
-    //    its distinct-PMT form
-    uint16_t *seed_cnt = cx.seed_cnt();
-    if (tp.count_distinct) {
-        count_distinct_pmts<CAP, NC, NB>(cx, pk, n, ns, seed_idx, bsh, seed_cnt);
-    } else {
-        count_causal<CAP, NC, 2u, NB>(cx, pk, n, ns, seed_idx, bsh, seed_cnt);
-    }
-    cons_sync<NC>();
-    PHASE_MARK(kPhF);
-    auto count_of = [&](uint32_t k) -> uint32_t { return seed_cnt[k]; };
-
-    // G. emit the fired seeds in order: warp w takes a contiguous range of
-    //    the seed list and adds up the fired totals of the warps before it.
-    const uint32_t threshold = tp.threshold;
-    const uint32_t per_w = (ns + NW - 1) / NW;
-    const uint32_t k_begin = min(ns, warp * per_w), k_end = min(ns, k_begin + per_w);
-    uint32_t my_f = 0;
-    for (uint32_t k0 = k_begin; k0 < k_end; k0 += 32) {
-        const uint32_t k = k0 + lane;
-        my_f += __popc(__ballot_sync(0xffffffffu, k < k_end && count_of(k) >= threshold));
-    }
-    uint32_t *ftot = s_tot + NW;                          // [NW]: fired per warp, then their prefix
-    if (lane == 0) ftot[warp] = my_f;
-    cons_sync<NC>();
-    if (warp == 0) {
-        const uint32_t v = lane < NW ? ftot[lane] : 0u;
-        const uint32_t vi = warp_incl_scan(v);
-        if (lane < NW) ftot[lane] = vi - v;
-        if (lane == NW - 1) s_red[0] = vi;
-    }
-    cons_sync<NC>();
-    const uint32_t n_fired = s_red[0];
-    uint32_t F = ftot[warp];
-    trig_trigger *dst = out + (out_at_c0 ? c0 : 0u);
-    for (uint32_t k0 = k_begin; k0 < k_end; k0 += 32) {
-        const uint32_t k = k0 + lane;
-        const uint32_t cnt_k = k < k_end ? count_of(k) : 0u;
-        const bool fired = k < k_end && cnt_k >= threshold;
-        const uint32_t m = __ballot_sync(0xffffffffu, fired);
-        if (fired) {
-            const uint32_t i = seed_idx[k];
-            const uint32_t ks = pk[i];
-            const uint32_t q = chg[i];
-            const uint32_t o_ = F + __popc(m & ((1u << lane) - 1u));
-            trig_trigger tr;
-            tr.t_ns = tb + (int64_t)(ks >> 12);
-            tr.pmt = (uint16_t)(ks & 0xfffu);
-            tr.charge = (uint16_t)q;
-            tr.count = cnt_k;
-            if (CHECK(3, o_, c1 - c0)) {
-                dst[o_] = tr;
-                // the merged ranks of the first hit of the seed's event
-                // window [t - h, t + h] and of the first hit past it, where
-                // that bound lies in the staged range (else kRankUnknown:
-                // the window pass searches for it)
-                const uint32_t ts = ks >> 12, wh = tp.win_half;
-                const uint32_t r_lo = ts >= wh ? rank_base + keys_before<NB, 12>(pk, cnt, n, ts - wh, bsh, span)
-                                               : kRankUnknown;
-                const uint32_t r_hi = ts + wh + 1u <= span
-                                          ? rank_base + keys_before<NB, 12>(pk, cnt, n, ts + wh + 1u, bsh, span)
-                                          : kRankUnknown;
-                *reinterpret_cast<uint2 *>(wr + 2 * ((out_at_c0 ? c0 : 0u) + o_)) = make_uint2(r_lo, r_hi);
-            }
-        }
-        F += __popc(m);
-    }
-    // optional row outputs: the merged core rows
-    // (verification, and the merged stream of event extraction) and each
-    // row's causal count (verification only); rows are indexed by merged
-    // rank minus the rank of the slice's first owned hit
-    if (tp.dbg_merged) {
-        const uint64_t dbg_base = (uint64_t)(dbg_rank_lo + (int64_t)c0);
-        for (uint32_t i = tid; i < c1 - c0; i += NC) {
-            const uint32_t k = pk[c0 + i];
-            trig_hit h;
-            h.t_ns = tb + (int64_t)(k >> 12);
-            h.pmt = (uint16_t)(k & 0xfffu);
-            h.charge = chg[c0 + i];
-            h.reserved = 0;
-            tp.dbg_merged[dbg_base + i] = h;
-            if (tp.dbg_seedcnt) tp.dbg_seedcnt[dbg_base + i] = 0xffffffffu;
-        }
-        if (tp.dbg_seedcnt) {
-            cons_sync<NC>();
-            for (uint32_t k = tid; k < ns; k += NC) tp.dbg_seedcnt[dbg_base + (seed_idx[k] - c0)] = seed_cnt[k];
-        }
-    }
-    // leave the bucket counts and the seed mask zero for the next tile
-    // (after every warp's last read of the offsets: the window ranks above)
-    cons_sync<NC>();
-    for (uint32_t i = tid; i < NB; i += NC) cnt[i] = 0;
-    for (uint32_t w = w_lo + tid; w < w_hi; w += NC) mask[w] = 0;
-    cons_sync<NC>();
-    PHASE_MARK(kPhG);
-#undef PHASE_MARK
-    CoreOut co;
-    co.n_fired = n_fired;
-    co.n_seeds = ns;
-    co.c0 = c0;
-    return co;
-}
-
 // Causal count c(s) = #{ j : |t_j - t_s| <= min(dt_max[p_s][p_j], W) } over
 // each seed's scan range keys [j0, j1) (seed_range), a group of 2^lg lanes
 // per seed; a fired seed sets its position in mask.
@@ -1552,11 +1020,10 @@ __device__ CoreOut sorted_pass(SortCtx<CAP> &cx, const uint64_t *stage, uint32_t
 // earlier buckets, more than dmax_row(p_s) >= dt before t_s, those from j1
 // on in later buckets, and the four end keys past the last key are beyond
 // any dt as well, so whole groups of four from j0 rounded down are taken.
-template <int CAP, int NC, bool NARROW, uint32_t NB>
-__device__ __forceinline__ void count_seeds(const TileCtx<CAP, NARROW> &cx, uint32_t n, uint32_t ns, uint32_t bsh,
-                                            uint32_t lg, uint32_t threshold)
+template <uint32_t NB, int NC, bool EXT, class C>
+__device__ __forceinline__ void count_seeds(const C &cx, uint32_t n, uint32_t ns, uint32_t bsh, uint32_t lg,
+                                            uint32_t threshold, uint32_t dt_mask)
 {
-    using C = TileCtx<CAP, NARROW>;
     const uint32_t tid = threadIdx.x, G = 1u << lg, gl = tid & (G - 1u), gid = tid >> lg, NG = NC >> lg;
     const uint32_t *pk = cx.pk();
     const uint32_t *seeds = cx.seeds();
@@ -1571,17 +1038,10 @@ __device__ __forceinline__ void count_seeds(const TileCtx<CAP, NARROW> &cx, uint
             uint32_t j0, j1;
             seed_range<NB>(cx, ts, ps, bsh, j0, j1);
             if (CHECK(12, j1, n + 1) && CHECK(13, ps, cx.P)) {
-                const uint32_t row_s = (uint32_t)TileCtx<CAP, NARROW>::L::oDt + ps * kDtRow;
-                const uint16_t *row_g = cx.dt_g + (size_t)ps * cx.P;
+                const auto row = cx.row(ps);
                 auto causal = [&](uint32_t kj) -> uint32_t {
-                    uint32_t lim;
-                    if (NARROW) {
-                        lim = *reinterpret_cast<const uint16_t *>(g_tile_smem + (row_s | (kj & C::kPmtMask)));
-                    } else {
-                        const uint32_t pj = C::key_p(kj);
-                        if (!CHECK(11, pj, cx.P)) return 0u;
-                        lim = __ldg(row_g + pj);
-                    }
+                    if (!CHECK(11, C::key_p(kj), cx.P)) return 0u;
+                    const uint32_t lim = EXT ? row.at(kj) & dt_mask : row.at(kj);
                     return __usad(C::key_t(kj), ts, 0u) <= lim;
                 };
                 uint32_t ca = 0, cb = 0, cc = 0, cd = 0;
@@ -1603,9 +1063,14 @@ __device__ __forceinline__ void count_seeds(const TileCtx<CAP, NARROW> &cx, uint
     }
 }
 
-// One staged tile through the whole trigger, default rule: the n records of
-// `stage` (16 bytes each, any order) span [tb, tb + span); the core is
-// t - tb in [lo_t, hi_t).
+// One staged tile through the whole trigger: the n records of `stage` (16
+// bytes each, any order) span [tb, tb + span); the core is t - tb in
+// [lo_t, hi_t).  The default builds take the default seed rule alone; the
+// extended ones (EXT) level 0, seed rule 1, the distinct count, row outputs
+// and event extraction as well (on 52 M hits with dt rows in shared memory
+// and unsorted buckets where order is not needed: the ladder 4.61 ms, 5.38
+// with a full sort and dt rows through the cache, the distinct count 1.67,
+// 2.30 before, both in 4096-hit tiles).
 //
 //  A. every record becomes a packed key (TileCtx::key), is counted in its
 //     time bucket (t - tb) >> bsh and marked in its floor cell (floor, and
@@ -1614,10 +1079,13 @@ __device__ __forceinline__ void count_seeds(const TileCtx<CAP, NARROW> &cx, uint
 //     cell with another hit in it or in a neighbouring cell;
 //  C. the k-way merge of the PMT runs ("DAQ system of NEMO Phase II"): keys
 //     scattered to bucket order, about one key per bucket.  A core hit
-//     over the charge threshold or in a marked cell becomes a candidate;
+//     over the charge threshold or in a marked cell becomes a candidate.
+//     For level 0 and row outputs the keys of a bucket are also sorted by
+//     (t, pmt, charge);
 //  D. floor coincidences ("Sorting and triggering in GPU": another PMT of
 //     the same floor within tau): each candidate looks through the buckets
-//     of [t - tau, t + tau];
+//     of [t - tau, t + tau].  EXT: seed rule 1 (coincidence_seed) tests
+//     every core key instead, and level 0 each seed;
 //  E. the causal counts (count_seeds);
 //  F. the fired seeds to out, in (t, pmt, charge) order: a seed's rank is
 //     the number of fired positions before it, corrected inside its bucket.
@@ -1632,12 +1100,12 @@ __device__ __forceinline__ void count_seeds(const TileCtx<CAP, NARROW> &cx, uint
 // 4.43 ms with the search from every hit and an ordered seed list; the
 // 2688-PMT slice 1.22 ms, 2.05 before.
 // The bucket counts, cells and mask are zero on entry and on return.
-template <int CAP, int NC, bool NARROW, bool DENSE>
-__device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span,
-                             uint32_t lo_t, uint32_t hi_t, const TrigParams &tp, trig_trigger *out, uint32_t *wr,
-                             bool out_at_c0, uint32_t rank_base, uint64_t *release_bar)
+template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE>
+__device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *stage, uint32_t n, int64_t tb,
+                             uint32_t span, uint32_t lo_t, uint32_t hi_t, const TrigParams &tp, trig_trigger *out,
+                             uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo, uint64_t *release_bar)
 {
-    using C = TileCtx<CAP, NARROW>;
+    using C = TileCtx<CAP, NC, NARROW, EXT>;
     using L = typename C::L;
     constexpr uint32_t NW = NC / 32;
     constexpr int PER = CAP / NC;
@@ -1647,7 +1115,7 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
     const uint32_t bsh = bucket_shift<NB>(span);
     const uint32_t tau = tp.tau;
     __shared__ uint32_t s_red[NW];
-    __shared__ uint32_t s_n[3];             // candidates, seeds, keys before the core
+    __shared__ uint32_t s_n[4];             // candidates, seeds, keys before the core, before its end
     uint32_t *cnt = cx.cnt(), *mask = cx.mask(), *cells = cx.cells();
     uint32_t *pk = cx.pk(), *seeds = cx.seeds(), *cand = cx.cand();
     const uint16_t *fl = cx.floor_s();
@@ -1668,6 +1136,10 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
 #define PHASE_MARK(i) ((void)0)
 #endif
 
+    // seed rule 1 looks through time, not floor cells; level 0 and the row
+    // outputs need the keys of a bucket in order
+    const bool rule1 = EXT && tp.seed_rule == 1, sorted = EXT && (tp.l0_hits || tp.dbg_merged);
+
     // A. keys, bucket counts, floor cells
     uint32_t key[PER], cs[PER], hc[PER];  // packed key; charge << 16 | slot in the bucket; floor cell
     if (tid == 0) s_n[0] = s_n[1] = 0;
@@ -1684,6 +1156,7 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
             cs[r] = (v.z & 0xffff0000u) | atomicAdd(&cnt[tr >> bsh], 1u);
             const uint32_t h = (fl[p] * fstep + (tr >> csh)) & (M - 1u), bit = 1u << (2u * (h & 15u));
             hc[r] = h;
+            if (rule1) continue;
             if (atomicOr(&cells[h >> 4], bit) & bit) atomicOr(&cells[h >> 4], bit << 1);
         }
     }
@@ -1752,20 +1225,55 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
     PHASE_MARK(kPhB);
 
     // C. bucket order and candidates (charge << 16 | position, with bit 15
-    //    set for a charge over the threshold)
+    //    set for a charge over the threshold); where they are needed sorted,
+    //    each key then goes to its rank inside its bucket, in place
     {
+        uint32_t pos[PER];
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            pos[r] = 0;
+            if (key[r] != kPkNone) {
+                pos[r] = cnt[C::key_t(key[r]) >> bsh] + (cs[r] & 0xffffu);
+                if (CHECK(22, pos[r], CAP)) {
+                    pk[pos[r]] = key[r];
+                    if (EXT) cx.chg()[pos[r]] = (uint16_t)(cs[r] >> 16);
+                }
+            }
+        }
+        if (sorted) {
+            const uint16_t *chg = cx.chg();
+            cons_sync<NC>();
+#pragma unroll
+            for (int r = 0; r < PER; ++r) {
+                if (key[r] == kPkNone) continue;
+                const uint32_t k = key[r], b = C::key_t(k) >> bsh, q = cs[r] >> 16;
+                const uint32_t s0 = cnt[b], s1 = cnt[b + 1];
+                uint32_t rk = s0;
+                for (uint32_t m = s0; m < s1; ++m) {
+                    const uint32_t o = pk[m];
+                    rk += o < k;
+                    if (o == k) rk += chg[m] < q || (chg[m] == q && m < pos[r]);     // equal time and PMT
+                }
+                pos[r] = rk;
+            }
+            cons_sync<NC>();
+#pragma unroll
+            for (int r = 0; r < PER; ++r)
+                if (key[r] != kPkNone && CHECK(23, pos[r], CAP)) {
+                    pk[pos[r]] = key[r];
+                    cx.chg()[pos[r]] = (uint16_t)(cs[r] >> 16);
+                }
+        }
         uint32_t m[PER], total = 0;
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             bool c = false;
-            if (key[r] != kPkNone) {
+            if (key[r] != kPkNone && !rule1) {
                 const uint32_t tr = C::key_t(key[r]);
-                const uint32_t pos = cnt[tr >> bsh] + (cs[r] & 0xffffu);
-                if (CHECK(22, pos, CAP)) pk[pos] = key[r];
                 if (tr - lo_t < hi_t - lo_t) {
                     const bool over = (cs[r] >> 16) >= tp.q_seed;
                     c = over || ((cells[hc[r] >> 4] >> (2u * (hc[r] & 15u))) & 1u);
-                    cs[r] = (cs[r] & 0xffff0000u) | pos | (over ? 0x8000u : 0u);
+                    cs[r] = (cs[r] & 0xffff0000u) | pos[r] | (over ? 0x8000u : 0u);
                 }
             }
             m[r] = __ballot_sync(0xffffffffu, c);
@@ -1786,11 +1294,19 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
     // D. floor coincidences of the candidates, four keys of the range at a
     //    time; the seeds take the cells' place
     {
-        const uint32_t nc = s_n[0];
+        // seed rule 1 tests every key of the core's buckets instead
+        const uint32_t k0 = rule1 ? cnt[bucket_of<NB>(lo_t, bsh)] : 0u;
+        const uint32_t nc = rule1 ? cnt[bucket_of<NB>(hi_t - 1u, bsh) + 1] - k0 : s_n[0];
         for (uint32_t x = warp * 32; x < nc; x += NC) {
             bool seed = false;
             uint32_t e = 0;
-            if (x + lane < nc) {
+            if (rule1) {
+                if (x + lane < nc) {
+                    const uint32_t i = k0 + x + lane, ti = C::key_t(pk[i]);
+                    e = (uint32_t)cx.chg()[EXT ? i : 0] << 16 | i;
+                    seed = ti - lo_t < hi_t - lo_t && coincidence_seed<NB>(cx, tp, i, bsh);
+                }
+            } else if (x + lane < nc) {
                 e = cand[x + lane];
                 seed = (e >> 15) & 1u;
                 e &= 0xffff7fffu;
@@ -1810,6 +1326,20 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
                     }
                 }
             }
+            if (EXT && tp.l0_hits) {
+                // level 0 (N hits within TW) before the seed triggers count
+                if (tp.l0_distinct && cx.P > 128) {
+                    // a warp per seed, marking its PMTs in a shared-memory set
+                    for (uint32_t todo = __ballot_sync(0xffffffffu, seed); todo; todo &= todo - 1u) {
+                        const uint32_t b = __ffs(todo) - 1;
+                        const uint32_t i = __shfl_sync(0xffffffffu, e, b) & 0xffffu;
+                        const bool ok = level0_distinct_warp<C>(pk, n, i, tp.l0_hits, tp.l0_window, cx.P, cx.pmt_set(warp));
+                        if (lane == b) seed = ok;
+                    }
+                } else if (seed) {
+                    seed = level0_pass<C>(pk, n, e & 0xffffu, tp.l0_hits, tp.l0_window, tp.l0_distinct != 0);
+                }
+            }
             const uint32_t m = __ballot_sync(0xffffffffu, seed);
             uint32_t at = 0;
             if (lane == 0 && m) at = atomicAdd(&s_n[1], __popc(m));
@@ -1818,6 +1348,7 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
         }
         // keys before the core: the fired seeds' place in the slice's staging
         if (tid == NC - 1) s_n[2] = keys_before<NB, C::kShift>(pk, cnt, n, lo_t, bsh, span);
+        if (EXT && tid == NC - 33) s_n[3] = keys_before<NB, C::kShift>(pk, cnt, n, hi_t, bsh, span);
     }
     cons_sync<NC>();
     PHASE_MARK(kPhD);
@@ -1832,7 +1363,8 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
         lg = 2;
         while (lg < 5 && (ns << (lg + 1)) <= NC) ++lg;
     }
-    count_seeds<CAP, NC, NARROW, NB>(cx, n, ns, bsh, lg, tp.threshold);
+    if (EXT && tp.count_distinct) count_distinct_pmts<NB, NC>(cx, n, ns, bsh, tp.threshold, tp.dt_mask);
+    else count_seeds<NB, NC, EXT>(cx, n, ns, bsh, lg, tp.threshold, tp.dt_mask);
     cons_sync<NC>();
     PHASE_MARK(kPhE);
 
@@ -1888,6 +1420,27 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NARROW> &cx, const uint64_t *stage, ui
         // the trigger's two halves: time; PMT, charge and count
         const uint64_t half = side ? (uint64_t)c << 32 | (e & 0xffff0000u) | C::key_p(ks) : (uint64_t)(tb + (int64_t)ts);
         reinterpret_cast<uint64_t *>(out + out_at + o)[side] = half;
+    }
+    // optional row outputs: the merged core rows (verification, and the
+    // merged stream of event extraction) and each row's causal count
+    // (verification only); rows are indexed by merged rank minus the rank of
+    // the slice's first owned hit
+    if (EXT && tp.dbg_merged) {
+        const uint32_t c1 = s_n[3];
+        const uint64_t dbg_base = (uint64_t)(dbg_rank_lo + (int64_t)c0);
+        for (uint32_t i = tid; i < c1 - c0; i += NC) {
+            const uint32_t k = pk[c0 + i];
+            // (8-byte stores: the rows may be the caller's buffer)
+            uint64_t *row = reinterpret_cast<uint64_t *>(tp.dbg_merged + dbg_base + i);
+            row[0] = (uint64_t)(tb + (int64_t)C::key_t(k));
+            row[1] = C::key_p(k) | (uint32_t)cx.chg()[c0 + i] << 16;
+            if (tp.dbg_seedcnt) tp.dbg_seedcnt[dbg_base + i] = 0xffffffffu;
+        }
+        if (tp.dbg_seedcnt) {
+            cons_sync<NC>();
+            for (uint32_t k = tid; k < ns; k += NC)
+                tp.dbg_seedcnt[dbg_base + ((seeds[k] & 0xffffu) - c0)] = cx.counts()[k];
+        }
     }
     // leave the bucket counts, cells and mask zero for the next tile
     cons_sync<NC>();
@@ -2045,26 +1598,23 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                                                                           uint32_t max_pmt)
 {
     constexpr uint32_t NW = NC / 32;
-    using L = TileLayout<CAP, EXT>;
-    constexpr uint32_t NSTG = L::NS;
-    __shared__ uint64_t full_bar[2], empty_bar[2];
-    __shared__ ItemInfo info[2];
+    using C = TileCtx<CAP, NC, SMEM_DT, EXT>;
+    using L = typename C::L;
+    __shared__ uint64_t full_bar, empty_bar;
+    __shared__ ItemInfo info;
     __shared__ __align__(16) uint32_t red[64 + 64];
     __shared__ int64_t stk[128];
 
-    std::conditional_t<EXT, SortCtx<CAP>, TileCtx<CAP, SMEM_DT>> cx;
+    C cx;
     cx.pp = (max_pmt + 7) & ~7u;
     cx.dt_g = nullptr;
     cx.P = 0;
-    if constexpr (!EXT) cx.tab = (uint32_t)L::tab(max_pmt, SMEM_DT);
-    auto stage_of = [&](uint32_t b) { return reinterpret_cast<uint64_t *>(g_tile_smem + (size_t)b * L::kStage); };
+    cx.tab = (uint32_t)L::tab(max_pmt);
 
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     if (tid == 0) {
-        mbar_init(&full_bar[0], 1);
-        mbar_init(&full_bar[1], 1);
-        mbar_init(&empty_bar[0], 1);
-        mbar_init(&empty_bar[1], 1);
+        mbar_init(&full_bar, 1);
+        mbar_init(&empty_bar, 1);
         fence_mbar_init();
     }
     __syncthreads();
@@ -2087,7 +1637,6 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
         if (lane == 0) item = atomicAdd(&hdr->queue, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
         for (uint32_t it = 0;; ++it) {
-            const uint32_t b = it % NSTG, use = it / NSTG;
 #ifdef TRIG_PHASE_STATS
             const long long tp0 = clock64();
 #endif
@@ -2161,14 +1710,14 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             if (lane == 0) PHASE_ADD(kPhProdItem, tw0 - tp0);
 #endif
             uint32_t free_ok = 1;
-            if (it >= NSTG && lane == 0) {
+            if (it >= 1 && lane == 0) {
 #ifdef TRIG_PHASE_STATS
                 uint32_t pr = 0;
-                free_ok = mbar_wait(&empty_bar[b], (use - 1) & 1u, wait_ns, &pr) ? 1u : 0u;
+                free_ok = mbar_wait(&empty_bar, (it - 1) & 1u, wait_ns, &pr) ? 1u : 0u;
                 PHASE_ADD(kPhProdWait, clock64() - tw0);
                 PHASE_ADD(kPhProdWaitRounds, pr);
 #else
-                free_ok = mbar_wait(&empty_bar[b], (use - 1) & 1u, wait_ns) ? 1u : 0u;
+                free_ok = mbar_wait(&empty_bar, (it - 1) & 1u, wait_ns) ? 1u : 0u;
 #endif
             }
             free_ok = __shfl_sync(0xffffffffu, free_ok, 0);
@@ -2179,27 +1728,27 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             }
             if (item >= n_items) {
                 if (lane == 0) {
-                    info[b].item = -1;
-                    mbar_arrive(&full_bar[b]);
+                    info.item = -1;
+                    mbar_arrive(&full_bar);
                 }
                 break;
             }
             if (lane == 0) {
-                info[b].item = (int32_t)item;
-                info[b].slice = s;
-                info[b].g = g;
-                info[b].n = min(tot, (uint32_t)CAP);
-                info[b].rank_lo = rlo;
-                info[b].mode = mode;
-                info[b].lo_t = lo_t;
-                info[b].span = span;
-                if (mode == 0) mbar_arrive_expect_tx(&full_bar[b], tot * 16u);
-                else mbar_arrive(&full_bar[b]);
+                info.item = (int32_t)item;
+                info.slice = s;
+                info.g = g;
+                info.n = min(tot, (uint32_t)CAP);
+                info.rank_lo = rlo;
+                info.mode = mode;
+                info.lo_t = lo_t;
+                info.span = span;
+                if (mode == 0) mbar_arrive_expect_tx(&full_bar, tot * 16u);
+                else mbar_arrive(&full_bar);
             }
             __syncwarp();
             if (mode == 0 && wide) {
                 if (lane == 0 && CHECK(7, (uint64_t)rlo + tot, d->n_hits + 1))
-                    bulk_g2s(stage_of(b), d->tbuf + rlo, tot * 16u, &full_bar[b]);
+                    bulk_g2s(cx.stage(), d->tbuf + rlo, tot * 16u, &full_bar);
             } else if (mode == 0) {
                 uint32_t dst = 0;
 #pragma unroll
@@ -2207,7 +1756,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                     const uint32_t len = rl[r], a = ra[r];
                     const uint32_t incl = warp_incl_scan(len);
                     if (len && CHECK(6, dst + incl, CAP + 1) && CHECK(7, (uint64_t)a + len, d->n_hits + 1))
-                        bulk_g2s(stage_of(b) + 2 * (size_t)(dst + incl - len), d->hits + a, len * 16u, &full_bar[b]);
+                        bulk_g2s(cx.stage() + 2 * (size_t)(dst + incl - len), d->hits + a, len * 16u, &full_bar);
                     dst += __shfl_sync(0xffffffffu, incl, 31);
                 }
             }
@@ -2220,11 +1769,10 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     }
 
     // ---------------------------------------------------- consumer warps
-    // the tile pass expects zero bucket counts, masks and bitmaps (and leaves them so)
+    // the tile pass expects zero bucket counts, mask and cells (and leaves them so)
     for (uint32_t i = tid; i < (uint32_t)L::NBK; i += NC) cx.cnt()[i] = 0;
     for (uint32_t i = tid; i < (uint32_t)CAP / 32; i += NC) cx.mask()[i] = 0;
-    if constexpr (!EXT)
-        for (uint32_t i = tid; i < L::kCells / 16; i += NC) cx.cells()[i] = 0;
+    for (uint32_t i = tid; i < L::kCells / 16; i += NC) cx.cells()[i] = 0;
     cons_sync<NC>();
     const SliceDesc *loaded = nullptr;
     // the slice's trigger parameters live in shared memory (written by one
@@ -2236,34 +1784,29 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     auto pass = [&](const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span, uint32_t lo_t, uint32_t hi_t,
                     trig_trigger *out, uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo,
                     uint64_t *release_bar) {
-        if constexpr (EXT)
-            return sorted_pass<CAP, NC>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0, rank_base,
-                                        dbg_rank_lo, release_bar);
-        else
-            return tile_pass<CAP, NC, SMEM_DT, DENSE>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0,
-                                                      rank_base, release_bar);
+        return tile_pass<CAP, NC, SMEM_DT, EXT, DENSE>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0, rank_base,
+                                                       dbg_rank_lo, release_bar);
     };
     for (uint32_t it = 0;; ++it) {
-        const uint32_t b = it % NSTG, use = it / NSTG;
         // every thread waits (bounded) for the staged tile; the barrier
         // ANDs their results, so the block never splits on a timeout
 #ifdef TRIG_PHASE_STATS
         const long long tw0 = clock64();
         uint32_t cr = 0;
-        const bool cwait_ok = mbar_wait(&full_bar[b], use & 1u, wait_ns, &cr);
+        const bool cwait_ok = mbar_wait(&full_bar, it & 1u, wait_ns, &cr);
         if (tid == 0) {
             PHASE_ADD(kPhConsWait, clock64() - tw0);
             PHASE_ADD(kPhConsWaitRounds, cr);
             PHASE_ADD(kPhTiles, 1);
         }
 #else
-        const bool cwait_ok = mbar_wait(&full_bar[b], use & 1u, wait_ns);
+        const bool cwait_ok = mbar_wait(&full_bar, it & 1u, wait_ns);
 #endif
         if (!named_sync_and(kBarCons, NC, cwait_ok)) {
             if (tid == 0) atomicOr(&hdr->err, TRIG_FLAG_TIMEOUT);
             break;
         }
-        const ItemInfo &inf = info[b];      // stable until this buffer is released
+        const ItemInfo &inf = info;      // stable until this buffer is released
         if (inf.item < 0) break;
         const SliceDesc &d = desc[inf.slice];
         if (&d != loaded) {
@@ -2274,8 +1817,11 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 cx.floor_s()[p] = d.floor[p];
                 cx.dmax_s()[p] = d.dmax_row[p];
             }
-            if constexpr (!EXT && SMEM_DT)
-                for (uint32_t i = tid; i < P * P; i += NC) cx.dt_s()[(i / P) * (kDtRow / 2) + i % P] = d.dt[i];
+            // seed rule 1: the PMT relation above a dt that leaves it room
+            const bool pack = EXT && SMEM_DT && d.rel_in_dt;
+            if (SMEM_DT)
+                for (uint32_t i = tid; i < P * P; i += NC)
+                    cx.dt_s()[(i / P) * (kDtRow / 2) + i % P] = (uint16_t)(d.dt[i] | (pack ? (uint32_t)d.rel[i] << kRelShift : 0u));
             cx.dt_g = d.dt;
             cx.P = P;
             loaded = &d;
@@ -2293,6 +1839,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 tp.fc_w = d.fc_w;
                 tp.afc_w = d.afc_w;
                 tp.count_distinct = d.count_distinct;
+                tp.dt_mask = pack ? (1u << kRelShift) - 1u : 0xffffu;
                 tp.rel = d.rel;
                 tp.dbg_merged = d.dbg_merged;
                 tp.dbg_seedcnt = d.dbg_seedcnt;
@@ -2311,7 +1858,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 d.tile_rank[inf.g] = 0;
             }
         } else if (inf.mode == 1) {
-            tile_overflow<CAP, NC>(pass, stage_of(b), d, inf.g, red, stk);
+            tile_overflow<CAP, NC>(pass, cx.stage(), d, inf.g, red, stk);
         } else {
             const int64_t W = sl[0];
             const uint32_t g = inf.g, n_st = inf.n, rank_lo = inf.rank_lo, span = inf.span;
@@ -2324,8 +1871,8 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             // the pass hands the buffer back as soon as it has read it (inf
             // is not read after that); the core's first hit has merged rank
             // rank_lo + c0
-            CoreOut co = pass(stage_of(b), n_st, tb, span, lo_t, hi_t, d.stage + rank_lo, d.wrank + 2 * (size_t)rank_lo,
-                              true, rank_lo, (int64_t)rank_lo - sl[3], &empty_bar[b]);
+            CoreOut co = pass(cx.stage(), n_st, tb, span, lo_t, hi_t, d.stage + rank_lo, d.wrank + 2 * (size_t)rank_lo,
+                              true, rank_lo, (int64_t)rank_lo - sl[3], &empty_bar);
             const uint32_t tile_rank = rank_lo + co.c0;
             if (tid == 0 && CHECK(14, (uint64_t)tile_rank + co.n_fired, d.n_hits + 1) && CHECK(15, g, d.n_tiles)) {
                 d.tile_nfired[g] = co.n_fired;
@@ -2338,7 +1885,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
         // accesses before its next bulk copy into the same buffer
         fence_proxy_async_smem();
         cons_sync<NC>();
-        if (tid == 0) mbar_arrive(&empty_bar[b]);
+        if (tid == 0) mbar_arrive(&empty_bar);
     }
 }
 
@@ -3164,7 +2711,7 @@ template <int CAP, int NC, bool SMEM_DT, bool EXT = false, bool DENSE = false>
 static cudaError_t launch_tile(BatchHeader *hdr, SliceDesc *desc, uint32_t max_pmt, cudaStream_t st)
 {
     static bool limit_set[64] = {};
-    size_t smem = TileLayout<CAP, EXT>::bytes(max_pmt, SMEM_DT);
+    size_t smem = TileLayout<CAP, NC, SMEM_DT, EXT>::bytes(max_pmt);
     auto kern = k_tile<CAP, NC, SMEM_DT, EXT, DENSE>;
     cudaError_t e = raise_smem_limit(kern, limit_set);
     if (e != cudaSuccess) return e;
@@ -3217,17 +2764,23 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
     const bool smem_dt = any_smem_dt && max_pmt <= kSmemDtMaxPmt;
     if (any_ext || any_events || rows) {
         // level 0, seed rule 1, distinct count, and every batch that needs
-        // the merged rows (event extraction, row outputs): the build that
-        // puts each tile in full (t, pmt, charge) order, one per shape, dt
-        // rows read through the cache
+        // the merged rows (event extraction, row outputs): the builds that
+        // put each tile in full (t, pmt, charge) order
         if (cfg.cap == 1024)
-            e = launch_tile<1024, 128, false, true>(d_hdr, d_desc, max_pmt, st);
+            e = smem_dt ? launch_tile<1024, 128, true, true>(d_hdr, d_desc, max_pmt, st)
+                        : launch_tile<1024, 128, false, true>(d_hdr, d_desc, max_pmt, st);
+        else if (cfg.cap == 2048 && cfg.warps == 16)
+            e = smem_dt ? launch_tile<2048, 512, true, true>(d_hdr, d_desc, max_pmt, st)
+                        : launch_tile<2048, 512, false, true>(d_hdr, d_desc, max_pmt, st);
         else if (cfg.cap == 2048)
-            e = cfg.warps == 16 ? launch_tile<2048, 512, false, true>(d_hdr, d_desc, max_pmt, st)
-                                : launch_tile<2048, 256, false, true>(d_hdr, d_desc, max_pmt, st);
+            e = smem_dt ? launch_tile<2048, 256, true, true>(d_hdr, d_desc, max_pmt, st)
+                        : launch_tile<2048, 256, false, true>(d_hdr, d_desc, max_pmt, st);
+        else if (cfg.warps == 8)
+            e = smem_dt ? launch_tile<4096, 256, true, true>(d_hdr, d_desc, max_pmt, st)
+                        : launch_tile<4096, 256, false, true>(d_hdr, d_desc, max_pmt, st);
         else
-            e = cfg.warps == 8 ? launch_tile<4096, 256, false, true>(d_hdr, d_desc, max_pmt, st)
-                               : launch_tile<4096, 512, false, true>(d_hdr, d_desc, max_pmt, st);
+            e = smem_dt ? launch_tile<4096, 512, true, true>(d_hdr, d_desc, max_pmt, st)
+                        : launch_tile<4096, 512, false, true>(d_hdr, d_desc, max_pmt, st);
     } else if (dense) {
         // a warp per seed in the causal count; dt rows read through the cache
         if (cfg.cap == 1024)
