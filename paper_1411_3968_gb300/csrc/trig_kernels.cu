@@ -631,10 +631,16 @@ struct ItemInfo {
     uint32_t g;
     uint32_t n;         // staged hits
     uint32_t rank_lo;   // merged rank of the first staged hit
-    uint32_t mode;      // 0 staged, 1 overflow (split path), 2 skip (bad slice or empty)
-    uint32_t lo_t;      // B_g minus the time of the staged range's start
-    uint32_t span;      // length of the staged time range (ns)
+    uint32_t mode;      // kItem*
+    uint32_t off;       // start of the core, from the tile's (ns)
+    uint32_t core;      // length of the core
+    uint32_t lo_t;      // start of the core, from the staged range's
+    uint32_t span;      // length of the staged range
 };
+// A whole staged tile; one with more hits than fit, left to tile_overflow
+// (wide slices); nothing to do (bad slice or empty); a staged piece of a
+// tile, and the end of a tile's pieces.
+enum : uint32_t { kItemTile, kItemOverflow, kItemSkip, kItemPiece, kItemEnd };
 
 // Shared memory of the tile kernel, in this order: the staging buffer (handed
 // back after its first read, so the next tile's copy overlaps the rest of the
@@ -1461,7 +1467,8 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
     return co;
 }
 
-// Overflow path: the tile holds more than CAP hits with its halo.  Split
+// Overflow path of the wide slices (a narrow one's tile is split by the
+// stager): the tile holds more than CAP hits with its halo.  Split
 // its core in halves until each piece fits; pieces are staged with plain
 // loads after per-PMT binary searches.  A 1 ns core that still does not
 // fit is reported (TRIG_FLAG_TILE_FULL) and skipped.
@@ -1592,6 +1599,117 @@ __device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint
     cons_sync<NC>();
 }
 
+// The stager's side of the hand-over of the one staging buffer.
+struct Stager {
+    uint64_t *full, *empty;
+    ItemInfo *info;
+    uint64_t *stage;
+    uint32_t it;                // hand-overs so far
+    // lane 0 waits (bounded) for the buffer and decides for the warp
+    __device__ __forceinline__ bool wait_free(BatchHeader *hdr, uint64_t wait_ns)
+    {
+        uint32_t ok = 1;
+        if (it >= 1 && lane_id() == 0) {
+#ifdef TRIG_PHASE_STATS
+            const long long tw0 = clock64();
+            uint32_t pr = 0;
+            ok = mbar_wait(empty, (it - 1) & 1u, wait_ns, &pr) ? 1u : 0u;
+            PHASE_ADD(kPhProdWait, clock64() - tw0);
+            PHASE_ADD(kPhProdWaitRounds, pr);
+#else
+            ok = mbar_wait(empty, (it - 1) & 1u, wait_ns) ? 1u : 0u;
+#endif
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();
+        if (!ok && lane_id() == 0) atomicOr(&hdr->err, TRIG_FLAG_TIMEOUT);
+        ++it;
+        return ok != 0;
+    }
+    // the item's description; with n > 0 hits to come by bulk copies
+    __device__ __forceinline__ void hand_over(const ItemInfo &x, uint32_t n)
+    {
+        if (lane_id() == 0) {
+            *info = x;
+            info->n = n;
+            if (n) mbar_arrive_expect_tx(full, n * 16u);
+            else mbar_arrive(full);
+        }
+        __syncwarp();
+    }
+    // one copy of a PMT run of len hits from a, at dst of the tile's (the
+    // lanes' runs follow each other); dst moves past the warp's
+    __device__ __forceinline__ void copy_run(const trig_hit *hits, uint64_t n_hits, uint32_t a, uint32_t len, uint32_t cap,
+                                             uint32_t &dst)
+    {
+        const uint32_t incl = warp_incl_scan(len);
+        if (len && CHECK(6, dst + incl, cap + 1) && CHECK(7, (uint64_t)a + len, n_hits + 1))
+            bulk_g2s(stage + 2 * (size_t)(dst + incl - len), hits + a, len * 16u, full);
+        dst += __shfl_sync(0xffffffffu, incl, 31);
+    }
+};
+
+constexpr uint32_t kStageRuns = 4;          // PMT runs per lane of the stager (narrow slices have at most 128)
+constexpr uint32_t kMaxPieces = 24;         // open halves of a core below 2^20 ns
+
+// A tile of a narrow slice with more hits than fit (a burst): its core is
+// halved until each piece fits with its halo; the pieces' runs are found
+// inside the tile's (runs: start and end of each PMT's, in shared memory).  A
+// 1 ns piece that still does not fit is reported and left out.  Returns
+// false when a wait ran out.
+__device__ __forceinline__ bool stage_pieces(Stager &sg, ItemInfo x, uint32_t cap, const SliceDesc *d, const uint2 *runs,
+                                          uint2 *pieces, BatchHeader *hdr)
+{
+    const uint32_t lane = lane_id(), H = d->halo, rlo = x.rank_lo;
+    const uint64_t wait_ns = hdr->wait_ns;
+    const int64_t Bg = d->t0 + (int64_t)x.g * d->tile_w;
+    uint32_t depth = 1;
+    if (lane == 0) pieces[0] = make_uint2(0u, x.core);
+    __syncwarp();
+    while (depth) {
+        const uint32_t lo = pieces[depth - 1].x, hi = pieces[depth - 1].y;
+        __syncwarp();
+        --depth;
+        uint32_t pa[kStageRuns], pe[kStageRuns], n = 0, rank = 0;
+#pragma unroll
+        for (uint32_t r = 0; r < kStageRuns; ++r) {
+            const uint2 run = runs[r * 32 + lane];
+            pa[r] = (uint32_t)lb_time(d->hits, run.x, run.y, Bg + lo - (int64_t)H);
+            pe[r] = (uint32_t)lb_time(d->hits, pa[r], run.y, Bg + hi + (int64_t)H);
+            n += pe[r] - pa[r];
+            rank += pa[r] - run.x;
+        }
+        n = __reduce_add_sync(0xffffffffu, n);
+        rank = __reduce_add_sync(0xffffffffu, rank);
+        if (n > cap) {
+            if (hi - lo > 1 && depth + 2 <= kMaxPieces) {
+                const uint32_t mid = lo + (hi - lo) / 2;
+                if (lane == 0) {
+                    pieces[depth] = make_uint2(mid, hi);            // right half below,
+                    pieces[depth + 1] = make_uint2(lo, mid);        // left half on top
+                }
+                __syncwarp();
+                depth += 2;
+            } else if (lane == 0) {
+                report(*d, TRIG_FLAG_TILE_FULL);
+            }
+            continue;
+        }
+        if (n == 0) continue;
+        if (!sg.wait_free(hdr, wait_ns)) return false;
+        x.rank_lo = rlo + rank;
+        x.off = lo, x.core = hi - lo, x.lo_t = H, x.span = hi - lo + 2 * H;
+        sg.hand_over(x, n);
+        uint32_t dst = 0;
+#pragma unroll
+        for (uint32_t r = 0; r < kStageRuns; ++r) sg.copy_run(d->hits, d->n_hits, pa[r], pe[r] - pa[r], cap, dst);
+    }
+    if (!sg.wait_free(hdr, wait_ns)) return false;
+    x.mode = kItemEnd;
+    sg.hand_over(x, 0);
+    return true;
+}
+
 template <int CAP, int NC, bool SMEM_DT, bool EXT, bool DENSE>
 __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 1)) k_tile(BatchHeader *__restrict__ hdr,
                                                                           const SliceDesc *__restrict__ desc,
@@ -1604,6 +1722,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     __shared__ ItemInfo info;
     __shared__ __align__(16) uint32_t red[64 + 64];
     __shared__ int64_t stk[128];
+    __shared__ uint2 pieces[kMaxPieces], runs[32 * kStageRuns];
 
     C cx;
     cx.pp = (max_pmt + 7) & ~7u;
@@ -1632,15 +1751,16 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
         uint32_t s = 0;
         bool bad = false;
         const SliceDesc *d = nullptr;
-        constexpr int R = 4;                       // PMTs per lane kept in registers
+        constexpr int R = kStageRuns;              // PMTs per lane kept in registers
         uint32_t item = 0;
         if (lane == 0) item = atomicAdd(&hdr->queue, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
-        for (uint32_t it = 0;; ++it) {
+        Stager sg{&full_bar, &empty_bar, &info, cx.stage(), 0u};
+        for (;;) {
 #ifdef TRIG_PHASE_STATS
             const long long tp0 = clock64();
 #endif
-            uint32_t g = 0, P = 0, mode = 2, lo_t = 0, span = 0;
+            uint32_t g = 0, P = 0, mode = kItemSkip, lo_t = 0, span = 0;
             uint32_t ra[R], rl[R];                  // hit indices are below 2^32 - 16
             uint32_t tot = 0, rlo = 0;
             bool wide = false;
@@ -1697,67 +1817,38 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                     tot = __reduce_add_sync(0xffffffffu, tot);
                     rlo = __reduce_add_sync(0xffffffffu, rlo);
                 }
-                mode = bad ? 2u : (tot > (uint32_t)CAP ? 1u : (tot == 0 ? 2u : 0u));
+                mode = bad || tot == 0 ? kItemSkip : tot <= (uint32_t)CAP ? kItemTile : wide ? kItemOverflow : kItemPiece;
             }
             uint32_t next = 0;
             if (item < n_items) {
                 if (lane == 0) next = atomicAdd(&hdr->queue, 1u);
                 next = __shfl_sync(0xffffffffu, next, 0);
             }
-            // lane 0 waits (bounded) for the buffer and decides for the warp
 #ifdef TRIG_PHASE_STATS
-            const long long tw0 = clock64();
-            if (lane == 0) PHASE_ADD(kPhProdItem, tw0 - tp0);
+            if (lane == 0) PHASE_ADD(kPhProdItem, clock64() - tp0);
 #endif
-            uint32_t free_ok = 1;
-            if (it >= 1 && lane == 0) {
-#ifdef TRIG_PHASE_STATS
-                uint32_t pr = 0;
-                free_ok = mbar_wait(&empty_bar, (it - 1) & 1u, wait_ns, &pr) ? 1u : 0u;
-                PHASE_ADD(kPhProdWait, clock64() - tw0);
-                PHASE_ADD(kPhProdWaitRounds, pr);
-#else
-                free_ok = mbar_wait(&empty_bar, (it - 1) & 1u, wait_ns) ? 1u : 0u;
-#endif
-            }
-            free_ok = __shfl_sync(0xffffffffu, free_ok, 0);
-            __syncwarp();
-            if (!free_ok) {
-                if (lane == 0) atomicOr(&hdr->err, TRIG_FLAG_TIMEOUT);
-                break;
-            }
             if (item >= n_items) {
-                if (lane == 0) {
-                    info.item = -1;
-                    mbar_arrive(&full_bar);
-                }
+                if (sg.wait_free(hdr, wait_ns)) sg.hand_over(ItemInfo{-1}, 0);
                 break;
             }
-            if (lane == 0) {
-                info.item = (int32_t)item;
-                info.slice = s;
-                info.g = g;
-                info.n = min(tot, (uint32_t)CAP);
-                info.rank_lo = rlo;
-                info.mode = mode;
-                info.lo_t = lo_t;
-                info.span = span;
-                if (mode == 0) mbar_arrive_expect_tx(&full_bar, tot * 16u);
-                else mbar_arrive(&full_bar);
-            }
-            __syncwarp();
-            if (mode == 0 && wide) {
-                if (lane == 0 && CHECK(7, (uint64_t)rlo + tot, d->n_hits + 1))
-                    bulk_g2s(cx.stage(), d->tbuf + rlo, tot * 16u, &full_bar);
-            } else if (mode == 0) {
-                uint32_t dst = 0;
+            const int64_t W = d->tile_w, Bg = d->t0 + (int64_t)g * W;
+            const uint32_t core = (uint32_t)(min(Bg + W, d->t0 + d->slice_ns) - Bg);
+            const ItemInfo x{(int32_t)item, s, g, 0, rlo, mode, 0, core, lo_t, span};
+            if (mode == kItemPiece) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const uint32_t len = rl[r], a = ra[r];
-                    const uint32_t incl = warp_incl_scan(len);
-                    if (len && CHECK(6, dst + incl, CAP + 1) && CHECK(7, (uint64_t)a + len, d->n_hits + 1))
-                        bulk_g2s(cx.stage() + 2 * (size_t)(dst + incl - len), d->hits + a, len * 16u, &full_bar);
-                    dst += __shfl_sync(0xffffffffu, incl, 31);
+                for (int r = 0; r < R; ++r) runs[r * 32 + lane] = make_uint2(ra[r], ra[r] + rl[r]);
+                __syncwarp();
+                if (!stage_pieces(sg, x, CAP, d, runs, pieces, hdr)) break;
+            } else {
+                if (!sg.wait_free(hdr, wait_ns)) break;
+                sg.hand_over(x, mode == kItemTile ? tot : 0u);
+                if (mode == kItemTile && wide) {
+                    if (lane == 0 && CHECK(7, (uint64_t)rlo + tot, d->n_hits + 1))
+                        bulk_g2s(cx.stage(), d->tbuf + rlo, tot * 16u, &full_bar);
+                } else if (mode == kItemTile) {
+                    uint32_t dst = 0;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) sg.copy_run(d->hits, d->n_hits, ra[r], rl[r], CAP, dst);
                 }
             }
 #ifdef TRIG_PHASE_STATS
@@ -1778,9 +1869,62 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     // the slice's trigger parameters live in shared memory (written by one
     // thread when the slice changes), keeping registers for the tile phases
     __shared__ TrigParams tp;
-    // the loaded slice's tile width, t0, length and merged rank of its first
-    // owned hit, also kept in shared memory
-    __shared__ int64_t sl[4];
+    // the loaded slice's tile width, t0 and merged rank of its first owned
+    // hit, also kept in shared memory
+    __shared__ int64_t sl[3];
+    // the tables of a slice's detector (kept while the next slice has the
+    // same) and its parameters
+    auto load_slice = [&](const SliceDesc &d) {
+        if (cx.dt_g != d.dt) {
+            const uint32_t P = d.n_pmt;
+            for (uint32_t p = tid; p < P; p += NC) {
+                cx.floor_s()[p] = d.floor[p];
+                cx.dmax_s()[p] = d.dmax_row[p];
+            }
+            // seed rule 1: the PMT relation above a dt that leaves it room
+            const bool pack = EXT && SMEM_DT && d.rel_in_dt;
+            if (SMEM_DT)
+                for (uint32_t p = warp; p < P; p += NW)
+                    for (uint32_t q = lane; q < P; q += 32) {
+                        uint32_t v = d.dt[p * P + q];
+                        if (pack) v |= (uint32_t)d.rel[p * P + q] << kRelShift;
+                        cx.dt_s()[p * (kDtRow / 2) + q] = (uint16_t)v;
+                    }
+            cx.dt_g = d.dt;
+            cx.P = P;
+        }
+        loaded = &d;
+        if (tid == 0) {
+            tp.H = d.halo;
+            tp.win_half = d.win_half;
+            tp.tau = d.tau;
+            tp.q_seed = d.q_seed;
+            tp.threshold = d.threshold;
+            tp.l0_hits = d.l0_hits;
+            tp.l0_window = d.l0_window;
+            tp.l0_distinct = d.l0_distinct;
+            tp.seed_rule = d.seed_rule;
+            tp.sc_w = d.sc_w;
+            tp.fc_w = d.fc_w;
+            tp.afc_w = d.afc_w;
+            tp.count_distinct = d.count_distinct;
+            tp.dt_mask = EXT && SMEM_DT && d.rel_in_dt ? (1u << kRelShift) - 1u : 0xffffu;
+            tp.rel = d.rel;
+            tp.dbg_merged = d.dbg_merged;
+            tp.dbg_seedcnt = d.dbg_seedcnt;
+            sl[0] = d.tile_w;
+            sl[1] = d.t0;
+            sl[2] = (int64_t)d.dbg_rank0;
+        }
+    };
+    // while the first tile is looked up and copied: the slice it is in if the
+    // blocks take the first items in turn
+    if (n_items) load_slice(desc[find_slice_by_item(desc, n_slices, min(blockIdx.x, n_items - 1u))]);
+    // the tile whose pieces are coming: its fired seeds so far, where they
+    // start, and whether a piece was seen (thread 0 writes after a pass; the
+    // next tile's barrier publishes it)
+    __shared__ uint32_t pc[3];
+    if (tid < 3) pc[tid] = 0;
     auto pass = [&](const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span, uint32_t lo_t, uint32_t hi_t,
                     trig_trigger *out, uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo,
                     uint64_t *release_bar) {
@@ -1810,73 +1954,41 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
         if (inf.item < 0) break;
         const SliceDesc &d = desc[inf.slice];
         if (&d != loaded) {
-            // (re)load the detector tables of this slice
             cons_sync<NC>();
-            const uint32_t P = d.n_pmt;
-            for (uint32_t p = tid; p < P; p += NC) {
-                cx.floor_s()[p] = d.floor[p];
-                cx.dmax_s()[p] = d.dmax_row[p];
-            }
-            // seed rule 1: the PMT relation above a dt that leaves it room
-            const bool pack = EXT && SMEM_DT && d.rel_in_dt;
-            if (SMEM_DT)
-                for (uint32_t i = tid; i < P * P; i += NC)
-                    cx.dt_s()[(i / P) * (kDtRow / 2) + i % P] = (uint16_t)(d.dt[i] | (pack ? (uint32_t)d.rel[i] << kRelShift : 0u));
-            cx.dt_g = d.dt;
-            cx.P = P;
-            loaded = &d;
-            if (tid == 0) {
-                tp.H = d.halo;
-                tp.win_half = d.win_half;
-                tp.tau = d.tau;
-                tp.q_seed = d.q_seed;
-                tp.threshold = d.threshold;
-                tp.l0_hits = d.l0_hits;
-                tp.l0_window = d.l0_window;
-                tp.l0_distinct = d.l0_distinct;
-                tp.seed_rule = d.seed_rule;
-                tp.sc_w = d.sc_w;
-                tp.fc_w = d.fc_w;
-                tp.afc_w = d.afc_w;
-                tp.count_distinct = d.count_distinct;
-                tp.dt_mask = pack ? (1u << kRelShift) - 1u : 0xffffu;
-                tp.rel = d.rel;
-                tp.dbg_merged = d.dbg_merged;
-                tp.dbg_seedcnt = d.dbg_seedcnt;
-            }
-            if (tid == 0) {
-                sl[0] = d.tile_w;
-                sl[1] = d.t0;
-                sl[2] = d.slice_ns;
-                sl[3] = (int64_t)d.dbg_rank0;
-            }
+            load_slice(d);
             cons_sync<NC>();
         }
-        if (inf.mode == 2) {
+        if (inf.mode == kItemSkip || inf.mode == kItemEnd) {
             if (tid == 0) {
-                d.tile_nfired[inf.g] = 0;
-                d.tile_rank[inf.g] = 0;
+                d.tile_nfired[inf.g] = pc[0];
+                d.tile_rank[inf.g] = pc[1];
+                pc[0] = pc[1] = pc[2] = 0;
             }
-        } else if (inf.mode == 1) {
+        } else if (inf.mode == kItemOverflow) {
             tile_overflow<CAP, NC>(pass, cx.stage(), d, inf.g, red, stk);
         } else {
-            const int64_t W = sl[0];
-            const uint32_t g = inf.g, n_st = inf.n, rank_lo = inf.rank_lo, span = inf.span;
-            const int64_t Bg = sl[1] + (int64_t)g * W;
-            const int64_t core_end = min(Bg + W, sl[1] + sl[2]);
+            const uint32_t g = inf.g, n_st = inf.n, rank_lo = inf.rank_lo, span = inf.span, lo_t = inf.lo_t;
+            const uint32_t hi_t = lo_t + inf.core;
+            const bool piece = inf.mode == kItemPiece;
             // the staged range starts lo_t (>= H) before the core
-            const uint32_t lo_t = inf.lo_t;
-            const int64_t tb = Bg - (int64_t)lo_t;
-            const uint32_t hi_t = lo_t + (uint32_t)(core_end - Bg);
-            // the pass hands the buffer back as soon as it has read it (inf
-            // is not read after that); the core's first hit has merged rank
-            // rank_lo + c0
-            CoreOut co = pass(cx.stage(), n_st, tb, span, lo_t, hi_t, d.stage + rank_lo, d.wrank + 2 * (size_t)rank_lo,
-                              true, rank_lo, (int64_t)rank_lo - sl[3], &empty_bar);
+            const int64_t tb = sl[1] + (int64_t)g * sl[0] + (int64_t)inf.off - (int64_t)lo_t;
+            // a tile's (or its first piece's) fired seeds go to the merged
+            // rank of its first core hit, rank_lo + c0; the other pieces'
+            // follow them.  The pass hands the buffer back as soon as it has
+            // read it (inf is not read after that)
+            const bool seen = pc[2] != 0;
+            const size_t at = seen ? pc[1] + pc[0] : rank_lo;
+            const CoreOut co = pass(cx.stage(), n_st, tb, span, lo_t, hi_t, d.stage + at, d.wrank + 2 * at, !seen, rank_lo,
+                                    (int64_t)rank_lo - sl[2], &empty_bar);
             const uint32_t tile_rank = rank_lo + co.c0;
             if (tid == 0 && CHECK(14, (uint64_t)tile_rank + co.n_fired, d.n_hits + 1) && CHECK(15, g, d.n_tiles)) {
-                d.tile_nfired[g] = co.n_fired;
-                d.tile_rank[g] = tile_rank;
+                if (!piece) {
+                    d.tile_nfired[g] = co.n_fired;
+                    d.tile_rank[g] = tile_rank;
+                } else {
+                    if (!pc[2]) pc[1] = tile_rank, pc[2] = 1;
+                    pc[0] += co.n_fired;
+                }
                 atomicAdd(reinterpret_cast<unsigned long long *>(&d.stats->n_seeds), (unsigned long long)co.n_seeds);
             }
             continue;
