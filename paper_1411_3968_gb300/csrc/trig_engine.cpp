@@ -80,8 +80,12 @@ extern "C" int trig_host_free(void *ptr)
 static std::atomic<uint64_t> g_launches{0};
 extern "C" uint64_t trig_kernel_launch_count(void) { return g_launches.load(); }
 
+// Launch shape of untuned detectors: the caller's (trig_set_tile_config), or,
+// until the first such call, the library's own choice for each batch (spread
+// 1, see spread_tiles).
 static std::mutex g_cfg_mu;
 static TileConfig g_cfg{4096, 16, 60};
+static bool g_cfg_set = false;
 
 extern "C" int trig_set_tile_config(uint32_t cap, uint32_t warps, uint32_t fill_pct)
 {
@@ -90,6 +94,7 @@ extern "C" int trig_set_tile_config(uint32_t cap, uint32_t warps, uint32_t fill_
                                  "(1024,4)}, fill_pct in [10, 95]");
     std::lock_guard<std::mutex> lk(g_cfg_mu);
     g_cfg = TileConfig{cap, warps, fill_pct};
+    g_cfg_set = true;
     return TRIG_OK;
 }
 
@@ -118,7 +123,7 @@ extern "C" int trig_set_device_wait(uint64_t limit_ns, int stall)
 static TileConfig current_cfg()
 {
     std::lock_guard<std::mutex> lk(g_cfg_mu);
-    return g_cfg;
+    return g_cfg_set ? g_cfg : kOwnShape;
 }
 
 static bool tune_cache_lookup(uint32_t n_pmt, TileConfig &out);
@@ -388,16 +393,44 @@ struct Plan {
     TileConfig shape{};         // launch shape of this batch
 };
 
+// Hits that a tile's core should hold at most when the library chooses the
+// shape itself: the batch's hits in whole waves of equal tiles over the
+// resident blocks (two of the 2048-hit shape on an SM), so that a small
+// batch uses every SM and none waits for a last wave that is nearly empty.
+// A tile has a cost of its own (about 4 us of barriers and look-ups), so
+// below 128 hits a tile is not cut smaller; and where a few waves are all
+// there is, a tile that a burst overfills would be the last to end, so they
+// are filled to 65 % (three PMTs at 500 kHz add a third to a tower's hits).
+// 0: no bound.
+static double spread_tiles(const trig_slice_dev *sl, uint32_t n, const TileConfig &cfg)
+{
+    if (!cfg.spread) return 0.0;
+    double hits = 0.0, full = 0.0, roomy = 0.0;
+    for (uint32_t s = 0; s < n; ++s) {
+        const trig_detector *det = sl[s].det;
+        if (!det || det->tuned) continue;
+        const double span = (double)det->par.slice_ns + 2.0 * (double)det->in_halo;
+        const double halo = 2.0 * det->tile_halo * (double)sl[s].n_hits / span;
+        hits += (double)sl[s].n_hits;
+        full += (double)sl[s].n_hits / std::max((double)cfg.cap * cfg.fill_pct / 100.0 - halo, 64.0);
+        roomy += (double)sl[s].n_hits / std::max((double)cfg.cap * 0.65 - halo, 64.0);
+    }
+    const double slots = 2.0 * device_sm_count();
+    if (full > 8.0 * slots) return 0.0;             // the work queue evens out many waves
+    return std::max(128.0, std::ceil(hits / (slots * std::max(std::ceil(roomy / slots), 1.0))));
+}
+
 // Tile width W (ns): a tile plus its two halos is expected to hold fill% of
-// the tile capacity at the slice's mean rate; W >= 256 ns and at most 2^20
-// tiles per slice.
-static int64_t choose_tile_w(const trig_detector *det, uint64_t n_hits, const TileConfig &cfg)
+// the tile capacity at the slice's mean rate, and its core at most core_max
+// hits (0: no bound); W >= 256 ns and at most 2^20 tiles per slice.
+static int64_t choose_tile_w(const trig_detector *det, uint64_t n_hits, const TileConfig &cfg, double core_max)
 {
     const double span = (double)det->par.slice_ns + 2.0 * (double)det->in_halo;
     const double rate = n_hits > 0 ? (double)n_hits / span : 1e-9;       // hits per ns
     const uint32_t fill = det->tuned ? det->tile.fill_pct : cfg.fill_pct;
     const double target = (double)cfg.cap * fill / 100.0;
     double w = target / rate - 2.0 * det->tile_halo;
+    if (core_max > 0.0 && !det->tuned) w = std::min(w, core_max / rate);
     const double w_min = std::max(256.0, (double)det->par.slice_ns / (double)kMaxTilesPerSlice + 1.0);
     if (w < w_min) w = w_min;
     if (w > (double)det->par.slice_ns) w = (double)det->par.slice_ns;
@@ -416,7 +449,7 @@ struct WideGrid {
     uint32_t wb, hh, m, lead, nb;
 };
 
-static WideGrid wide_grid(const trig_detector *det, uint64_t n_hits, const TileConfig &cfg)
+static WideGrid wide_grid(const trig_detector *det, uint64_t n_hits, const TileConfig &cfg, double core_max)
 {
     const double S = (double)det->par.slice_ns;
     const double span = S + 2.0 * (double)det->in_halo;
@@ -431,6 +464,7 @@ static WideGrid wide_grid(const trig_detector *det, uint64_t n_hits, const TileC
     g.wb = (uint32_t)std::min(wb, 1e9);
     g.hh = H ? (H + g.wb - 1) / g.wb : 0;
     double m = std::floor(target / ((double)g.wb * rate)) - 2.0 * g.hh;
+    if (core_max > 0.0 && !det->tuned) m = std::min(m, std::ceil(core_max / ((double)g.wb * rate)));
     m = std::min(m, std::ceil(S / g.wb));
     m = std::min(m, std::floor((double)(kMaxTileSpan - 1) / g.wb) - 2.0 * g.hh);   // staged span below 2^20 ns
     m = std::max(1.0, m);
@@ -454,6 +488,7 @@ static TileConfig batch_shape(const trig_slice_dev *sl, uint32_t n, const TileCo
             best = sl[s].n_hits;
             out.cap = det->tile.cap;
             out.warps = det->tile.warps;
+            out.spread = 0;
         }
     }
     return out;
@@ -468,6 +503,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
     if (!sl || n == 0) return fail(TRIG_EINVAL, "no slices");
     const TileConfig cfg = batch_shape(sl, n, cfg_in);
     if (shape_out) *shape_out = cfg;
+    const double core_max = spread_tiles(sl, n, cfg);
     size_t off = align256(sizeof(BatchHeader));
     off += align256(sizeof(SliceDesc) * n);
     uint32_t items = 0, chunks = 0, fins = 0;
@@ -523,7 +559,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
         }
         int64_t W = 0;
         if (wide) {
-            const WideGrid wg = wide_grid(det, x.n_hits, cfg);
+            const WideGrid wg = wide_grid(det, x.n_hits, cfg, core_max);
             if ((uint64_t)(wg.m + 2 * wg.hh) * wg.wb >= (uint64_t)kMaxTileSpan)
                 return fail(TRIG_EINVAL, "slice too long for this detector's tiles");
             W = (int64_t)wg.m * wg.wb;
@@ -537,7 +573,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             d.bkt32 = (uint64_t)wg.nb * wg.wb < ((uint64_t)1 << 31);
             d.bkt_origin = x.t0_ns - (int64_t)wg.lead * wg.wb;
         } else {
-            W = choose_tile_w(det, x.n_hits, cfg);
+            W = choose_tile_w(det, x.n_hits, cfg, core_max);
         }
         d.tile_w = W;
         d.w_magic = (uint32_t)((((uint64_t)1 << 32) + (uint64_t)W - 1) / (uint64_t)W);
@@ -1022,7 +1058,8 @@ extern "C" int trig_autotune(trig_detector *det, const trig_slice_dev *slices, u
 extern "C" int trig_detector_tile_config(const trig_detector *det, uint32_t *cap, uint32_t *warps, uint32_t *fill_pct)
 {
     if (!det) return fail(TRIG_EINVAL, "NULL detector");
-    const TileConfig c = det->tuned ? det->tile : current_cfg();
+    TileConfig c = det->tuned ? det->tile : current_cfg();
+    if (c.spread) trig_get_tile_config(&c.cap, &c.warps, &c.fill_pct);
     if (cap) *cap = c.cap;
     if (warps) *warps = c.warps;
     if (fill_pct) *fill_pct = c.fill_pct;
