@@ -893,30 +893,63 @@ __device__ __forceinline__ void count_distinct_pmts(const CTX &cx, uint32_t n, u
     }
 }
 
-// Level 0 at sorted index i: some window [t_j, t_j + TW) with
-// t_i - TW < t_j <= t_i holds at least N hits, or hits of N different PMTs
-// (P <= 128 here; above, level0_distinct_warp).  Only the first index of each time starts a window; every
-// hit within TW of a core hit is staged (the tile halo covers TW).  The
-// distinct count slides the window back start by start, keeping per-PMT
-// counts, so it reads each hit within 2 TW once.
+// A window-edge rank the tile pass could not read off its staged keys.
+constexpr uint32_t kRankUnknown = 0xffffffffu;
+
+// Staged keys with time below x (relative to the staged range's start, x
+// in [0, span]): the buckets before x's bucket, plus the keys of that bucket
+// below x.  The keys of a bucket are contiguous in bucket order and in
+// sorted order alike.
+template <uint32_t NB, uint32_t SHIFT>
+__device__ __forceinline__ uint32_t keys_before(const uint32_t *pk, const uint32_t *cnt, uint32_t n, uint32_t x,
+                                                uint32_t bsh, uint32_t span)
+{
+    if (x >= span) return n;
+    const uint32_t b = bucket_of<NB>(x, bsh);
+    uint32_t c = cnt[b];
+    const uint32_t e = cnt[b + 1];
+    for (uint32_t m = c; m < e; ++m) c += (pk[m] >> SHIFT) < x;
+    return c;
+}
+
+// Level 0 for the key at position i: some window [t_j, t_j + TW) with
+// t_i - TW < t_j <= t_i holds at least N hits.  The hits of a window are the
+// difference of two exact ranks, so the keys of a bucket need no order; the
+// whole buckets inside the window that starts at t_i already hold N hits
+// where the tower is busy.  Every hit within TW of a core hit is staged (the
+// tile halo covers TW).
+template <uint32_t NB, class CTX>
+__device__ __noinline__ bool level0_pass(const CTX &cx, uint32_t n, uint32_t i, uint32_t N, uint32_t TW, uint32_t bsh,
+                                         uint32_t span)
+{
+    const uint32_t *pk = cx.pk(), *cnt = cx.cnt();
+    const uint32_t ts = CTX::key_t(pk[i]);
+    const uint32_t b0 = (ts >> bsh) + 1u, b1 = bucket_of<NB>(ts + TW, bsh);
+    if (b1 > b0 && cnt[b1] - cnt[b0] >= N) return true;
+    auto busy = [&](uint32_t tj) {
+        return keys_before<NB, CTX::kShift>(pk, cnt, n, tj + TW, bsh, span) -
+                   keys_before<NB, CTX::kShift>(pk, cnt, n, tj, bsh, span) >=
+               N;
+    };
+    if (busy(ts)) return true;
+    // the windows that start at an earlier hit
+    const uint32_t lo = ts >= TW ? ts - TW + 1u : 0u;
+    for (uint32_t j = cnt[lo >> bsh], je = cnt[b0]; j < je; ++j) {
+        const uint32_t tj = CTX::key_t(pk[j]);
+        if (tj >= lo && tj < ts && busy(tj)) return true;
+    }
+    return false;
+}
+
+// The same with hits of at least N different PMTs (up to 128 PMTs; above,
+// level0_distinct_warp), on sorted keys: the window slides back start by
+// start, keeping per-PMT counts, so it reads each hit within 2 TW once.
 template <class CTX>
-__device__ __noinline__ bool level0_pass(const uint32_t *pk, uint32_t n, uint32_t i, uint32_t N, uint32_t TW,
-                                         bool distinct)
+__device__ __noinline__ bool level0_distinct(const uint32_t *pk, uint32_t n, uint32_t i, uint32_t N, uint32_t TW)
 {
     const uint32_t ts = CTX::key_t(pk[i]);
     uint32_t j = i;
     while (j > 0 && CTX::key_t(pk[j - 1]) == ts) --j;             // first index of t_i
-    if (!distinct) {
-        for (;;) {
-            const uint32_t tj = CTX::key_t(pk[j]);
-            if (j + N - 1 < n && CTX::key_t(pk[j + N - 1]) - tj < TW) return true;
-            if (j == 0) return false;
-            const uint32_t tp = CTX::key_t(pk[j - 1]);
-            if (ts - tp >= TW) return false;
-            for (--j; j > 0 && CTX::key_t(pk[j - 1]) == tp; --j) {
-            }
-        }
-    }
     uint16_t cnt[128];
     for (uint32_t p = 0; p < 128; ++p) cnt[p] = 0;
     uint32_t distinct_n = 0, e = j;
@@ -982,25 +1015,6 @@ __device__ __noinline__ bool level0_distinct_warp(const uint32_t *pk, uint32_t n
         for (--j; j > 0 && CTX::key_t(pk[j - 1]) == tp; --j) {
         }
     }
-}
-
-// A window-edge rank the tile pass could not read off its staged keys.
-constexpr uint32_t kRankUnknown = 0xffffffffu;
-
-// Staged keys with time below x (relative to the staged range's start, x
-// in [0, span]): the buckets before x's bucket, plus the keys of that bucket
-// below x.  The keys of a bucket are contiguous in bucket order and in
-// sorted order alike.
-template <uint32_t NB, uint32_t SHIFT>
-__device__ __forceinline__ uint32_t keys_before(const uint32_t *pk, const uint32_t *cnt, uint32_t n, uint32_t x,
-                                                uint32_t bsh, uint32_t span)
-{
-    if (x >= span) return n;
-    const uint32_t b = bucket_of<NB>(x, bsh);
-    uint32_t c = cnt[b];
-    const uint32_t e = cnt[b + 1];
-    for (uint32_t m = c; m < e; ++m) c += (pk[m] >> SHIFT) < x;
-    return c;
 }
 
 // Bucket shift of a staged range of `span` ns: buckets of 2^bsh ns, NBK of
@@ -1086,12 +1100,13 @@ __device__ __forceinline__ void count_seeds(const C &cx, uint32_t n, uint32_t ns
 //  C. the k-way merge of the PMT runs ("DAQ system of NEMO Phase II"): keys
 //     scattered to bucket order, about one key per bucket.  A core hit
 //     over the charge threshold or in a marked cell becomes a candidate.
-//     For level 0 and row outputs the keys of a bucket are also sorted by
-//     (t, pmt, charge);
+//     For row outputs and level 0 over different PMTs the keys of a bucket
+//     are also sorted by (t, pmt, charge);
 //  D. floor coincidences ("Sorting and triggering in GPU": another PMT of
 //     the same floor within tau): each candidate looks through the buckets
-//     of [t - tau, t + tau].  EXT: seed rule 1 (coincidence_seed) tests
-//     every core key instead, and level 0 each seed;
+//     of [t - tau, t + tau].  EXT: or for seed rule 1 (coincidence_seed; it
+//     needs a hit of its own floor within SC or FC), and level 0 tests each
+//     seed;
 //  E. the causal counts (count_seeds);
 //  F. the fired seeds to out, in (t, pmt, charge) order: a seed's rank is
 //     the number of fired positions before it, corrected inside its bucket.
@@ -1125,9 +1140,12 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
     uint32_t *cnt = cx.cnt(), *mask = cx.mask(), *cells = cx.cells();
     uint32_t *pk = cx.pk(), *seeds = cx.seeds(), *cand = cx.cand();
     const uint16_t *fl = cx.floor_s();
-    // floor cells of 2^csh ns; the floors' ranges of cells follow each other,
-    // taken modulo M (two hits that share a cell by chance only cost a search)
-    const uint32_t csh = 32u - __clz(tau), fstep = (span >> csh) + 2u;
+    // floor cells of 2^csh ns, more than the floor coincidence (under seed
+    // rule 1, the wider of SC and FC); the floors' ranges of cells follow
+    // each other, taken modulo M (two hits that share a cell by chance only
+    // cost a search)
+    const bool rule1 = EXT && tp.seed_rule == 1;
+    const uint32_t csh = 32u - __clz(rule1 ? max(tp.sc_w, tp.fc_w) : tau), fstep = (span >> csh) + 2u;
 #ifdef TRIG_PHASE_STATS
     long long t_ph = clock64();
 #define PHASE_MARK(i)                                   \
@@ -1142,9 +1160,9 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
 #define PHASE_MARK(i) ((void)0)
 #endif
 
-    // seed rule 1 looks through time, not floor cells; level 0 and the row
-    // outputs need the keys of a bucket in order
-    const bool rule1 = EXT && tp.seed_rule == 1, sorted = EXT && (tp.l0_hits || tp.dbg_merged);
+    // level 0 over different PMTs and the row outputs need the keys of a
+    // bucket in order
+    const bool sorted = EXT && ((tp.l0_hits && tp.l0_distinct) || tp.dbg_merged);
 
     // A. keys, bucket counts, floor cells
     uint32_t key[PER], cs[PER], hc[PER];  // packed key; charge << 16 | slot in the bucket; floor cell
@@ -1162,7 +1180,6 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
             cs[r] = (v.z & 0xffff0000u) | atomicAdd(&cnt[tr >> bsh], 1u);
             const uint32_t h = (fl[p] * fstep + (tr >> csh)) & (M - 1u), bit = 1u << (2u * (h & 15u));
             hc[r] = h;
-            if (rule1) continue;
             if (atomicOr(&cells[h >> 4], bit) & bit) atomicOr(&cells[h >> 4], bit << 1);
         }
     }
@@ -1255,11 +1272,12 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
                 const uint32_t k = key[r], b = C::key_t(k) >> bsh, q = cs[r] >> 16;
                 const uint32_t s0 = cnt[b], s1 = cnt[b + 1];
                 uint32_t rk = s0;
-                for (uint32_t m = s0; m < s1; ++m) {
-                    const uint32_t o = pk[m];
-                    rk += o < k;
-                    if (o == k) rk += chg[m] < q || (chg[m] == q && m < pos[r]);     // equal time and PMT
-                }
+                if (s1 - s0 > 1)
+                    for (uint32_t m = s0; m < s1; ++m) {
+                        const uint32_t o = pk[m];
+                        rk += o < k;
+                        if (o == k && m != pos[r]) rk += chg[m] < q || (chg[m] == q && m < pos[r]);   // equal time, PMT
+                    }
                 pos[r] = rk;
             }
             cons_sync<NC>();
@@ -1274,10 +1292,10 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             bool c = false;
-            if (key[r] != kPkNone && !rule1) {
+            if (key[r] != kPkNone) {
                 const uint32_t tr = C::key_t(key[r]);
                 if (tr - lo_t < hi_t - lo_t) {
-                    const bool over = (cs[r] >> 16) >= tp.q_seed;
+                    const bool over = !rule1 && (cs[r] >> 16) >= tp.q_seed;
                     c = over || ((cells[hc[r] >> 4] >> (2u * (hc[r] & 15u))) & 1u);
                     cs[r] = (cs[r] & 0xffff0000u) | pos[r] | (over ? 0x8000u : 0u);
                 }
@@ -1300,23 +1318,16 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
     // D. floor coincidences of the candidates, four keys of the range at a
     //    time; the seeds take the cells' place
     {
-        // seed rule 1 tests every key of the core's buckets instead
-        const uint32_t k0 = rule1 ? cnt[bucket_of<NB>(lo_t, bsh)] : 0u;
-        const uint32_t nc = rule1 ? cnt[bucket_of<NB>(hi_t - 1u, bsh) + 1] - k0 : s_n[0];
+        const uint32_t nc = s_n[0];
         for (uint32_t x = warp * 32; x < nc; x += NC) {
             bool seed = false;
             uint32_t e = 0;
-            if (rule1) {
-                if (x + lane < nc) {
-                    const uint32_t i = k0 + x + lane, ti = C::key_t(pk[i]);
-                    e = (uint32_t)cx.chg()[EXT ? i : 0] << 16 | i;
-                    seed = ti - lo_t < hi_t - lo_t && coincidence_seed<NB>(cx, tp, i, bsh);
-                }
-            } else if (x + lane < nc) {
+            if (x + lane < nc) {
                 e = cand[x + lane];
                 seed = (e >> 15) & 1u;
                 e &= 0xffff7fffu;
-                if (!seed) {
+                if (rule1) seed = coincidence_seed<NB>(cx, tp, e & 0xffffu, bsh);
+                else if (!seed) {
                     const uint32_t ki = pk[e & 0xffffu], ti = C::key_t(ki), pi = C::key_p(ki), fi = fl[pi];
                     uint32_t j = cnt[(ti > tau ? ti - tau : 0u) >> bsh];
                     const uint32_t je = cnt[bucket_of<NB>(ti + tau, bsh) + 1];
@@ -1343,7 +1354,8 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
                         if (lane == b) seed = ok;
                     }
                 } else if (seed) {
-                    seed = level0_pass<C>(pk, n, e & 0xffffu, tp.l0_hits, tp.l0_window, tp.l0_distinct != 0);
+                    seed = tp.l0_distinct ? level0_distinct<C>(pk, n, e & 0xffffu, tp.l0_hits, tp.l0_window)
+                                          : level0_pass<NB>(cx, n, e & 0xffffu, tp.l0_hits, tp.l0_window, bsh, span);
                 }
             }
             const uint32_t m = __ballot_sync(0xffffffffu, seed);

@@ -83,3 +83,42 @@ def test_tile_pass_edges(pkg, params, shape, n_pmt, n, slice_ns, step, extra):
     for f in ("lo", "hi", "n_hits", "n_triggers"):
         assert np.array_equal(win[f], ref.windows[f]), f
     det.close()
+
+
+@pytest.mark.parametrize("n_pmt", [84, 129, 336])
+@pytest.mark.parametrize("cluster_ns", [40, 4_000, 30_000])
+@pytest.mark.parametrize("rule", [{}, dict(seed_rule=1, l0_hits=7, l0_window_ns=1000, threshold=1)])
+def test_bursts_split_tiles(pkg, params, n_pmt, cluster_ns, rule):
+    """Clusters that overfill tiles of every path, at the start, inside and at
+    the end of the slice: the pieces' seeds, ranks and windows are the
+    oracle's."""
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(n_pmt + cluster_ns))
+    par = dict(params, slice_ns=600_000, **rule)
+    t0, n = 1_000_000, 9000
+    xyz, floor = _detector(n_pmt)
+    hits, _ = _hits(rng, n, n_pmt, t0 - 3000, t0 + par["slice_ns"] + 3000)
+    for at, share in ((t0, 0), (t0 + 250_000, 1500), (t0 + par["slice_ns"] - cluster_ns, 3000)):
+        hits["t"][share:share + 1500] = at + rng.integers(0, cluster_ns, 1500)
+    hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    det = pkg.Detector(xyz, floor, par)
+    b = DeviceBatch([SliceIn(det, t0, hits, off)], events=True)
+    old = pkg.trig_get_tile_config()
+    for events, shape in ((True, (2048, 16, 90)), (False, (2048, 16, 90)), (False, (4096, 16, 95))):
+        pkg.trig_set_tile_config(*shape)
+        try:
+            b.set_events(events)
+            b.run()
+            (stats, trig, win), = b.results()
+        finally:
+            pkg.trig_set_tile_config(*old)
+        ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+        assert int(stats["status"]) == 0, shape
+        assert int(stats["n_seeds"]) == len(ref.seeds) and len(trig) == len(ref.triggers)
+        for f in ("t", "pmt", "charge", "count"):
+            assert np.array_equal(trig[f], ref.triggers[f]), (shape, f)
+        for f in ("lo", "hi", "n_hits", "n_triggers"):
+            assert np.array_equal(win[f], ref.windows[f]), (shape, f)
+    det.close()
