@@ -192,6 +192,39 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
 
 int device_sm_count();
 
+#ifdef __CUDACC__
+// The pipeline's kernels are launched as programmatic dependents: one may
+// start while its predecessor runs, sets up what needs no input, and waits
+// here until every kernel before it has ended and its writes are visible.
+// Every block of such a kernel waits, so a kernel's end implies that of all
+// before it.
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Lets the next kernel's blocks come in as soon as all of this one's have
+// started.
+__device__ __forceinline__ void let_next_kernel_in() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launches a kernel of the pipeline as a programmatic dependent of the one
+// before it on the stream (wait_for_previous_kernel).
+template <typename... P, typename... A>
+inline cudaError_t launch_next(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+#endif
+
+
 // Continuation submissions: the combined slice (resident tail of each PMT,
 // then the submission's hits of that PMT) into out / out_off.
 cudaError_t launch_prepend(const trig_hit *tail, const uint64_t *tail_off, uint64_t n_tail, const trig_hit *fresh,

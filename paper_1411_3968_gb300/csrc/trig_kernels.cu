@@ -503,6 +503,8 @@ __device__ __noinline__ void bounds_chunks_long(const SliceDesc &d, uint32_t c, 
 __global__ void __launch_bounds__(kBoundsThreads, 3) k_bounds(const BatchHeader *__restrict__ hdr,
                                                            const SliceDesc *__restrict__ desc)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t n_slices = hdr->n_slices, n_chunks = hdr->n_chunks;
     // no run of seeds is published yet (k_final)
     for (uint32_t i = blockIdx.x * kBoundsThreads + threadIdx.x; i < hdr->n_fin; i += gridDim.x * kBoundsThreads)
@@ -531,6 +533,8 @@ __global__ void __launch_bounds__(kBktChunk) k_bsum(const BatchHeader *__restric
 {
     __shared__ uint32_t wsum[32];
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     for (uint32_t s = 0; s < hdr->n_slices; ++s) {
         const SliceDesc &d = desc[s];
         if (!d.wide) continue;
@@ -558,6 +562,8 @@ __global__ void __launch_bounds__(kBktChunk) k_bscan(const BatchHeader *__restri
     __shared__ uint32_t base;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     constexpr uint32_t NW = kBktChunk / 32;
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     for (uint32_t s = 0; s < hdr->n_slices; ++s) {
         const SliceDesc &d = desc[s];
         if (!d.wide) continue;
@@ -605,6 +611,8 @@ __global__ void __launch_bounds__(kBktChunk) k_bscan(const BatchHeader *__restri
 // malformed input (flagged by the structure pass) are skipped.
 __global__ void __launch_bounds__(256) k_scatter(const BatchHeader *__restrict__ hdr, const SliceDesc *__restrict__ desc)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t n_slices = hdr->n_slices, n_chunks = hdr->n_chunks;
     for (uint32_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
         const SliceDesc &d = desc[find_slice_by_chunk(desc, n_slices, c)];
@@ -1749,6 +1757,8 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
         fence_mbar_init();
     }
     __syncthreads();
+    wait_for_previous_kernel();
+    let_next_kernel_in();
 
     const uint32_t n_slices = hdr->n_slices, n_items = hdr->n_items;
     const uint64_t wait_ns = hdr->wait_ns;
@@ -2184,6 +2194,7 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_final(BatchHeader *__restric
     __shared__ uint32_t s_chunk, s_err, s_off[kFinTiles + 1], s_rank[kFinTiles];
     __shared__ FinRun s_run[NW], s_before;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, lt = (1u << lane) - 1u;
+    wait_for_previous_kernel();
     const uint32_t n_slices = hdr->n_slices, n_chunks = hdr->n_fin;
     for (;;) {
         if (tid == 0) {
@@ -2782,6 +2793,7 @@ static_assert(sizeof(PutPlan<kPutSlices>) <= 32000, "kernel parameter space");
 template <uint32_t K>
 __global__ void __launch_bounds__(256) k_put(const __grid_constant__ PutPlan<K> plan, BatchHeader *hdr, SliceDesc *desc)
 {
+    let_next_kernel_in();
     const uint32_t tid = threadIdx.x, at = blockIdx.x * 256 + tid;
     const uint32_t *src_h = reinterpret_cast<const uint32_t *>(&plan.hdr);
     const uint32_t *src_d = reinterpret_cast<const uint32_t *>(plan.desc);
@@ -2879,8 +2891,7 @@ static cudaError_t launch_tile(BatchHeader *hdr, SliceDesc *desc, uint32_t max_p
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NC + 32, smem);
     if (per_sm < 1) per_sm = 1;
-    kern<<<device_sm_count() * per_sm, NC + 32, smem, st>>>(hdr, desc, max_pmt);
-    return cudaGetLastError();
+    return launch_next(kern, device_sm_count() * per_sm, NC + 32, smem, st, hdr, desc, max_pmt);
 }
 
 const char *const kKernelNames[kPipelineKernels] = {"k_put",    "k_bounds", "k_bsum",  "k_bscan",  "k_scatter", "k_tile",
@@ -2903,7 +2914,7 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
     mark(0);
     if ((e = launch_put(hdr, desc, d_hdr, d_desc, st, &nl)) != cudaSuccess) return e;
     mark(1);
-    k_bounds<<<sms * 6, kBoundsThreads, 0, st>>>(d_hdr, d_desc);
+    if ((e = launch_next(k_bounds, sms * 6, kBoundsThreads, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
     nl += 1;
     if (rows) {
         k_rank0<<<n_slices, 256, 0, st>>>(d_hdr, d_desc);
@@ -2911,11 +2922,11 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
     }
     mark(2);
     if (any_wide) {
-        k_bsum<<<sms * 2, kBktChunk, 0, st>>>(d_hdr, d_desc);
+        if ((e = launch_next(k_bsum, sms * 2, kBktChunk, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
         mark(3);
-        k_bscan<<<sms * 2, kBktChunk, 0, st>>>(d_hdr, d_desc);
+        if ((e = launch_next(k_bscan, sms * 2, kBktChunk, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
         mark(4);
-        k_scatter<<<sms * 8, 256, 0, st>>>(d_hdr, d_desc);
+        if ((e = launch_next(k_scatter, sms * 8, 256, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
         nl += 3;
     } else {
         mark(3);
@@ -2983,7 +2994,9 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
     }
     mark(7);
     // at most as many blocks as there are chunks of tiles
-    k_final<<<std::min<uint32_t>(hdr.n_fin, (uint32_t)sms * 8), kFinThreads, 0, st>>>(d_hdr, d_desc);
+    if ((e = launch_next(k_final, std::min<uint32_t>(hdr.n_fin, (uint32_t)sms * 8), kFinThreads, 0, st, d_hdr, d_desc)) !=
+        cudaSuccess)
+        return e;
     mark(8);
     if (any_events) {
         k_escan<<<sb, 1024, 0, st>>>(d_hdr, d_desc);
