@@ -576,8 +576,6 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             W = choose_tile_w(det, x.n_hits, cfg, core_max);
         }
         d.tile_w = W;
-        d.w_magic = (uint32_t)((((uint64_t)1 << 32) + (uint64_t)W - 1) / (uint64_t)W);
-        d.span32 = (det->par.slice_ns + 2 * det->in_halo + 2 * (int64_t)det->tile_halo + 2 * W) < ((int64_t)1 << 31);
         const uint64_t ng = x.n_hits ? (uint64_t)((det->par.slice_ns + W - 1) / W) : 0;
         if (ng > kMaxTilesPerSlice) return fail(TRIG_EINVAL, "too many tiles");
         d.n_tiles = (uint32_t)ng;
@@ -586,15 +584,27 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
         items += d.n_tiles;
         chunks += (uint32_t)((x.n_hits + kChunkHits - 1) / kChunkHits);
         if (wide) {
-            d.bkt_cnt = reinterpret_cast<uint32_t *>(base + off);
-            off += align256((size_t)d.n_bkt * 4);
+            // segments of about 8 hits per PMT (a run of 128 bytes), at least
+            // 4096 hits, at most kSegBuckets buckets and 2^31 ns
+            const double rate = (double)x.n_hits / ((double)d.n_bkt * d.bkt_w);
+            const double hits = std::max(8.0 * P, 4096.0);
+            const double want = rate > 0.0 ? hits / (rate * d.bkt_w) : (double)kSegBuckets;
+            d.seg_bkt = (uint32_t)std::max(1.0, std::min({want, (double)kSegBuckets, (double)d.n_bkt,
+                                                          std::floor(2147483647.0 / d.bkt_w)}));
+            d.edge_w = d.seg_bkt * d.bkt_w;
+            d.edge_org = d.bkt_origin;
+            d.n_edges = (d.n_bkt + d.seg_bkt - 1) / d.seg_bkt + 1;
+            d.span32 = d.bkt32 && (uint64_t)d.edge_w * d.n_edges < ((uint64_t)1 << 31);
+            d.edge = reinterpret_cast<uint32_t *>(base + off);
+            off += align256((size_t)d.n_edges * P * 4);
             d.bkt_off = reinterpret_cast<uint32_t *>(base + off);
             off += align256(((size_t)d.n_bkt + 1) * 4);
-            d.bkt_part = reinterpret_cast<uint32_t *>(base + off);
-            off += align256(((size_t)d.n_bkt + kBktChunk - 1) / kBktChunk * 4);
             d.tbuf = reinterpret_cast<trig_hit *>(base + off);
             off += align256((size_t)x.n_hits * sizeof(trig_hit));
         } else {
+            d.edge_w = (uint32_t)W;
+            d.edge_org = x.t0_ns - (int64_t)d.halo;
+            d.span32 = (det->par.slice_ns + 2 * det->in_halo + 2 * (int64_t)det->tile_halo + 2 * W) < ((int64_t)1 << 31);
             const uint32_t D = 2u * d.halo + (uint32_t)W;
             d.edge_a = D / (uint32_t)W;
             d.edge_b = D % (uint32_t)W;
@@ -602,6 +612,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             d.edge = reinterpret_cast<uint32_t *>(base + off);
             off += align256((size_t)d.n_edges * P * 4);
         }
+        d.w_magic = (uint32_t)((((uint64_t)1 << 32) + d.edge_w - 1) / d.edge_w);
         d.tile_nfired = reinterpret_cast<uint32_t *>(base + off);
         off += align256((size_t)d.n_tiles * 4);
         d.tile_rank = reinterpret_cast<uint32_t *>(base + off);

@@ -15,7 +15,7 @@ constexpr uint32_t kMaxPmt = 4096;          // PMTs per detector
 constexpr uint32_t kSmemDtMaxPmt = 96;      // dt table lives in shared memory up to this P
 constexpr uint32_t kDtRow = 256;            // bytes of a dt row in shared memory (128 PMTs)
 constexpr uint32_t kWideMinPmt = 129;       // from this P on, slices are staged from a bucketed copy
-constexpr uint32_t kBktChunk = 1024;        // buckets per block of the bucket scan
+constexpr uint32_t kSegBuckets = 4096;      // buckets of a segment at most (k_scatter)
 // A tile plus its halos spans less than 2^20 ns, so a hit's time within the
 // staged range and its PMT (< 2^12) pack into 32 bits.  The limit keeps
 // 65536 ns (more than any dt, <= 60000 ns) between the last staged time and
@@ -68,14 +68,17 @@ struct SliceDesc {
     int64_t in_lo, in_hi;   // accepted hit times [in_lo, in_hi)
     uint64_t n_hits;
     int64_t tile_w;         // tile width W (ns); tile g owns [t0 + g W, t0 + (g+1) W)
-    uint32_t w_magic;       // ceil(2^32 / W): 32-bit quotient estimate when span32
-    uint32_t span32;        // all in-range times are < 2^31 ns past t0 - H
+    uint32_t w_magic;       // ceil(2^32 / edge_w): 32-bit quotient estimate when span32
+    uint32_t span32;        // all in-range times are < 2^31 ns past the first edge
     uint32_t n_tiles;       // NG (<= 2^20)
     uint32_t item0;         // first work item (tile) of this slice
     uint32_t chunk0;        // first structure-pass chunk of this slice
     uint32_t *edge;         // [n_edges][P] first hit index at or past each tile edge (narrow slices):
                             //   edge 2g is B_g - H, edge 2 (g + edge_a) + 1 is B_{g+1} + H
     uint32_t n_edges, edge_a, edge_b;       // 2H + W = edge_a W + edge_b
+    int64_t edge_org;       // time of the first edge
+    uint32_t edge_w;        // W; wide slices: the length of a segment of seg_bkt buckets, whose
+    uint32_t seg_bkt;       //   starts are their edges
     // Wide slices (P >= kWideMinPmt): the hits are also copied, grouped by
     // time bucket [O + b Wb, O + (b+1) Wb), into tbuf; tile g's core is the
     // buckets [lead + g m, lead + (g+1) m) and it stages those plus `hh`
@@ -89,9 +92,7 @@ struct SliceDesc {
     uint32_t n_bkt;         // NB
     uint32_t bkt32;         // every in-range time is < 2^31 ns past O
     int64_t bkt_origin;     // O = t0 - lead * Wb
-    uint32_t *bkt_cnt;      // [NB] hits per bucket, then fill cursors
-    uint32_t *bkt_off;      // [NB + 1] exclusive prefix of the counts
-    uint32_t *bkt_part;     // [ceil(NB / kBktChunk)] sums of the counts per chunk
+    uint32_t *bkt_off;      // [NB + 1] merged rank of each bucket's first hit
     trig_hit *tbuf;         // [n_hits] hits in bucket order
     trig_trigger *stage;    // [n_hits] fired seeds at their merged rank
     uint32_t *wrank;        // [n_hits][2] beside each staged fired seed: the merged ranks of the
@@ -173,12 +174,12 @@ inline bool valid_tile_shape(uint32_t cap, uint32_t warps)
 }
 constexpr uint32_t kMaxTilesPerSlice = 1u << 20;
 
-constexpr int kPipelineKernels = 11;
+constexpr int kPipelineKernels = 9;
 extern const char *const kKernelNames[kPipelineKernels];
 
 // Enqueues the batch pipeline, the copy of its header and descriptors to
-// d_hdr and d_desc included.  hdr.any_wide: the bucket sums, scan and scatter
-// kernels run only then; any_events: the halo, event-offset, event-copy and
+// d_hdr and d_desc included.  hdr.any_wide: the scatter kernel runs only
+// then; any_events: the halo, event-offset, event-copy and
 // status kernels run only then; any_ext: the tile kernel built with level 0,
 // seed rule 1 and the distinct count runs, else the one without them; dense:
 // the tile kernel built with a warp per seed in the causal count runs.  ev

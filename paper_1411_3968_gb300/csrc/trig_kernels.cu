@@ -361,10 +361,13 @@ static_assert(kBoundsPerWarp == 31 * kBoundsUnroll, "a warp steps through 31 hit
 // 2 q + 1 + (r >= b): edge 2g is tile g's lo edge, edge 2 (g + a) + 1 its hi
 // edge (the odd ones below 2a + 1 are no tile's).  One number per hit then
 // tells both, and passing either kind of edge is the same store.
+// A wide slice (WIDE) has the starts of its segments of buckets instead, one
+// edge every edge_w ns.
+template <bool WIDE>
 struct EdgeCount {
     uint32_t W, magic, b, NE;
     __device__ __forceinline__ explicit EdgeCount(const SliceDesc &d)
-        : W((uint32_t)d.tile_w), magic(d.w_magic), b(d.edge_b), NE(d.n_edges)
+        : W(d.edge_w), magic(d.w_magic), b(d.edge_b), NE(d.n_edges)
     {
     }
     // x below 2^31: the high half of x * ceil(2^32 / W) is the quotient or
@@ -375,14 +378,14 @@ struct EdgeCount {
         uint32_t q = __umulhi((uint32_t)x, magic);
         uint32_t r = (uint32_t)x - q * W;
         if ((int32_t)r < 0) --q, r += W;
-        return min(2u * q + (r >= b ? 2u : 1u), NE);
+        return min(WIDE ? q + 1u : 2u * q + (r >= b ? 2u : 1u), NE);
     }
     __device__ __forceinline__ uint32_t of64(int64_t x) const
     {
         if (x < 0) return 0u;
         const int64_t q = x / (int64_t)W;
-        if (q >= (int64_t)(NE / 2u)) return NE;
-        return min(2u * (uint32_t)q + (x - q * (int64_t)W >= (int64_t)b ? 2u : 1u), NE);
+        if (q >= (int64_t)(WIDE ? NE : NE / 2u)) return NE;
+        return min(WIDE ? (uint32_t)q + 1u : 2u * (uint32_t)q + (x - q * (int64_t)W >= (int64_t)b ? 2u : 1u), NE);
     }
 };
 
@@ -400,19 +403,22 @@ __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
     trig_hit l = h;
     if (li > 0) l = load_hit(d.hits + li - 1);
     const uint32_t p = h.pmt, pl = l.pmt;
-    const bool is_first = li == 0 || pl != p, narrow = !d.wide;
-    uint32_t e = 0, el = 0;
-    if (narrow) {
-        const EdgeCount ec(d);
-        const int64_t x0 = d.t0 - (int64_t)d.halo;
-        e = ec.of64(h.t_ns - x0);
-        el = ec.of64(l.t_ns - x0);
+    const bool is_first = li == 0 || pl != p;
+    uint32_t e, el;
+    if (d.wide) {
+        const EdgeCount<true> ec(d);
+        e = ec.of64(h.t_ns - d.edge_org);
+        el = ec.of64(l.t_ns - d.edge_org);
+    } else {
+        const EdgeCount<false> ec(d);
+        e = ec.of64(h.t_ns - d.edge_org);
+        el = ec.of64(l.t_ns - d.edge_org);
     }
     uint32_t bad = 0;
     if (is_first && li > 0 && pl < P) {
         // hit li - 1 was the last of PMT pl's run
         if (poff[pl + 1] != li) bad |= TRIG_FLAG_BAD_PMT;
-        if (narrow) fill_run_end(d.edge, poff, P, NE, pl, el, (uint32_t)li);
+        fill_run_end(d.edge, poff, P, NE, pl, el, (uint32_t)li);
     }
     if (p >= P) bad |= TRIG_FLAG_BAD_PMT;
     else {
@@ -423,10 +429,6 @@ __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
     if (!is_first && l.t_ns > h.t_ns) bad |= TRIG_FLAG_UNSORTED;
     if (bad) {
         report(d, bad);
-        return;
-    }
-    if (!narrow) {
-        atomicAdd(&d.bkt_cnt[bkt_index(d, h.t_ns)], 1u);
         return;
     }
     fill_edges(d.edge, P, p, is_first ? 0u : el, e, (uint32_t)li);
@@ -453,8 +455,8 @@ __device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, ui
     const trig_hit *__restrict__ hits = d.hits;
     const int64_t in_lo = d.in_lo;
     const T in_span = (T)(d.in_hi - in_lo);
-    const T x0 = (T)(d.t0 - (int64_t)d.halo - in_lo);           // the first edge, from in_lo
-    const EdgeCount ec(d);
+    const T x0 = (T)(d.edge_org - in_lo);                       // the first edge, from in_lo
+    const EdgeCount<WIDE> ec(d);
     for (; c < c_end; ++c) {
         const uint32_t wbase = (c - d.chunk0) * kChunkHits + warp * kBoundsPerWarp;
         if (wbase >= n_hits) continue;
@@ -468,20 +470,18 @@ __device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, ui
 #pragma unroll
         for (int u = 0; u < kBoundsUnroll; ++u) {
             const uint32_t li = wbase + u * 31 + lane - 1u;
-            const int64_t t = (int64_t)(((uint64_t)v[u].y << 32) | v[u].x);
-            const uint64_t rel = (uint64_t)t - (uint64_t)in_lo;
+            const uint64_t rel = (((uint64_t)v[u].y << 32) | v[u].x) - (uint64_t)in_lo;
             const T r = (T)rel;
             const bool valid = li < n_hits, in = S32 ? (rel >> 32) == 0 && r < in_span : rel < (uint64_t)in_span;
             // PMT label; bits 16, 17: out of range, no such hit
             const uint32_t p = v[u].z & 0xffffu, pc = valid ? (in ? p : p | 0x10000u) : 0x2ffffu;
             uint32_t e = 0;
-            if (!WIDE && in) e = S32 ? ec.of32((int32_t)(r - x0)) : ec.of64((int64_t)(r - x0));
+            if (in) e = S32 ? ec.of32((int32_t)(r - x0)) : ec.of64((int64_t)(r - x0));
             const uint32_t pcl = __shfl_up_sync(0xffffffffu, pc, 1);
             const T rl = __shfl_up_sync(0xffffffffu, r, 1);
-            const uint32_t el = WIDE ? 0u : __shfl_up_sync(0xffffffffu, e, 1);
+            const uint32_t el = __shfl_up_sync(0xffffffffu, e, 1);
             if (lane == 0 || !valid) continue;
             if (pc != pcl || rl > r || !in || li + 1 == n_hits) special |= 1u << u;
-            else if (WIDE) atomicAdd(&d.bkt_cnt[bkt_index(d, t)], 1u);
             else if (e != el && p < P) fill_edges(d.edge, P, p, el, e, li);
         }
         for (; special; special &= special - 1u)
@@ -492,13 +492,14 @@ __device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, ui
 // Slices longer than about two seconds, in 64-bit times.
 __device__ __noinline__ void bounds_chunks_long(const SliceDesc &d, uint32_t c, uint32_t c_end)
 {
-    bounds_chunks<false, false>(d, c, c_end);
+    if (d.wide) bounds_chunks<true, false>(d, c, c_end);
+    else bounds_chunks<false, false>(d, c, c_end);
 }
 
 // Structure pass: one read of every hit.  The CSR layout and the time order
 // are checked (run starts and ends against pmt_off, each hit against its
-// predecessor); narrow slices record where each PMT's stream crosses the
-// tile edges, wide ones count their time buckets.  Each block takes a
+// predecessor), and where each PMT's stream crosses the tile edges (wide
+// slices: the edges of their segments of buckets) is recorded.  Each block takes a
 // contiguous share of the chunks, so it looks its slice up once.
 __global__ void __launch_bounds__(kBoundsThreads, 3) k_bounds(const BatchHeader *__restrict__ hdr,
                                                            const SliceDesc *__restrict__ desc)
@@ -515,118 +516,114 @@ __global__ void __launch_bounds__(kBoundsThreads, 3) k_bounds(const BatchHeader 
     for (uint32_t s = find_slice_by_chunk(desc, n_slices, c); c < c1; ++s) {
         const SliceDesc &d = desc[s];
         const uint32_t end = min(c1, s + 1 < n_slices ? desc[s + 1].chunk0 : n_chunks);
-        if (d.wide) bounds_chunks<true, false>(d, c, end);
-        else if (d.span32) bounds_chunks<false, true>(d, c, end);
-        else bounds_chunks_long(d, c, end);
+        if (!d.span32) bounds_chunks_long(d, c, end);
+        else if (d.wide) bounds_chunks<true, true>(d, c, end);
+        else bounds_chunks<false, true>(d, c, end);
         c = end;
-    }
-}
-
-// ----------------------------------------------------------- k_bsum, k_bscan
-
-// Wide slices: bucket offsets = exclusive prefix of the bucket counts, in
-// two grid-wide passes over chunks of kBktChunk buckets (a block per chunk):
-// the chunk sums, then each chunk's scan from the sums of the chunks before
-// it.  The counts are reset to serve as fill cursors of the scatter.
-__global__ void __launch_bounds__(kBktChunk) k_bsum(const BatchHeader *__restrict__ hdr,
-                                                    const SliceDesc *__restrict__ desc)
-{
-    __shared__ uint32_t wsum[32];
-    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    wait_for_previous_kernel();
-    let_next_kernel_in();
-    for (uint32_t s = 0; s < hdr->n_slices; ++s) {
-        const SliceDesc &d = desc[s];
-        if (!d.wide) continue;
-        const uint32_t nb = d.n_bkt, nch = (nb + kBktChunk - 1) / kBktChunk;
-        for (uint32_t c = blockIdx.x; c < nch; c += gridDim.x) {
-            const uint32_t i = c * kBktChunk + tid;
-            uint32_t v = i < nb ? d.bkt_cnt[i] : 0u;
-            v = __reduce_add_sync(0xffffffffu, v);
-            if (lane == 0) wsum[warp] = v;
-            __syncthreads();
-            if (warp == 0) {
-                uint32_t t = lane < kBktChunk / 32 ? wsum[lane] : 0u;
-                t = __reduce_add_sync(0xffffffffu, t);
-                if (lane == 0) d.bkt_part[c] = t;
-            }
-            __syncthreads();
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kBktChunk) k_bscan(const BatchHeader *__restrict__ hdr,
-                                                     const SliceDesc *__restrict__ desc)
-{
-    __shared__ uint32_t wsum[33];
-    __shared__ uint32_t base;
-    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    constexpr uint32_t NW = kBktChunk / 32;
-    wait_for_previous_kernel();
-    let_next_kernel_in();
-    for (uint32_t s = 0; s < hdr->n_slices; ++s) {
-        const SliceDesc &d = desc[s];
-        if (!d.wide) continue;
-        const uint32_t nb = d.n_bkt, nch = (nb + kBktChunk - 1) / kBktChunk;
-        for (uint32_t c = blockIdx.x; c < nch; c += gridDim.x) {
-            // sum of the chunks before c
-            uint32_t pre = 0;
-            for (uint32_t q = tid; q < c; q += kBktChunk) pre += d.bkt_part[q];
-            pre = __reduce_add_sync(0xffffffffu, pre);
-            if (lane == 0) wsum[warp] = pre;
-            __syncthreads();
-            if (warp == 0) {
-                uint32_t t = lane < NW ? wsum[lane] : 0u;
-                t = __reduce_add_sync(0xffffffffu, t);
-                if (lane == 0) base = t;
-            }
-            __syncthreads();
-            // the chunk's own exclusive scan
-            const uint32_t i = c * kBktChunk + tid;
-            const uint32_t v = i < nb ? d.bkt_cnt[i] : 0u;
-            const uint32_t incl = warp_incl_scan(v);
-            if (lane == 31) wsum[warp] = incl;
-            __syncthreads();
-            if (warp == 0) {
-                const uint32_t w = lane < NW ? wsum[lane] : 0u;
-                const uint32_t wi = warp_incl_scan(w);
-                if (lane < NW) wsum[lane] = wi - w;
-                if (lane == NW - 1) wsum[32] = wi;
-            }
-            __syncthreads();
-            if (i < nb) {
-                d.bkt_off[i] = base + wsum[warp] + incl - v;
-                d.bkt_cnt[i] = 0;
-            }
-            if (c == nch - 1 && tid == 0) d.bkt_off[nb] = base + wsum[32];
-            __syncthreads();
-        }
     }
 }
 
 // --------------------------------------------------------------- k_scatter
 
 // Wide slices: every hit copied to its time bucket's range of tbuf (the
-// order inside a bucket is arbitrary; the tile pass sorts).  Slices with
-// malformed input (flagged by the structure pass) are skipped.
-__global__ void __launch_bounds__(256) k_scatter(const BatchHeader *__restrict__ hdr, const SliceDesc *__restrict__ desc)
+// order inside a bucket is arbitrary; the tile pass sorts), and the buckets'
+// offsets.  A block takes one segment of seg_bkt buckets at a time: it reads
+// each PMT's run in the segment (eight hits on average, sixteen lanes a run),
+// counts them per bucket in shared memory, scans the counts from the
+// segment's merged rank (the sum of the runs' places), and reads the runs
+// again, from L2, to write them.  The writes of a block land in one window
+// of tbuf (8 P hits), so L2 fills whole lines; the global counters that a
+// hit-by-hit copy needs took 0.51 ms for the 2688-PMT slice (29.6 M hits)
+// and 0.24 of the structure pass, against 0.42 and 0.13.  Bound by the
+// latency of the short runs' loads.
+// Slices with malformed input (flagged by the structure pass) are skipped.
+constexpr uint32_t kScatThreads = 512;
+
+__global__ void __launch_bounds__(kScatThreads, 2) k_scatter(const BatchHeader *__restrict__ hdr,
+                                                          const SliceDesc *__restrict__ desc)
 {
+    constexpr uint32_t NW = kScatThreads / 32;
+    __shared__ uint32_t cnt[kSegBuckets], red[NW + 1];
     wait_for_previous_kernel();
     let_next_kernel_in();
-    const uint32_t n_slices = hdr->n_slices, n_chunks = hdr->n_chunks;
-    for (uint32_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-        const SliceDesc &d = desc[find_slice_by_chunk(desc, n_slices, c)];
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    for (uint32_t s = 0; s < hdr->n_slices; ++s) {
+        const SliceDesc &d = desc[s];
         if (!d.wide) continue;
         if (d.stats->flags & (TRIG_FLAG_BAD_PMT | TRIG_FLAG_UNSORTED | TRIG_FLAG_OUT_OF_RANGE)) continue;
-        const uint64_t first = (uint64_t)(c - d.chunk0) * kChunkHits;
-        for (uint32_t k = threadIdx.x; k < kChunkHits; k += blockDim.x) {
-            const uint64_t li = first + k;
-            if (li >= d.n_hits) break;
-            const int4 v = *reinterpret_cast<const int4 *>(d.hits + li);
-            const int64_t t = (int64_t)(((uint64_t)(uint32_t)v.y << 32) | (uint32_t)v.x);
-            const uint32_t b = bkt_index(d, t);
-            const uint32_t pos = d.bkt_off[b] + atomicAdd(&d.bkt_cnt[b], 1u);
-            if (CHECK(17, pos, d.n_hits)) *reinterpret_cast<int4 *>(d.tbuf + pos) = v;
+        const uint32_t P = d.n_pmt, K = d.seg_bkt, n_seg = d.n_edges - 1u;
+        for (uint32_t g = blockIdx.x; g < n_seg; g += gridDim.x) {
+            const uint32_t *ea = d.edge + (size_t)g * P, *eb = ea + P;
+            const uint32_t b0 = g * K, nb = min(K, d.n_bkt - b0);
+            const int64_t org = d.bkt_origin + (int64_t)b0 * d.bkt_w;
+            for (uint32_t b = tid; b < nb; b += kScatThreads) cnt[b] = 0;
+            __syncthreads();
+            // bucket in the segment; a segment is shorter than 2^31 ns
+            auto bucket = [&](const int4 &v) {
+                const uint32_t rel = (uint32_t)((((uint64_t)(uint32_t)v.y << 32) | (uint32_t)v.x) - (uint64_t)org);
+                uint32_t q = __umulhi(rel, d.bkt_magic);
+                if (q * d.bkt_w > rel) --q;
+                return min(q, nb - 1u);
+            };
+            // each half warp takes four runs at a time, their loads in flight
+            // together
+            auto each = [&](auto &&f) {
+                for (uint32_t p0 = 2u * warp + (lane >> 4); p0 < P; p0 += 8u * NW) {
+                    uint32_t i[4], e[4];
+                    int4 v[4];
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) {
+                        const uint32_t p = p0 + u * 2u * NW;
+                        i[u] = p < P ? ea[p] + (lane & 15u) : 0u;
+                        e[u] = p < P ? eb[p] : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u)
+                        if (i[u] < e[u]) v[u] = *reinterpret_cast<const int4 *>(d.hits + i[u]);
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) {
+                        if (i[u] < e[u]) f(v[u]);
+                        for (uint32_t k = i[u] + 16u; k < e[u]; k += 16u) f(*reinterpret_cast<const int4 *>(d.hits + k));
+                    }
+                }
+            };
+            each([&](const int4 &v) { atomicAdd(&cnt[bucket(v)], 1u); });
+            // merged rank of the segment's first hit
+            uint32_t base = 0;
+            for (uint32_t p = tid; p < P; p += kScatThreads) base += ea[p] - (uint32_t)d.pmt_off[p];
+            base = __reduce_add_sync(0xffffffffu, base);
+            if (lane == 0) red[warp] = base;
+            __syncthreads();
+            base = __reduce_add_sync(0xffffffffu, lane < NW ? red[lane] : 0u);
+            __syncthreads();
+            // exclusive scan of the counts, kSegBuckets / threads each
+            constexpr uint32_t V = kSegBuckets / kScatThreads;
+            uint32_t v[V], own = 0;
+#pragma unroll
+            for (uint32_t i = 0; i < V; ++i) {
+                v[i] = tid * V + i < nb ? cnt[tid * V + i] : 0u;
+                own += v[i];
+            }
+            const uint32_t incl = warp_incl_scan(own);
+            if (lane == 31) red[warp] = incl;
+            __syncthreads();
+            uint32_t run = base + __reduce_add_sync(0xffffffffu, lane < warp ? red[lane % NW] : 0u) + incl - own;
+#pragma unroll
+            for (uint32_t i = 0; i < V; ++i) {
+                const uint32_t b = tid * V + i;
+                if (b < nb) {
+                    cnt[b] = run;
+                    d.bkt_off[b0 + b] = run;
+                }
+                run += v[i];
+            }
+            if (g + 1 == n_seg && tid == kScatThreads - 1) d.bkt_off[d.n_bkt] = run;
+            __syncthreads();
+            each([&](const int4 &v) {
+                const uint32_t pos = atomicAdd(&cnt[bucket(v)], 1u);
+                if (CHECK(17, pos, d.n_hits)) *reinterpret_cast<int4 *>(d.tbuf + pos) = v;
+            });
+            __syncthreads();
         }
     }
 }
@@ -2779,8 +2776,7 @@ cudaError_t static_scratch(void **ptr, size_t *bytes)
 // the kernel's parameter, copied when it is launched or captured: nothing is
 // read from host memory later, no copy waits on the caller's stream, and a
 // captured graph names no host or device allocation but through the kernels'
-// own pointers.  The same launch zeroes what a run starts from: the slices'
-// counters and the wide slices' bucket counts.
+// own pointers.  The same launch zeroes the slices' counters.
 template <uint32_t K>
 struct PutPlan {
     BatchHeader hdr;
@@ -2805,12 +2801,6 @@ __global__ void __launch_bounds__(256) k_put(const __grid_constant__ PutPlan<K> 
         z.n_hits = plan.desc[at].n_hits;
         *plan.desc[at].stats = z;
     }
-    for (uint32_t s = 0; plan.hdr.any_wide && s < plan.n; ++s) {
-        if (!plan.desc[s].wide) continue;
-        uint32_t *cnt = plan.desc[s].bkt_cnt;
-        const uint32_t nb = plan.desc[s].n_bkt;
-        for (uint32_t i = blockIdx.x * 256 + tid; i < nb; i += gridDim.x * 256) cnt[i] = 0;
-    }
 }
 
 template <uint32_t K>
@@ -2825,7 +2815,7 @@ static cudaError_t put_part(const BatchHeader &hdr, const SliceDesc *desc, uint3
     std::memcpy(plan.desc, desc + first, n * sizeof(SliceDesc));
     // a block per two descriptors (reads of the parameter by 32 different
     // addresses take turns: 17 us for 64 of them in one block)
-    k_put<K><<<hdr.any_wide ? device_sm_count() * 2 : (n + 1) / 2, 256, 0, st>>>(plan, d_hdr, d_desc);
+    k_put<K><<<(n + 1) / 2, 256, 0, st>>>(plan, d_hdr, d_desc);
     return cudaGetLastError();
 }
 
@@ -2894,8 +2884,8 @@ static cudaError_t launch_tile(BatchHeader *hdr, SliceDesc *desc, uint32_t max_p
     return launch_next(kern, device_sm_count() * per_sm, NC + 32, smem, st, hdr, desc, max_pmt);
 }
 
-const char *const kKernelNames[kPipelineKernels] = {"k_put",    "k_bounds", "k_bsum",  "k_bscan",  "k_scatter", "k_tile",
-                                                     "k_evhalo", "k_final",  "k_escan", "k_events", "k_status"};
+const char *const kKernelNames[kPipelineKernels] = {"k_put",   "k_bounds", "k_scatter", "k_tile",  "k_evhalo",
+                                                     "k_final", "k_escan",  "k_events",  "k_status"};
 
 cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHeader *d_hdr, SliceDesc *d_desc,
                          uint32_t max_pmt, bool any_smem_dt, const TileConfig &cfg, cudaStream_t st, uint64_t *launches,
@@ -2922,17 +2912,10 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
     }
     mark(2);
     if (any_wide) {
-        if ((e = launch_next(k_bsum, sms * 2, kBktChunk, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
-        mark(3);
-        if ((e = launch_next(k_bscan, sms * 2, kBktChunk, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
-        mark(4);
-        if ((e = launch_next(k_scatter, sms * 8, 256, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
-        nl += 3;
-    } else {
-        mark(3);
-        mark(4);
+        if ((e = launch_next(k_scatter, sms * 4, kScatThreads, 0, st, d_hdr, d_desc)) != cudaSuccess) return e;
+        nl += 1;
     }
-    mark(5);
+    mark(3);
     const bool smem_dt = any_smem_dt && max_pmt <= kSmemDtMaxPmt;
     if (any_ext || any_events || rows) {
         // level 0, seed rule 1, distinct count, and every batch that needs
@@ -2979,7 +2962,7 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
         e = smem_dt ? launch_tile<4096, 512, true>(d_hdr, d_desc, max_pmt, st)
                     : launch_tile<4096, 512, false>(d_hdr, d_desc, max_pmt, st);
     if (e != cudaSuccess) return e;
-    mark(6);
+    mark(4);
     if (any_events) {
         static bool ev_limit_set[64] = {};
         int dev = 0;
@@ -2992,24 +2975,24 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
         k_evhalo<<<sb, kEvHaloThreads, ev_smem, st>>>(d_hdr, d_desc);
         nl += 1;
     }
-    mark(7);
+    mark(5);
     // at most as many blocks as there are chunks of tiles
     if ((e = launch_next(k_final, std::min<uint32_t>(hdr.n_fin, (uint32_t)sms * 8), kFinThreads, 0, st, d_hdr, d_desc)) !=
         cudaSuccess)
         return e;
-    mark(8);
+    mark(6);
     if (any_events) {
         k_escan<<<sb, 1024, 0, st>>>(d_hdr, d_desc);
-        mark(9);
+        mark(7);
         k_events<<<sms * 8, 256, 0, st>>>(d_hdr, d_desc);
-        mark(10);
+        mark(8);
         k_status<<<1, 256, 0, st>>>(d_hdr, d_desc);
         nl += 3;
     } else {
-        mark(9);
-        mark(10);
+        mark(7);
+        mark(8);
     }
-    mark(11);
+    mark(9);
     nl += 2;
     if (launches) *launches += nl;
     return cudaGetLastError();
