@@ -643,7 +643,7 @@ struct ItemInfo {
     uint32_t span;      // length of the staged range
 };
 // A whole staged tile; one with more hits than fit, left to tile_overflow
-// (wide slices); nothing to do (bad slice or empty); a staged piece of a
+// (wide slices whose single buckets do not fit); nothing to do (bad slice or empty); a staged piece of a
 // tile, and the end of a tile's pieces.
 enum : uint32_t { kItemTile, kItemOverflow, kItemSkip, kItemPiece, kItemEnd };
 
@@ -1484,8 +1484,8 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
     return co;
 }
 
-// Overflow path of the wide slices (a narrow one's tile is split by the
-// stager): the tile holds more than CAP hits with its halo.  Split
+// Last resort of the wide slices (other tiles are split by the stager): a
+// single bucket with its halo holds more than CAP hits.  Split
 // its core in halves until each piece fits; pieces are staged with plain
 // loads after per-PMT binary searches.  A 1 ns core that still does not
 // fit is reported (TRIG_FLAG_TILE_FULL) and skipped.
@@ -1727,6 +1727,59 @@ __device__ __forceinline__ bool stage_pieces(Stager &sg, ItemInfo x, uint32_t ca
     return true;
 }
 
+// The staged buckets [b_lo, b_hi) of a wide slice's core buckets [c, c + k).
+struct BucketRange {
+    uint32_t b_lo, b_hi, lead;
+    __device__ __forceinline__ BucketRange(const SliceDesc *d, uint32_t c, uint32_t k)
+        : b_lo(c > d->bkt_halo ? c - d->bkt_halo : 0u), b_hi(min(c + k + d->bkt_halo, d->n_bkt)), lead(c - b_lo)
+    {
+    }
+    __device__ __forceinline__ uint32_t hits(const SliceDesc *d) const
+    {
+        return __ldg(d->bkt_off + b_hi) - __ldg(d->bkt_off + b_lo);
+    }
+};
+
+// A wide slice's tile with more hits than fit (a muon in a full tile): the
+// largest piece of core buckets, halved from the tile's, that fits
+// everywhere in the tile; 0 if not even one bucket does.
+__device__ __forceinline__ uint32_t piece_buckets(const SliceDesc *d, uint32_t c_lo, uint32_t cap)
+{
+    const uint32_t m = d->bkt_per_tile;
+    for (uint32_t k = m; k > 1;) {
+        k = (k + 1) / 2;
+        uint32_t most = 0;
+        for (uint32_t j = 0; j < m; j += k) most = max(most, BucketRange(d, c_lo + j, min(k, m - j)).hits(d));
+        if (most <= cap) return k;
+    }
+    return 0;
+}
+
+__device__ __forceinline__ bool stage_buckets(Stager &sg, ItemInfo x, const SliceDesc *d, uint32_t c_lo, uint32_t k,
+                                              BatchHeader *hdr)
+{
+    const uint32_t m = d->bkt_per_tile, core = x.core;
+    const uint64_t wait_ns = hdr->wait_ns;
+    for (uint32_t j = 0; j < m; j += k) {
+        const uint32_t kk = min(k, m - j), off = j * d->bkt_w;
+        if (off >= core) break;                                     // past the slice's end
+        const BucketRange r(d, c_lo + j, kk);
+        const uint32_t n = r.hits(d);
+        if (n == 0) continue;
+        if (!sg.wait_free(hdr, wait_ns)) return false;
+        x.rank_lo = __ldg(d->bkt_off + r.b_lo);
+        x.off = off, x.core = min(kk * d->bkt_w, core - off);
+        x.lo_t = r.lead * d->bkt_w, x.span = (r.b_hi - r.b_lo) * d->bkt_w;
+        sg.hand_over(x, n);
+        if (lane_id() == 0 && CHECK(7, (uint64_t)x.rank_lo + n, d->n_hits + 1))
+            bulk_g2s(sg.stage, d->tbuf + x.rank_lo, n * 16u, sg.full);
+    }
+    if (!sg.wait_free(hdr, wait_ns)) return false;
+    x.mode = kItemEnd;
+    sg.hand_over(x, 0);
+    return true;
+}
+
 template <int CAP, int NC, bool SMEM_DT, bool EXT, bool DENSE>
 __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 1)) k_tile(BatchHeader *__restrict__ hdr,
                                                                           const SliceDesc *__restrict__ desc,
@@ -1781,7 +1834,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
 #endif
             uint32_t g = 0, P = 0, mode = kItemSkip, lo_t = 0, span = 0;
             uint32_t ra[R], rl[R];                  // hit indices are below 2^32 - 16
-            uint32_t tot = 0, rlo = 0;
+            uint32_t tot = 0, rlo = 0, c_lo = 0, piece = 0;
             bool wide = false;
             if (item < n_items) {
                 // items arrive in increasing order: walk the slice index forward
@@ -1797,15 +1850,14 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 if (wide) {
                     // one contiguous range of the bucketed copy: the core
                     // buckets and hh buckets of halo on each side
-                    const uint32_t hh = d->bkt_halo, m = d->bkt_per_tile;
-                    const uint32_t c_lo = d->bkt_lead + g * m;
-                    const uint32_t b_lo = c_lo > hh ? c_lo - hh : 0u;
-                    const uint32_t b_hi = min(c_lo + m + hh, d->n_bkt);
-                    lo_t = (c_lo - b_lo) * d->bkt_w;
-                    span = (b_hi - b_lo) * d->bkt_w;
+                    c_lo = d->bkt_lead + g * d->bkt_per_tile;
+                    const BucketRange r(d, c_lo, d->bkt_per_tile);
+                    lo_t = r.lead * d->bkt_w;
+                    span = (r.b_hi - r.b_lo) * d->bkt_w;
                     if (!bad) {
-                        rlo = __ldg(d->bkt_off + b_lo);
-                        tot = __ldg(d->bkt_off + b_hi) - rlo;
+                        rlo = __ldg(d->bkt_off + r.b_lo);
+                        tot = r.hits(d);
+                        if (tot > (uint32_t)CAP) piece = piece_buckets(d, c_lo, CAP);
                     }
                 } else {
                     // the PMTs' runs [lb(B_g - H), lb(B_{g+1} + H)), P <= 32 R
@@ -1836,7 +1888,10 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                     tot = __reduce_add_sync(0xffffffffu, tot);
                     rlo = __reduce_add_sync(0xffffffffu, rlo);
                 }
-                mode = bad || tot == 0 ? kItemSkip : tot <= (uint32_t)CAP ? kItemTile : wide ? kItemOverflow : kItemPiece;
+                mode = bad || tot == 0                ? kItemSkip
+                       : tot <= (uint32_t)CAP    ? kItemTile
+                       : wide && piece == 0      ? kItemOverflow
+                                                 : kItemPiece;
             }
             uint32_t next = 0;
             if (item < n_items) {
@@ -1853,7 +1908,9 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             const int64_t W = d->tile_w, Bg = d->t0 + (int64_t)g * W;
             const uint32_t core = (uint32_t)(min(Bg + W, d->t0 + d->slice_ns) - Bg);
             const ItemInfo x{(int32_t)item, s, g, 0, rlo, mode, 0, core, lo_t, span};
-            if (mode == kItemPiece) {
+            if (mode == kItemPiece && wide) {
+                if (!stage_buckets(sg, x, d, c_lo, piece, hdr)) break;
+            } else if (mode == kItemPiece) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) runs[r * 32 + lane] = make_uint2(ra[r], ra[r] + rl[r]);
                 __syncwarp();
