@@ -181,6 +181,8 @@ template <bool ONES>
 __global__ void __launch_bounds__(1024) k_scan_part(const uint32_t *in, const uint32_t *n_ptr, uint32_t *part)
 {
     __shared__ uint32_t red[33];
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t n = *n_ptr, base = blockIdx.x * kScanBlock;
     if (base >= n && blockIdx.x > 0) return;
     uint32_t sum = 0;
@@ -194,6 +196,8 @@ __global__ void __launch_bounds__(1024) k_scan_part(const uint32_t *in, const ui
 __global__ void __launch_bounds__(1024) k_scan_top(const uint32_t *n_ptr, uint32_t *part, uint32_t *total)
 {
     __shared__ uint32_t red[33];
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t nb = (*n_ptr + kScanBlock - 1) / kScanBlock;
     uint32_t carry = 0;
     for (uint32_t b0 = 0; b0 < nb; b0 += 1024) {
@@ -212,6 +216,8 @@ __global__ void __launch_bounds__(1024) k_scan_final(const uint32_t *in, const u
                                                     const uint32_t *total, uint32_t *out)
 {
     __shared__ uint32_t red[33];
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t n = *n_ptr, base = blockIdx.x * kScanBlock;
     if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = *total;
     if (base >= n) return;
@@ -236,25 +242,37 @@ void launch_scan(const uint32_t *in, const uint32_t *n_ptr, uint64_t n_max, uint
                  uint32_t *out, cudaStream_t st, uint64_t &launches)
 {
     const uint32_t nb = (uint32_t)std::max<uint64_t>(1, (n_max + kScanBlock - 1) / kScanBlock);
-    k_scan_part<ONES><<<nb, 1024, 0, st>>>(in, n_ptr, part);
-    k_scan_top<<<1, 1024, 0, st>>>(n_ptr, part, total);
-    k_scan_final<ONES><<<nb, 1024, 0, st>>>(in, n_ptr, part, total, out);
+    launch_next(k_scan_part<ONES>, nb, 1024, 0, st, in, n_ptr, part);
+    launch_next(k_scan_top, 1, 1024, 0, st, n_ptr, part, total);
+    launch_next(k_scan_final<ONES>, nb, 1024, 0, st, in, n_ptr, part, total, out);
     launches += 3;
 }
 
 // ------------------------------------------------------------ selection
 
-// one thread per tower (blockDim.x = kMaxTowers)
-__global__ void k_acount(AHeader *h, const ATower *tw)
+// The selection's descriptors travel as this kernel's parameter; then one
+// thread per tower (blockDim.x = kMaxTowers) counts its triggers.
+struct APlan {
+    AHeader h;
+    ATower tw[kMaxTowers];
+};
+static_assert(sizeof(APlan) <= 32000 && sizeof(AHeader) % 4 == 0 && sizeof(ATower) % 4 == 0, "a kernel parameter of words");
+
+__global__ void k_acount(const __grid_constant__ APlan plan, AHeader *h, ATower *tw)
 {
     __shared__ uint32_t n_s[kMaxTowers];
     __shared__ uint32_t fl;
     const uint32_t b = threadIdx.x;
+    let_next_kernel_in();
+    for (uint32_t i = b; i < sizeof(AHeader) / 4; i += kMaxTowers)
+        reinterpret_cast<uint32_t *>(h)[i] = reinterpret_cast<const uint32_t *>(&plan.h)[i];
+    for (uint32_t i = b; i < plan.h.nt * (uint32_t)(sizeof(ATower) / 4); i += kMaxTowers)
+        reinterpret_cast<uint32_t *>(tw)[i] = reinterpret_cast<const uint32_t *>(plan.tw)[i];
     if (b == 0) fl = 0;
     __syncthreads();
-    if (b < h->nt) {
-        const trig_slice_stats *s = tw[b].stats;
-        const uint64_t n = s->n_triggers < tw[b].trig_cap ? s->n_triggers : tw[b].trig_cap;
+    if (b < plan.h.nt) {
+        const trig_slice_stats *s = plan.tw[b].stats;
+        const uint64_t n = s->n_triggers < plan.tw[b].trig_cap ? s->n_triggers : plan.tw[b].trig_cap;
         n_s[b] = (uint32_t)n;
         h->n[b] = (uint32_t)n;
         if (s->status != 0) atomicOr(&fl, TRIG_AFLAG_TOWER_INCOMPLETE);
@@ -277,41 +295,64 @@ __global__ void k_acount(AHeader *h, const ATower *tw)
     }
 }
 
+// Lanes that share a trigger in the searches over the towers' lists: a lane
+// per tower where they fit, so that the searches (14 dependent loads each)
+// run side by side (for 98 k triggers of eight towers k_amerge takes 12 us,
+// 23 with a thread per trigger, and k_aselect, which also scans the muons'
+// clusters, 30, 33 before).
+__device__ __forceinline__ uint32_t lanes_per_item(uint32_t nt) { return nt <= 8 ? 8u : nt <= 16 ? 16u : 32u; }
+
+__device__ __forceinline__ uint32_t group_sum(uint32_t v, uint32_t G)
+{
+    for (uint32_t o = G >> 1; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 __global__ void k_aselect(AHeader *h, const ATower *tw)
 {
-    const uint32_t nt = h->nt, total = h->n_trig, K = h->K;
+    wait_for_previous_kernel();
+    let_next_kernel_in();
+    const uint32_t nt = h->nt, total = h->n_trig, K = h->K, G = lanes_per_item(nt), lane = threadIdx.x & 31u;
+    const uint32_t per = 32u / G, gl = lane & (G - 1u);
+    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     const int64_t W = h->W;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const uint32_t a = tower_of(h->off, nt, i);
-        const trig_trigger s = tw[a].trig[i - h->off[a]];
+    for (uint64_t i0 = (uint64_t)gw * per; i0 < total; i0 += (uint64_t)nw * per) {
+        const uint32_t i = (uint32_t)i0 + lane / G;
         uint32_t cnt = 0;
-        if (s.pmt < tw[a].n_pmt) {
-            const uint16_t *row = h->dt + (size_t)(tw[a].base + s.pmt) * h->pt;
-            for (uint32_t b = 0; b < nt; ++b) {
-                if (b == a) {
-                    ++cnt;                  // s itself: |0| <= dt_max[p][p]
-                    continue;
-                }
-                const trig_trigger *L = tw[b].trig;
-                const uint32_t nb = h->n[b];
-                for (uint32_t j = trig_bound(L, nb, s.t_ns - W, false); j < nb; ++j) {
-                    const trig_trigger u = L[j];
-                    if (u.t_ns > s.t_ns + W) break;
-                    if (u.pmt >= tw[b].n_pmt) continue;
-                    const int64_t d = u.t_ns > s.t_ns ? u.t_ns - s.t_ns : s.t_ns - u.t_ns;
-                    if (d <= (int64_t)__ldg(row + tw[b].base + u.pmt)) {
-                        ++cnt;
-                        break;
+        if (i < total) {
+            const uint32_t a = tower_of(h->off, nt, i);
+            const trig_trigger s = tw[a].trig[i - h->off[a]];
+            if (s.pmt < tw[a].n_pmt) {
+                const uint16_t *row = h->dt + (size_t)(tw[a].base + s.pmt) * h->pt;
+                for (uint32_t b = gl; b < nt; b += G) {
+                    if (b == a) {
+                        ++cnt;                  // s itself: |0| <= dt_max[p][p]
+                        continue;
+                    }
+                    const trig_trigger *L = tw[b].trig;
+                    const uint32_t nb = h->n[b];
+                    for (uint32_t j = trig_bound(L, nb, s.t_ns - W, false); j < nb; ++j) {
+                        const trig_trigger u = L[j];
+                        if (u.t_ns > s.t_ns + W) break;
+                        if (u.pmt >= tw[b].n_pmt) continue;
+                        const int64_t d = u.t_ns > s.t_ns ? u.t_ns - s.t_ns : s.t_ns - u.t_ns;
+                        if (d <= (int64_t)__ldg(row + tw[b].base + u.pmt)) {
+                            ++cnt;
+                            break;
+                        }
                     }
                 }
             }
         }
-        h->sel_flag[i] = cnt >= K ? cnt : 0u;
+        cnt = group_sum(cnt, G);
+        if (i < total && gl == 0) h->sel_flag[i] = cnt >= K ? cnt : 0u;
     }
 }
 
 __global__ void k_apack(AHeader *h, const ATower *tw)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t nt = h->nt, total = h->n_trig;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const uint32_t f = h->sel_flag[i];
@@ -329,6 +370,8 @@ __global__ void k_apack(AHeader *h, const ATower *tw)
 
 __global__ void k_aseloff(AHeader *h)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t b = threadIdx.x, nt = h->nt;
     if (b <= nt) h->soff[b] = h->sel_pos[h->off[b]];        // sel_pos[n_trig] is the total
     if (b == 0) h->n_sel = h->sel_pos[h->n_trig];
@@ -336,15 +379,27 @@ __global__ void k_aseloff(AHeader *h)
 
 __global__ void k_amerge(AHeader *h)
 {
-    const uint32_t nt = h->nt, M = h->n_sel;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-        const uint32_t a = tower_of(h->soff, nt, i), k = i - h->soff[a];
-        const trig_array_seed s = h->sel[i];
-        uint64_t g = k;
-        for (uint32_t b = 0; b < nt; ++b)
-            if (b != a) g += seed_bound(h->sel + h->soff[b], h->soff[b + 1] - h->soff[b], s.t_ns, b < a);
-        h->merged_t[g] = s.t_ns;
-        if (g < h->seed_cap) h->seeds[g] = s;
+    wait_for_previous_kernel();
+    let_next_kernel_in();
+    const uint32_t nt = h->nt, M = h->n_sel, G = lanes_per_item(nt), lane = threadIdx.x & 31u;
+    const uint32_t per = 32u / G, gl = lane & (G - 1u);
+    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (uint64_t i0 = (uint64_t)gw * per; i0 < M; i0 += (uint64_t)nw * per) {
+        const uint32_t i = (uint32_t)i0 + lane / G;
+        uint32_t g = 0;
+        trig_array_seed s{};
+        if (i < M) {
+            const uint32_t a = tower_of(h->soff, nt, i);
+            s = h->sel[i];
+            if (gl == 0) g = i - h->soff[a];
+            for (uint32_t b = gl; b < nt; b += G)
+                if (b != a) g += seed_bound(h->sel + h->soff[b], h->soff[b + 1] - h->soff[b], s.t_ns, b < a);
+        }
+        g = group_sum(g, G);
+        if (i < M && gl == 0) {
+            h->merged_t[g] = s.t_ns;
+            if (g < h->seed_cap) h->seeds[g] = s;
+        }
     }
 }
 
@@ -352,6 +407,8 @@ __global__ void k_amerge(AHeader *h)
 
 __global__ void k_ahead(AHeader *h)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t M = h->n_sel;
     const int64_t gap = 2 * h->h + 1;
     for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < M; g += gridDim.x * blockDim.x)
@@ -360,6 +417,8 @@ __global__ void k_ahead(AHeader *h)
 
 __global__ void k_awin_a(AHeader *h)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t M = h->n_sel;
     for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < M; g += gridDim.x * blockDim.x)
         if (h->head[g]) h->win_first[h->head_pos[g]] = g;
@@ -380,6 +439,8 @@ __global__ void k_awin_a(AHeader *h)
 
 __global__ void k_awin_b(AHeader *h)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t M = h->n_sel, nw = h->n_win, ns = h->n_win_stored;
     for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < ns; w += gridDim.x * blockDim.x) {
         const uint32_t first = h->win_first[w], next = w + 1 < nw ? h->win_first[w + 1] : M;
@@ -396,6 +457,8 @@ __global__ void k_awin_b(AHeader *h)
 
 __global__ void k_azero(AHeader *h)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t n = h->n_cells;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) h->cell_cnt[i] = 0;
 }
@@ -416,6 +479,8 @@ __device__ __forceinline__ uint32_t first_ending_at(const int64_t *whi, uint32_t
 // bkt_win[j] .. bkt_win[j + 1].
 __global__ void k_abkt(AHeader *h)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t ns = h->n_win_stored, nb = h->n_bkt;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j <= nb; j += gridDim.x * blockDim.x)
         h->bkt_win[j] = first_ending_at(h->whi, 0, ns, h->bkt_org + ((int64_t)j << h->bkt_shift));
@@ -434,6 +499,8 @@ __device__ __forceinline__ uint32_t window_of(const AHeader *h, uint32_t ns, int
 
 __global__ void k_amark(AHeader *h, const ATower *tw)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t nt = h->nt, ns = h->n_win_stored, pt = h->pt;
     const uint64_t n = h->n_hits;
     for (uint64_t gi = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < n;
@@ -456,6 +523,8 @@ __global__ void k_amark(AHeader *h, const ATower *tw)
 
 __global__ void k_afrag(AHeader *h, const ATower *tw)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t nt = h->nt, ns = h->n_win_stored, pt = h->pt;
     const uint32_t total = h->cell_off[h->n_cells];
     const uint32_t stride = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -473,20 +542,35 @@ __global__ void k_afrag(AHeader *h, const ATower *tw)
     }
 }
 
+// Every hit inside a window to its place; a thread takes four hits at once.
+constexpr uint32_t kMarkPer = 4;
+
 __global__ void k_acopy(AHeader *h, const ATower *tw)
 {
+    wait_for_previous_kernel();
+    let_next_kernel_in();
     const uint32_t nt = h->nt, pt = h->pt;
-    const uint64_t n = h->n_hits;
-    for (uint64_t gi = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < n;
-         gi += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t w = h->win_id[gi];
-        if (w == kNone) continue;
-        const uint32_t b = tower_of_hit(tw, nt, gi);
-        const uint64_t i = gi - tw[b].hit0;
-        const trig_hit x = tw[b].hits[i];
-        const size_t cell = (size_t)w * pt + tw[b].base + x.pmt;
-        const uint64_t dst = (uint64_t)h->cell_off[cell] + (i - (uint64_t)h->cell_first[cell]);
-        if (dst < h->hit_cap) h->hits[dst] = x;
+    const uint64_t n = h->n_hits, nth = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g0 < n; g0 += nth * kMarkPer) {
+        uint32_t w[kMarkPer];
+#pragma unroll
+        for (uint32_t u = 0; u < kMarkPer; ++u) w[u] = g0 + u * nth < n ? h->win_id[g0 + u * nth] : kNone;
+#pragma unroll
+        for (uint32_t u = 0; u < kMarkPer; ++u) {
+            if (w[u] == kNone) continue;
+            const uint64_t gi = g0 + u * nth;
+            const uint32_t b = tower_of_hit(tw, nt, gi);
+            const uint64_t i = gi - tw[b].hit0;
+            const int4 x = *reinterpret_cast<const int4 *>(tw[b].hits + i);
+            const size_t cell = (size_t)w[u] * pt + tw[b].base + ((uint32_t)x.z & 0xffffu);
+            const uint64_t dst = (uint64_t)h->cell_off[cell] + (i - (uint64_t)h->cell_first[cell]);
+            // (8-byte stores: the buffer is the caller's)
+            if (dst < h->hit_cap) {
+                uint2 *o = reinterpret_cast<uint2 *>(h->hits + dst);
+                o[0] = make_uint2((uint32_t)x.x, (uint32_t)x.y);
+                o[1] = make_uint2((uint32_t)x.z, (uint32_t)x.w);
+            }
+        }
     }
 }
 
@@ -661,7 +745,8 @@ extern "C" int trig_array_select(trig_array *a, const trig_slice_dev *slices, co
         return report_error(TRIG_EINVAL, "trig_array_select: scratch must be 256-byte aligned device memory");
     if (scratch_bytes < L.bytes) return report_error(TRIG_ECAPACITY, "trig_array_select: scratch too small");
     char *sp = static_cast<char *>(scratch);
-    AHeader hd{};
+    APlan plan{};
+    AHeader &hd = plan.h;
     hd.nt = a->nt;
     hd.pt = a->pt;
     hd.K = a->par.min_towers;
@@ -695,7 +780,7 @@ extern "C" int trig_array_select(trig_array *a, const trig_slice_dev *slices, co
     hd.bkt_org = slices[0].t0_ns - (int64_t)a->par.win_half_ns;
     hd.bkt_shift = L.bkt_shift;
     hd.n_bkt = L.n_bkt;
-    ATower tw[kMaxTowers];
+    ATower *tw = plan.tw;
     uint64_t hit0 = 0;
     for (uint32_t b = 0; b < a->nt; ++b) {
         tw[b].trig = slices[b].triggers;
@@ -711,31 +796,27 @@ extern "C" int trig_array_select(trig_array *a, const trig_slice_dev *slices, co
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     AHeader *d_h = reinterpret_cast<AHeader *>(sp + L.hdr);
     ATower *d_t = reinterpret_cast<ATower *>(sp + L.towers);
-    // pageable sources: both copies are staged before the calls return
-    cudaError_t e = cudaMemcpyAsync(d_h, &hd, sizeof hd, cudaMemcpyHostToDevice, st);
-    if (!e) e = cudaMemcpyAsync(d_t, tw, sizeof(ATower) * a->nt, cudaMemcpyHostToDevice, st);
-    if (e) return report_cuda_error(e, "trig_array_select: copy descriptors");
     const int sms = device_sm_count();
     const unsigned grid = (unsigned)sms * 4;
     uint64_t nl = 0;
     uint32_t *scan_total = &d_h->scan_total;
-    k_acount<<<1, kMaxTowers, 0, st>>>(d_h, d_t);
-    k_aselect<<<grid, 256, 0, st>>>(d_h, d_t);
+    k_acount<<<1, kMaxTowers, 0, st>>>(plan, d_h, d_t);
+    launch_next(k_aselect, grid * 2, 256, 0, st, d_h, d_t);
     launch_scan<true>(hd.sel_flag, &d_h->n_trig, L.cap, hd.part, scan_total, hd.sel_pos, st, nl);
-    k_apack<<<grid, 256, 0, st>>>(d_h, d_t);
-    k_aseloff<<<1, kMaxTowers + 32, 0, st>>>(d_h);
-    k_amerge<<<grid, 256, 0, st>>>(d_h);
-    k_ahead<<<grid, 256, 0, st>>>(d_h);
+    launch_next(k_apack, grid, 256, 0, st, d_h, d_t);
+    launch_next(k_aseloff, 1, kMaxTowers + 32, 0, st, d_h);
+    launch_next(k_amerge, grid * 2, 256, 0, st, d_h);
+    launch_next(k_ahead, grid, 256, 0, st, d_h);
     launch_scan<false>(hd.head, &d_h->n_sel, L.cap, hd.part, scan_total, hd.head_pos, st, nl);
-    k_awin_a<<<grid, 256, 0, st>>>(d_h);
-    k_awin_b<<<grid, 256, 0, st>>>(d_h);
-    k_abkt<<<grid, 256, 0, st>>>(d_h);
-    k_azero<<<grid * 2, 256, 0, st>>>(d_h);
-    k_amark<<<grid * 2, 256, 0, st>>>(d_h, d_t);
+    launch_next(k_awin_a, grid, 256, 0, st, d_h);
+    launch_next(k_awin_b, grid, 256, 0, st, d_h);
+    launch_next(k_abkt, grid, 256, 0, st, d_h);
+    launch_next(k_azero, grid * 2, 256, 0, st, d_h);
+    launch_next(k_amark, grid * 2, 256, 0, st, d_h, d_t);
     launch_scan<false>(hd.cell_cnt, &d_h->n_cells, L.cells, hd.part, scan_total, hd.cell_off, st, nl);
-    k_afrag<<<grid, 256, 0, st>>>(d_h, d_t);
-    k_acopy<<<grid * 2, 256, 0, st>>>(d_h, d_t);
+    launch_next(k_afrag, grid, 256, 0, st, d_h, d_t);
+    launch_next(k_acopy, grid * 2, 256, 0, st, d_h, d_t);
     count_launches(nl + 13);
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     return e ? report_cuda_error(e, "trig_array_select: launch") : TRIG_OK;
 }
