@@ -1298,6 +1298,10 @@ struct Slot {
 };
 
 constexpr int kSlots = 3;
+// With a batch in flight the worker looks for its events without sleeping
+// until this long after the last progress (a sleep of 20 us lasts about 70,
+// twice a batch: one 84-PMT slice 0.35 against 0.27 ms); a longer batch is waited for in sleeps.
+constexpr std::chrono::microseconds kSpin(300);
 constexpr uint32_t kMaxBatchSlices = 256;
 
 struct Engine {
@@ -1668,12 +1672,14 @@ void Engine::run()
 {
     cudaSetDevice(device);
     std::unique_lock<std::mutex> lk(mu);
+    Clock::time_point progress = Clock::now();
     for (;;) {
         bool busy = false;
         for (auto &s : slots) busy |= s.state != 0;
         if (stop && !busy && pending.empty()) break;
         if (!busy && (pending.empty() || hold)) {
             cv.wait(lk);
+            progress = Clock::now();
             continue;
         }
         // progress in-flight slots; a CUDA error fails the slot's slices
@@ -1681,11 +1687,13 @@ void Engine::run()
         for (auto &s : slots) {
             if (s.state == 1) {
                 cudaError_t q = cudaEventQuery(s.ev_stats);
+                if (q != cudaErrorNotReady) progress = Clock::now();
                 if (q == cudaSuccess) collect_stats(s);
                 else if (q != cudaErrorNotReady) fail_slot(s, q);
             }
             if (s.state == 2) {
                 cudaError_t q = cudaEventQuery(s.ev_done);
+                if (q != cudaErrorNotReady) progress = Clock::now();
                 if (q == cudaSuccess) finish(s);
                 else if (q != cudaErrorNotReady) fail_slot(s, q);
             }
@@ -1730,7 +1738,19 @@ void Engine::run()
                 break;
             }
         }
-        if (!launched) cv.wait_for(lk, std::chrono::microseconds(20));
+        if (launched) {
+            progress = Clock::now();
+        } else if (busy && Clock::now() - progress < kSpin) {
+            // a query every 5 us: more of them hold up the submitting
+            // threads' copies (12 slices 1.48 against 1.36 ms)
+            lk.unlock();
+            const auto t = Clock::now();
+            do std::this_thread::yield();
+            while (Clock::now() - t < std::chrono::microseconds(5));
+            lk.lock();
+        } else {
+            cv.wait_for(lk, std::chrono::microseconds(20));
+        }
     }
 }
 
