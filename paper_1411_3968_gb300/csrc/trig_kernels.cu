@@ -443,9 +443,11 @@ __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
 // hit has its predecessor's PMT and edge count, in order and in range, is
 // done after that comparison; one that passes a tile edge writes its index.
 // Bound by instruction issue (nearly every step of 31 hits has a lane on the
-// edge path), then by HBM: the 64 slices of both towers (205 M hits) take
-// 0.95 ms, 1.42 with two edge counts per hit carried along walks of 512
-// hits; one 320 k-hit slice 8 us, 13 before.
+// edge path; its first store is predicated, the loop behind it rare), then
+// by HBM: the 64 slices of both towers (205 M hits) take 0.86 ms, 1.42 with
+// two edge counts per hit carried along walks of 512 hits (0.95 with a loop
+// over the edges alone); one 320 k-hit slice 8 us, 13 before.  Four blocks an
+// SM instead of three would spill: 254 against 210 us for 52 M hits.
 template <bool WIDE, bool S32>
 __device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, uint32_t c_end)
 {
@@ -453,6 +455,7 @@ __device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, ui
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, P = d.n_pmt;
     const uint32_t n_hits = (uint32_t)d.n_hits;                 // below 2^32 - 16
     const trig_hit *__restrict__ hits = d.hits;
+    uint32_t *__restrict__ edge = d.edge;
     const int64_t in_lo = d.in_lo;
     const T in_span = (T)(d.in_hi - in_lo);
     const T x0 = (T)(d.edge_org - in_lo);                       // the first edge, from in_lo
@@ -482,7 +485,10 @@ __device__ __forceinline__ void bounds_chunks(const SliceDesc &d, uint32_t c, ui
             const uint32_t el = __shfl_up_sync(0xffffffffu, e, 1);
             if (lane == 0 || !valid) continue;
             if (pc != pcl || rl > r || !in || li + 1 == n_hits) special |= 1u << u;
-            else if (e != el && p < P) fill_edges(d.edge, P, p, el, e, li);
+            else if (e != el && p < P) {
+                edge[(size_t)el * P + p] = li;          // most pass one edge at most
+                if (e - el > 1u) fill_edges(edge, P, p, el + 1u, e, li);
+            }
         }
         for (; special; special &= special - 1u)
             bounds_special(&d, wbase + (__ffs(special) - 1) * 31 + lane - 1u);
@@ -2079,29 +2085,39 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
 
 // ------------------------------------------------------------ window ranks
 
-// Hit rank of time x in PMT p's stream, narrowed by the tile edges the
-// structure pass recorded: x between the edges B_g - H and B_{g+1} - H lies
-// between the PMT's offsets there, so the binary search covers a handful of
-// hits.  Outside the edges the first or last one bounds it.
-__device__ __forceinline__ uint64_t rank_in_pmt(const SliceDesc &d, uint32_t p, int64_t x, uint64_t sp, uint64_t ep)
+// Where the first hit of PMT p's stream at or past time x can be, narrowed by
+// the tile edges the structure pass recorded: x between the edges B_g - H and
+// B_{g+1} - H lies between the PMT's offsets there, so a binary search covers
+// a handful of hits.  Outside the edges the first or last one bounds it.
+__device__ __forceinline__ void rank_range(const SliceDesc &d, uint32_t p, int64_t x, uint32_t sp, uint32_t ep, uint32_t &lo,
+                                           uint32_t &hi)
 {
     const int64_t rel = x - (d.t0 - (int64_t)d.halo);
-    uint64_t lo = sp, hi = ep;
+    lo = sp;
+    hi = ep;
     if (rel >= 0) {
         const int64_t g = min(rel / d.tile_w, (int64_t)d.n_tiles);
         const uint32_t *at = d.edge + (size_t)(2 * g) * d.n_pmt + p;
-        lo = max(lo, min((uint64_t)at[0], ep));
-        if (g < (int64_t)d.n_tiles) hi = min(hi, max((uint64_t)at[2 * (size_t)d.n_pmt], lo));
+        lo = max(lo, min(at[0], ep));
+        if (g < (int64_t)d.n_tiles) hi = min(hi, max(at[2 * (size_t)d.n_pmt], lo));
     } else if (d.n_tiles) {
-        hi = min(hi, max((uint64_t)d.edge[p], lo));
+        hi = min(hi, max(d.edge[p], lo));
     }
+}
+
+// That first hit's index.
+__device__ __forceinline__ uint64_t rank_in_pmt(const SliceDesc &d, uint32_t p, int64_t x, uint64_t sp, uint64_t ep)
+{
+    uint32_t lo, hi;
+    rank_range(d, p, x, (uint32_t)sp, (uint32_t)ep, lo, hi);
     return lb_time(d.hits, lo, hi, x);
 }
 
 // Merged rank of time x (the hits of the submission with t < x), by the
-// warp: per-PMT searches, or for a wide slice the bucket offsets plus the
-// edge bucket's hits below x.
-__device__ uint64_t warp_rank_of(const SliceDesc &d, int64_t x)
+// warp: per-PMT searches, a lane's four side by side (one after the other
+// they were the longest chain behind a slice's windows), or for a wide slice
+// the bucket offsets plus the edge bucket's hits below x.
+__device__ __noinline__ uint64_t warp_rank_of(const SliceDesc &d, int64_t x)
 {
     const uint32_t lane = lane_id();
     uint64_t r = 0;
@@ -2111,10 +2127,38 @@ __device__ uint64_t warp_rank_of(const SliceDesc &d, int64_t x)
         if (lane == 0) r = e0;
         for (uint32_t j = e0 + lane; j < e1; j += 32) r += d.tbuf[j].t_ns < x;
     } else {
-        for (uint32_t p = lane; p < d.n_pmt; p += 32) {
-            const uint64_t sp = d.pmt_off[p], ep = d.pmt_off[p + 1];
-            r += rank_in_pmt(d, p, x, sp, ep) - sp;
+        constexpr uint32_t R = (kWideMinPmt + 30) / 32;
+        uint32_t lo[R], hi[R], own = 0;
+        bool more = false;
+#pragma unroll
+        for (uint32_t k = 0; k < R; ++k) {
+            const uint32_t p = k * 32 + lane;
+            lo[k] = hi[k] = 0;
+            if (p < d.n_pmt) {
+                const uint32_t sp = (uint32_t)d.pmt_off[p];
+                rank_range(d, p, x, sp, (uint32_t)d.pmt_off[p + 1], lo[k], hi[k]);
+                own -= sp;
+            }
+            more |= lo[k] < hi[k];
         }
+        while (more) {
+            int64_t t[R];
+#pragma unroll
+            for (uint32_t k = 0; k < R; ++k)
+                if (lo[k] < hi[k]) t[k] = d.hits[lo[k] + ((hi[k] - lo[k]) >> 1)].t_ns;
+            more = false;
+#pragma unroll
+            for (uint32_t k = 0; k < R; ++k) {
+                if (lo[k] >= hi[k]) continue;
+                const uint32_t mid = lo[k] + ((hi[k] - lo[k]) >> 1);
+                if (t[k] < x) lo[k] = mid + 1u;
+                else hi[k] = mid;
+                more |= lo[k] < hi[k];
+            }
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < R; ++k) own += lo[k];
+        r = own;                        // the lane's sum: at most its hits, so below 2^32
     }
     return warp_sum_u64(r);
 }
@@ -2240,7 +2284,7 @@ __device__ __forceinline__ void fin_window(const SliceDesc &d, bool have, uint64
 // slices of 12 M triggers.  Bound by the latency of its chain (ticket, tile
 // counts, two reads of the seeds around the look-back).
 constexpr uint32_t kFinThreads = 256;
-constexpr uint32_t kFinUnroll = 4;          // loads of a warp's pass in flight
+constexpr uint32_t kFinUnroll = 2;          // loads of a warp's pass in flight (four spill)
 
 __global__ void __launch_bounds__(kFinThreads, 3) k_final(BatchHeader *__restrict__ hdr, const SliceDesc *__restrict__ desc)
 {
