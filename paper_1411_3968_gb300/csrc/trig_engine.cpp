@@ -587,7 +587,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             // segments of about 8 hits per PMT (a run of 128 bytes), at least
             // 4096 hits, at most kSegBuckets buckets and 2^31 ns
             const double rate = (double)x.n_hits / ((double)d.n_bkt * d.bkt_w);
-            const double hits = std::max(8.0 * P, 4096.0);
+            const double hits = std::max((cfg.lean ? 64.0 : 8.0) * P, 4096.0);
             const double want = rate > 0.0 ? hits / (rate * d.bkt_w) : (double)kSegBuckets;
             d.seg_bkt = (uint32_t)std::max(1.0, std::min({want, (double)kSegBuckets, (double)d.n_bkt,
                                                           std::floor(2147483647.0 / d.bkt_w)}));
@@ -1114,6 +1114,15 @@ extern "C" int trig_batch_run_noalloc(const trig_slice_dev *slices, uint32_t n_s
     int rc = plan_into(slices, n_slices, (uintptr_t)scratch, cfg, hdr, desc, bytes, max_pmt, smem_dt,
                        any_wide, &shape);
     if (rc) return rc;
+    if (bytes > cap) {
+        // the largest batches only fit with larger tiles and segments
+        TileConfig lean = cfg;
+        if (cfg.spread) trig_get_tile_config(&lean.cap, &lean.warps, &lean.fill_pct);
+        lean.spread = 0;
+        lean.lean = 1;
+        rc = plan_into(slices, n_slices, (uintptr_t)scratch, lean, hdr, desc, bytes, max_pmt, smem_dt, any_wide, &shape);
+        if (rc) return rc;
+    }
     if (bytes > cap) return fail(TRIG_ECAPACITY, "trig_batch_run_noalloc: batch needs more than TRIG_NOALLOC_SCRATCH_BYTES of scratch");
     BatchHeader *d_hdr = reinterpret_cast<BatchHeader *>(scratch);
     SliceDesc *d_desc = reinterpret_cast<SliceDesc *>((char *)scratch + align256(sizeof(BatchHeader)));

@@ -162,6 +162,7 @@ struct TileConfig {
     uint32_t warps;
     uint32_t fill_pct;
     uint32_t spread = 0;    // tiles cut smaller so that a small batch fills the GPU (kOwnShape)
+    uint32_t lean = 0;      // the smallest side tables (a batch at the edge of a fixed scratch)
 };
 // The library's own choice: the shape the autotuner ends at for towers and
 // the 2688-PMT array, with two blocks on an SM (4096-hit tiles leave room for

@@ -7,15 +7,17 @@
 //              of every hit: validates the CSR layout and ordering, and for
 //              every tile g and PMT p records where p's stream crosses
 //              the tile's halo edges B_g - H and B_{g+1} + H.
-//   k_tile     persistent, warp-specialised: a producer warp dequeues tiles
-//              and stages each tile's hits (one contiguous run per PMT) into
-//              shared memory with bulk TMA copies (cp.async.bulk + mbarrier,
-//              double-buffered); 16 consumer warps merge the runs into time
-//              order (bucket sort on the time key), select seeds (charge
-//              threshold or floor coincidence, "Sorting and triggering in
-//              GPU"), count causally related hits per seed with warp
-//              ballot/popc against the integer dt_max table ("Muon trigger
-//              strategy"), and emit the fired seeds at their merged rank.
+//   k_scatter  detectors above 128 PMTs: the hits copied to time buckets,
+//              whose ranges then stand in for the PMT runs.
+//   k_tile     persistent, warp-specialised: a stager warp dequeues tiles and
+//              brings each tile's hits (one contiguous run per PMT) into
+//              shared memory with bulk TMA copies (cp.async.bulk + mbarrier);
+//              up to 16 consumer warps merge the runs into time order (bucket
+//              sort on the time key), select seeds (charge threshold or
+//              floor coincidence, "Sorting and triggering in GPU"), count
+//              causally related hits per seed against the integer dt_max
+//              table ("Muon trigger strategy"), and emit the fired seeds at
+//              their merged rank.
 //   k_final    stream compaction of the fired seeds, and the +-3 us windows
 //              around the triggers, merged while lo_next <= hi_cur + 1, with
 //              the hit count inside each: the difference of two merged ranks
@@ -2844,7 +2846,7 @@ extern "C" int trig_check_record(unsigned *site, unsigned *count, unsigned long 
 
 // Scratch of trig_batch_run_noalloc: a fixed device array, present on every
 // device that loads the library until the process exits.  Calls share it
-// and it keeps the previous call's contents; k_prep clears the counters
+// and it keeps the previous call's contents; k_put clears the counters
 // that must start at zero, and everything else is written before it is
 // read.  Calls that overlap on the GPU race on it.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[TRIG_NOALLOC_SCRATCH_BYTES];

@@ -121,4 +121,63 @@ def test_bursts_split_tiles(pkg, params, n_pmt, cluster_ns, rule):
             assert np.array_equal(trig[f], ref.triggers[f]), (shape, f)
         for f in ("lo", "hi", "n_hits", "n_triggers"):
             assert np.array_equal(win[f], ref.windows[f]), (shape, f)
+        if events:
+            (ev, n_ev, full), = b.event_hits()
+            want = oracle.events(hits, ref.windows)
+            assert not full and n_ev == len(want)
+            for f in ("t", "pmt", "charge"):
+                assert np.array_equal(ev[f], want[f]), (shape, f)
+    det.close()
+
+
+def test_more_slices_than_one_descriptor_launch_carries(pkg, params):
+    """70 slices (k_put carries 64 at a time), plain and as a graph replay,
+    empty ones among them: every slice the oracle's."""
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(70))
+    par = dict(params, slice_ns=50_000)
+    xyz, floor = _detector(84)
+    det = pkg.Detector(xyz, floor, par)
+    slices = []
+    for k in range(70):
+        t0 = 1_000_000 + k * par["slice_ns"]
+        hits, off = _hits(rng, 0 if k % 23 == 5 else 300 + 20 * k, 84, t0 - 3000, t0 + par["slice_ns"] + 3000)
+        slices.append(SliceIn(det, t0, hits, off))
+    b = DeviceBatch(slices)
+    for graph in (False, True, True):
+        b.run(graph=graph)
+        for s, (stats, trig, win) in zip(slices, b.results()):
+            ref = oracle.run(xyz, floor, par, s.hits, [s.t0])[0]
+            assert int(stats["status"]) == 0 and int(stats["n_hits"]) == len(s.hits)
+            assert int(stats["n_seeds"]) == len(ref.seeds)
+            for f in ("t", "pmt", "charge", "count"):
+                assert np.array_equal(trig[f], ref.triggers[f]), f
+            for f in ("lo", "hi", "n_hits", "n_triggers"):
+                assert np.array_equal(win[f], ref.windows[f]), f
+    det.close()
+
+
+@pytest.mark.parametrize("n_pmt,n", [(84, 2_750_000), (336, 1_635_000)])
+def test_noalloc_takes_the_largest_batches(pkg, params, n_pmt, n):
+    """A slice close to what the static scratch holds (about 24 bytes a hit, 40
+    above 128 PMTs) is planned with larger tiles and segments instead of
+    being refused."""
+    import torch
+    from paper_1411_3968_gb300 import _lib
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(n))
+    par = dict(params, slice_ns=200_000_000)
+    xyz, floor = _detector(n_pmt)
+    det = pkg.Detector(xyz, floor, par)
+    hits, off = _hits(rng, n, n_pmt, 1_000_000 - 3000, 1_000_000 + par["slice_ns"] + 3000)
+    b = DeviceBatch([SliceIn(det, 1_000_000, hits, off)])
+    b.run()
+    (stats, trig, win), = b.results()
+    b.trig[0].zero_()
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    _lib.trig_batch_run_noalloc(b.descs, st.cuda_stream)
+    (stats2, trig2, win2), = b.results()
+    assert int(stats2["status"]) == 0 and stats2 == stats
+    assert np.array_equal(trig2, trig) and np.array_equal(win2, win)
     det.close()
