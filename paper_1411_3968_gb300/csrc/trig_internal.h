@@ -169,6 +169,8 @@ struct TileConfig {
 // one: 15.7 against 20.3 us for 320 k hits, 72 against 83 us for 2.8 M, 1.33
 // against 1.68 ms for 52 M under the distinct count).
 constexpr TileConfig kOwnShape{2048, 16, 90, 1};
+// Many tiles of an array so dense that halos crowd the tile (see halo_heavy).
+constexpr TileConfig kOwnDenseShape{4096, 16, 90, 0};
 inline bool valid_tile_shape(uint32_t cap, uint32_t warps)
 {
     return ((cap == 4096 || cap == 2048) && (warps == 16 || warps == 8)) || (cap == 1024 && warps == 4);

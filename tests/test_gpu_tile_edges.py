@@ -181,3 +181,49 @@ def test_noalloc_takes_the_largest_batches(pkg, params, n_pmt, n):
     assert int(stats2["status"]) == 0 and stats2 == stats
     assert np.array_equal(trig2, trig) and np.array_equal(win2, win)
     det.close()
+
+
+_OWN_SHAPE = """
+import sys
+sys.path[:0] = {path!r}
+import numpy as np, torch
+import paper_1411_3968_gb300 as pkg, workload
+from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+pkg.load()
+torch.cuda.init()
+rng = np.random.Generator(np.random.PCG64({n}))
+k = np.arange(2016)
+xyz = np.stack([1000 * (k % 6), np.zeros_like(k), 40_000 * (k // 6)], 1).astype(np.int32)
+par = dict({par!r}, slice_ns={slice_ns})
+hits = np.zeros({n}, workload.HIT_DTYPE)
+hits["t"] = 1_000_000 - 3000 + rng.integers(0, par["slice_ns"] + 6000, {n})
+hits["pmt"] = rng.integers(0, 2016, {n})
+hits["charge"] = rng.integers(1, 320, {n})
+hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+off = np.zeros(2017, np.uint64)
+np.cumsum(np.bincount(hits["pmt"], minlength=2016), out=off[1:])
+b = DeviceBatch([SliceIn(pkg.Detector(xyz, (k // 6).astype(np.uint32), par), 1_000_000, hits, off)])
+res = []
+for shape in (None, (2048, 16, 90)):
+    if shape:
+        pkg.trig_set_tile_config(*shape)
+    b.run()
+    res.append(b.results()[0])
+    b.trig[0].zero_()
+(s0, t0, w0), (s1, t1, w1) = res
+assert int(s0["status"]) == 0 and s0 == s1 and len(t0) > 1000
+assert np.array_equal(t0, t1) and np.array_equal(w0, w1)
+print("same")
+"""
+
+
+@pytest.mark.parametrize("slice_ns,n", [(32_000_000, 4_800_000), (60_000_000, 5_400_000)])
+def test_own_shape_of_dense_arrays(pkg, params, slice_ns, n):
+    """The library's own shape above and below the rate at which halos take a
+    quarter of a tile (a process of its own: no shape is set before): what a
+    set shape gives."""
+    import subprocess
+    import sys
+    src = _OWN_SHAPE.format(path=sys.path, par=dict(params), slice_ns=slice_ns, n=n)
+    r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
