@@ -544,7 +544,8 @@ __global__ void __launch_bounds__(kBoundsThreads, 3) k_bounds(const BatchHeader 
 // hit-by-hit copy needs took 0.51 ms for the 2688-PMT slice (29.6 M hits)
 // and 0.24 of the structure pass, against 0.42 and 0.13.  Bound by the
 // latency of the short runs' loads.
-// Slices with malformed input (flagged by the structure pass) are skipped.
+// Slices with malformed input (flagged by the structure pass) are skipped, and
+// so are those without hits, whose edges the structure pass never writes.
 constexpr uint32_t kScatThreads = 512;
 
 __global__ void __launch_bounds__(kScatThreads, 2) k_scatter(const BatchHeader *__restrict__ hdr,
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_scatter(const BatchHeader *
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     for (uint32_t s = 0; s < hdr->n_slices; ++s) {
         const SliceDesc &d = desc[s];
-        if (!d.wide) continue;
+        if (!d.wide || d.n_hits == 0) continue;
         if (d.stats->flags & (TRIG_FLAG_BAD_PMT | TRIG_FLAG_UNSORTED | TRIG_FLAG_OUT_OF_RANGE)) continue;
         const uint32_t P = d.n_pmt, K = d.seg_bkt, n_seg = d.n_edges - 1u;
         for (uint32_t g = blockIdx.x; g < n_seg; g += gridDim.x) {
@@ -2594,7 +2595,7 @@ __global__ void __launch_bounds__(kEvHaloThreads) k_evhalo(const BatchHeader *__
     uint32_t *psum = reinterpret_cast<uint32_t *>(keys + TRIG_EV_HALO_MAX);
     for (uint32_t s = blockIdx.x; s < hdr->n_slices; s += gridDim.x) {
         const SliceDesc &d = desc[s];
-        if (!d.ev || d.ev_cap == 0) continue;
+        if (!d.ev || d.ev_cap == 0 || d.n_hits == 0) continue;
         if (d.stats->flags & (TRIG_FLAG_BAD_PMT | TRIG_FLAG_UNSORTED | TRIG_FLAG_OUT_OF_RANGE)) continue;
         ev_halo_side(d, true, keys, psum, d.in_lo, d.t0);
         ev_halo_side(d, false, keys, psum, d.t0 + d.slice_ns, d.t0 + d.slice_ns);

@@ -1,0 +1,135 @@
+"""Slices whose input is at the edge of what a call takes, beside ordinary
+ones of the same batch: no hits at all.  The neighbours' results are the
+oracle's, whatever the scratch held before."""
+import numpy as np
+import pytest
+
+import oracle
+import workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+    import paper_1411_3968_gb300 as p
+    from paper_1411_3968_gb300 import build
+    build.build()
+    p.load()
+    torch.cuda.init()
+    return p
+
+
+def _detector(n_pmt, per_floor=6):
+    k = np.arange(n_pmt)
+    xyz = np.stack([1000 * (k % per_floor), np.zeros_like(k), 40_000 * (k // per_floor)], 1).astype(np.int32)
+    return xyz, (k // per_floor).astype(np.uint32)
+
+
+def _stream(hits, n_pmt):
+    hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    return hits, off
+
+
+def _hits(rng, n, n_pmt, lo, hi, step=1):
+    hits = np.zeros(n, workload.HIT_DTYPE)
+    hits["t"] = lo + rng.integers(0, max(1, (hi - lo) // step), n) * step
+    hits["pmt"] = rng.integers(0, n_pmt, n)
+    hits["charge"] = rng.integers(1, 400, n)
+    return _stream(hits, n_pmt)
+
+
+def _assert_same(res, ref, ctx=""):
+    stats, trig, win = res
+    assert int(stats["status"]) == 0, ctx
+    assert int(stats["n_seeds"]) == len(ref.seeds), ctx
+    assert len(trig) == len(ref.triggers) and len(win) == len(ref.windows), ctx
+    for f in ("t", "pmt", "charge", "count"):
+        assert np.array_equal(trig[f], ref.triggers[f]), (ctx, f)
+    for f in ("lo", "hi", "n_hits", "n_triggers"):
+        assert np.array_equal(win[f], ref.windows[f]), (ctx, f)
+
+
+def _assert_result(r, ref, ctx=""):
+    assert r.status == 0 and r.n_seeds == len(ref.seeds), ctx
+    for f in ("t", "pmt", "charge", "count"):
+        assert np.array_equal(r.triggers[f], ref.triggers[f]), (ctx, f)
+    for f in ("lo", "hi", "n_hits", "n_triggers"):
+        assert np.array_equal(r.windows[f], ref.windows[f]), (ctx, f)
+
+
+def _mixed(pkg, n_pmt, par, empty, n=4000):
+    """Five slices, the ones in `empty` without hits, and the others' oracle results."""
+    from paper_1411_3968_gb300.runner import SliceIn
+    rng = np.random.Generator(np.random.PCG64(n_pmt))
+    xyz, floor = _detector(n_pmt)
+    det = pkg.Detector(xyz, floor, par)
+    slices, refs = [], []
+    for k in range(5):
+        t0 = 1_000_000 + k * par["slice_ns"]
+        hits, off = _hits(rng, 0 if k in empty else n + 100 * k, n_pmt, t0 - 3000, t0 + par["slice_ns"] + 3000)
+        slices.append(SliceIn(det, t0, hits, off))
+        refs.append(oracle.run(xyz, floor, par, hits, [t0])[0])
+    return det, slices, refs
+
+
+@pytest.mark.parametrize("n_pmt", [84, 129, 672, 2688])
+@pytest.mark.parametrize("empty", [(0, 3), (4,), (0, 1, 2, 3, 4)])
+def test_empty_slices_beside_full_ones(pkg, params, n_pmt, empty):
+    import torch
+    from paper_1411_3968_gb300 import _lib
+    from paper_1411_3968_gb300.runner import DeviceBatch
+    par = dict(params, slice_ns=300_000)
+    det, slices, refs = _mixed(pkg, n_pmt, par, empty)
+    b = DeviceBatch(slices)
+    stream = torch.cuda.Stream()
+
+    def noalloc():
+        torch.cuda.synchronize()
+        _lib.trig_batch_run_noalloc(b.descs, stream.cuda_stream)
+
+    for name, run in (("plain", b.run), ("graph", lambda: b.run(graph=True)), ("replay", lambda: b.run(graph=True)),
+                      ("noalloc", noalloc)):
+        b.scratch.fill_(0x3f)
+        for t in b.trig + b.win:
+            t.zero_()
+        run()
+        for k, (res, ref) in enumerate(zip(b.results(), refs)):
+            _assert_same(res, ref, (name, k))
+            assert int(res[0]["n_hits"]) == len(slices[k].hits)
+    det.close()
+
+
+@pytest.mark.parametrize("n_pmt", [84, 672])
+def test_empty_slices_with_events(pkg, params, n_pmt):
+    from paper_1411_3968_gb300.runner import DeviceBatch
+    par = dict(params, slice_ns=300_000)
+    det, slices, refs = _mixed(pkg, n_pmt, par, (1, 4))
+    b = DeviceBatch(slices, events=True)
+    b.scratch.fill_(0x3f)
+    b.run()
+    for k, (res, ev, ref) in enumerate(zip(b.results(), b.event_hits(), refs)):
+        _assert_same(res, ref, k)
+        want = oracle.events(slices[k].hits, ref.windows)
+        assert not ev[2] and ev[1] == len(want), k
+        for f in ("t", "pmt", "charge"):
+            assert np.array_equal(ev[0][f], want[f]), (k, f)
+    det.close()
+
+
+@pytest.mark.parametrize("n_pmt", [84, 672])
+def test_empty_slices_through_the_engine(pkg, params, n_pmt):
+    par = dict(params, slice_ns=300_000)
+    det, slices, refs = _mixed(pkg, n_pmt, par, (0, 3))
+    for _ in range(2):                      # the second time on an arena full of the first one's bytes
+        pkg.trig_engine_hold(True)
+        ids = [pkg.trig_submit_slice(det, s.t0, s.hits, s.pmt_off) for s in slices]
+        pkg.trig_engine_hold(False)
+        for k, ref in enumerate(refs):
+            r = pkg.trig_poll(det, 30_000)
+            assert r is not None and r.slice_id == ids[k]
+            _assert_result(r, ref, k)
+    det.close()
