@@ -52,7 +52,8 @@ extern "C" {
 #define TRIG_ECAPACITY  (-6)  /* output capacity or tile capacity exceeded      */
 
 /* Slice status bits reported by the device (trig_slice_stats.flags). */
-#define TRIG_FLAG_BAD_PMT      0x01u  /* hit.pmt >= n_pmt or outside its CSR row  */
+#define TRIG_FLAG_BAD_PMT      0x01u  /* hit.pmt >= n_pmt or outside its CSR row, or
+                                         a pmt_off entry not at its PMT's place  */
 #define TRIG_FLAG_UNSORTED     0x02u  /* a PMT stream is not time-ordered         */
 #define TRIG_FLAG_OUT_OF_RANGE 0x04u  /* hit outside [t0 - halo, t0 + S + halo)   */
 #define TRIG_FLAG_TILE_FULL    0x08u  /* > tile capacity hits inside one 1 ns core

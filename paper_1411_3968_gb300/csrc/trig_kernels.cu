@@ -344,12 +344,18 @@ __device__ __forceinline__ void fill_edges(uint32_t *e, uint32_t P, uint32_t p, 
         if (CHECK(1, (size_t)g * P + p, (size_t)g1 * P)) e[(size_t)g * P + p] = v;
 }
 
-// Edges after a PMT's last hit, and all edges of the empty PMTs that follow.
-__device__ __noinline__ void fill_run_end(uint32_t *edge, const uint64_t *poff, uint32_t P, uint32_t NE, uint32_t p,
-                                          uint32_t from, uint32_t ep)
+// The edges of the empty PMTs [q0, q1) before hit v of the slice (or past its
+// last) are all v, if their offsets and that of q1 are; returns whether they
+// are.  (No PMT has two places, so wrong offsets cost no more stores than
+// right ones.)
+__device__ __forceinline__ bool fill_empty(uint32_t *edge, const uint64_t *poff, uint32_t P, uint32_t NE, uint32_t q0,
+                                           uint32_t q1, uint32_t v)
 {
-    fill_edges(edge, P, p, from, NE, ep);
-    for (uint32_t q = p + 1; q < P && poff[q] == poff[q + 1]; ++q) fill_edges(edge, P, q, 0, NE, ep);
+    for (uint32_t q = q0; q < q1; ++q) {
+        if (poff[q] != v) return false;
+        fill_edges(edge, P, q, 0, NE, v);
+    }
+    return poff[q1] == v;
 }
 
 constexpr int kBoundsThreads = 256;
@@ -395,6 +401,11 @@ struct EdgeCount {
 // first or last hit of a PMT's run or of the slice, an out-of-range time, a
 // step back.  It looks at the hit and its predecessor again (a run has
 // thousands of hits, so few come here).
+// A slice with hits that leaves here without a flag has its PMTs in order and
+// every one of its P + 1 offsets at the place where that PMT's hits start:
+// each run's first hit checks its own and those of the empty PMTs before it,
+// the last hit those after it.  What follows takes offsets and edges as
+// indices without a further look.
 __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
 {
     const SliceDesc &d = *dp;
@@ -417,15 +428,10 @@ __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
         el = ec.of64(l.t_ns - d.edge_org);
     }
     uint32_t bad = 0;
-    if (is_first && li > 0 && pl < P) {
-        // hit li - 1 was the last of PMT pl's run
-        if (poff[pl + 1] != li) bad |= TRIG_FLAG_BAD_PMT;
-        fill_run_end(d.edge, poff, P, NE, pl, el, (uint32_t)li);
-    }
-    if (p >= P) bad |= TRIG_FLAG_BAD_PMT;
-    else {
-        if (is_first && poff[p] != li) bad |= TRIG_FLAG_BAD_PMT;
-        if (li + 1 == n_hits && (poff[p + 1] != n_hits || poff[P] != n_hits)) bad |= TRIG_FLAG_BAD_PMT;
+    if (p >= P || (li > 0 && pl > p)) bad |= TRIG_FLAG_BAD_PMT;
+    else if (is_first) {
+        if (!fill_empty(d.edge, poff, P, NE, li > 0 ? pl + 1u : 0u, p, (uint32_t)li)) bad |= TRIG_FLAG_BAD_PMT;
+        else if (li > 0) fill_edges(d.edge, P, pl, el, NE, (uint32_t)li);       // hit li - 1 ended PMT pl's run
     }
     if (h.t_ns < d.in_lo || h.t_ns >= d.in_hi) bad |= TRIG_FLAG_OUT_OF_RANGE;
     if (!is_first && l.t_ns > h.t_ns) bad |= TRIG_FLAG_UNSORTED;
@@ -434,9 +440,10 @@ __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
         return;
     }
     fill_edges(d.edge, P, p, is_first ? 0u : el, e, (uint32_t)li);
-    if (li + 1 == n_hits) fill_run_end(d.edge, poff, P, NE, p, e, (uint32_t)n_hits);
-    if (li == 0)
-        for (uint32_t q = 0; q < p; ++q) fill_edges(d.edge, P, q, 0, NE, 0u);       // empty PMTs before the first hit
+    if (li + 1 == n_hits) {
+        if (!fill_empty(d.edge, poff, P, NE, p + 1u, P, (uint32_t)n_hits)) report(d, TRIG_FLAG_BAD_PMT);
+        else fill_edges(d.edge, P, p, e, NE, (uint32_t)n_hits);
+    }
 }
 
 // Chunks [c, c_end) of one slice, block-wide.  A warp takes 31 new hits per
@@ -2717,7 +2724,8 @@ __global__ void k_rank0(const BatchHeader *__restrict__ hdr, SliceDesc *__restri
     if (s >= hdr->n_slices) return;
     SliceDesc &d = desc[s];
     uint64_t r = 0, r1 = 0;
-    for (uint32_t p = threadIdx.x; p < d.n_pmt; p += blockDim.x) {
+    const bool offsets = d.n_hits && !(d.stats->flags & TRIG_FLAG_BAD_PMT);       // checked, and not found wrong
+    for (uint32_t p = threadIdx.x; offsets && p < d.n_pmt; p += blockDim.x) {
         uint64_t sp = d.pmt_off[p], ep = d.pmt_off[p + 1];
         uint64_t a = lb_time(d.hits, sp, ep, d.t0);
         r += a - sp;

@@ -1,6 +1,7 @@
-"""Slices whose input is at the edge of what a call takes, beside ordinary
-ones of the same batch: no hits at all.  The neighbours' results are the
-oracle's, whatever the scratch held before."""
+"""Slices whose input is at the edge of what a call takes, or past it, beside
+ordinary ones of the same batch: no hits at all, PMTs without hits, offsets
+that are wrong where no hit is.  The neighbours' results are the oracle's,
+whatever the scratch held before."""
 import numpy as np
 import pytest
 
@@ -132,4 +133,77 @@ def test_empty_slices_through_the_engine(pkg, params, n_pmt):
             r = pkg.trig_poll(det, 30_000)
             assert r is not None and r.slice_id == ids[k]
             _assert_result(r, ref, k)
+    det.close()
+
+
+def _sparse(rng, n_pmt, used, n, lo, hi):
+    """Hits of the PMTs `used` alone."""
+    hits, _ = _hits(rng, n, len(used), lo, hi)
+    hits["pmt"] = np.asarray(used, np.uint16)[hits["pmt"]]
+    return _stream(hits, n_pmt)
+
+
+def _used(n_pmt):
+    """Most of the PMTs, with empty ones before the first, after the last and in runs between."""
+    return [p for p in range(2, n_pmt - 3) if p % 7 not in (3, 4) and not n_pmt // 2 <= p < n_pmt // 2 + 9]
+
+
+@pytest.mark.parametrize("n_pmt", [84, 128, 129, 672])
+def test_runs_of_empty_pmts(pkg, params, n_pmt):
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(n_pmt + 5))
+    par = dict(params, slice_ns=300_000)
+    xyz, floor = _detector(n_pmt)
+    det = pkg.Detector(xyz, floor, par)
+    t0 = 1_000_000
+    for used in (_used(n_pmt), [n_pmt - 1], [0], [0, n_pmt - 1]):
+        hits, off = _sparse(rng, n_pmt, used, 3000, t0 - 3000, t0 + par["slice_ns"] + 3000)
+        b = DeviceBatch([SliceIn(det, t0, hits, off)])
+        b.scratch.fill_(0x3f)
+        b.run()
+        _assert_same(b.results()[0], oracle.run(xyz, floor, par, hits, [t0])[0], used[:3])
+    det.close()
+
+
+def _bad_offsets(off, n_pmt):
+    """Offsets that disagree with the hits at empty PMTs only, where no hit's own run start or end shows it."""
+    n = int(off[-1])
+    mid = n_pmt // 2 + 4                        # inside the empty run of _used
+    return {"first": (0, 1), "second": (1, n), "low": (mid, int(off[mid]) - 1), "high": (mid, int(off[mid]) + 1),
+            "far": (mid, 2 ** 40), "wrapped": (mid, 2 ** 64 - 1), "after": (n_pmt - 1, n - 1), "past": (n_pmt - 2, n + 7)}
+
+
+@pytest.mark.parametrize("n_pmt", [84, 129, 672])
+def test_offsets_of_empty_pmts_are_checked(pkg, params, n_pmt):
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(n_pmt + 9))
+    par = dict(params, slice_ns=300_000)
+    xyz, floor = _detector(n_pmt)
+    det = pkg.Detector(xyz, floor, par)
+    t0 = 1_000_000
+    hits, off = _sparse(rng, n_pmt, _used(n_pmt), 3000, t0 - 3000, t0 + par["slice_ns"] + 3000)
+    ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+    slices = [SliceIn(det, t0, hits, off)]
+    for at, value in _bad_offsets(off, n_pmt).values():
+        wrong = off.copy()
+        wrong[at] = value
+        slices.append(SliceIn(det, t0, hits, wrong))
+    # runs out of order, each at its own PMT's offset
+    swapped = np.concatenate([hits[hits["pmt"] == 9], hits[hits["pmt"] == 5]])
+    so = np.full(n_pmt + 1, len(swapped), np.uint64)
+    n9 = int((swapped["pmt"] == 9).sum())
+    so[:10], so[5], so[6], so[9], so[10] = 0, n9, len(swapped), 0, n9
+    slices.append(SliceIn(det, t0, swapped, so))
+    slices.append(slices[0])
+    b = DeviceBatch(slices)
+    b.scratch.fill_(0x3f)
+    for graph in (False, True):
+        b.run(graph=graph)
+        res = b.results()
+        for k in (0, len(slices) - 1):
+            _assert_same(res[k], ref, k)
+        for stats, trig, win in res[1:-1]:
+            assert int(stats["status"]) == pkg.TRIG_EINVAL and int(stats["flags"]) & 0x01
+            assert len(trig) == 0 and len(win) == 0 and int(stats["n_seeds"]) == 0
+    assert all(len(b.rows(i)[0]) == 0 for i in range(1, len(slices) - 1))
     det.close()
