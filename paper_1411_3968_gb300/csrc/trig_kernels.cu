@@ -1752,33 +1752,38 @@ struct BucketRange {
     }
     __device__ __forceinline__ uint32_t hits(const SliceDesc *d) const
     {
+        if (!CHECK(28, max(b_lo, b_hi), d->n_bkt + 1u)) return 0;
         return __ldg(d->bkt_off + b_hi) - __ldg(d->bkt_off + b_lo);
     }
 };
 
-// A wide slice's tile with more hits than fit (a muon in a full tile): the
-// largest piece of core buckets, halved from the tile's, that fits
-// everywhere in the tile; 0 if not even one bucket does.
-__device__ __forceinline__ uint32_t piece_buckets(const SliceDesc *d, uint32_t c_lo, uint32_t cap)
+// Buckets of a tile's core: the slice's last tile may end before its width.
+__device__ __forceinline__ uint32_t core_buckets(const SliceDesc *d, uint32_t core)
 {
-    const uint32_t m = d->bkt_per_tile;
-    for (uint32_t k = m; k > 1;) {
-        k = (k + 1) / 2;
+    return (core + d->bkt_w - 1u) / d->bkt_w;
+}
+
+// A wide slice's tile with more hits than fit (a muon in a full tile): the
+// largest piece of its core buckets, halved from all of them, that fits
+// everywhere in the core; 0 if not even one bucket does.
+__device__ __forceinline__ uint32_t piece_buckets(const SliceDesc *d, uint32_t c_lo, uint32_t core, uint32_t cap)
+{
+    const uint32_t m = core_buckets(d, core);
+    for (uint32_t k = m;; k = (k + 1) / 2) {
         uint32_t most = 0;
         for (uint32_t j = 0; j < m; j += k) most = max(most, BucketRange(d, c_lo + j, min(k, m - j)).hits(d));
         if (most <= cap) return k;
+        if (k == 1) return 0;
     }
-    return 0;
 }
 
 __device__ __forceinline__ bool stage_buckets(Stager &sg, ItemInfo x, const SliceDesc *d, uint32_t c_lo, uint32_t k,
                                               BatchHeader *hdr)
 {
-    const uint32_t m = d->bkt_per_tile, core = x.core;
+    const uint32_t core = x.core, m = core_buckets(d, core);
     const uint64_t wait_ns = hdr->wait_ns;
     for (uint32_t j = 0; j < m; j += k) {
         const uint32_t kk = min(k, m - j), off = j * d->bkt_w;
-        if (off >= core) break;                                     // past the slice's end
         const BucketRange r(d, c_lo + j, kk);
         const uint32_t n = r.hits(d);
         if (n == 0) continue;
@@ -1848,7 +1853,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
 #ifdef TRIG_PHASE_STATS
             const long long tp0 = clock64();
 #endif
-            uint32_t g = 0, P = 0, mode = kItemSkip, lo_t = 0, span = 0;
+            uint32_t g = 0, P = 0, mode = kItemSkip, lo_t = 0, span = 0, core = 0;
             uint32_t ra[R], rl[R];                  // hit indices are below 2^32 - 16
             uint32_t tot = 0, rlo = 0, c_lo = 0, piece = 0;
             bool wide = false;
@@ -1863,6 +1868,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 g = item - d->item0;
                 P = d->n_pmt;
                 wide = d->wide != 0;
+                core = (uint32_t)min(d->tile_w, d->slice_ns - (int64_t)g * d->tile_w);
                 if (wide) {
                     // one contiguous range of the bucketed copy: the core
                     // buckets and hh buckets of halo on each side
@@ -1873,7 +1879,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                     if (!bad) {
                         rlo = __ldg(d->bkt_off + r.b_lo);
                         tot = r.hits(d);
-                        if (tot > (uint32_t)CAP) piece = piece_buckets(d, c_lo, CAP);
+                        if (tot > (uint32_t)CAP) piece = piece_buckets(d, c_lo, core, CAP);
                     }
                 } else {
                     // the PMTs' runs [lb(B_g - H), lb(B_{g+1} + H)), P <= 32 R
@@ -1921,8 +1927,6 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 if (sg.wait_free(hdr, wait_ns)) sg.hand_over(ItemInfo{-1}, 0);
                 break;
             }
-            const int64_t W = d->tile_w, Bg = d->t0 + (int64_t)g * W;
-            const uint32_t core = (uint32_t)(min(Bg + W, d->t0 + d->slice_ns) - Bg);
             const ItemInfo x{(int32_t)item, s, g, 0, rlo, mode, 0, core, lo_t, span};
             if (mode == kItemPiece && wide) {
                 if (!stage_buckets(sg, x, d, c_lo, piece, hdr)) break;

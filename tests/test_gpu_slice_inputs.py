@@ -207,3 +207,45 @@ def test_offsets_of_empty_pmts_are_checked(pkg, params, n_pmt):
             assert len(trig) == 0 and len(win) == 0 and int(stats["n_seeds"]) == 0
     assert all(len(b.rows(i)[0]) == 0 for i in range(1, len(slices) - 1))
     det.close()
+
+
+# at 20 hits a microsecond a tile of 2048 hits filled to 90 % has a core of 57
+# buckets of 1500 ns, and the seventh tile of these slices one of 1 to 26
+LAST_TILE_SLICES = tuple(6 * 57 * 1500 + 1500 * k for k in (1, 2, 7, 26))
+
+
+def _last_tile_burst(n_pmt, slice_ns, cluster_ns):
+    rng = np.random.Generator(np.random.PCG64(n_pmt + slice_ns))
+    t0 = 1_000_000
+    hits, _ = _hits(rng, (slice_ns + 6000) // 50, n_pmt, t0 - 3000, t0 + slice_ns + 3000)
+    hits["t"][:1890] = t0 + slice_ns - cluster_ns + rng.integers(0, cluster_ns, 1890)
+    return _stream(hits, n_pmt)
+
+
+@pytest.mark.parametrize("n_pmt", [129, 336])
+@pytest.mark.parametrize("slice_ns", LAST_TILE_SLICES)
+@pytest.mark.parametrize("cluster_ns", [1_200, 8_000])
+def test_burst_in_a_short_last_tile(pkg, params, n_pmt, slice_ns, cluster_ns):
+    """The last tile of a wide slice is overfull and its core far shorter than
+    the others': its pieces end with the slice."""
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    par = dict(params, slice_ns=slice_ns)
+    t0 = 1_000_000
+    xyz, floor = _detector(n_pmt)
+    hits, off = _last_tile_burst(n_pmt, slice_ns, cluster_ns)
+    det = pkg.Detector(xyz, floor, par)
+    b = DeviceBatch([SliceIn(det, t0, hits, off)])
+    ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+    old = pkg.trig_get_tile_config()
+    for shape in ((2048, 16, 90), (2048, 16, 60), (1024, 4, 90)):
+        pkg.trig_set_tile_config(*shape)
+        try:
+            b.run()
+            res, = b.results()
+        finally:
+            pkg.trig_set_tile_config(*old)
+        if shape[0] == 1024:        # more than 1024 of the burst's hits within 3 us of any of its 1 ns cores
+            assert int(res[0]["status"]) == pkg.TRIG_ECAPACITY and int(res[0]["flags"]) & 0x08
+        else:
+            _assert_same(res, ref, shape)
+    det.close()
