@@ -668,7 +668,8 @@ enum : uint32_t { kItemTile, kItemOverflow, kItemSkip, kItemPiece, kItemEnd };
 // pass); the keys in bucket order (+16 bytes of end keys that the causal
 // count's 16-byte loads may read past the last key); the floor cells, two
 // bits each, whose place the seed list takes; the candidate list (position
-// and charge), whose place the seeds' counts take; the bucket offsets; the
+// and charge), whose place the seeds' counts and the fired seeds' charges by
+// position take; the bucket offsets; the
 // mask of fired positions; the extended builds' (EXT) charges in key order
 // and, for detectors above 128 PMTs, a 4096-bit PMT set per warp; the dt rows
 // (kDtRow bytes each, 256-byte aligned) when the detector's table fits
@@ -711,6 +712,8 @@ struct TileCtx {
     __device__ __forceinline__ uint32_t *seeds() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCell); }
     __device__ __forceinline__ uint32_t *cand() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCand); }
     __device__ __forceinline__ uint16_t *counts() const { return reinterpret_cast<uint16_t *>(g_tile_smem + L::oCand); }
+    // a fired seed's charge at its position (the extended builds have every key's)
+    __device__ __forceinline__ uint16_t *fired_charge() const { return EXT ? chg() : counts() + CAP; }
     __device__ __forceinline__ uint32_t *cnt() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCnt); }
     __device__ __forceinline__ uint32_t *cells() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oCell); }
     __device__ __forceinline__ uint32_t *mask() const { return reinterpret_cast<uint32_t *>(g_tile_smem + L::oMask); }
@@ -1071,10 +1074,10 @@ __device__ __forceinline__ void count_seeds(const C &cx, uint32_t n, uint32_t ns
     const uint32_t rounds = (ns + NG - 1) / NG;
     for (uint32_t r = 0; r < rounds; ++r) {
         const uint32_t k = r * NG + gid;
-        uint32_t c = 0, pos = 0;
+        uint32_t c = 0, e = 0;
         if (k < ns) {
-            pos = seeds[k] & 0xffffu;
-            const uint32_t ks = pk[pos];
+            e = seeds[k];
+            const uint32_t ks = pk[e & 0xffffu];
             const uint32_t ts = C::key_t(ks), ps = C::key_p(ks);
             uint32_t j0, j1;
             seed_range<NB>(cx, ts, ps, bsh, j0, j1);
@@ -1099,7 +1102,11 @@ __device__ __forceinline__ void count_seeds(const C &cx, uint32_t n, uint32_t ns
         for (uint32_t off = G >> 1; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
         if (k < ns && gl == 0) {
             cx.counts()[k] = (uint16_t)c;
-            if (c >= threshold) atomicOr(&cx.mask()[pos >> 5], 1u << (pos & 31u));
+            if (c >= threshold) {
+                const uint32_t pos = e & 0xffffu;
+                if (!EXT) cx.fired_charge()[pos] = (uint16_t)(e >> 16);
+                atomicOr(&cx.mask()[pos >> 5], 1u << (pos & 31u));
+            }
         }
     }
 }
@@ -1443,12 +1450,11 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
             if (j == pos || !((mask[j >> 5] >> (j & 31u)) & 1u)) continue;
             const uint32_t kj = pk[j];
             bool less = kj < ks, more = kj > ks;
-            if (kj == ks)                        // the same time and PMT: by charge (kept in the list)
-                for (uint32_t y = 0; y < ns; ++y)
-                    if ((seeds[y] & 0xffffu) == j) {
-                        less = (seeds[y] >> 16) < (e >> 16);
-                        more = (seeds[y] >> 16) > (e >> 16);
-                    }
+            if (kj == ks) {                      // the same time and PMT: by charge
+                const uint32_t qj = cx.fired_charge()[j];
+                less = qj < (e >> 16);
+                more = qj > (e >> 16);
+            }
             o += j > pos && less ? 1u : 0u;
             o -= j < pos && more ? 1u : 0u;
         }

@@ -227,3 +227,51 @@ def test_own_shape_of_dense_arrays(pkg, params, slice_ns, n):
     src = _OWN_SHAPE.format(path=sys.path, par=dict(params), slice_ns=slice_ns, n=n)
     r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("shape", [(4096, 8, 90), (2048, 16, 90)])
+@pytest.mark.parametrize("n_pmt,rule", [(84, {}), (129, {}), (84, dict(count_distinct_pmts=1, threshold=1)),
+                                        (84, dict(l0_hits=2, l0_window_ns=1000, l0_distinct_pmts=1, threshold=1))])
+def test_tiles_of_equal_records(pkg, params, shape, n_pmt, rule):
+    """Nearly a tile of hits at one time on one PMT (some charges equal too),
+    and at one time and the next on the floor's other PMTs: every seed's place
+    among its equals, in a time that grows with their square (12 ms for 3800
+    of them) and not with their cube (0.75 s for 1750)."""
+    import torch
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(shape[0] + n_pmt))
+    par = dict(params, slice_ns=300_000, **rule)
+    t0 = 1_000_000
+    xyz, floor = _detector(n_pmt)
+    hits, _ = _hits(rng, shape[0] - 600, n_pmt, t0 + 100_000, t0 + 100_001)
+    hits["pmt"] = 7
+    hits["charge"] = rng.integers(300, 900, len(hits))
+    hits["t"][::9] += 1
+    hits["pmt"][::9] = 6 + 2 * rng.integers(0, 2, len(hits[::9]))
+    other, _ = _hits(rng, 600, n_pmt, t0 - 3000, t0 + par["slice_ns"] + 3000)
+    hits = np.sort(np.concatenate([hits, other]), order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    det = pkg.Detector(xyz, floor, par)
+    b = DeviceBatch([SliceIn(det, t0, hits, off)])
+    old = pkg.trig_get_tile_config()
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    try:
+        pkg.trig_set_tile_config(*shape)
+        b.run()
+        torch.cuda.synchronize()
+        ev[0].record()
+        b.run()
+        ev[1].record()
+        (stats, trig, win), = b.results()
+    finally:
+        pkg.trig_set_tile_config(*old)
+    ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+    assert int(stats["status"]) == 0
+    assert int(stats["n_seeds"]) == len(ref.seeds) and len(trig) == len(ref.triggers) and len(win) == len(ref.windows)
+    for f in ("t", "pmt", "charge", "count"):
+        assert np.array_equal(trig[f], ref.triggers[f]), f
+    for f in ("lo", "hi", "n_hits", "n_triggers"):
+        assert np.array_equal(win[f], ref.windows[f]), f
+    assert ev[0].elapsed_time(ev[1]) < 100.0
+    det.close()
