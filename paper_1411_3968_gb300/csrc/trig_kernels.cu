@@ -956,11 +956,18 @@ __device__ __noinline__ bool level0_pass(const CTX &cx, uint32_t n, uint32_t i, 
                N;
     };
     if (busy(ts)) return true;
-    // the windows that start at an earlier hit
+    // the windows that start at an earlier hit; those of a bucket are looked at
+    // one by one only if all the buckets they may touch hold N hits together
+    // (else hits that share a few buckets, as under a coarse clock, would each
+    // be counted against all of them)
     const uint32_t lo = ts >= TW ? ts - TW + 1u : 0u;
-    for (uint32_t j = cnt[lo >> bsh], je = cnt[b0]; j < je; ++j) {
-        const uint32_t tj = CTX::key_t(pk[j]);
-        if (tj >= lo && tj < ts && busy(tj)) return true;
+    for (uint32_t b = lo >> bsh; b < b0; ++b) {
+        const uint32_t j0 = cnt[b], j1 = cnt[b + 1];
+        if (j0 == j1 || cnt[bucket_of<NB>(((b + 1u) << bsh) - 1u + TW, bsh) + 1u] - j0 < N) continue;
+        for (uint32_t j = j0; j < j1; ++j) {
+            const uint32_t tj = CTX::key_t(pk[j]);
+            if (tj >= lo && tj < ts && busy(tj)) return true;
+        }
     }
     return false;
 }

@@ -275,3 +275,46 @@ def test_tiles_of_equal_records(pkg, params, shape, n_pmt, rule):
         assert np.array_equal(win[f], ref.windows[f]), f
     assert ev[0].elapsed_time(ev[1]) < 100.0
     det.close()
+
+
+@pytest.mark.parametrize("n_pmt", [84, 129])
+@pytest.mark.parametrize("l0_hits", [2600, 1900, 1300, 40])
+def test_level0_over_crowded_buckets(pkg, params, n_pmt, l0_hits):
+    """Three clusters of 1200 hits in 24 ns, 700 ns apart, under a level 0 that
+    none, some or all of their hits pass: each seed's windows are searched in
+    a time that does not grow with the clusters' square."""
+    import torch
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(l0_hits + n_pmt))
+    par = dict(params, slice_ns=300_000, l0_hits=l0_hits, l0_window_ns=1000, q_seed_adc=0, threshold=1)
+    t0 = 1_000_000
+    xyz, floor = _detector(n_pmt)
+    hits, _ = _hits(rng, 3900, n_pmt, t0 - 3000, t0 + par["slice_ns"] + 3000)
+    for k in range(3):
+        hits["t"][1200 * k:1200 * (k + 1)] = t0 + 100_000 + 700 * k + rng.integers(0, 24, 1200)
+    hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    det = pkg.Detector(xyz, floor, par)
+    b = DeviceBatch([SliceIn(det, t0, hits, off)])
+    old = pkg.trig_get_tile_config()
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    try:
+        pkg.trig_set_tile_config(4096, 8, 90)
+        b.run()
+        torch.cuda.synchronize()
+        ev[0].record()
+        b.run()
+        ev[1].record()
+        (stats, trig, win), = b.results()
+    finally:
+        pkg.trig_set_tile_config(*old)
+    ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+    assert int(stats["status"]) == 0
+    assert int(stats["n_seeds"]) == len(ref.seeds) and len(trig) == len(ref.triggers) and len(win) == len(ref.windows)
+    for f in ("t", "pmt", "charge", "count"):
+        assert np.array_equal(trig[f], ref.triggers[f]), f
+    for f in ("lo", "hi", "n_hits", "n_triggers"):
+        assert np.array_equal(win[f], ref.windows[f]), f
+    assert ev[0].elapsed_time(ev[1]) < 50.0
+    det.close()
