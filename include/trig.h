@@ -57,7 +57,9 @@ extern "C" {
 #define TRIG_FLAG_UNSORTED     0x02u  /* a PMT stream is not time-ordered         */
 #define TRIG_FLAG_OUT_OF_RANGE 0x04u  /* hit outside [t0 - halo, t0 + S + halo)   */
 #define TRIG_FLAG_TILE_FULL    0x08u  /* > tile capacity hits inside one 1 ns core
-                                         plus its halo; results incomplete       */
+                                         plus its halo; results incomplete.  The
+                                         capacity is 4096, less only in shapes
+                                         set or tuned to (2048, 8) or (1024, 4) */
 #define TRIG_FLAG_TRIG_FULL    0x10u  /* more triggers than trig_cap             */
 #define TRIG_FLAG_WIN_FULL     0x20u  /* more windows than win_cap               */
 #define TRIG_FLAG_TIMEOUT      0x40u  /* a bounded device wait gave up            */

@@ -658,10 +658,10 @@ struct ItemInfo {
     uint32_t lo_t;      // start of the core, from the staged range's
     uint32_t span;      // length of the staged range
 };
-// A whole staged tile; one with more hits than fit, left to tile_overflow
-// (wide slices whose single buckets do not fit); nothing to do (bad slice or empty); a staged piece of a
-// tile, and the end of a tile's pieces.
-enum : uint32_t { kItemTile, kItemOverflow, kItemSkip, kItemPiece, kItemEnd };
+// A whole staged tile; nothing to do (bad slice or empty); a staged piece of a
+// tile, and the end of a tile's pieces; a tile put off until the block has no
+// others, for tile_overflow (what was done of its pieces is dropped).
+enum : uint32_t { kItemTile, kItemSkip, kItemPiece, kItemEnd, kItemDefer };
 
 // Shared memory of the tile kernel, in this order: the staging buffer (handed
 // back after its first read, so the next tile's copy overlaps the rest of the
@@ -674,20 +674,28 @@ enum : uint32_t { kItemTile, kItemOverflow, kItemSkip, kItemPiece, kItemEnd };
 // and, for detectors above 128 PMTs, a 4096-bit PMT set per warp; the dt rows
 // (kDtRow bytes each, 256-byte aligned) when the detector's table fits
 // (NARROW); the PMT tables (floor, row maximum of dt).
-template <int CAP, int NC, bool NARROW, bool EXT>
+// CROWD: the layout of crowd_pass, which takes twice the hits in the same
+// memory: no staging buffer (its records, 8 bytes each, lie where the keys and
+// candidates come later), half as many buckets and cells for a hit; the PMT
+// sets and tables stay where they are.
+template <int CAP, int NC, bool NARROW, bool EXT, bool CROWD = false>
 struct TileLayout {
-    static constexpr uint32_t kCells = 16u * CAP;          // floor cells
-    static constexpr int NBK = CAP;                        // time buckets
-    static constexpr size_t kStage = (size_t)CAP * 16;
+    static constexpr int NBK = CROWD ? CAP / 2 : CAP;      // time buckets
+    static constexpr uint32_t kCells = 16u * NBK;          // floor cells
+    static constexpr size_t kStage = CROWD ? 0 : (size_t)CAP * 16;
     static constexpr size_t oPk = kStage;
-    static constexpr size_t oCell = oPk + (size_t)CAP * 4 + 16;
-    static constexpr size_t oCand = oCell + (size_t)CAP * 4;
-    static constexpr size_t oCnt = oCand + (size_t)CAP * 4;
+    static constexpr size_t kLists = (size_t)CAP * 4;      // the cells (or seeds), and the candidates
+    static constexpr size_t oCell = oPk + (size_t)CAP * 4 + 16 + (CROWD ? kLists : 0);
+    static constexpr size_t oCand = CROWD ? oPk + (size_t)CAP * 4 + 16 : oCell + kLists;
+    static constexpr size_t oCnt = oPk + (size_t)CAP * 4 + 16 + 2 * kLists;
     static constexpr size_t oMask = oCnt + (size_t)(NBK + 1) * 4;
-    static_assert(kCells / 4 == (size_t)CAP * 4, "the cells and the seed list share their place");
+    static_assert(kCells / 4 <= kLists, "the cells and the seed list share their place");
     static constexpr size_t oChg = oMask + (size_t)(CAP / 32) * 4;
-    static constexpr size_t oSet = oChg + (EXT ? (size_t)CAP * 2 : 0);
-    static constexpr size_t oDt = (oSet + (EXT && !NARROW ? (size_t)NC / 32 * 512 : 0) + kDtRow - 1) & ~(size_t)(kDtRow - 1);
+    static constexpr size_t oEnd = oChg + (EXT ? (size_t)CAP * 2 : 0);
+    static constexpr size_t tables(size_t set) { return (set + (EXT && !NARROW ? (size_t)NC / 32 * 512 : 0) + kDtRow - 1) & ~(size_t)(kDtRow - 1); }
+    static constexpr size_t oSet = CROWD ? TileLayout<CAP / (CROWD ? 2 : 1), NC, NARROW, EXT, false>::oSet : oEnd;
+    static constexpr size_t oDt = tables(oSet);
+    static_assert(oEnd <= oSet, "fits below what it leaves in place");
     static_assert(oCnt % 16 == 0 && oCell % 16 == 0, "cleared and scanned as 16-byte vectors");
     __host__ __device__ static size_t tab(uint32_t P) { return oDt + (NARROW ? (size_t)P * kDtRow : 0); }
     static size_t bytes(uint32_t P) { return (tab(P) + 2 * (size_t)((P + 7) & ~7u) * 2 + 127) & ~(size_t)127; }
@@ -700,9 +708,9 @@ extern __shared__ __align__(256) unsigned char g_tile_smem[];
 // addresses are recomputed where used instead of living in registers through
 // every phase; only the PMT tables' place depends on the launch.  NARROW: at
 // most kSmemDtMaxPmt PMTs in the batch and every dt table in shared memory.
-template <int CAP, int NC, bool NARROW, bool EXT>
+template <int CAP, int NC, bool NARROW, bool EXT, bool CROWD = false>
 struct TileCtx {
-    using L = TileLayout<CAP, NC, NARROW, EXT>;
+    using L = TileLayout<CAP, NC, NARROW, EXT, CROWD>;
     uint32_t P;             // PMTs of the loaded slice
     uint32_t tab;           // offset of the PMT tables
     uint32_t pp;            // their stride
@@ -759,6 +767,7 @@ template <int NC>
 __device__ __forceinline__ void cons_sync() { named_sync(kBarCons, NC); }
 
 constexpr uint32_t kPkNone = 0xffffffffu;       // "no hit", above every key
+constexpr uint32_t kNoItem = 0xffffffffu;       // end of the list of tiles put off
 
 // Bucket of a time relative to the tile base: t_rel >> bsh, the last of
 // the NB buckets taking everything beyond.
@@ -1156,12 +1165,12 @@ __device__ __forceinline__ void count_seeds(const C &cx, uint32_t n, uint32_t ns
 // 4.43 ms with the search from every hit and an ordered seed list; the
 // 2688-PMT slice 1.22 ms, 2.05 before.
 // The bucket counts, cells and mask are zero on entry and on return.
-template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE>
-__device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *stage, uint32_t n, int64_t tb,
+template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE, bool CROWD = false>
+__device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT, CROWD> &cx, const uint64_t *stage, uint32_t n, int64_t tb,
                              uint32_t span, uint32_t lo_t, uint32_t hi_t, const TrigParams &tp, trig_trigger *out,
                              uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo, uint64_t *release_bar)
 {
-    using C = TileCtx<CAP, NC, NARROW, EXT>;
+    using C = TileCtx<CAP, NC, NARROW, EXT, CROWD>;
     using L = typename C::L;
     constexpr uint32_t NW = NC / 32;
     constexpr int PER = CAP / NC;
@@ -1208,11 +1217,18 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
         key[r] = kPkNone;
         cs[r] = hc[r] = 0;
         if (i < n) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(stage + 2 * i);
-            // t - tb in 32 bits (the staged range spans less than 2^20 ns)
-            const uint32_t tr = min(v.x - (uint32_t)tb, span - 1u), p = v.z & 0xfffu;
+            uint32_t tr, pq;            // time from tb, PMT and charge
+            if (CROWD) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(stage + i);
+                tr = v.x, pq = v.y;
+            } else {
+                const uint4 v = *reinterpret_cast<const uint4 *>(stage + 2 * i);
+                // in 32 bits (the staged range spans less than 2^20 ns)
+                tr = min(v.x - (uint32_t)tb, span - 1u), pq = v.z;
+            }
+            const uint32_t p = pq & 0xfffu;
             key[r] = C::key(tr, p);
-            cs[r] = (v.z & 0xffff0000u) | atomicAdd(&cnt[tr >> bsh], 1u);
+            cs[r] = (pq & 0xffff0000u) | atomicAdd(&cnt[tr >> bsh], 1u);
             const uint32_t h = (fl[p] * fstep + (tr >> csh)) & (M - 1u), bit = 1u << (2u * (h & 15u));
             hc[r] = h;
             if (atomicOr(&cells[h >> 4], bit) & bit) atomicOr(&cells[h >> 4], bit << 1);
@@ -1500,6 +1516,7 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
     {
         uint4 *z = reinterpret_cast<uint4 *>(cnt);
         uint4 *y = reinterpret_cast<uint4 *>(cells);
+        static_assert(M / 16 == NB, "as many words of cells as of bucket counts");
         for (uint32_t i = tid; i < NB / 4; i += NC) z[i] = y[i] = make_uint4(0, 0, 0, 0);
         for (uint32_t i = tid; i < (uint32_t)CAP / 32; i += NC) mask[i] = 0;
     }
@@ -1513,13 +1530,91 @@ __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT> &cx, const uint64_t *
     return co;
 }
 
-// Last resort of the wide slices (other tiles are split by the stager): a
-// single bucket with its halo holds more than CAP hits.  Split
-// its core in halves until each piece fits; pieces are staged with plain
-// loads after per-PMT binary searches.  A 1 ns core that still does not
-// fit is reported (TRIG_FLAG_TILE_FULL) and skipped.
-template <int CAP, int NC, class PASS>
-__device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint32_t g, uint32_t *red, int64_t *stk)
+// What a block's shared memory holds for crowd_pass: the library's own tiles
+// of 2048 hits take pieces of up to 4096 (the shape untuned detectors always
+// had room for); other shapes have none.
+template <int CAP, int NC>
+constexpr uint32_t kCrowdCap = CAP == 2048 && NC == 512 ? 2u * CAP : CAP;
+
+// A piece of core_ns with n > cap hits is left to crowd_pass if it fits there
+// and halving it would not help much: nearly all of its hits are halo.
+__device__ __forceinline__ bool crowded(uint64_t n, uint32_t core_ns, uint32_t H, uint32_t crowd_cap)
+{
+    return n <= crowd_cap && (core_ns == 1 || core_ns <= H / 4u);
+}
+
+// A piece [lo, hi) of a core whose hits, halos included, do not fit in a tile
+// and whose core cannot usefully be split further: a burst so dense that the
+// halos alone nearly fill a tile.  The tile pass on a layout for twice the
+// hits, over the whole of the block's memory (the stager's buffer too: the
+// stager is done).  The hits of [lo - H, hi + H), at most
+// 2 CAP, are collected with plain loads after per-PMT searches.
+// 18 k hits of 84 PMTs in 30 us take 2.9 ms, 3.9 in 4096-hit tiles; 2048-hit
+// tiles without it refused them.
+// Its fired seeds go to the merged rank `at` of the slice's staging (at_c0: to
+// that of the first core hit, `at` being the first collected hit's).
+template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE>
+__device__ CoreOut crowd_pass(const TileCtx<CAP, NC, NARROW, EXT> &host, const SliceDesc &d, int64_t lo, int64_t hi,
+                              const TrigParams &tp, uint32_t at, bool at_c0, uint32_t rank_lo)
+{
+    using C = TileCtx<2 * CAP, NC, NARROW, EXT, true>;
+    using L = typename C::L;
+    using H = TileLayout<CAP, NC, NARROW, EXT>;
+    constexpr uint32_t NW = NC / 32, kCap = 2 * CAP;
+    __shared__ uint32_t s_n;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, P = d.n_pmt;
+    C cx;
+    cx.P = host.P;
+    cx.tab = host.tab;
+    cx.pp = host.pp;
+    cx.dt_g = host.dt_g;
+    auto clear = [&](size_t from, size_t to) {
+        uint32_t *w = reinterpret_cast<uint32_t *>(g_tile_smem);
+        for (uint32_t i = (uint32_t)from / 4 + tid; i < (uint32_t)to / 4; i += NC) w[i] = 0;
+    };
+    const int64_t tb = lo - (int64_t)tp.H, te = hi + (int64_t)tp.H;
+    if (tid == 0) s_n = 0;
+    clear(L::oCell, L::oChg);
+    cons_sync<NC>();
+    uint2 *rec = reinterpret_cast<uint2 *>(cx.stage());
+    for (uint32_t p0 = warp * 32; p0 < P; p0 += NW * 32) {
+        uint64_t a = 0;
+        uint32_t len = 0;
+        if (p0 + lane < P) {
+            const uint64_t ep = d.pmt_off[p0 + lane + 1];
+            a = lb_time(d.hits, d.pmt_off[p0 + lane], ep, tb);
+            len = (uint32_t)(lb_time(d.hits, a, ep, te) - a);
+        }
+        const uint32_t incl = warp_incl_scan(len);
+        uint32_t to = 0;
+        if (lane == 31) to = atomicAdd(&s_n, incl);
+        to = __shfl_sync(0xffffffffu, to, 31) + incl - len;
+        for (uint32_t q = 0; q < 32; ++q) {
+            const uint64_t qa = __shfl_sync(0xffffffffu, a, q);
+            const uint32_t ql = __shfl_sync(0xffffffffu, len, q), qd = __shfl_sync(0xffffffffu, to, q);
+            for (uint32_t e = lane; e < ql; e += 32) {
+                const trig_hit h = load_hit(d.hits + qa + e);
+                if (qd + e < kCap) rec[qd + e] = make_uint2((uint32_t)(h.t_ns - tb), h.pmt | (uint32_t)h.charge << 16);
+            }
+        }
+    }
+    cons_sync<NC>();
+    const CoreOut co = tile_pass<kCap, NC, NARROW, EXT, DENSE, true>(
+        cx, cx.stage(), min(s_n, kCap), tb, (uint32_t)(te - tb), tp.H, tp.H + (uint32_t)(hi - lo), tp, d.stage + at,
+        d.wrank + 2 * (size_t)at, at_c0, rank_lo, (int64_t)rank_lo - (int64_t)d.dbg_rank0, nullptr);
+    clear(H::oPk, H::oChg);             // the tile pass's counts, cells and mask
+    cons_sync<NC>();
+    return co;
+}
+
+// Last resort of the tiles that the stager cannot split: a single bucket of a
+// wide slice with its halo holds more than CAP hits, or a piece of a narrow
+// one is crowded.  Split its core in halves until each piece fits; pieces are
+// staged with plain loads after per-PMT binary searches.  A 1 ns core that
+// still does not fit, nor in crowd_pass, is reported (TRIG_FLAG_TILE_FULL) and
+// skipped.
+template <int CAP, int NC, class PASS, class CROWD>
+__device__ void tile_overflow(PASS pass, CROWD crowd, uint64_t *buf, const SliceDesc &d, uint32_t g, uint32_t *red, int64_t *stk)
 {
     constexpr uint32_t NW = NC / 32;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
@@ -1580,7 +1675,8 @@ __device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint
             red[2] = T > 0xffffffffull ? 0xffffffffu : (uint32_t)T;
             red[3] = (uint32_t)R;
             red[7] = depth - 1;                      // pop
-            if (T > (uint64_t)CAP) {
+            red[1] = T > (uint64_t)CAP && crowded(T, (uint32_t)(hi - lo), H, kCrowdCap<CAP, NC>);
+            if (T > (uint64_t)CAP && !red[1]) {
                 if (hi - lo > 1 && depth + 1 < 64) {
                     int64_t mid = lo + (hi - lo) / 2;
                     stk[2 * (depth - 1)] = mid;          // right half below ...
@@ -1594,9 +1690,18 @@ __device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint
             }
         }
         cons_sync<NC>();
-        const uint32_t total = red[2];
+        const uint32_t total = red[2], rank_lo = red[3];
+        if (red[1]) {
+            const uint32_t fired0 = red[5];
+            const CoreOut co = crowd(lo, hi, tile_rank + fired0, false, rank_lo);
+            if (tid == 0) {
+                red[5] = fired0 + co.n_fired;
+                red[6] += co.n_seeds;
+            }
+            cons_sync<NC>();
+            continue;
+        }
         if (total > (uint32_t)CAP) continue;         // split (or skipped)
-        const uint32_t rank_lo = red[3];
         // stage the piece: PMTs in order, warps take groups of 32 PMTs
         uint32_t dst = 0;
         for (uint32_t p0 = 0; p0 < P; p0 += 32) {
@@ -1630,7 +1735,7 @@ __device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint
         const uint32_t fired0 = red[5];
         CoreOut co = pass(buf, total, tb, span, H, H + (uint32_t)(hi - lo), d.stage + tile_rank + fired0,
                           d.wrank + 2 * (size_t)(tile_rank + fired0), false, rank_lo,
-                          (int64_t)rank_lo - (int64_t)d.dbg_rank0, nullptr);
+                          (int64_t)rank_lo - (int64_t)d.dbg_rank0);
         if (tid == 0) {
             red[5] = fired0 + co.n_fired;
             red[6] += co.n_seeds;
@@ -1643,6 +1748,53 @@ __device__ void tile_overflow(PASS pass, uint64_t *buf, const SliceDesc &d, uint
         atomicAdd(reinterpret_cast<unsigned long long *>(&d.stats->n_seeds), (unsigned long long)red[6]);
     }
     cons_sync<NC>();
+}
+
+// A tile put off (k_tile).  Where its code stands decides how many of the tile
+// pass's registers it costs in builds of 56 a thread: in the extended ones it
+// is inlined after the loop over the tiles, with crowd_pass a call (16 slices
+// with events 2.01 ms, 2.05 all inlined, 2.08 all a call, 1.99 without any of
+// it), in the default ones one call (a 320 k-hit slice 31.4, 32.4, 31.4, 31.6 us;
+// 64 slices 4.79, 4.76, 4.79, 4.73 ms).
+template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE>
+__device__ __noinline__ void crowd_call(uint32_t pmts, uint32_t tab, uint32_t pp, const uint16_t *dt_g, const SliceDesc *d, int64_t lo,
+                                        int64_t hi, const TrigParams *tp, uint32_t at, bool at_c0, uint32_t rank_lo, CoreOut *res)
+{
+    TileCtx<CAP, NC, NARROW, EXT> cx;
+    cx.P = pmts, cx.tab = tab, cx.pp = pp, cx.dt_g = dt_g;
+    const CoreOut co = crowd_pass<CAP, NC, NARROW, EXT, DENSE>(cx, *d, lo, hi, *tp, at, at_c0, rank_lo);
+    if (threadIdx.x == 0) *res = co;
+    cons_sync<NC>();
+}
+
+template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE>
+__device__ __forceinline__ void put_off_tile(TileCtx<CAP, NC, NARROW, EXT> &cx, const SliceDesc &d, uint32_t g, const TrigParams &tp)
+{
+    __shared__ __align__(16) uint32_t red[64 + 64];
+    __shared__ int64_t stk[128];
+    __shared__ CoreOut res;
+    auto pass = [&](const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span, uint32_t lo_t, uint32_t hi_t, trig_trigger *out,
+                    uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo) {
+        return tile_pass<CAP, NC, NARROW, EXT, DENSE>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0, rank_base,
+                                                      dbg_rank_lo, nullptr);
+    };
+    auto crowd = [&](int64_t lo, int64_t hi, uint32_t at, bool at_c0, uint32_t rank_lo) {
+        if constexpr (kCrowdCap<CAP, NC> == CAP) return CoreOut{};
+        else if constexpr (EXT) {
+            crowd_call<CAP, NC, NARROW, EXT, DENSE>(cx.P, cx.tab, cx.pp, cx.dt_g, &d, lo, hi, &tp, at, at_c0, rank_lo, &res);
+            return res;
+        } else return crowd_pass<CAP, NC, NARROW, EXT, DENSE>(cx, d, lo, hi, tp, at, at_c0, rank_lo);
+    };
+    tile_overflow<CAP, NC>(pass, crowd, cx.stage(), d, g, red, stk);
+}
+
+template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE>
+__device__ __noinline__ void put_off_call(uint32_t pmts, uint32_t tab, uint32_t pp, const uint16_t *dt_g, const SliceDesc *d, uint32_t g,
+                                          const TrigParams *tp)
+{
+    TileCtx<CAP, NC, NARROW, EXT> cx;
+    cx.P = pmts, cx.tab = tab, cx.pp = pp, cx.dt_g = dt_g;
+    put_off_tile<CAP, NC, NARROW, EXT, DENSE>(cx, *d, g, *tp);
 }
 
 // The stager's side of the hand-over of the one staging buffer.
@@ -1701,10 +1853,10 @@ constexpr uint32_t kMaxPieces = 24;         // open halves of a core below 2^20 
 // A tile of a narrow slice with more hits than fit (a burst): its core is
 // halved until each piece fits with its halo; the pieces' runs are found
 // inside the tile's (runs: start and end of each PMT's, in shared memory).  A
-// 1 ns piece that still does not fit is reported and left out.  Returns
-// false when a wait ran out.
-__device__ __forceinline__ bool stage_pieces(Stager &sg, ItemInfo x, uint32_t cap, const SliceDesc *d, const uint2 *runs,
-                                          uint2 *pieces, BatchHeader *hdr)
+// tile with a crowded piece is put off; a 1 ns piece that fits nowhere is
+// reported and left out.  Returns false when a wait ran out.
+__device__ __forceinline__ bool stage_pieces(Stager &sg, ItemInfo x, uint32_t cap, uint32_t crowd_cap, const SliceDesc *d,
+                                          const uint2 *runs, uint2 *pieces, BatchHeader *hdr)
 {
     const uint32_t lane = lane_id(), H = d->halo, rlo = x.rank_lo;
     const uint64_t wait_ns = hdr->wait_ns;
@@ -1728,7 +1880,12 @@ __device__ __forceinline__ bool stage_pieces(Stager &sg, ItemInfo x, uint32_t ca
         n = __reduce_add_sync(0xffffffffu, n);
         rank = __reduce_add_sync(0xffffffffu, rank);
         if (n > cap) {
-            if (hi - lo > 1 && depth + 2 <= kMaxPieces) {
+            if (cap < crowd_cap && crowded(n, hi - lo, H, crowd_cap)) {
+                if (!sg.wait_free(hdr, wait_ns)) return false;
+                x.mode = kItemDefer;
+                sg.hand_over(x, 0);
+                return true;
+            } else if (hi - lo > 1 && depth + 2 <= kMaxPieces) {
                 const uint32_t mid = lo + (hi - lo) / 2;
                 if (lane == 0) {
                     pieces[depth] = make_uint2(mid, hi);            // right half below,
@@ -1824,8 +1981,6 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     using L = typename C::L;
     __shared__ uint64_t full_bar, empty_bar;
     __shared__ ItemInfo info;
-    __shared__ __align__(16) uint32_t red[64 + 64];
-    __shared__ int64_t stk[128];
     __shared__ uint2 pieces[kMaxPieces], runs[32 * kStageRuns];
 
     C cx;
@@ -1925,7 +2080,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
                 }
                 mode = bad || tot == 0                ? kItemSkip
                        : tot <= (uint32_t)CAP    ? kItemTile
-                       : wide && piece == 0      ? kItemOverflow
+                       : wide && piece == 0      ? kItemDefer
                                                  : kItemPiece;
             }
             uint32_t next = 0;
@@ -1947,7 +2102,7 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
 #pragma unroll
                 for (int r = 0; r < R; ++r) runs[r * 32 + lane] = make_uint2(ra[r], ra[r] + rl[r]);
                 __syncwarp();
-                if (!stage_pieces(sg, x, CAP, d, runs, pieces, hdr)) break;
+                if (!stage_pieces(sg, x, CAP, kCrowdCap<CAP, NC>, d, runs, pieces, hdr)) break;
             } else {
                 if (!sg.wait_free(hdr, wait_ns)) break;
                 sg.hand_over(x, mode == kItemTile ? tot : 0u);
@@ -2030,16 +2185,15 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
     // blocks take the first items in turn
     if (n_items) load_slice(desc[find_slice_by_item(desc, n_slices, min(blockIdx.x, n_items - 1u))]);
     // the tile whose pieces are coming: its fired seeds so far, where they
-    // start, and whether a piece was seen (thread 0 writes after a pass; the
-    // next tile's barrier publishes it)
-    __shared__ uint32_t pc[3];
-    if (tid < 3) pc[tid] = 0;
-    auto pass = [&](const uint64_t *stage, uint32_t n, int64_t tb, uint32_t span, uint32_t lo_t, uint32_t hi_t,
-                    trig_trigger *out, uint32_t *wr, bool out_at_c0, uint32_t rank_base, int64_t dbg_rank_lo,
-                    uint64_t *release_bar) {
-        return tile_pass<CAP, NC, SMEM_DT, EXT, DENSE>(cx, stage, n, tb, span, lo_t, hi_t, tp, out, wr, out_at_c0, rank_base,
-                                                       dbg_rank_lo, release_bar);
-    };
+    // start, whether a piece was seen, and its seeds (thread 0 writes after a
+    // pass; the next tile's barrier publishes it)
+    __shared__ uint32_t pc[4];
+    if (tid < 4) pc[tid] = 0;
+    // the block's tiles that are put off, the last one first: the item before
+    // each stands in its tile_nfired
+    __shared__ uint32_t deferred;
+    if (tid == 0) deferred = kNoItem;
+    bool done = false;
     for (uint32_t it = 0;; ++it) {
         // every thread waits (bounded) for the staged tile; the barrier
         // ANDs their results, so the block never splits on a timeout
@@ -2060,21 +2214,28 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             break;
         }
         const ItemInfo &inf = info;      // stable until this buffer is released
-        if (inf.item < 0) break;
+        if (inf.item < 0) {
+            done = true;
+            break;
+        }
         const SliceDesc &d = desc[inf.slice];
         if (&d != loaded) {
             cons_sync<NC>();
             load_slice(d);
             cons_sync<NC>();
         }
-        if (inf.mode == kItemSkip || inf.mode == kItemEnd) {
+        if (inf.mode == kItemSkip || inf.mode == kItemEnd || inf.mode == kItemDefer) {
             if (tid == 0) {
-                d.tile_nfired[inf.g] = pc[0];
-                d.tile_rank[inf.g] = pc[1];
-                pc[0] = pc[1] = pc[2] = 0;
+                if (inf.mode == kItemDefer) {
+                    d.tile_nfired[inf.g] = deferred;
+                    deferred = (uint32_t)inf.item;
+                } else {
+                    d.tile_nfired[inf.g] = pc[0];
+                    d.tile_rank[inf.g] = pc[1];
+                    if (pc[3]) atomicAdd(reinterpret_cast<unsigned long long *>(&d.stats->n_seeds), (unsigned long long)pc[3]);
+                }
+                pc[0] = pc[1] = pc[2] = pc[3] = 0;
             }
-        } else if (inf.mode == kItemOverflow) {
-            tile_overflow<CAP, NC>(pass, cx.stage(), d, inf.g, red, stk);
         } else {
             const uint32_t g = inf.g, n_st = inf.n, rank_lo = inf.rank_lo, span = inf.span, lo_t = inf.lo_t;
             const uint32_t hi_t = lo_t + inf.core;
@@ -2087,18 +2248,20 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
             // read it (inf is not read after that)
             const bool seen = pc[2] != 0;
             const size_t at = seen ? pc[1] + pc[0] : rank_lo;
-            const CoreOut co = pass(cx.stage(), n_st, tb, span, lo_t, hi_t, d.stage + at, d.wrank + 2 * at, !seen, rank_lo,
-                                    (int64_t)rank_lo - sl[2], &empty_bar);
+            const CoreOut co = tile_pass<CAP, NC, SMEM_DT, EXT, DENSE>(cx, cx.stage(), n_st, tb, span, lo_t, hi_t, tp, d.stage + at,
+                                                                       d.wrank + 2 * at, !seen, rank_lo,
+                                                                       (int64_t)rank_lo - sl[2], &empty_bar);
             const uint32_t tile_rank = rank_lo + co.c0;
             if (tid == 0 && CHECK(14, (uint64_t)tile_rank + co.n_fired, d.n_hits + 1) && CHECK(15, g, d.n_tiles)) {
                 if (!piece) {
                     d.tile_nfired[g] = co.n_fired;
                     d.tile_rank[g] = tile_rank;
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&d.stats->n_seeds), (unsigned long long)co.n_seeds);
                 } else {
                     if (!pc[2]) pc[1] = tile_rank, pc[2] = 1;
                     pc[0] += co.n_fired;
+                    pc[3] += co.n_seeds;
                 }
-                atomicAdd(reinterpret_cast<unsigned long long *>(&d.stats->n_seeds), (unsigned long long)co.n_seeds);
             }
             continue;
         }
@@ -2107,6 +2270,17 @@ __global__ void __launch_bounds__(NC + 32, (CAP <= 1024 ? 4 : CAP <= 2048 ? 2 : 
         fence_proxy_async_smem();
         cons_sync<NC>();
         if (tid == 0) mbar_arrive(&empty_bar);
+    }
+    if (!done) return;                   // a wait ran out
+    // the tiles put off: out of the loop above, whose registers they would take
+    for (uint32_t item; (item = deferred) != kNoItem; cons_sync<NC>()) {
+        const SliceDesc &d = desc[find_slice_by_item(desc, n_slices, item)];
+        cons_sync<NC>();                 // every thread has read `deferred`
+        if (&d != loaded) load_slice(d);
+        if (tid == 0) deferred = d.tile_nfired[item - d.item0];
+        cons_sync<NC>();
+        if constexpr (EXT) put_off_tile<CAP, NC, SMEM_DT, EXT, DENSE>(cx, d, item - d.item0, tp);
+        else put_off_call<CAP, NC, SMEM_DT, EXT, DENSE>(cx.P, cx.tab, cx.pp, cx.dt_g, &d, item - d.item0, &tp);
     }
 }
 

@@ -318,3 +318,76 @@ def test_level0_over_crowded_buckets(pkg, params, n_pmt, l0_hits):
         assert np.array_equal(win[f], ref.windows[f]), f
     assert ev[0].elapsed_time(ev[1]) < 50.0
     det.close()
+
+
+def _check_slice(pkg, det, xyz, floor, par, t0, hits, off, events):
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    b = DeviceBatch([SliceIn(det, t0, hits, off)], events=events)
+    old = pkg.trig_get_tile_config()
+    try:
+        pkg.trig_set_tile_config(2048, 16, 90)
+        b.run()
+        (stats, trig, win), = b.results()
+    finally:
+        pkg.trig_set_tile_config(*old)
+    ref = oracle.run(xyz, floor, par, hits, [t0])[0]
+    assert int(stats["status"]) == 0, int(stats["flags"])
+    assert int(stats["n_seeds"]) == len(ref.seeds) and len(trig) == len(ref.triggers) and len(win) == len(ref.windows)
+    for f in ("t", "pmt", "charge", "count"):
+        assert np.array_equal(trig[f], ref.triggers[f]), f
+    for f in ("lo", "hi", "n_hits", "n_triggers"):
+        assert np.array_equal(win[f], ref.windows[f]), f
+    if events:
+        (ev, n_ev, full), = b.event_hits()
+        want = oracle.events(hits, ref.windows)
+        assert not full and n_ev == len(want)
+        for f in ("t", "pmt", "charge"):
+            assert np.array_equal(ev[f], want[f]), f
+
+
+_CROWD_RULES = [{}, dict(seed_rule=1, l0_hits=7, l0_window_ns=1000, threshold=1), dict(count_distinct_pmts=1),
+                dict(l0_hits=9, l0_window_ns=400, l0_distinct_pmts=1)]
+
+
+@pytest.mark.parametrize("n_pmt", [32, 84, 97, 128, 129, 336])
+@pytest.mark.parametrize("slice_ns", [60_000, 1_000_000])
+@pytest.mark.parametrize("rule", range(len(_CROWD_RULES)))
+def test_bursts_whose_halos_crowd_a_tile(pkg, params, n_pmt, slice_ns, rule):
+    """A burst of 0.6 hits/ns, 3600 within the halos of any nanosecond of it:
+    2048-hit tiles take what 4096-hit tiles would.  In the short slice the
+    burst sets the slice's own rate (the builds with a warp per seed)."""
+    rng = np.random.Generator(np.random.PCG64(n_pmt + slice_ns + rule))
+    par = dict(params, slice_ns=slice_ns, **_CROWD_RULES[rule])
+    t0, n, burst = 1_000_000, 12_000, 9_000
+    xyz, floor = _detector(n_pmt)
+    hits, _ = _hits(rng, n, n_pmt, t0 - 3000, t0 + slice_ns + 3000)
+    hits["t"][:burst] = t0 + slice_ns - 20_000 + rng.integers(0, 15_000, burst)
+    hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    det = pkg.Detector(xyz, floor, par)
+    for events in (False, True):
+        _check_slice(pkg, det, xyz, floor, par, t0, hits, off, events)
+    det.close()
+
+
+@pytest.mark.parametrize("n_pmt", [84, 129])
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 3000, 4095, 4096, 4097])
+@pytest.mark.parametrize("where", ["start", "inside", "end"])
+def test_pileups_up_to_two_tiles(pkg, params, n_pmt, n, where):
+    """n hits within 2 ns: up to 4096 they are processed, one more is
+    reported; so too at the slice's first and last nanosecond, with half of
+    them in the halo."""
+    rng = np.random.Generator(np.random.PCG64(n + n_pmt))
+    par = dict(params, slice_ns=300_000)
+    t0 = 1_000_000
+    at = {"start": t0 - 1, "inside": t0 + 100_000, "end": t0 + par["slice_ns"] - 1}[where]
+    xyz, floor = _detector(n_pmt)
+    hits, off = _hits(rng, n, n_pmt, at, at + 2)
+    det = pkg.Detector(xyz, floor, par)
+    if n <= 4096:
+        _check_slice(pkg, det, xyz, floor, par, t0, hits, off, False)
+    else:
+        with pytest.raises(AssertionError, match="8"):
+            _check_slice(pkg, det, xyz, floor, par, t0, hits, off, False)
+    det.close()
