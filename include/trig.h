@@ -442,11 +442,11 @@ int trig_slice_rows(const trig_slice_dev *slice, trig_hit *merged_out, uint32_t 
  * consumer warps per block and target fill (percent of the capacity a tile
  * plus its halos should hold at the slice's mean rate; it sets the tile
  * width).  (cap, warps) must be (4096, 16), (4096, 8), (2048, 16), (2048, 8)
- * or (1024, 4);
- * fill_pct in [10, 95].  Applies to later runs in this process.  Until the
- * first call the library chooses the shape for each batch by its size, and
- * trig_get_tile_config reports the nominal (4096, 16, 60).  Results do not
- * depend on the shape. */
+ * or (1024, 4); fill_pct in [10, 95].  Applies to later runs in this
+ * process.  (4096, 16, 60), which trig_get_tile_config reports until another
+ * shape is set, stands for the library's own choice for each batch by its
+ * size; setting it gives that choice back.  Results do not depend on the
+ * shape. */
 int trig_set_tile_config(uint32_t cap, uint32_t warps, uint32_t fill_pct);
 int trig_get_tile_config(uint32_t *cap, uint32_t *warps, uint32_t *fill_pct);
 

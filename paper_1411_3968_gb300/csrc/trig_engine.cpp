@@ -80,12 +80,13 @@ extern "C" int trig_host_free(void *ptr)
 static std::atomic<uint64_t> g_launches{0};
 extern "C" uint64_t trig_kernel_launch_count(void) { return g_launches.load(); }
 
-// Launch shape of untuned detectors: the caller's (trig_set_tile_config), or,
-// until the first such call, the library's own choice for each batch (spread
-// 1, see spread_tiles).
+// Launch shape of untuned detectors: the caller's (trig_set_tile_config), or
+// the nominal one, which stands for the library's own choice for each batch
+// (spread 1, see spread_tiles) and is what it is reported as, so that a
+// caller who puts back the shape that was reported gets the choice back.
+static constexpr TileConfig kNominalShape{4096, 16, 60};
 static std::mutex g_cfg_mu;
-static TileConfig g_cfg{4096, 16, 60};
-static bool g_cfg_set = false;
+static TileConfig g_cfg = kNominalShape;
 
 extern "C" int trig_set_tile_config(uint32_t cap, uint32_t warps, uint32_t fill_pct)
 {
@@ -94,7 +95,6 @@ extern "C" int trig_set_tile_config(uint32_t cap, uint32_t warps, uint32_t fill_
                                  "(1024,4)}, fill_pct in [10, 95]");
     std::lock_guard<std::mutex> lk(g_cfg_mu);
     g_cfg = TileConfig{cap, warps, fill_pct};
-    g_cfg_set = true;
     return TRIG_OK;
 }
 
@@ -123,7 +123,9 @@ extern "C" int trig_set_device_wait(uint64_t limit_ns, int stall)
 static TileConfig current_cfg()
 {
     std::lock_guard<std::mutex> lk(g_cfg_mu);
-    return g_cfg_set ? g_cfg : kOwnShape;
+    const bool nominal = g_cfg.cap == kNominalShape.cap && g_cfg.warps == kNominalShape.warps &&
+                         g_cfg.fill_pct == kNominalShape.fill_pct;
+    return nominal ? kOwnShape : g_cfg;
 }
 
 static bool tune_cache_lookup(uint32_t n_pmt, TileConfig &out);
@@ -1088,7 +1090,7 @@ extern "C" int trig_detector_tile_config(const trig_detector *det, uint32_t *cap
 {
     if (!det) return fail(TRIG_EINVAL, "NULL detector");
     TileConfig c = det->tuned ? det->tile : current_cfg();
-    if (c.spread) trig_get_tile_config(&c.cap, &c.warps, &c.fill_pct);
+    if (c.spread) c = kNominalShape;
     if (cap) *cap = c.cap;
     if (warps) *warps = c.warps;
     if (fill_pct) *fill_pct = c.fill_pct;
@@ -1134,9 +1136,7 @@ extern "C" int trig_batch_run_noalloc(const trig_slice_dev *slices, uint32_t n_s
     if (rc) return rc;
     if (bytes > cap) {
         // the largest batches only fit with larger tiles and segments
-        TileConfig lean = cfg;
-        if (cfg.spread) trig_get_tile_config(&lean.cap, &lean.warps, &lean.fill_pct);
-        lean.spread = 0;
+        TileConfig lean = cfg.spread ? kNominalShape : cfg;
         lean.lean = 1;
         rc = plan_into(slices, n_slices, (uintptr_t)scratch, lean, hdr, desc, bytes, max_pmt, smem_dt, any_wide, &shape);
         if (rc) return rc;

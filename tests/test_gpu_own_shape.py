@@ -1,0 +1,77 @@
+"""The tile shape that the library chooses by itself: how it is left and given
+back, and where its choice changes."""
+import numpy as np
+import pytest
+
+import oracle
+import workload
+
+pytestmark = pytest.mark.gpu
+
+NOMINAL = (4096, 16, 60)
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+    import paper_1411_3968_gb300 as p
+    from paper_1411_3968_gb300 import build
+    build.build()
+    p.load()
+    torch.cuda.init()
+    return p
+
+
+def _scratch(pkg, det, n_hits, n_slices=1):
+    """Scratch bytes of a batch of such slices (its buffers are only named)."""
+    from paper_1411_3968_gb300 import _lib
+    d = [_lib.slice_dev(det, 4096, 4096, n_hits, 1_000_000, 4096, 1, 4096, 1, 4096) for _ in range(n_slices)]
+    return pkg.trig_batch_scratch_bytes(d)
+
+
+def test_the_reported_shape_gives_the_choice_back(pkg, params):
+    g = workload.km3_tower()
+    det = pkg.Detector(g.xyz_mm, g.floor_id, params)
+    assert pkg.trig_get_tile_config() == NOMINAL
+    for n in (40_000, 3_000_000):
+        own = _scratch(pkg, det, n)
+        pkg.trig_set_tile_config(1024, 4, 40)
+        assert pkg.trig_get_tile_config() == (1024, 4, 40)
+        other = _scratch(pkg, det, n)
+        pkg.trig_set_tile_config(*NOMINAL)
+        assert pkg.trig_get_tile_config() == NOMINAL
+        assert pkg.trig_detector_tile_config(det) == dict(cap=4096, warps=16, fill_pct=60, tuned=False)
+        assert _scratch(pkg, det, n) == own != other
+    # the choice follows the batch: small ones are cut into more tiles a hit
+    assert _scratch(pkg, det, 40_000) > _scratch(pkg, det, 3_000_000) * 40_000 / 3_000_000
+    det.close()
+
+
+@pytest.mark.parametrize("rate,n_slices", [(2e3, 1), (60e3, 3), (300e3, 1)])
+def test_own_shape_gives_the_oracles_results(pkg, params, rate, n_slices):
+    """A short batch, a few uneven slices, and one of more than eight waves of
+    tiles (25 MHz of hits for 200 ms), each after another shape was set and
+    taken back."""
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    g = workload.km3_tower()
+    par = dict(params, slice_ns=200_000_000 if n_slices == 1 else 20_000_000)
+    det = pkg.Detector(g.xyz_mm, g.floor_id, par)
+    slices, refs = [], []
+    for k in range(n_slices):
+        t0 = workload.T_ORIGIN_NS + k * par["slice_ns"]
+        st = workload.gen_stream(g, t0 - 3000, t0 + par["slice_ns"] + 3000, rate / (1 + 2 * k), n_muons=20, seed=6 + k,
+                                 stream=200 + k)
+        slices.append(SliceIn(det, t0, st.hits, st.pmt_off))
+        refs.append(oracle.run(g.xyz_mm, g.floor_id, par, st.hits, [t0])[0])
+    old = pkg.trig_get_tile_config()
+    pkg.trig_set_tile_config(2048, 8, 50)
+    pkg.trig_set_tile_config(*old)
+    b = DeviceBatch(slices)
+    b.run()
+    for (stats, trig, win), ref in zip(b.results(), refs):
+        assert int(stats["status"]) == 0 and int(stats["n_seeds"]) == len(ref.seeds)
+        for f in ("t", "pmt", "charge", "count"):
+            assert np.array_equal(trig[f], ref.triggers[f]), f
+        for f in ("lo", "hi", "n_hits", "n_triggers"):
+            assert np.array_equal(win[f], ref.windows[f]), f
+    det.close()
