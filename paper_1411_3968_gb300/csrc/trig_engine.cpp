@@ -496,19 +496,20 @@ static TileConfig batch_shape(const trig_slice_dev *sl, uint32_t n, const TileCo
     return out;
 }
 
-// Whether every slice's halo hits, at its mean rate, take a quarter of a
-// tile or more (about 106 MHz of merged hits at H = 2414 ns) under the
+// Whether every slice's halo hits, at its mean rate, take two sevenths of a
+// tile or more (585 of 2048: 97 MHz of merged hits at H = 3000 ns) under the
 // default rule.  A larger tile reads fewer halos twice, but only one block
 // fits on an SM.  Time of a 200 ms slice with 2048- and 4096-hit tiles at
-// 90 %: 714 halo hits 1679 and 1471 us, 487 944 and 911, 454 807 and 844,
-// 357 599 and 637, 180 279 and 304.
+// 90 %, by halo hits: 2688 PMTs 484 709 and 719 us, 548 831 and 831, 581 890
+// and 880, 613 972 and 940, 774 1337 and 1185; 2016 PMTs 569 880 and 883, 605
+// 960 and 928; 1344 PMTs 581 898 and 951, 613 975 and 940.
 static bool halo_heavy(const trig_slice_dev *sl, uint32_t n, const TileConfig &cfg)
 {
     for (uint32_t s = 0; s < n; ++s) {
         const trig_detector *det = sl[s].det;
         if (!det || det->par.l0_hits || det->par.seed_rule || det->par.count_distinct_pmts) return false;
         const double span = (double)det->par.slice_ns + 2.0 * (double)det->in_halo;
-        if (2.0 * det->tile_halo * (double)sl[s].n_hits / span < cfg.cap / 4.0) return false;
+        if (2.0 * det->tile_halo * (double)sl[s].n_hits / span < cfg.cap * 2.0 / 7.0) return false;
     }
     return true;
 }

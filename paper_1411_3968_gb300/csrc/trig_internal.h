@@ -164,10 +164,10 @@ struct TileConfig {
     uint32_t spread = 0;    // tiles cut smaller so that a small batch fills the GPU (kOwnShape)
     uint32_t lean = 0;      // the smallest side tables (a batch at the edge of a fixed scratch)
 };
-// The library's own choice: the shape the autotuner ends at for towers and
-// the 2688-PMT array, with two blocks on an SM (4096-hit tiles leave room for
-// one: 15.7 against 20.3 us for 320 k hits, 72 against 83 us for 2.8 M, 1.33
-// against 1.68 ms for 52 M under the distinct count).
+// The library's own choice: the shape the autotuner ends at for towers, with
+// two blocks on an SM (4096-hit tiles leave room for one: 15.7 against 20.3 us
+// for 320 k hits, 72 against 83 us for 2.8 M, 1.33 against 1.68 ms for 52 M
+// under the distinct count); for dense arrays it is kOwnDenseShape.
 constexpr TileConfig kOwnShape{2048, 16, 90, 1};
 // Many tiles of an array so dense that halos crowd the tile (see halo_heavy).
 constexpr TileConfig kOwnDenseShape{4096, 16, 90, 0};

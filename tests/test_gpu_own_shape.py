@@ -75,3 +75,25 @@ def test_own_shape_gives_the_oracles_results(pkg, params, rate, n_slices):
         for f in ("lo", "hi", "n_hits", "n_triggers"):
             assert np.array_equal(win[f], ref.windows[f]), f
     det.close()
+
+
+@pytest.mark.parametrize("n_pmt", [1344, 2688])
+@pytest.mark.parametrize("halo_hits,cap", [(300, 2048), (520, 2048), (575, 2048), (595, 4096), (900, 4096)])
+def test_dense_arrays_take_larger_tiles_from_585_halo_hits(pkg, params, n_pmt, halo_hits, cap):
+    """The rule counts the hits of both halos of H = 3000 ns, as wide as the
+    array's dt allows: of a 200 ms slice, which tiles it is planned with."""
+    k = np.arange(n_pmt)
+    xyz = np.stack([1000 * (k % 6), np.zeros_like(k), 40_000 * (k // 6)], 1).astype(np.int32)
+    par = dict(params, slice_ns=200_000_000)
+    det = pkg.Detector(xyz, (k // 6).astype(np.uint32), par)
+    assert det.halo_ns == 3000
+    n = int(halo_hits * (par["slice_ns"] + 6000) / 6000)
+    own = _scratch(pkg, det, n)
+    try:
+        pkg.trig_set_tile_config(cap, 16, 90)
+        assert _scratch(pkg, det, n) == own
+        pkg.trig_set_tile_config(6144 - cap, 16, 90)
+        assert _scratch(pkg, det, n) != own
+    finally:
+        pkg.trig_set_tile_config(*NOMINAL)
+    det.close()
