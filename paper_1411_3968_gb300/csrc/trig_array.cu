@@ -561,14 +561,15 @@ __global__ void k_acopy(AHeader *h, const ATower *tw)
             const uint64_t gi = g0 + u * nth;
             const uint32_t b = tower_of_hit(tw, nt, gi);
             const uint64_t i = gi - tw[b].hit0;
-            const int4 x = *reinterpret_cast<const int4 *>(tw[b].hits + i);
-            const size_t cell = (size_t)w[u] * pt + tw[b].base + ((uint32_t)x.z & 0xffffu);
+            // (8-byte loads and stores: the buffers are the caller's)
+            const uint2 *in = reinterpret_cast<const uint2 *>(tw[b].hits + i);
+            const uint2 x0 = in[0], x1 = in[1];
+            const size_t cell = (size_t)w[u] * pt + tw[b].base + (x1.x & 0xffffu);
             const uint64_t dst = (uint64_t)h->cell_off[cell] + (i - (uint64_t)h->cell_first[cell]);
-            // (8-byte stores: the buffer is the caller's)
             if (dst < h->hit_cap) {
                 uint2 *o = reinterpret_cast<uint2 *>(h->hits + dst);
-                o[0] = make_uint2((uint32_t)x.x, (uint32_t)x.y);
-                o[1] = make_uint2((uint32_t)x.z, (uint32_t)x.w);
+                o[0] = x0;
+                o[1] = x1;
             }
         }
     }

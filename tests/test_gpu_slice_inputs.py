@@ -249,3 +249,38 @@ def test_burst_in_a_short_last_tile(pkg, params, n_pmt, slice_ns, cluster_ns):
         else:
             _assert_same(res, ref, shape)
     det.close()
+
+
+def test_selection_takes_hits_at_any_8_bytes(pkg, params):
+    """trig_array_select reads hits by their 8-byte members: towers whose hits
+    start 8 bytes past a 16-byte boundary give what aligned ones do."""
+    import torch
+    from paper_1411_3968_gb300 import _lib
+    from paper_1411_3968_gb300.runner import ArrayBatch, SliceIn
+    wl = workload.cfg_towers8()
+    subs = wl.submissions[:3]
+    dets = [pkg.Detector(wl.detectors[s.det_index].xyz_mm, wl.detectors[s.det_index].floor_id, params) for s in subs]
+    arr = pkg.Array(dets, min_towers=1, corr_window_ns=3000, win_half_ns=3000)
+    ab = ArrayBatch(arr, [SliceIn(d, s.t0, s.stream.hits, s.stream.pmt_off) for d, s in zip(dets, subs)])
+    ab.run()
+    want = ab.results()
+    assert int(want[0]["status"]) == 0 and len(want[4]) > 10_000
+    shifted = []
+    for k, (d, s) in enumerate(zip(ab.batch.descs, subs)):
+        nbytes = len(s.stream.hits) * 16
+        buf = torch.empty(nbytes + 24, dtype=torch.uint8, device="cuda")
+        buf[8:8 + nbytes].copy_(ab.batch.hits[k][:nbytes])
+        assert (buf.data_ptr() + 8) % 16 == 8
+        shifted.append((buf, _lib.slice_dev(dets[k], buf.data_ptr() + 8, ab.batch.offs[k].data_ptr(), len(s.stream.hits), s.t0,
+                                            ab.batch.trig[k].data_ptr(), ab.batch.trig_cap[k], ab.batch.win[k].data_ptr(),
+                                            ab.batch.win_cap[k], ab.batch.stats.data_ptr() + k * _lib.STATS_DTYPE.itemsize)))
+    ab.hits.zero_()
+    st = torch.cuda.current_stream()
+    _lib.trig_array_select(arr, [x[1] for x in shifted], ab.out, ab.scratch.data_ptr(), ab.scratch_bytes, st.cuda_stream)
+    got = ab.results()
+    assert got[0] == want[0]
+    for a, b in zip(got[1:], want[1:]):
+        assert np.array_equal(a, b)
+    arr.close()
+    for d in dets:
+        d.close()
