@@ -2643,11 +2643,13 @@ __global__ void __launch_bounds__(kFinThreads, 3) k_final(BatchHeader *__restric
                 fin_window(d, lane == 0 && z.n > 0, z.heads, (inner ? z.t_head : z.t_first) - half, z.t_last + half,
                            inner ? z.r : z.r_first, z.r_last, z.n - (inner ? z.k : 0u));
                 if (lane == 0) {
-                    const uint64_t nw = z.n ? (uint64_t)z.heads + 1u : 0u;
-                    uint32_t f = d.stats->flags | __ldcg(&hdr->err);
-                    if (z.n > d.trig_cap) f |= TRIG_FLAG_TRIG_FULL;
+                    // (a wait that ran out before: the sums are not valid)
+                    const uint32_t err = __ldcg(&hdr->err), nt = err ? 0u : z.n;
+                    const uint64_t nw = nt ? (uint64_t)z.heads + 1u : 0u;
+                    uint32_t f = d.stats->flags | err;
+                    if (nt > d.trig_cap) f |= TRIG_FLAG_TRIG_FULL;
                     if (nw > d.win_cap) f |= TRIG_FLAG_WIN_FULL;
-                    d.stats->n_triggers = z.n;
+                    d.stats->n_triggers = nt;
                     d.stats->n_windows = nw;
                     d.stats->flags = f;
                     d.stats->status = status_of(f);
