@@ -158,7 +158,9 @@ typedef struct {
     uint32_t flags;             /* TRIG_FLAG_* bits                          */
     uint64_t n_hits;            /* hits submitted (owned range and halos)    */
     uint64_t n_seeds;
-    uint64_t n_triggers;        /* may exceed trig_cap (then TRIG_FLAG_TRIG_FULL) */
+    uint64_t n_triggers;        /* may exceed trig_cap (then TRIG_FLAG_TRIG_FULL:
+                                   the first trig_cap are stored; the windows are
+                                   those of all triggers)                         */
     uint64_t n_windows;         /* may exceed win_cap  (then TRIG_FLAG_WIN_FULL)  */
     uint64_t n_events;          /* hits inside the merged windows (event runs
                                    only; may exceed ev_cap, then TRIG_FLAG_EV_FULL) */
@@ -308,8 +310,9 @@ int trig_engine_trace(uint32_t capacity);
 int trig_engine_trace_read(trig_trace_rec *out, uint32_t max, uint32_t *n_out);
 
 /* Bounded device waits.  Every wait of the tile pass (the stager waiting
- * for a free buffer, the consumers waiting for a staged tile) gives up after
- * limit_ns of the GPU's global timer (default 1 s; 0 restores it, at most
+ * for a free buffer, the consumers waiting for a staged tile) and of the
+ * final pass (a block waiting for what comes before its triggers) gives up
+ * after limit_ns of the GPU's global timer (default 1 s; 0 restores it, at most
  * 600 s), sets TRIG_FLAG_TIMEOUT and ends the pass; the batch's slices then
  * report TRIG_ETIMEOUT with no output, and the device stays usable.
  * stall = 1 is a test control: later batches stage no tile, so the first

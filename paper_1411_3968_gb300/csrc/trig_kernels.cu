@@ -451,9 +451,9 @@ __device__ __noinline__ void bounds_special(const SliceDesc *dp, uint64_t li)
 // is its neighbour's and nothing is carried from step to step.  A lane whose
 // hit has its predecessor's PMT and edge count, in order and in range, is
 // done after that comparison; one that passes a tile edge writes its index.
-// Bound by instruction issue (nearly every step of 31 hits has a lane on the
-// edge path; its first store is predicated, the loop behind it rare), then
-// by HBM: the 64 slices of both towers (205 M hits) take 0.86 ms, 1.42 with
+// Bound by the latency of its loads and checks (issue 53 %, DRAM 51 %; nearly
+// every step of 31 hits has a lane on the edge path, whose first store is
+// predicated, the loop behind it rare): the 64 slices of both towers (205 M hits) take 0.91 ms, 1.42 with
 // two edge counts per hit carried along walks of 512 hits (0.95 with a loop
 // over the edges alone); one 320 k-hit slice 8 us, 13 before.  Four blocks an
 // SM instead of three would spill: 254 against 210 us for 52 M hits.
@@ -1155,15 +1155,15 @@ __device__ __forceinline__ void count_seeds(const C &cx, uint32_t n, uint32_t ns
 //  F. the fired seeds to out, in (t, pmt, charge) order: a seed's rank is
 //     the number of fired positions before it, corrected inside its bucket.
 //
-// Bound by the shared-memory pipe (60 % busy) and the latency of the phases'
-// chains of lookups, then by instruction issue (54 %), not by HBM (11 %).  So
+// Bound by the shared-memory pipe (65 % busy) and the latency of the phases'
+// chains of lookups, then by instruction issue (59 %), not by HBM (13 %).  So
 // each phase reads shared memory as seldom as it can: the floor cells leave
 // about one hit in six for phase D's search (a search from every hit took a
 // third of the pass), charges travel with the candidates instead of being
 // scattered with every key, and two lanes share a seed's emission.  The 64
-// slices of both towers (205 M hits, tiles of 2048 at 90 %) take 3.50 ms,
-// 4.43 ms with the search from every hit and an ordered seed list; the
-// 2688-PMT slice 1.22 ms, 2.05 before.
+// slices of both towers (205 M hits, tiles of 2048 at 90 and 95 %) take 3.61
+// ms, 4.43 ms with the search from every hit and an ordered seed list; the
+// 2688-PMT slice 0.96 ms (4096 at 90 %; 1.12 in tiles of 2048), 2.05 before.
 // The bucket counts, cells and mask are zero on entry and on return.
 template <int CAP, int NC, bool NARROW, bool EXT, bool DENSE, bool CROWD = false>
 __device__ CoreOut tile_pass(TileCtx<CAP, NC, NARROW, EXT, CROWD> &cx, const uint64_t *stage, uint32_t n, int64_t tb,
@@ -2476,12 +2476,13 @@ __device__ __forceinline__ void fin_window(const SliceDesc &d, bool have, uint64
 // over the tiles' seeds: a block takes kFinTiles tiles of a slice at a time
 // (in order, by a ticket), reduces their seeds to a FinRun, publishes it,
 // gets the run of everything before from the published ones (decoupled
-// look-back: the tickets' order makes the blocks it waits for running ones;
-// the wait is bounded like the tile pass's), then copies the seeds to the
+// look-back, after Merrill and Garland, "Single-pass Parallel Prefix Scan with
+// Decoupled Look-back", NVIDIA 2016: the tickets' order makes the blocks it
+// waits for running ones; the wait is bounded like the tile pass's), then copies the seeds to the
 // dense list and writes each window from the head that follows it.  One
 // launch where a scan, a copy, a scan, a window pass, a count pass and a
 // status pass were six, each reading what the one before had written: 14 us
-// against 36 behind one 320 k-hit slice, 0.26 ms against 0.44 behind 64
+// against 36 behind one 320 k-hit slice, 0.27 ms against 0.44 behind 64
 // slices of 12 M triggers.  Bound by the latency of its chain (ticket, tile
 // counts, two reads of the seeds around the look-back).
 constexpr uint32_t kFinThreads = 256;
@@ -3224,8 +3225,9 @@ cudaError_t launch_batch(const BatchHeader &hdr, const SliceDesc *desc, BatchHea
     const bool smem_dt = any_smem_dt && max_pmt <= kSmemDtMaxPmt;
     if (any_ext || any_events || rows) {
         // level 0, seed rule 1, distinct count, and every batch that needs
-        // the merged rows (event extraction, row outputs): the builds that
-        // put each tile in full (t, pmt, charge) order
+        // the merged rows (event extraction, row outputs): the extended
+        // builds, which put a tile in full (t, pmt, charge) order for the
+        // rows and for level 0 over different PMTs
         if (cfg.cap == 1024)
             e = smem_dt ? launch_tile<1024, 128, true, true>(d_hdr, d_desc, max_pmt, st)
                         : launch_tile<1024, 128, false, true>(d_hdr, d_desc, max_pmt, st);
