@@ -422,6 +422,13 @@ static double spread_tiles(const trig_slice_dev *sl, uint32_t n, const TileConfi
     return std::max(128.0, std::ceil(hits / (slots * std::max(std::ceil(roomy / slots), 1.0))));
 }
 
+// Target fill of a detector's tiles (percent): its tuned shape's, else the
+// batch's; 95 under the smallest tables, which have the fewest tiles.
+static uint32_t fill_of(const trig_detector *det, const TileConfig &cfg)
+{
+    return cfg.lean > 1 ? 95u : det->tuned ? det->tile.fill_pct : cfg.fill_pct;
+}
+
 // Tile width W (ns): a tile plus its two halos is expected to hold fill% of
 // the tile capacity at the slice's mean rate, and its core at most core_max
 // hits (0: no bound); W >= 256 ns and at most 2^20 tiles per slice.
@@ -429,11 +436,10 @@ static int64_t choose_tile_w(const trig_detector *det, uint64_t n_hits, const Ti
 {
     const double span = (double)det->par.slice_ns + 2.0 * (double)det->in_halo;
     const double rate = n_hits > 0 ? (double)n_hits / span : 1e-9;       // hits per ns
-    const uint32_t fill = det->tuned ? det->tile.fill_pct : cfg.fill_pct;
-    const double target = (double)cfg.cap * fill / 100.0;
+    const double target = (double)cfg.cap * fill_of(det, cfg) / 100.0;
     double w = target / rate - 2.0 * det->tile_halo;
     if (core_max > 0.0 && !det->tuned) w = std::min(w, core_max / rate);
-    const double w_min = std::max(256.0, (double)det->par.slice_ns / (double)kMaxTilesPerSlice + 1.0);
+    const double w_min = std::max(cfg.lean > 1 ? 1024.0 : 256.0, (double)det->par.slice_ns / (double)kMaxTilesPerSlice + 1.0);
     if (w < w_min) w = w_min;
     if (w > (double)det->par.slice_ns) w = (double)det->par.slice_ns;
     // a tile plus its halos spans less than kMaxTileSpan ns
@@ -445,8 +451,8 @@ static int64_t choose_tile_w(const trig_detector *det, uint64_t n_hits, const Ti
 // Bucket grid of a wide slice: buckets of Wb ns from O = t0 - lead * Wb,
 // tiles of m buckets, hh buckets of halo on each side (hh * Wb >= H).  Wb
 // is about H / 2, smaller when a bucket would hold more than an eighth of a
-// tile at the slice's mean rate; m fills a tile with its halos to the
-// target fill.
+// tile at the slice's mean rate (under the smallest tables, an eighth of a
+// tile or 65536 ns); m fills a tile with its halos to the target fill.
 struct WideGrid {
     uint32_t wb, hh, m, lead, nb;
 };
@@ -456,10 +462,9 @@ static WideGrid wide_grid(const trig_detector *det, uint64_t n_hits, const TileC
     const double S = (double)det->par.slice_ns;
     const double span = S + 2.0 * (double)det->in_halo;
     const double rate = n_hits > 0 ? (double)n_hits / span : 1e-9;        // hits per ns
-    const uint32_t fill = det->tuned ? det->tile.fill_pct : cfg.fill_pct;
-    const double target = (double)cfg.cap * fill / 100.0;
+    const double target = (double)cfg.cap * fill_of(det, cfg) / 100.0;
     const uint32_t H = det->tile_halo;
-    double wb = std::max(64.0, std::ceil(H / 2.0));
+    double wb = cfg.lean > 1 ? 65536.0 : std::max(64.0, std::ceil(H / 2.0));
     wb = std::min(wb, std::max(64.0, std::floor(target / 8.0 / rate)));
     wb = std::max(wb, std::ceil(span / (double)(1u << 22)));                 // at most ~4M buckets
     WideGrid g{};
@@ -579,6 +584,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             dense |= (double)x.n_hits / span * (2.0 * det->tile_halo + 1.0) >= kDenseKeys;
         }
         int64_t W = 0;
+        bool edge_in_stage = false;
         if (wide) {
             const WideGrid wg = wide_grid(det, x.n_hits, cfg, core_max);
             if ((uint64_t)(wg.m + 2 * wg.hh) * wg.wb >= (uint64_t)kMaxTileSpan)
@@ -616,8 +622,11 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
             d.edge_org = d.bkt_origin;
             d.n_edges = (d.n_bkt + d.seg_bkt - 1) / d.seg_bkt + 1;
             d.span32 = d.bkt32 && (uint64_t)d.edge_w * d.n_edges < ((uint64_t)1 << 31);
+            // (the edges are done with when the tile pass first writes the
+            // stage: where the tables are to be small, they lie there)
+            edge_in_stage = cfg.lean && (size_t)d.n_edges * P * 4 <= (size_t)x.n_hits * sizeof(trig_trigger);
             d.edge = reinterpret_cast<uint32_t *>(base + off);
-            off += align256((size_t)d.n_edges * P * 4);
+            if (!edge_in_stage) off += align256((size_t)d.n_edges * P * 4);
             d.bkt_off = reinterpret_cast<uint32_t *>(base + off);
             off += align256(((size_t)d.n_bkt + 1) * 4);
             d.tbuf = reinterpret_cast<trig_hit *>(base + off);
@@ -641,6 +650,7 @@ static int plan_into(const trig_slice_dev *sl, uint32_t n, uintptr_t base, const
         d.fin0 = fins;
         fins += std::max(1u, (d.n_tiles + kFinTiles - 1) / kFinTiles);
         d.stage = reinterpret_cast<trig_trigger *>(base + off);
+        if (edge_in_stage) d.edge = reinterpret_cast<uint32_t *>(d.stage);
         off += align256((size_t)x.n_hits * sizeof(trig_trigger));
         d.wrank = reinterpret_cast<uint32_t *>(base + off);
         off += align256((size_t)x.n_hits * 8);
@@ -1135,11 +1145,12 @@ extern "C" int trig_batch_run_noalloc(const trig_slice_dev *slices, uint32_t n_s
     int rc = plan_into(slices, n_slices, (uintptr_t)scratch, cfg, hdr, desc, bytes, max_pmt, smem_dt,
                        any_wide, &shape);
     if (rc) return rc;
-    if (bytes > cap) {
-        // the largest batches only fit with larger tiles and segments
-        TileConfig lean = cfg.spread ? kNominalShape : cfg;
-        lean.lean = 1;
-        rc = plan_into(slices, n_slices, (uintptr_t)scratch, lean, hdr, desc, bytes, max_pmt, smem_dt, any_wide, &shape);
+    // the largest batches only fit with larger tiles and segments, and the
+    // last few of them only with full tiles and coarse buckets
+    for (uint32_t lean = 1; bytes > cap && lean <= 2; ++lean) {
+        TileConfig small = cfg.spread ? kNominalShape : cfg;
+        small.lean = lean;
+        rc = plan_into(slices, n_slices, (uintptr_t)scratch, small, hdr, desc, bytes, max_pmt, smem_dt, any_wide, &shape);
         if (rc) return rc;
     }
     if (bytes > cap) return fail(TRIG_ECAPACITY, "trig_batch_run_noalloc: batch needs more than TRIG_NOALLOC_SCRATCH_BYTES of scratch");

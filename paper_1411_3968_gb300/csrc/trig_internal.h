@@ -162,7 +162,7 @@ struct TileConfig {
     uint32_t warps;
     uint32_t fill_pct;
     uint32_t spread = 0;    // tiles cut smaller so that a small batch fills the GPU (kOwnShape)
-    uint32_t lean = 0;      // the smallest side tables (a batch at the edge of a fixed scratch)
+    uint32_t lean = 0;      // smaller side tables (1), the smallest (2): a batch at the edge of a fixed scratch
 };
 // The library's own choice: the shape the autotuner ends at for towers, with
 // two blocks on an SM (4096-hit tiles leave room for one: 15.7 against 20.3 us

@@ -97,3 +97,40 @@ def test_dense_arrays_take_larger_tiles_from_585_halo_hits(pkg, params, n_pmt, h
     finally:
         pkg.trig_set_tile_config(*NOMINAL)
     det.close()
+
+
+@pytest.mark.parametrize("n_pmt,n_slices,slice_ns,n", [(2688, 16, 5_000_000, 103_952), (2688, 1, 5_000_000, 1_673_664),
+                                                       (4096, 16, 2_000_000, 104_464), (128, 16, 300_000, 123_696),
+                                                       (672, 16, 20_000_000, 101_456)])
+def test_noalloc_takes_what_the_nominal_tables_left_room_for(pkg, params, n_pmt, n_slices, slice_ns, n):
+    """Batches that fill the static scratch to within 1 KB when every slice
+    has tiles of 4096 hits filled to 60 %, with two offsets a PMT, or two
+    counters a bucket: they are taken, and give what trig_batch_run does."""
+    import torch
+    from paper_1411_3968_gb300 import _lib
+    from paper_1411_3968_gb300.runner import DeviceBatch, SliceIn
+    rng = np.random.Generator(np.random.PCG64(n))
+    k = np.arange(n_pmt)
+    xyz = np.stack([1000 * (k % 6), np.zeros_like(k), 40_000 * (k // 6)], 1).astype(np.int32)
+    par = dict(params, slice_ns=slice_ns)
+    det = pkg.Detector(xyz, (k // 6).astype(np.uint32), par)
+    t0 = 1_000_000
+    hits = np.zeros(n, workload.HIT_DTYPE)
+    hits["t"] = t0 - 3000 + rng.integers(0, slice_ns + 6000, n)
+    hits["pmt"] = rng.integers(0, n_pmt, n)
+    hits["charge"] = rng.integers(1, 320, n)
+    hits = np.sort(hits, order=["pmt", "t", "charge"], kind="stable")
+    off = np.zeros(n_pmt + 1, np.uint64)
+    np.cumsum(np.bincount(hits["pmt"], minlength=n_pmt), out=off[1:])
+    b = DeviceBatch([SliceIn(det, t0, hits, off)] * n_slices)
+    b.run()
+    want = b.results()
+    assert all(int(w[0]["status"]) == 0 for w in want) and len(want[0][1]) > 100
+    for t in b.trig + b.win:
+        t.zero_()
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    _lib.trig_batch_run_noalloc(b.descs, st.cuda_stream)
+    for (s1, t1, w1), (s0, t0_, w0) in zip(b.results(), want):
+        assert s1 == s0 and np.array_equal(t1, t0_) and np.array_equal(w1, w0)
+    det.close()
